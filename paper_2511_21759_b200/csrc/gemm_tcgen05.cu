@@ -627,6 +627,12 @@ static int target_ctas() {
     return v;
 }
 
+int gemm_whole_splits(int splits, int nkb) {
+    if (splits < 1) splits = 1;
+    while (splits > 1 && ((nkb + splits - 1) / splits) * (splits - 1) >= nkb) --splits;
+    return splits;
+}
+
 int gemm_pick_splits(int M, int N, int K) {
     const int n_tiles = (N + kBM - 1) / kBM;
     const int bn = pick_bn(M, use_pair(M, n_tiles));
@@ -644,15 +650,12 @@ int gemm_pick_splits(int M, int N, int K) {
         }
         int sp = tiles >= big_target ? 1 : big_target / tiles;
         if (sp > nkb / 8) sp = nkb / 8;
-        return sp < 1 ? 1 : sp;
+        return gemm_whole_splits(sp, nkb);
     }
     int splits = target_ctas() / tiles;
     if (splits > nkb / 4) splits = nkb / 4;
     if (splits > 16) splits = 16;
-    if (splits < 1) splits = 1;
-    // no empty split: ceil(nkb/splits) * (splits-1) < nkb
-    while (splits > 1 && ((nkb + splits - 1) / splits) * (splits - 1) >= nkb) --splits;
-    return splits;
+    return gemm_whole_splits(splits, nkb);
 }
 
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
@@ -660,8 +663,10 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     // The gate/up projection has no K split to balance its CTAs over the SMs (192 tiles on 148 SMs at the 8B
     // shape: some SMs stage for two CTAs), so from 65 rows up it also runs as pairs, each CTA staging half of
     // the activation rows (measured at 128 rows: step 4.84 -> 4.72 ms; at 32 rows pairs lose, 3.27 vs 3.26).
-    const bool pair = use_pair(a.M, swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM) ||
-                      (swiglu && a.M > 64 && pair_enabled() && (((a.N + 63) / 64) & 1) == 0);
+    static const bool rows_on = !(getenv("ODB_GEMM_ROWS") && getenv("ODB_GEMM_ROWS")[0] == '0');
+    const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
+    if (rows_on && use_pair(a.M, n_tiles) && gemm_rows_supported(a, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
+    const bool pair = use_pair(a.M, n_tiles) || (swiglu && a.M > 64 && pair_enabled() && (n_tiles & 1) == 0);
     const int bn = pick_bn(a.M, pair);
     if (swiglu) {
         if (a.splits != 1) return cudaErrorInvalidValue;

@@ -615,7 +615,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             cap = L.tp_recv_slot / sizeof(float) / (static_cast<size_t>(rows) * N * R);
             if (cap > static_cast<size_t>(16 / R)) cap = 16 / R;
         }
-        if (static_cast<size_t>(sp) > cap) sp = static_cast<int>(cap < 1 ? 1 : cap);
+        if (static_cast<size_t>(sp) > cap) sp = gemm_whole_splits(static_cast<int>(cap < 1 ? 1 : cap), (K + 63) / 64);
         return sp;
     };
     // An exchange of kind `kind`: the projection that produces the data raises this rank's flags when its last CTA

@@ -302,6 +302,8 @@ struct GemmArgs {
     int* status;           // device status word
 };
 int gemm_pick_splits(int M, int N, int K);
+// the largest number of K splits <= splits that leaves none of them empty: ceil(nkb / splits) * (splits - 1) < nkb
+int gemm_whole_splits(int splits, int nkb);
 
 // Test entry: one block performs the consumers' flag wait (tensor_parallel.cu).
 cudaError_t launch_tp_wait(const TpWait& tw, cudaStream_t st);
@@ -314,6 +316,9 @@ cudaError_t make_gate_up_tmap(CUtensorMap* out, const void* w_packed, int F, int
 cudaError_t launch_pack_gate_up(const void* src_gate_then_up, void* dst_packed, int F, int K, cudaStream_t st);
 cudaError_t launch_pack_weight(const void* src_row_major, void* dst_packed, int N, int K, cudaStream_t st);
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
+// many-row projections with the activation rows on the M side of the tile (gemm_rows.cu)
+bool gemm_rows_supported(const GemmArgs& a, int n_tiles);
+cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stride, float* out, size_t n,
                                    cudaStream_t st);
 
