@@ -572,7 +572,14 @@ bool use_pair(int M, int n_tiles) {
     return pair_enabled() && M > min_rows && (n_tiles & 1) == 0;
 }
 
+bool rows_enabled() {
+    static const bool on = !(getenv("ODB_GEMM_ROWS") && getenv("ODB_GEMM_ROWS")[0] == '0');
+    return on;
+}
+
 }  // namespace
+
+bool gemm_rows_usable(int M, int N) { return M > 128 && rows_enabled() && use_pair(M, (N + kBM - 1) / kBM); }
 
 cudaError_t make_weight_tmap(CUtensorMap* out, const void* w, int N, int K) { return make_tmap_packed(out, w, N, K); }
 
@@ -663,9 +670,9 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     // The gate/up projection has no K split to balance its CTAs over the SMs (192 tiles on 148 SMs at the 8B
     // shape: some SMs stage for two CTAs), so from 65 rows up it also runs as pairs, each CTA staging half of
     // the activation rows (measured at 128 rows: step 4.84 -> 4.72 ms; at 32 rows pairs lose, 3.27 vs 3.26).
-    static const bool rows_on = !(getenv("ODB_GEMM_ROWS") && getenv("ODB_GEMM_ROWS")[0] == '0');
     const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
-    if (rows_on && use_pair(a.M, n_tiles) && gemm_rows_supported(a, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
+    if (rows_enabled() && use_pair(a.M, n_tiles) && gemm_rows_supported(a, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
+    if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of that kernel only
     const bool pair = use_pair(a.M, n_tiles) || (swiglu && a.M > 64 && pair_enabled() && (n_tiles & 1) == 0);
     const int bn = pick_bn(a.M, pair);
     if (swiglu) {

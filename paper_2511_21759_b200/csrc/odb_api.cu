@@ -71,7 +71,7 @@ void vocab_shard(const odb_config& c, int rank, int* tile0, int* rows) {
 // odb_session_create so that both always agree.
 struct Layout {
     size_t rows, lm_chunk, tiles, partial_rows, attn_rows;
-    size_t rope, state, results, status, loop, x, row_tok, row_pos, row_seq, row_copy, row_flags, lm_rows, tile_buf, big_tile_buf, step_tile_buf;
+    size_t rope, rope_t, state, results, status, loop, x, row_tok, row_pos, row_seq, row_copy, row_flags, lm_rows, tile_buf, big_tile_buf, step_tile_buf;
     size_t h, a, inv, q, k, v, o, g, partial, logits, conf, tok, conf_part, part_o, part_ml, ptable, pbars, noise;
     size_t tp_recv, tp_recv_slot, tp_flags, conf_part_bytes;   // tensor parallelism: two receive slots for partial sums, the flag words
     size_t total;
@@ -93,6 +93,7 @@ Layout make_layout(const odb_config& c) {
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     L.rope = take(static_cast<size_t>(c.max_seq) * (c.head_dim / 2) * sizeof(float2));
+    L.rope_t = take(static_cast<size_t>(c.max_seq) * (c.head_dim / 2) * sizeof(float2));
     L.state = take(sizeof(SeqState) * c.max_batch);
     L.results = take(sizeof(odb_result) * c.max_batch);
     L.status = take(sizeof(int));
@@ -347,17 +348,20 @@ int32_t odb_session_create(odb_model* m, void* kv, size_t kv_bytes, void* worksp
     if (e == cudaSuccess) e = cudaMallocHost(&s->pinned_results, sizeof(odb_result) * c.max_batch);
     if (e == cudaSuccess) e = cudaMallocHost(&s->pinned_status, sizeof(int));
     // RoPE table: angle(pos, i) = pos * theta^(-2i/hd), evaluated in double, stored as fp32 (cos, sin)
-    std::vector<float2> rope(static_cast<size_t>(c.max_seq) * (c.head_dim / 2));
+    std::vector<float2> rope(static_cast<size_t>(c.max_seq) * (c.head_dim / 2)), rope_t(rope.size());
     for (int i = 0; i < c.head_dim / 2; ++i) {
         const double inv = pow(static_cast<double>(c.rope_theta), -2.0 * i / c.head_dim);
         for (int p = 0; p < c.max_seq; ++p) {
             const double ang = p * inv;
-            rope[static_cast<size_t>(p) * (c.head_dim / 2) + i] = make_float2(static_cast<float>(cos(ang)),
-                                                                              static_cast<float>(sin(ang)));
+            const float2 cs = make_float2(static_cast<float>(cos(ang)), static_cast<float>(sin(ang)));
+            rope[static_cast<size_t>(p) * (c.head_dim / 2) + i] = cs;
+            rope_t[static_cast<size_t>(i) * c.max_seq + p] = cs;
         }
     }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->ws + L.rope, rope.data(), rope.size() * sizeof(float2), cudaMemcpyHostToDevice, s->st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->ws + L.rope_t, rope_t.data(), rope_t.size() * sizeof(float2), cudaMemcpyHostToDevice, s->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->ws + L.state, 0, L.x - L.state, s->st);   // state, results, status
     // The tensor-core attention loads whole 64-row boxes: cache rows that are not keys of a work item are masked
     // in its softmax but still enter the P V product with weight zero, so they must hold finite values; the
@@ -741,17 +745,33 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d,
                                                         hint_of(m->p_qkv[l], qkv_bytes, 0), st, res_wait));
         int sp = plan_splits(M, 3 * da, d, false);
-        ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_qkv[l], a, partial, M, 3 * da, d, sp));
         QkvRopeArgs qa;
         qa.partial = partial; qa.splits = sp; qa.pstride = static_cast<size_t>(M) * 3 * da;
         qa.scale = inv_scale;
         qa.rope = s->at<float2>(L.rope);
+        qa.rope_t = s->at<float2>(L.rope_t);
         qa.row_pos = s->cb.row_pos; qa.row_seq = s->cb.row_seq;
         qa.q = q; qa.k = k; qa.v = v;
         qa.cache = write_cache ? s->kv : nullptr;
         qa.layer = l; qa.n_layers = c.n_layers; qa.H = H; qa.hd = hd; qa.max_seq = c.max_seq; qa.M = M;
         qa.pf = hint_of(m->p_o[l], o_bytes, 0);
-        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_qkv_rope(qa, st));
+        if (sp == 1 && gemm_rows_usable(M, 3 * da)) {
+            // many rows: RoPE, the bf16 rows and the cache scatter in the projection's epilogue, no fp32 rows in memory
+            GemmArgs ga;
+            ga.tmap_w = m->tm_qkv[l];
+            ga.x = a;
+            ga.partial = nullptr;
+            ga.act_out = nullptr;
+            ga.qkv = &qa;
+            ga.row_scale = inv_scale;
+            ga.M = M; ga.N = 3 * da; ga.K = d;
+            ga.splits = 1;
+            ga.status = status;
+            ODB_FWD(ODB_KIND_GEMM, launch_gemm(ga, st));
+        } else {
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_qkv[l], a, partial, M, 3 * da, d, sp));
+            ODB_FWD(ODB_KIND_ELEMENTWISE, launch_qkv_rope(qa, st));
+        }
         if (n_step_tiles > 0) {
             // several copies: one work item serves all copies of a block, cached K/V loaded once
             StepAttnArgs sa;

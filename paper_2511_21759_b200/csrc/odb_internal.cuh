@@ -287,6 +287,19 @@ __device__ __forceinline__ void tp_wait_flags(const TpWait& tw) {
 }
 #endif
 
+// Split reduction of a QKV projection, RoPE and the places its rows go to.
+struct QkvRopeArgs {
+    const float* partial; int splits; size_t pstride;      // [splits][M][3d]
+    RowScale scale;                                        // scalar of the preceding RMSNorm
+    const float2* rope;                                    // [max_seq][hd/2] (cos, sin)
+    const float2* rope_t;                                  // the same table as [hd/2][max_seq]
+    const int32_t* row_pos; const int32_t* row_seq;
+    __nv_bfloat16 *q, *k, *v;                              // [M][d]
+    __nv_bfloat16* cache;                                  // NULL: do not write the cache
+    int layer, n_layers, H, hd, max_seq, M;
+    L2Prefetch pf;
+};
+
 // Weight-streaming GEMM: partial[s][M][N] (fp32) = x[M][K_s] * w[N][K_s]^T for each K split s.
 struct GemmArgs {
     CUtensorMap tmap_w;    // packed bf16 weight tiles [n_tile * k_blocks][128][64], 128B swizzle
@@ -296,6 +309,9 @@ struct GemmArgs {
     ConfEpilogue conf;                  // conf.part non-null: LM head fused with the confidence statistics, splits == 1
     RowScale row_scale;                 // per activation row m: the output is multiplied by scale[m]
                                         // (the 1/rms of an RMSNorm folded behind the projection); needs splits == 1
+    const QkvRopeArgs* qkv = nullptr;   // non-null: QKV projection whose epilogue applies RoPE and writes q / k / v and the cache
+                                        // (many rows, gemm_rows_usable); splits == 1
+    float* add_to = nullptr;            // non-null: the product is added to fp32 [M][N] in place (likewise)
     PeerOut peers;                      // peers.n > 0: the partial tiles (or statistics) go to these buffers instead
     int M, N, K;
     int splits;
@@ -317,6 +333,7 @@ cudaError_t launch_pack_gate_up(const void* src_gate_then_up, void* dst_packed, 
 cudaError_t launch_pack_weight(const void* src_row_major, void* dst_packed, int N, int K, cudaStream_t st);
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
 // many-row projections with the activation rows on the M side of the tile (gemm_rows.cu)
+bool gemm_rows_usable(int M, int N);   // whether a projection of this size has the epilogues `qkv` and `add_to`
 bool gemm_rows_supported(const GemmArgs& a, int n_tiles);
 cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stride, float* out, size_t n,
@@ -341,16 +358,6 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
 // features); g[m][f] = bf16(silu(gate) * up) with gate, up = the split sums (split order) times the row scalar.
 cudaError_t launch_swiglu_combine(const float* partial, int splits, size_t pstride, const RowScale& scale, __nv_bfloat16* g,
                                   int M, int F, cudaStream_t st);
-struct QkvRopeArgs {
-    const float* partial; int splits; size_t pstride;      // [splits][M][3d]
-    RowScale scale;                                        // scalar of the preceding RMSNorm
-    const float2* rope;                                    // [max_seq][hd/2] (cos, sin)
-    const int32_t* row_pos; const int32_t* row_seq;
-    __nv_bfloat16 *q, *k, *v;                              // [M][d]
-    __nv_bfloat16* cache;                                  // NULL: do not write the cache
-    int layer, n_layers, H, hd, max_seq, M;
-    L2Prefetch pf;
-};
 cudaError_t launch_qkv_rope(const QkvRopeArgs& a, cudaStream_t st);
 cudaError_t launch_confidence_final(const ConfPartial* part, int chunks, int rows, float* conf, int32_t* tok,
                                     cudaStream_t st, const TpWait& tw = TpWait());
