@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(kThreads) attention_tc_kernel(const __grid_con
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int* cta_abort = &sh->abort;
 
-    pdl_launch_dependents();
     if ((smem_u32(smem_raw) & 1023u) != 0) {                // the swizzled tiles need 1024-byte alignment
         if (tid == 0) atomicExch(status, ODB_ERR_CUDA);
         pdl_wait();
@@ -237,6 +236,7 @@ __global__ void __launch_bounds__(kThreads) attention_tc_kernel(const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();                                // behind the TMEM allocation: the successor allocates for pairs
     const uint32_t tmem_s0 = sh->tmem_base;                // 64 columns
     const uint32_t tmem_o = sh->tmem_base + 64;            // 128 columns
     const uint32_t tmem_s1 = sh->tmem_base + 192;          // 64 columns

@@ -1,5 +1,5 @@
-// Many-row projection (more than 128 activation rows) as CTA pairs, with the ACTIVATION rows on the M side of the
-// tensor-core tile.
+// Many-row projections (more than 128 activation rows): persistent CTA pairs with the ACTIVATION rows on the M side of
+// the tensor-core tile.
 //
 // The pair kernel of gemm_tcgen05.cu gives the M side to the weights; its accumulator then has one weight row per
 // TMEM lane and an epilogue thread owns one output FEATURE of many rows: SwiGLU has to fetch the matching up value
@@ -9,19 +9,20 @@
 // CTA staging 128 activation rows (A) and one packed weight tile of 128 rows (its half of B), so the bytes staged and
 // the MMA rate are the ones of the other kernel, and lane r of a CTA's accumulator is its activation row r with 256
 // features in consecutive columns.  A thread owns a row: gate and up (a packed gate/up tile is 64 gate then 64 up
-// rows), the row's RMSNorm scalar and a whole vocabulary tile's logits are its own, the epilogue warps share no data
-// and meet at no barrier.  Results leave through a 4 KB patch of the (then idle) stage ring per warp, so that
-// stores are 16 bytes wide and cover whole 128-byte lines.  The sums are the same products in the same order.
+// rows), rotate-half partners, the row's RMSNorm scalar and a whole vocabulary tile's logits are its own; the eight
+// epilogue warps (two per 32 TMEM lanes, one packed weight tile each) share no data and meet at no barrier.  Results
+// leave through a 4 KB patch of shared memory per warp, so that stores are 16 bytes wide and cover whole 64- or
+// 128-byte lines.  The sums are the same products in the same order.
 //
-// Bound: tensor cores (operand staging 131 FLOP per byte).  Two CTAs per SM, 3 stages x 32 KB each.
-// Eight epilogue warps (two per 32 TMEM lanes, one packed weight tile each): with four, the QKV epilogue below took 20 us
-// longer at 768 rows, where the single wave of CTAs leaves it exposed (59 against 76 us).
-// Measured against the other kernel (8B shape, one launch each):
-//   SwiGLU at 768 / 4096 / 25568 rows        154 -> 111, 793 -> 573, 4523 -> 3604 us (1.39, 1.44, 1.43 PFLOP/s)
-//   LM head + statistics at 256 rows          321 -> 245 us
-//   QKV + RoPE + cache scatter, same rows      72 -> 59, 330 -> 300, 2170 -> 1868 us (projection and RoPE kernel before)
-#include <stdlib.h>
-
+// One pair per two SMs walks over the output tiles (6 stages x 32 KB, two accumulators in TMEM): the epilogue of a tile
+// runs under the main loop of the next.  With 227 KB of shared memory no other kernel that allocates TMEM fits beside a
+// CTA, and no second pair either: an allocation for a pair needs the same columns in both SMs, so two of them meeting on
+// one pair of SMs, or one meeting single-SM allocations of a successor, could wait for each other.
+//
+// Measured against the kernels this replaces (8B shape, one launch each, 768 / 4096 / 25568 rows):
+//   SwiGLU                                154 -> 108, 793 -> 554 us, 4.52 -> 3.5 ms (1.43, 1.49, 1.47 PFLOP/s; 1.66 is the peak)
+//   QKV + RoPE + cache scatter             72 -> 60, 330 -> 283 us, 2.17 -> 1.8 ms (projection and RoPE kernel before)
+//   LM head + statistics at 256 rows      321 -> 205 us
 #include "odb_internal.cuh"
 #include "tcgen05_common.cuh"
 
@@ -32,30 +33,55 @@ namespace {
 constexpr int kRowsN = 256;                              // weight rows of a pair's tile (two packed tiles)
 constexpr uint32_t kTileBytes = kBM * kBK * 2;           // 16 KB: a packed weight tile, and 128 activation rows
 constexpr uint32_t kRowsStageBytes = 2 * kTileBytes;
-constexpr int kRowsStages = 3;                           // 96 KB: two CTAs per SM
-constexpr uint32_t kRowsTmemCols = kRowsN;
-constexpr int kRowsThreads = 320;                        // TMA warp, MMA warp, eight epilogue warps (two per 32 TMEM lanes)
+constexpr int kRowsStages = 6;
+constexpr uint32_t kRowsTmemCols = 2 * kRowsN;           // two accumulators
+constexpr int kRowsThreads = 320;                        // TMA warp, MMA warp, eight epilogue warps
+constexpr uint32_t kPatchBytes = 4096;                   // per epilogue warp: 32 rows x 128 bytes
 
-constexpr int ROWS_SWIGLU = 0, ROWS_CONF = 1, ROWS_ADD = 2, ROWS_QKV64 = 3, ROWS_QKV128 = 4;
+constexpr int ROWS_SWIGLU = 0, ROWS_CONF = 1, ROWS_ADD = 2, ROWS_PARTIAL = 3, ROWS_QKV64 = 4, ROWS_QKV128 = 5;
 
 struct alignas(8) RowsShared {
     uint64_t full[kRowsStages];
     uint64_t empty[kRowsStages];
-    uint64_t acc_full;
+    uint64_t acc_full[2];
+    uint64_t acc_empty[2];       // the leader's counts the 16 epilogue warps of both CTAs
     uint32_t tmem_base;
     int abort;
 };
 
 struct RowsArgs {
+    float* partial;              // ROWS_PARTIAL: fp32 [splits][M][N]
     __nv_bfloat16* act_out;      // ROWS_SWIGLU: bf16 [M][N = F]
     ConfEpilogue ce;             // ROWS_CONF
     float* add_to;               // ROWS_ADD: fp32 [M][N], the residual stream
     QkvRopeArgs qkv;             // ROWS_QKV64 / ROWS_QKV128 (head dim)
     RowScale rs;
-    int M, N, nkb;
-    int n_pairs, m_tiles;        // pairs of weight tiles, tiles of 256 rows
+    int M, N, nkb_total, nkb_per_split;
+    int n_pairs, m_tiles, group, splits;   // pairs of weight tiles, tiles of 256 rows, row tiles that are walked side by side
+    uint64_t w_hint;             // L2 policy of the weight tiles
     int* status;
 };
+
+// The tiles in the order they are handed out, round robin, to the pairs: the row tiles of a group side by side on one
+// weight-tile pair (its weights come from HBM once, from L2 for the other row tiles), then the next weight-tile pair
+// (the group's activation rows, a few MB, stay in L2), then the next group, then the next K split.
+struct RowsItem {
+    int m_tile, pair, split, kb0, nkb;
+};
+__device__ __forceinline__ RowsItem rows_item(const RowsArgs& a, int item) {
+    RowsItem w;
+    const int per_split = a.m_tiles * a.n_pairs;
+    w.split = item / per_split;
+    item -= w.split * per_split;
+    const int g = item / (a.group * a.n_pairs), m_first = g * a.group;
+    const int in_group = min(a.group, a.m_tiles - m_first);
+    item -= m_first * a.n_pairs;
+    w.pair = item / in_group;
+    w.m_tile = m_first + item - w.pair * in_group;
+    w.kb0 = w.split * a.nkb_per_split;
+    w.nkb = min(a.nkb_per_split, a.nkb_total - w.kb0);   // >= 1: the launcher refuses empty splits
+    return w;
+}
 
 // 128-byte pieces of 32 rows, turned in shared memory (16-byte chunks, XOR-swizzled: no bank conflicts either way):
 // lane r puts its row's chunks, then eight lanes take one row's 128 bytes, so that a store covers whole lines.
@@ -80,15 +106,6 @@ __device__ __forceinline__ void take_rows(uint8_t* buf, int lane, Sink&& sink) {
         sink(r, c, x);
     }
 }
-// put, meet, take.  Callers alternate between two buffers, so that one warp barrier per piece is enough.
-template <class Sink>
-__device__ __forceinline__ void store_rows(uint8_t* buf, const uint32_t (&v)[32], int lane, Sink&& sink) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) put_chunk(buf, lane, c, v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-    __syncwarp();
-    take_rows(buf, lane, sink);
-}
-
 // four fp32 sums added to memory without a read back; every element has exactly one such add per launch, so the
 // result is the rounded sum whatever the order of the CTAs
 __device__ __forceinline__ void red_add4(float* p, const uint4& x) {
@@ -117,41 +134,39 @@ __device__ __forceinline__ void tmem_read32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ uint32_t leader_address(uint64_t* bar) {   // shared::cluster address of the leader's copy of `bar`
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(bar)));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
 template <int EPI>
-__global__ void __launch_bounds__(kRowsThreads, 2)
+__global__ void __launch_bounds__(kRowsThreads, 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RowsArgs a,
                  const __grid_constant__ PeerOut po) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    RowsShared* sh = reinterpret_cast<RowsShared*>(ring + kRowsStages * kRowsStageBytes);
+    uint8_t* patches = ring + kRowsStages * kRowsStageBytes;
+    RowsShared* sh = reinterpret_cast<RowsShared*>(patches + 8 * kPatchBytes);
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    // grid (2, row tiles of a group, weight-tile pairs x row-tile groups), scheduled in that order: the row
-    // tiles of a group run side by side on one weight-tile pair (its weights come from HBM once) and a group's
-    // activation rows (a few MB) stay in L2 while every weight-tile pair passes over them
-    const int pair = static_cast<int>(blockIdx.z) % a.n_pairs;
-    const int m_tile = static_cast<int>(blockIdx.z) / a.n_pairs * static_cast<int>(gridDim.y) + static_cast<int>(blockIdx.y);
-    if (m_tile >= a.m_tiles) {   // ragged last group: both CTAs of the pair leave together
-        if (po.n > 0 && threadIdx.x == 0) {
-            pdl_wait();   // the arrival counter is shared with the previous exchanging launch: count only once that one is complete
-            tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);
-        }
-        return;
-    }
-    const int nkb = a.nkb;
-    const int m0 = m_tile * 2 * kBM + static_cast<int>(rank) * kBM;   // first activation row of this CTA
-    const int wtile0 = (2 * pair + static_cast<int>(rank)) * nkb;
+    const int first = static_cast<int>(blockIdx.x) >> 1, step = static_cast<int>(gridDim.x) >> 1;
+    const int n_items = a.m_tiles * a.n_pairs * a.splits;
     volatile int* cta_abort = &sh->abort;
 
-    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kRowsStages; ++i) {
             mbar_init(&sh->full[i], 1);
             mbar_init(&sh->empty[i], 1);
         }
-        mbar_init(&sh->acc_full, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sh->acc_full[b], 1);
+            mbar_init(&sh->acc_empty[b], 16);
+        }
         sh->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -170,38 +185,53 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    cluster_barrier();   // the peer's barriers are initialised before anything signals them
+    cluster_barrier();         // the peer's barriers are initialised before anything signals them
+    pdl_launch_dependents();   // behind the allocation: no successor's allocation can come before it
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---- TMA producer: weight tiles first (they do not depend on the preceding kernel), then the rows ----
-            const int pre = nkb < kRowsStages ? nkb : kRowsStages;
+            // ---- TMA producer: weight tiles of the first stages first (they do not depend on the preceding kernel) ----
+            RowsItem w = rows_item(a, first);
+            const int pre = w.nkb < kRowsStages ? w.nkb : kRowsStages;
+            int wt = (2 * w.pair + static_cast<int>(rank)) * a.nkb_total + w.kb0;
+            int mrow = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM;
             for (int i = 0; i < pre; ++i) {
                 if (leader) mbar_expect_tx(&sh->full[i], 2 * kRowsStageBytes);   // the loads of both CTAs report to the leader
-                tma_load_3d_pair(ring + i * kRowsStageBytes, &tmap_w, &sh->full[i], 0, 0, wtile0 + i, kEvictFirst);
+                tma_load_3d_pair(ring + i * kRowsStageBytes, &tmap_w, &sh->full[i], 0, 0, wt + i, a.w_hint);
             }
             pdl_wait();
             for (int i = 0; i < pre; ++i)
-                tma_load_2d_pair(ring + i * kRowsStageBytes + kTileBytes, &tmap_x, &sh->full[i], i * kBK, m0, kEvictLast);
-            int st = 0, issued = pre;
-            uint32_t ph = 0;   // fills of the ring completed so far, parity
-            for (int i = pre; i < nkb; ++i) {
-                if (!mbar_wait(&sh->empty[st], ph, cta_abort, a.status)) break;
-                uint8_t* dst = ring + st * kRowsStageBytes;
-                if (leader) mbar_expect_tx(&sh->full[st], 2 * kRowsStageBytes);
-                tma_load_3d_pair(dst, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
-                tma_load_2d_pair(dst + kTileBytes, &tmap_x, &sh->full[st], i * kBK, m0, kEvictLast);
-                issued = i + 1;
-                if (++st == kRowsStages) { st = 0; ph ^= 1u; }
+                tma_load_2d_pair(ring + i * kRowsStageBytes + kTileBytes, &tmap_x, &sh->full[i], (w.kb0 + i) * kBK, mrow, kEvictLast);
+            int st = pre == kRowsStages ? 0 : pre;
+            uint32_t ph = pre == kRowsStages ? 1u : 0u;   // parity of the ring's current round
+            long long issued = pre;
+            bool ok = true;
+            int i = pre;
+            for (int item = first;;) {
+                for (; i < w.nkb && ok; ++i) {
+                    ok = mbar_wait(&sh->empty[st], ph ^ 1u, cta_abort, a.status);   // the first round's stages are free
+                    if (!ok) break;
+                    uint8_t* dst = ring + st * kRowsStageBytes;
+                    if (leader) mbar_expect_tx(&sh->full[st], 2 * kRowsStageBytes);
+                    tma_load_3d_pair(dst, &tmap_w, &sh->full[st], 0, 0, wt + i, a.w_hint);
+                    tma_load_2d_pair(dst + kTileBytes, &tmap_x, &sh->full[st], (w.kb0 + i) * kBK, mrow, kEvictLast);
+                    ++issued;
+                    if (++st == kRowsStages) { st = 0; ph ^= 1u; }
+                }
+                item += step;
+                if (!ok || item >= n_items) break;
+                w = rows_item(a, item);
+                wt = (2 * w.pair + static_cast<int>(rank)) * a.nkb_total + w.kb0;
+                mrow = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM;
+                i = 0;
             }
             if (*cta_abort && leader) {
                 // aborted: let the copies still in flight land before the CTA's shared memory goes away (the
                 // peer cannot observe its own copies; it is held by the cluster barrier at the end)
-                const int first = issued > kRowsStages ? issued - kRowsStages : 0;
-                for (int i = first; i < issued; ++i) {
+                for (long long j = issued > kRowsStages ? issued - kRowsStages : 0; j < issued; ++j) {
                     const long long t0 = clock64();
-                    while (!mbar_try_wait_parity(&sh->full[i % kRowsStages], static_cast<uint32_t>(i / kRowsStages) & 1u) &&
+                    while (!mbar_try_wait_parity(&sh->full[j % kRowsStages], static_cast<uint32_t>(j / kRowsStages) & 1u) &&
                            clock64() - t0 < kWaitLimitCycles / 8) {
                     }
                 }
@@ -212,39 +242,52 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             // ---- MMA issuer (the leader's, for both CTAs): A = activation rows, B = weight rows ----
             constexpr uint32_t idesc = make_instr_desc(2 * kBM, kRowsN);
             bool ok = true;
-            int st = 0;
+            int st = 0, n = 0;
             uint32_t ph = 0;
-            for (int i = 0; i < nkb; ++i) {
-                ok = mbar_wait(&sh->full[st], ph, cta_abort, a.status);
-                if (!ok) break;
+            for (int item = first; item < n_items && ok; item += step, ++n) {
+                const int nkb = rows_item(a, item).nkb, b = n & 1;
+                const uint32_t acc = tmem_acc + static_cast<uint32_t>(b * kRowsN);
+                ok = mbar_wait(&sh->acc_empty[b], ((n >> 1) & 1) ^ 1u, cta_abort, a.status);   // free at first
                 tc_fence_after();
-                const uint32_t w_addr = smem_u32(ring + st * kRowsStageBytes), x_addr = w_addr + kTileBytes;
+                for (int i = 0; i < nkb && ok; ++i) {
+                    ok = mbar_wait(&sh->full[st], ph, cta_abort, a.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t w_addr = smem_u32(ring + st * kRowsStageBytes), x_addr = w_addr + kTileBytes;
 #pragma unroll
-                for (int k = 0; k < kBK / kUmmaK; ++k)
-                    umma_bf16_pair(tmem_acc, make_smem_desc(x_addr + k * kUmmaK * 2), make_smem_desc(w_addr + k * kUmmaK * 2), idesc,
-                                   (i > 0 || k > 0) ? 1u : 0u);
-                umma_commit_pair(&sh->empty[st]);   // frees the stage in both CTAs once these MMAs have read it
-                if (++st == kRowsStages) { st = 0; ph ^= 1u; }
+                    for (int k = 0; k < kBK / kUmmaK; ++k)
+                        umma_bf16_pair(acc, make_smem_desc(x_addr + k * kUmmaK * 2), make_smem_desc(w_addr + k * kUmmaK * 2), idesc,
+                                       (i > 0 || k > 0) ? 1u : 0u);
+                    umma_commit_pair(&sh->empty[st]);   // frees the stage in both CTAs once these MMAs have read it
+                    if (++st == kRowsStages) { st = 0; ph ^= 1u; }
+                }
+                if (ok) umma_commit_pair(&sh->acc_full[b]);
             }
-            if (ok) umma_commit_pair(&sh->acc_full);
         }
     } else {
         // ---- epilogue: warps 2..9 own TMEM lanes 32 * (warp % 4) .. + 31 = activation rows, and the 128 columns of
         // packed weight tile 2 * pair + t ----
         const int q = warp & 3, t = (warp - 2) >> 2;
-        const int mw = m0 + q * 32;                          // the warp's first row
-        const int m = mw + lane;
-        const int tile = 2 * pair + t;
-        const uint32_t tmem = tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(t * kBM);
+        uint8_t* patch = patches + (warp - 2) * kPatchBytes;
+        const uint32_t free_bar = leader_address(&sh->acc_empty[0]);
         pdl_wait();   // the previous reader of the output buffer has finished; the predecessor's results are visible
-        const float sc = m < a.M ? row_scale_of(a.rs, m) : 1.0f;
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&sh->acc_full, 0, cta_abort, a.status));
-        if (ok) {
+        int n_done = 0;
+        for (int item = first; item < n_items; item += step, ++n_done) {
+            const RowsItem w = rows_item(a, item);
+            const int b = n_done & 1;
+            const int mw = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM + q * 32;   // the warp's first row
+            const int m = mw + lane;
+            const int tile = 2 * w.pair + t;
+            const uint32_t tmem = tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * kRowsN + t * kBM);
+            const float sc = m < a.M ? row_scale_of(a.rs, m) : 1.0f;
+            int pos = 0, seq = 0;
+            if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
+                if (m < a.M) { pos = a.qkv.row_pos[m]; seq = a.qkv.row_seq[m]; }
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[b], (n_done >> 1) & 1, cta_abort, a.status))) break;
             tc_fence_after();
-            // every MMA of both CTAs has completed, so the stage ring is free
-            uint8_t* patch = ring + (warp - 2) * 8192;
             if constexpr (EPI == ROWS_SWIGLU) {
-#pragma unroll 1
+#pragma unroll
                 for (int c = 0; c < 64; c += 16) {
                     uint32_t g[16], u[16];
                     tmem_ld16(tmem + c, g);
@@ -266,35 +309,55 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                     if (mw + r < a.M && f < a.N)             // F % 16 == 0
                         *reinterpret_cast<uint4*>(a.act_out + static_cast<size_t>(mw + r) * a.N + f) = x;
                 });
-            } else if constexpr (EPI == ROWS_ADD) {
+            } else if constexpr (EPI == ROWS_ADD || EPI == ROWS_PARTIAL) {
+                const size_t split_off = static_cast<size_t>(w.split) * a.M * a.N;
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
                     const int nc = tile * kBM + c * 32;
                     if (nc >= a.N) break;
                     uint32_t v[32];
                     tmem_read32(tmem + c * 32, v);
-                    store_rows(patch + (c & 1) * 4096, v, lane, [&](int r, int ch, const uint4& x) {
+                    if (EPI == ROWS_PARTIAL && a.rs.ssq) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
+                    }
+                    __syncwarp();                            // the previous piece has been taken
+#pragma unroll
+                    for (int ch = 0; ch < 8; ++ch) put_chunk(patch, lane, ch, v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
+                    __syncwarp();
+                    take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
                         const int n = nc + ch * 4;
-                        if (mw + r < a.M && n < a.N) red_add4(a.add_to + static_cast<size_t>(mw + r) * a.N + n, x);   // N % 4 == 0
+                        if (mw + r >= a.M || n >= a.N) return;       // N % 4 == 0
+                        const size_t off = static_cast<size_t>(mw + r) * a.N + n;
+                        if (EPI == ROWS_ADD) {
+                            red_add4(a.add_to + off, x);
+                        } else if (po.n == 0) {
+                            *reinterpret_cast<uint4*>(a.partial + split_off + off) = x;
+                        } else {   // tensor-parallel partial sums: the tile goes to the receive buffer of every rank
+#pragma unroll 1
+                            for (int p = 0; p < po.n; ++p) *reinterpret_cast<uint4*>(po.partial[p] + split_off + off) = x;
+                        }
                     });
                 }
             } else if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
                 // QKV projection: a head's q, k or v of this row is the thread's own, rotate-half partners included.
                 // The RMSNorm scalar, RoPE (q and k), bf16 rows and - in a refresh - the K/V cache.  The (cos, sin) table
-                // is read transposed ([pair][position]): the lanes' positions are neighbours, mostly.
+                // is read transposed ([pair][position]): the lanes' positions are neighbours, mostly.  A piece is 32
+                // dims of a head's lower half and the 32 they rotate with.
                 constexpr int HD = EPI == ROWS_QKV128 ? 128 : 64, kHalf = HD / 2;
                 const QkvRopeArgs& e = a.qkv;
-                const int pos = m < a.M ? e.row_pos[m] : 0, seq = m < a.M ? e.row_seq[m] : 0;
                 const long long crow = (static_cast<long long>(seq) * e.n_layers + e.layer) * 2 * e.H * e.max_seq + pos;
                 const float2* rope = e.rope_t + pos;
 #pragma unroll 1
-                for (int grp = 0; grp < kBM / HD; ++grp) {
+                for (int piece = 0; piece < kBM / 64; ++piece) {
+                    const int grp = HD == 128 ? 0 : piece, c0 = HD == 128 ? piece * 32 : 0;
                     const int g = tile * (kBM / HD) + grp;             // head of [Wq; Wk; Wv]
                     if (g >= 3 * e.H) break;
                     const int sec = g / e.H, head = g - sec * e.H;
-                    uint8_t* buf = patch + grp * 4096;                 // one group of two pieces, or two of one
+                    __syncwarp();                                      // the previous piece has been taken
 #pragma unroll 1
-                    for (int c = 0; c < kHalf; c += 16) {
+                    for (int cc = 0; cc < 32; cc += 16) {
+                        const int c = c0 + cc;
                         uint32_t lo[16], hi[16];
                         tmem_ld16(tmem + grp * HD + c, lo);
                         tmem_ld16(tmem + grp * HD + kHalf + c, hi);
@@ -317,24 +380,21 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                             pl[j / 2] = pack2(x0, x1);
                             ph[j / 2] = pack2(y0, y1);
                         }
-                        uint8_t* bh = HD == 128 ? buf + 4096 : buf;    // where the upper half of the head goes
-                        const int ch = c / 8, chh = HD == 128 ? ch : ch + 4;
-                        put_chunk(buf, lane, ch, pl[0], pl[1], pl[2], pl[3]);
-                        put_chunk(buf, lane, ch + 1, pl[4], pl[5], pl[6], pl[7]);
-                        put_chunk(bh, lane, chh, ph[0], ph[1], ph[2], ph[3]);
-                        put_chunk(bh, lane, chh + 1, ph[4], ph[5], ph[6], ph[7]);
+                        put_chunk(patch, lane, cc / 8, pl[0], pl[1], pl[2], pl[3]);
+                        put_chunk(patch, lane, cc / 8 + 1, pl[4], pl[5], pl[6], pl[7]);
+                        put_chunk(patch, lane, cc / 8 + 4, ph[0], ph[1], ph[2], ph[3]);
+                        put_chunk(patch, lane, cc / 8 + 5, ph[4], ph[5], ph[6], ph[7]);
                     }
                     __syncwarp();
                     __nv_bfloat16* fresh = (sec == 0 ? e.q : sec == 1 ? e.k : e.v) + head * HD;
                     const long long chead = static_cast<long long>((sec - 1) * e.H + head) * e.max_seq;
-#pragma unroll
-                    for (int piece = 0; piece < HD / 64; ++piece)
-                        take_rows(buf + piece * 4096, lane, [&](int r, int ch, const uint4& x) {
-                            const long long cr = __shfl_sync(0xffffffffu, crow, r);
-                            if (mw + r >= a.M) return;
-                            *reinterpret_cast<uint4*>(fresh + static_cast<size_t>(mw + r) * (e.H * HD) + piece * 64 + ch * 8) = x;
-                            if (e.cache && sec > 0) *reinterpret_cast<uint4*>(e.cache + (cr + chead) * HD + piece * 64 + ch * 8) = x;
-                        });
+                    take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
+                        const long long cr = __shfl_sync(0xffffffffu, crow, r);
+                        if (mw + r >= a.M) return;
+                        const int dim = c0 + (ch & 3) * 8 + (ch >> 2) * kHalf;
+                        *reinterpret_cast<uint4*>(fresh + static_cast<size_t>(mw + r) * (e.H * HD) + dim) = x;
+                        if (e.cache && sec > 0) *reinterpret_cast<uint4*>(e.cache + (cr + chead) * HD + dim) = x;
+                    });
                 }
             } else {
                 // LM head: softmax statistics of each 128-entry vocabulary tile of this thread's row: maximum and argmax
@@ -378,10 +438,14 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                     }
                 }
             }
+            // the accumulator has been read: the next but one tile may overwrite it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(free_bar + b * 8);
         }
-        if (EPI == ROWS_CONF && po.n > 0) {   // uniform: the stores of all eight warps, then one arrival for the CTA
+        if ((EPI == ROWS_CONF || EPI == ROWS_PARTIAL) && po.n > 0) {   // uniform: the stores of all eight warps, then one arrival for the CTA
             asm volatile("bar.sync 1, 256;" ::: "memory");
-            if (threadIdx.x == 64) tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);
+            if (threadIdx.x == 64) tp_arrive_and_signal(po, gridDim.x);
         }
     }
     pdl_wait();   // every thread: keeps completion of the launch chain transitive
@@ -395,37 +459,55 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     }
 }
 
+int sm_pairs() {
+    static std::atomic<int> n{0};
+    int v = n.load(std::memory_order_relaxed);
+    if (!v) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) v = sms / 2;
+        if (v < 1) v = 74;
+        n.store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
 template <int EPI>
 cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     CUtensorMap tmx;
     cudaError_t e = make_rows_tmap(&tmx, g.x, g.M, g.K, kBM);
     if (e != cudaSuccess) return e;
     RowsArgs a;
-    a.act_out = g.act_out; a.ce = g.conf; a.rs = g.row_scale;
-    a.add_to = g.add_to;
-    if (g.qkv) a.qkv = *g.qkv;
+    a.partial = g.partial; a.act_out = g.act_out; a.ce = g.conf; a.rs = g.row_scale; a.add_to = g.add_to;
+    a.qkv = g.qkv ? *g.qkv : QkvRopeArgs();
     a.M = g.M; a.N = g.N;
-    a.nkb = (g.K + kBK - 1) / kBK;
+    a.splits = g.splits;
+    a.nkb_total = (g.K + kBK - 1) / kBK;
+    a.nkb_per_split = (a.nkb_total + g.splits - 1) / g.splits;
+    if (a.nkb_per_split * (g.splits - 1) >= a.nkb_total) return cudaErrorInvalidValue;   // an empty split
     a.n_pairs = n_tiles / 2;
     a.m_tiles = (g.M + 2 * kBM - 1) / (2 * kBM);
+    // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (measured with two CTAs per SM at 128 row tiles: groups of
+    // 2 / 4 / 8 / 16 give 430 / 414 / 404 / 407 ms of GEMM time per refresh, no grouping 475)
+    a.group = a.m_tiles < 8 ? a.m_tiles : 8;
     a.status = g.status;
-    constexpr int smem = kRowsStages * kRowsStageBytes + sizeof(RowsShared) + 1024;
+    // with several row tiles a weight tile is read once per row tile of its group, by pairs a few microseconds apart:
+    // marked "first to be evicted", as in the single-pass kernels, it came from HBM 4.5 times per group (25568 rows,
+    // SwiGLU: 11.5 GB; refresh of 16 sequences 11.2 ms against 10.2)
+    a.w_hint = a.m_tiles > 1 ? kEvictNormal : kEvictFirst;
+    const long long items = static_cast<long long>(a.n_pairs) * a.m_tiles * g.splits;
+    if (items > (1ll << 30)) return cudaErrorInvalidValue;
+    constexpr int smem = kRowsStages * kRowsStageBytes + 8 * kPatchBytes + sizeof(RowsShared) + 1024;
+    static_assert(smem <= 227 * 1024, "one CTA per SM");
     static std::atomic<unsigned long long> attr_done{0};
     e = set_smem_limit_once(attr_done, gemm_rows_kernel<EPI>, smem);
     if (e != cudaSuccess) return e;
-    // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (measured at 128 row tiles: groups of 2 / 4 / 8 / 16
-    // give 430 / 414 / 404 / 407 ms of GEMM time per refresh, no grouping 475, one row tile per weight pass 462)
-    const int group = a.m_tiles < 8 ? a.m_tiles : 8;
-    const int m_groups = (a.m_tiles + group - 1) / group;
-    const size_t z = static_cast<size_t>(a.n_pairs) * m_groups;
-    if (z > 65535) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2, group, static_cast<unsigned>(z));
+    cfg.gridDim = dim3(2 * static_cast<unsigned>(items < sm_pairs() ? items : sm_pairs()));
     cfg.blockDim = dim3(kRowsThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;   // neighbouring weight tiles form the pair
+    attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
@@ -438,18 +520,22 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
 
 }  // namespace
 
-// Projections with an even number of weight tiles (pairs) and more than 128 rows whose epilogue gains from owning rows.
-// fp32 partial sums (K splits) stay with gemm_kernel: its epilogue (a feature per thread) stores them without a detour
-// and measured 3 % faster.  All row starts are 16-byte aligned: d, F multiples of 16, heads of 64 or 128.
+// Whether a projection with more than 128 rows runs here: an even number of weight tiles (pairs) and row starts on
+// 16-byte boundaries (always so inside a model: d, F multiples of 16, heads of 64 or 128; the GEMM entry points take any N).
 bool gemm_rows_supported(const GemmArgs& a, int n_tiles) {
-    return a.M > 128 && (n_tiles & 1) == 0 && a.splits == 1 && (a.act_out || a.conf.part || a.qkv || a.add_to);
+    if (a.M <= 128 || (n_tiles & 1)) return false;
+    if (a.act_out || a.conf.part || a.qkv || a.add_to) return a.splits == 1;
+    uintptr_t low = reinterpret_cast<uintptr_t>(a.partial);
+    for (int r = 0; r < a.peers.n; ++r) low |= reinterpret_cast<uintptr_t>(a.peers.partial[r]);
+    return (a.N & 3) == 0 && (low & 15) == 0;
 }
 
 cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st) {
     if (a.act_out) return launch_rows<ROWS_SWIGLU>(a, n_tiles, st);
     if (a.qkv) return a.qkv->hd == 128 ? launch_rows<ROWS_QKV128>(a, n_tiles, st) : launch_rows<ROWS_QKV64>(a, n_tiles, st);
     if (a.add_to) return launch_rows<ROWS_ADD>(a, n_tiles, st);
-    return launch_rows<ROWS_CONF>(a, n_tiles, st);
+    if (a.conf.part) return launch_rows<ROWS_CONF>(a, n_tiles, st);
+    return launch_rows<ROWS_PARTIAL>(a, n_tiles, st);
 }
 
 }  // namespace odb

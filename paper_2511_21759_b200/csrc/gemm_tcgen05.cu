@@ -92,7 +92,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     // packed weights: tile (n-tile, k-block) is the contiguous 16 KB chunk number n_tile * nkb_total + k_block
     const int wtile0 = n_tile * nkb_total + kb0;
 
-    pdl_launch_dependents();
+    if constexpr (!PAIR) pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < stages; ++i) {
             mbar_init(&sh->full[i], 1);
@@ -124,7 +124,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if constexpr (PAIR) cluster_barrier();   // the peer's barriers are initialised before anything signals them
+    if constexpr (PAIR) {
+        cluster_barrier();   // the peer's barriers are initialised before anything signals them
+        pdl_launch_dependents();   // a pair needs the same columns in both SMs: no successor may take any before it has them
+    }
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {
