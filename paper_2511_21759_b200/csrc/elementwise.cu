@@ -1,4 +1,4 @@
-// Small memory-bound kernels between the GEMMs: embedding gather, residual + split-K reduction
+// Small memory-bound kernels between the GEMMs: residual (at first: the embedding) + split-K reduction
 // + RMSNorm operand, split-K reduction + RoPE + K/V cache scatter, and the vocab-wide confidence
 // reduction (SwiGLU lives in the gate/up GEMM's epilogue).  All reductions run in a fixed order (bitwise reproducible).
 #include "odb_internal.cuh"
@@ -22,6 +22,14 @@ __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d) 
     return pk;
 }
 
+// x^2 + y^2 + z^2 + w^2 with the roundings spelled out, so that every variant of an RMSNorm kernel gives the same bits
+// (a last bit here flips bf16 roundings in every layer behind): SECOND_FIRST starts with y^2, as the few-row kernel does.
+template <bool SECOND_FIRST>
+__device__ __forceinline__ float squares4(const float4& v) {
+    const float t = SECOND_FIRST ? __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)) : __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x));
+    return __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, t));
+}
+
 // block-wide sum, same value returned to every thread; `red` has >= 32 floats
 __device__ __forceinline__ float block_sum(float v, float* red) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -34,17 +42,11 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
     return t;
 }
 
-__global__ void embed_kernel(const __nv_bfloat16* __restrict__ embed, const int32_t* __restrict__ row_tok,
-                             float* __restrict__ h, int d) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int row = blockIdx.x;
-    const __nv_bfloat16* src = embed + static_cast<size_t>(row_tok[row]) * d;
-    float* dst = h + static_cast<size_t>(row) * d;
-    for (int i = threadIdx.x * 2; i < d; i += blockDim.x * 2) {
-        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(src + i);
-        *reinterpret_cast<float2*>(dst + i) = __bfloat1622float2(v);
-    }
+// float4 i of the embedding row of row r's token
+__device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i, int d) {
+    const uint2 x = reinterpret_cast<const uint2*>(e.table + static_cast<size_t>(e.row_tok[r]) * d)[i];
+    return make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xffff0000u), __uint_as_float(x.y << 16),
+                       __uint_as_float(x.y & 0xffff0000u));
 }
 
 // grid (output rows, slices of kNormSliceCols columns), one float4 per thread: the part of RMSNorm that is
@@ -55,7 +57,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __re
                                                                      int splits, size_t pstride, const float* __restrict__ gain,
                                                                      __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                      const int32_t* __restrict__ row_map, int d, L2Prefetch pf,
-                                                                     TpWait tw) {
+                                                                     TpWait tw, EmbedSource emb) {
     __shared__ float red[32];
     pdl_launch_dependents();
     pdl_wait();
@@ -67,7 +69,8 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __re
     float ss = 0.f;
     if (i < (d >> 2)) {
         float* hr = h + static_cast<size_t>(row) * d;
-        float4 v = reinterpret_cast<const float4*>(hr)[i];
+        float4 v = emb.table ? embed_load4(emb, row, i, d) : reinterpret_cast<const float4*>(hr)[i];
+        if (emb.table) reinterpret_cast<float4*>(hr)[i] = v;   // first norm of a forward
         if (partial) {
             const float* p = partial + static_cast<size_t>(row) * d + 4 * i;
             float4 t[16];
@@ -79,7 +82,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __re
                 if (u < splits) { v.x += t[u].x; v.y += t[u].y; v.z += t[u].z; v.w += t[u].w; }
             reinterpret_cast<float4*>(hr)[i] = v;
         }
-        ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        ss = squares4<true>(v);
         const float4 g = reinterpret_cast<const float4*>(gain)[i];
         const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x * g.x, v.y * g.y);
         const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z * g.z, v.w * g.w);
@@ -97,20 +100,25 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __re
 // (768 rows x 4096, three splits: 21 -> 14.5 us per launch).  Same sums in the same order per row.
 constexpr int kNormRows = 4;
 constexpr int kNormRowsMaxSplits = 4;
+// SPLITS: most partials per row (0: the projection in front has added to the residual stream itself), a template
+// parameter because the loads in flight are registers: with room for four splits two blocks fit an SM, without any
+// eight do (25568 rows x 4096: 247 us with one partial in the four-split kernel, 90 us with none).
+// EMBED: the first norm of a forward; the residual stream is the embedding row of each row's token.
+template <int SPLITS, bool EMBED>
 __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float* __restrict__ h, const float* __restrict__ partial,
                                                                           int splits, size_t pstride,
                                                                           const float* __restrict__ gain,
                                                                           __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                           const int32_t* __restrict__ row_map, int rows_out, int d,
-                                                                          TpWait tw) {
+                                                                          TpWait tw, EmbedSource emb) {
     __shared__ float red[kNormRows][32];
     pdl_launch_dependents();
     pdl_wait();
-    tp_wait_flags(tw);
+    if (SPLITS > 0) tp_wait_flags(tw);
     const int i = blockIdx.y * (kNormSliceCols / 4) + threadIdx.x;   // float4 index within the row
     const int orow0 = blockIdx.x * kNormRows;
     const bool in = i < (d >> 2);
-    float4 v[kNormRows], t[kNormRows][kNormRowsMaxSplits];
+    float4 v[kNormRows], t[kNormRows][SPLITS > 0 ? SPLITS : 1];
     int row[kNormRows];
 #pragma unroll
     for (int r = 0; r < kNormRows; ++r) {
@@ -120,11 +128,11 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
 #pragma unroll
     for (int r = 0; r < kNormRows; ++r) {
         if (!in || row[r] < 0) continue;
-        v[r] = reinterpret_cast<const float4*>(h + static_cast<size_t>(row[r]) * d)[i];
-        if (partial) {
+        v[r] = EMBED ? embed_load4(emb, row[r], i, d) : reinterpret_cast<const float4*>(h + static_cast<size_t>(row[r]) * d)[i];
+        if (SPLITS > 0) {
             const float* p = partial + static_cast<size_t>(row[r]) * d + 4 * i;
 #pragma unroll
-            for (int u = 0; u < kNormRowsMaxSplits; ++u)
+            for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) t[r][u] = *reinterpret_cast<const float4*>(p + static_cast<size_t>(u) * pstride);
         }
     }
@@ -136,13 +144,13 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
         ss[r] = 0.f;
         if (!in || row[r] < 0) continue;
         float4 x = v[r];
-        if (partial) {
+        if (SPLITS > 0) {
 #pragma unroll
-            for (int u = 0; u < kNormRowsMaxSplits; ++u)
+            for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) { x.x += t[r][u].x; x.y += t[r][u].y; x.z += t[r][u].z; x.w += t[r][u].w; }
-            reinterpret_cast<float4*>(h + static_cast<size_t>(row[r]) * d)[i] = x;
         }
-        ss[r] = x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+        if (SPLITS > 0 || EMBED) reinterpret_cast<float4*>(h + static_cast<size_t>(row[r]) * d)[i] = x;
+        ss[r] = squares4<false>(x);
         reinterpret_cast<uint2*>(out + static_cast<size_t>(orow0 + r) * d)[i] = pack4_bf16(x.x * g.x, x.y * g.y, x.z * g.z, x.w * g.w);
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -485,25 +493,35 @@ cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink
     return cudaGetLastError();
 }
 
-// First kernel of a forward.  Launched WITHOUT programmatic stream serialization: it starts only when
-// everything enqueued before it (the row and tile tables, the previous accept) has completed, and every
-// later kernel of the chain starts after this one has started.  That is what allows the attention
-// kernels to read the tile table and the K/V cache before their own griddepcontrol.wait.
-cudaError_t launch_embed(const __nv_bfloat16* embed, const int32_t* row_tok, float* h, int M, int d, cudaStream_t st) {
-    embed_kernel<<<dim3(M), dim3(256), 0, st>>>(embed, row_tok, h, d);
-    return cudaGetLastError();
+template <int SPLITS, bool EMBED>
+static cudaError_t launch_norm_rows(bool first, float* h, const float* partial, int splits, size_t pstride, const float* gain,
+                                    __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, cudaStream_t st,
+                                    const TpWait& tw, const EmbedSource& emb) {
+    return launch_kernel_if(!first, rmsnorm_rows_kernel<SPLITS, EMBED>,
+                            dim3((rows_out + kNormRows - 1) / kNormRows, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4),
+                            0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, emb);
 }
 
+// The first norm (emb.table set) is the first kernel of a forward.  It is launched WITHOUT programmatic stream
+// serialization: it starts only when everything enqueued before it (the row and tile tables, the previous accept) has
+// completed, and every later kernel of the chain starts after this one has started.  That is what allows the
+// attention kernels to read the tile table and the K/V cache before their own griddepcontrol.wait.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw) {
+                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb) {
     if (splits > 16) return cudaErrorInvalidValue;
-    const int slices = (d + kNormSliceCols - 1) / kNormSliceCols;
-    if (rows_out >= 256 && splits <= kNormRowsMaxSplits)
-        return launch_kernel(rmsnorm_rows_kernel, dim3((rows_out + kNormRows - 1) / kNormRows, slices), dim3(kNormSliceCols / 4), 0,
-                             st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw);
-    return launch_kernel(rmsnorm_kernel, dim3(rows_out, slices), dim3(kNormSliceCols / 4), 0, st, h, partial, splits, pstride,
-                         gain, out, ssq, row_map, d, pf, tw);
+    const bool first = emb.table != nullptr;
+    if (first && (partial || row_map)) return cudaErrorInvalidValue;
+    if (rows_out >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
+        if (first) return launch_norm_rows<0, true>(true, h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb);
+        if (!partial) return launch_norm_rows<0, false>(false, h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb);
+        if (splits == 1)
+            return launch_norm_rows<1, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb);
+        return launch_norm_rows<kNormRowsMaxSplits, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
+                                                           tw, emb);
+    }
+    return launch_kernel_if(!first, rmsnorm_kernel, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
+                            st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb);
 }
 
 cudaError_t launch_qkv_rope(const QkvRopeArgs& a, cudaStream_t st) {

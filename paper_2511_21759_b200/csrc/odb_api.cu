@@ -661,6 +661,19 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         }
         return launch_gemm(ga, st);
     };
+    // many rows, no K split: the product goes straight into the residual stream, no partial sums in memory
+    auto gemm_add = [&](const CUtensorMap& tw, const __nv_bfloat16* x, int K) {
+        GemmArgs ga;
+        ga.tmap_w = tw;
+        ga.x = x;
+        ga.partial = nullptr;
+        ga.act_out = nullptr;
+        ga.add_to = h;
+        ga.M = M; ga.N = d; ga.K = K;
+        ga.splits = 1;
+        ga.status = status;
+        return launch_gemm(ga, st);
+    };
 #define ODB_LAUNCH(kind, call)          \
     do {                                \
         LaunchScope scope__(s, kind);   \
@@ -714,7 +727,6 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         }
         return ODB_OK;
     }
-    ODB_FWD(ODB_KIND_ELEMENTWISE, launch_embed(m->embed, s->cb.row_tok, h, M, d, st));
     const float* res = nullptr;   // split-K partials of the projection not yet added to the residual stream
     TpWait res_wait;              // tensor parallelism: the flags those partials are complete behind
     int res_splits = 0;
@@ -742,8 +754,10 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     const size_t qkv_bytes = packed_weight_bytes(3 * da, d), o_bytes = packed_weight_bytes(d, da),
                  gu_bytes = packed_gate_up_bytes(F, d);
     for (int l = 0; l < c.n_layers; ++l) {
+        EmbedSource emb;
+        if (l == 0) { emb.table = m->embed; emb.row_tok = s->cb.row_tok; }
         ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d,
-                                                        hint_of(m->p_qkv[l], qkv_bytes, 0), st, res_wait));
+                                                        hint_of(m->p_qkv[l], qkv_bytes, 0), st, res_wait, emb));
         int sp = plan_splits(M, 3 * da, d, false);
         QkvRopeArgs qa;
         qa.partial = partial; qa.splits = sp; qa.pstride = static_cast<size_t>(M) * 3 * da;
@@ -839,6 +853,9 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             o_wait = end_exchange(0);
             o_sum = tp.recv[c.tp_rank];
             o_parts = R * sp;
+        } else if (sp == 1 && gemm_rows_usable(M, d)) {
+            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->tm_o[l], o, da));
+            o_sum = nullptr;
         } else {
             ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_o[l], o, partial, M, d, da, sp));
         }
@@ -874,7 +891,10 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             res_wait = end_exchange(1);
             res = tp.recv[c.tp_rank] + L.tp_recv_slot / sizeof(float);
             res_splits = R * sp;
-        } else {
+        } else if (sp == 1 && gemm_rows_usable(M, d) && !(c.with_lm_head && l == c.n_layers - 1)) {
+            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->tm_d[l], g, F));
+            res = nullptr; res_splits = 0;
+        } else {   // also in front of the LM head, whose norm reads the response rows only
             ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_d[l], g, partial, M, d, F, sp));
             res = partial; res_splits = sp;
         }

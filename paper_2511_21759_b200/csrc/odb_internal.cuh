@@ -70,8 +70,8 @@ __device__ __forceinline__ void l2_prefetch_slice(const L2Prefetch& pf, int cta,
 #endif
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                          Args&&... args) {
+cudaError_t launch_kernel_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args&&... args) {   // early: with programmatic stream serialization
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -81,8 +81,12 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = early && pdl_enabled() ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    return launch_kernel_if(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -343,8 +347,11 @@ cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stri
 cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink, int grid, cudaStream_t st);
 // bulk-copy ring probe; *streamed = the bytes one launch reads (whole chunks per CTA); `status` is a device word
 cudaError_t launch_bulk_read_stream(const void* src, size_t bytes, int grid, int* status, size_t* streamed, cudaStream_t st);
-cudaError_t launch_embed(const __nv_bfloat16* embed, const int32_t* row_tok, float* h, int M, int d,
-                         cudaStream_t st);
+// table non-null: the residual stream of row r starts as the embedding of token row_tok[r] (first norm of a forward)
+struct EmbedSource {
+    const __nv_bfloat16* table = nullptr;
+    const int32_t* row_tok = nullptr;
+};
 // The part of RMSNorm that is not a row scalar, for rows r = map ? map[i] : i of the residual stream:
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's
 // operand, ssq[i][t] = sum of h[r]^2 over the t-th slice of kNormSliceCols columns; the projection's consumer
@@ -352,7 +359,7 @@ cudaError_t launch_embed(const __nv_bfloat16* embed, const int32_t* row_tok, flo
 // product).  splits <= 16.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw = TpWait());
+                           cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource());
 // SwiGLU of a gate/up projection that ran with K splits (few weight tiles: a tensor-parallel shard): partial is fp32
 // [splits][M][tiles * 128] in the packed gate/up order (tile t = gate features [64t, 64t+64), then the same up
 // features); g[m][f] = bf16(silu(gate) * up) with gate, up = the split sums (split order) times the row scalar.
