@@ -21,27 +21,29 @@ __global__ void build_refresh_rows_kernel(ControlBuffers c, int batch, BlockInde
         if (threadIdx.x == 0) st->in_fwd = 0;
         return;
     }
+    // what the sequences in front take: one thread per sequence (serially, sixteen sequences were 9 us of dependent loads)
     __shared__ int row0, lm0, tile0, big0;
-    if (threadIdx.x == 0) {
-        int r = 0, l = 0, t = 0, tb = 0;
-        for (int j = 0; j < seq; ++j) {
-            const SeqState* o = c.state + j;
-            if (!o->active || bp.block_index[j] < 0) continue;
-            const int sj = o->P + bp.block_index[j] * bp.block_len;
-            r += o->T;
-            l += o->T - sj;
-            t += (o->T + 63) / 64;
-            tb += (o->T + 127) / 128;
+    if (threadIdx.x == 0) row0 = lm0 = tile0 = big0 = 0;
+    __syncthreads();
+    if (threadIdx.x < seq) {
+        const SeqState* o = c.state + threadIdx.x;
+        if (o->active && bp.block_index[threadIdx.x] >= 0) {
+            atomicAdd(&row0, o->T);
+            atomicAdd(&lm0, o->T - (o->P + bp.block_index[threadIdx.x] * bp.block_len));
+            atomicAdd(&tile0, (o->T + 63) / 64);
+            atomicAdd(&big0, (o->T + 127) / 128);
         }
-        row0 = r; lm0 = l; tile0 = t; big0 = tb;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         const int s = st->P + bp.block_index[seq] * bp.block_len;
         st->in_fwd = 1;
         st->block_idx = bp.block_index[seq];
         st->s = s;
         st->e = min(s + bp.block_len, st->T);
-        st->row0 = r;
+        st->row0 = row0;
         st->n_rows = st->T;
-        st->lm_row0 = l;
+        st->lm_row0 = lm0;
         st->lm_s = s;
         st->lm_n = st->T - s;
         st->n_ranks = 0;
@@ -49,7 +51,6 @@ __global__ void build_refresh_rows_kernel(ControlBuffers c, int batch, BlockInde
         st->copy_mask[0] = 0;
         st->stage2 = 0;
     }
-    __syncthreads();
     const int T = st->T;
     const int s = st->P + bp.block_index[seq] * bp.block_len;
     const int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
@@ -97,35 +98,45 @@ __device__ int step_tiles_of(const SeqState* st) {
     return step_tiles_of_counts(st->n_copies, B, st->stage2 ? st->n_masked : B);
 }
 
-__global__ void build_step_rows_kernel(ControlBuffers c, int batch, int mask_id) {
-    const int seq = blockIdx.x;
-    SeqState* st = c.state + seq;
+// One block per sequence.  The state is worked on in shared memory and the sequences in front are counted by one thread
+// each: written as one thread's walk over global memory this was 6 us at batch 1 and 22 us at batch 16.
+__global__ void __launch_bounds__(64) build_step_rows_kernel(ControlBuffers c, int batch, int mask_id) {
+    const int seq = blockIdx.x, tid = threadIdx.x;
+    __shared__ SeqState sst;
+    __shared__ int xs[kMaxBlock];      // the block's committed tokens
+    __shared__ unsigned masked_w[2];   // bit i: position i of the block is masked
+    __shared__ int row_base, tile_base, stile_base;
+    __shared__ StepTile items[ODB_MAX_COPIES];
+    {
+        const int* gs = reinterpret_cast<const int*>(c.state + seq);
+        for (int i = tid; i < static_cast<int>(sizeof(SeqState) / 4); i += 64) reinterpret_cast<int*>(&sst)[i] = gs[i];
+        if (tid == 0) row_base = tile_base = stile_base = 0;
+    }
+    __syncthreads();
+    SeqState* st = &sst;
     if (!st->active || st->n_masked <= 0) {
-        if (threadIdx.x == 0) st->in_fwd = 0;
+        if (tid == 0) c.state[seq].in_fwd = 0;
         return;
     }
-    __shared__ int xs[kMaxBlock];      // the block's committed tokens
-    __shared__ int mpre[kMaxBlock];    // masked positions before position i of the block
-    __shared__ int row_base, tile_base;
     const int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
-    const int s = st->s, e = st->e, B = e - s;
-    for (int i = threadIdx.x; i < B; i += blockDim.x) xs[i] = x[s + i];
+    const int s = st->s, e = st->e, B = e - s;   // B <= kMaxBlock = blockDim
+    const int my_tok = tid < B ? x[s + tid] : 0;
+    if (tid < seq) {
+        const SeqState* o = c.state + tid;
+        if (o->active && o->n_masked > 0) {
+            atomicAdd(&row_base, step_rows_of(o));
+            atomicAdd(&tile_base, o->n_copies);
+            atomicAdd(&stile_base, step_tiles_of(o));
+        }
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, tid < B && my_tok == mask_id);
+    if ((tid & 31) == 0) masked_w[tid >> 5] = bal;
+    xs[tid] = my_tok;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
+        const int nm = __popc(masked_w[0]) + __popc(masked_w[1]);
+        int row = row_base;
         st->in_fwd = 1;
-        int row = 0, tile = 0;
-        for (int j = 0; j < seq; ++j) {
-            const SeqState* o = c.state + j;
-            if (!o->active || o->n_masked <= 0) continue;
-            row += step_rows_of(o);
-            tile += o->n_copies;
-        }
-        int nm = 0;
-        for (int i = 0; i < B; ++i) {
-            mpre[i] = nm;
-            nm += xs[i] == mask_id;
-        }
-        row_base = row; tile_base = tile;
         st->row0 = row;
         // copy 0 holds the whole block; a speculative copy the whole block or, in the decoded-share layout, the
         // positions still masked
@@ -134,15 +145,18 @@ __global__ void build_step_rows_kernel(ControlBuffers c, int batch, int mask_id)
             st->copy_nrows[cp] = (st->stage2 && cp > 0) ? nm : B;
             row += st->copy_nrows[cp];
         }
+        st->n_rows = row - st->row0;
+        st->lm_row0 = st->row0;
     }
     __syncthreads();
+    const unsigned long long masked = static_cast<unsigned long long>(masked_w[1]) << 32 | masked_w[0];
     // one thread per (copy, position): the rows of the copies, copy after copy
-    for (int it = threadIdx.x; it < st->n_copies * B; it += blockDim.x) {
+    for (int it = tid; it < st->n_copies * B; it += 64) {
         const int cp = it / B, i = it % B;
-        const bool decoded = xs[i] != mask_id;
+        const bool decoded = !((masked >> i) & 1ull);
         const bool shared = st->stage2 && cp > 0;
         if (shared && decoded) continue;
-        const int row = st->copy_row0[cp] + (shared ? mpre[i] : i);
+        const int row = st->copy_row0[cp] + (shared ? __popcll(masked & ((1ull << i) - 1ull)) : i);
         int tok = xs[i];
         for (int r = 0; r < st->n_ranks; ++r)
             if (((st->copy_mask[cp] >> r) & 1) && st->rank_off[r] == i) tok = st->rank_tok[r];
@@ -153,11 +167,8 @@ __global__ void build_step_rows_kernel(ControlBuffers c, int batch, int mask_id)
         c.row_flags[row] = decoded ? kRowDecoded : 0;
         c.lm_rows[row] = row;
     }
-    if (threadIdx.x != 0) return;
-    int row = row_base;
-    const int tile = tile_base;
-    for (int cp = 0; cp < st->n_copies; ++cp) {
-        row += st->copy_nrows[cp];
+    if (tid < st->n_copies) {
+        const int cp = tid;
         QTile q;
         q.q_row0 = st->copy_row0[cp];
         q.nq = st->copy_nrows[cp];
@@ -167,77 +178,94 @@ __global__ void build_step_rows_kernel(ControlBuffers c, int batch, int mask_id)
         const bool shared = st->stage2 && cp > 0;
         q.f1 = shared ? st->copy_row0[0] : 0;
         q.n1 = shared ? st->copy_nrows[0] : 0;
-        c.tiles[tile + cp] = q;
+        c.tiles[tile_base + cp] = q;
     }
-    st->n_rows = row - st->row0;
-    st->lm_row0 = st->row0;
     // attention work items that share the cached K/V among copies: copies are packed, in order, into
     // items of at most 8 slabs of 16 rows (the host counts them with the same rule, step_tiles_of)
-    int stile = 0;
-    for (int j = 0; j < seq; ++j) {
-        const SeqState* o = c.state + j;
-        if (!o->active || o->n_masked <= 0) continue;
-        stile += step_tiles_of(o);
-    }
-    StepTile cur{};
-    int have = 0;
-    auto add_src = [&](int cp) {
-        for (int i = 0; i < cur.n_src; ++i)
-            if (cur.src_copy[i] == cp) return;
-        cur.src_copy[cur.n_src] = cp;
-        cur.src_row0[cur.n_src] = st->copy_row0[cp];
-        cur.src_n[cur.n_src] = st->copy_nrows[cp];
-        ++cur.n_src;
-    };
-    auto flush = [&]() {
-        if (st->stage2) add_src(0);   // copy 0's decoded rows are visible to every speculative copy
-        c.step_tiles[stile++] = cur;
-        have = 0;
-    };
-    for (int cp = 0; cp < st->n_copies; ++cp) {
-        const int slabs = (st->copy_nrows[cp] + 15) / 16;
-        if (have && cur.n_slabs + slabs > 8) flush();
-        if (!have) {
-            cur.seq = seq; cur.cA = s; cur.cB0 = e; cur.cB1 = st->T;
-            cur.n_slabs = 0; cur.n_src = 0; cur.stage2 = st->stage2;
-            have = 1;
+    __shared__ int n_items;
+    if (tid == 32) {
+        int have = 0, n = 0;
+        StepTile* cur = items;
+        auto add_src = [&](int cp) {
+            for (int i = 0; i < cur->n_src; ++i)
+                if (cur->src_copy[i] == cp) return;
+            cur->src_copy[cur->n_src] = cp;
+            cur->src_row0[cur->n_src] = st->copy_row0[cp];
+            cur->src_n[cur->n_src] = st->copy_nrows[cp];
+            ++cur->n_src;
+        };
+        auto flush = [&]() {
+            if (st->stage2) add_src(0);   // copy 0's decoded rows are visible to every speculative copy
+            ++cur; ++n;
+            have = 0;
+        };
+        for (int cp = 0; cp < st->n_copies; ++cp) {
+            const int slabs = (st->copy_nrows[cp] + 15) / 16;
+            if (have && cur->n_slabs + slabs > 8) flush();
+            if (!have) {
+                cur->seq = seq; cur->cA = s; cur->cB0 = e; cur->cB1 = st->T;
+                cur->n_slabs = 0; cur->n_src = 0; cur->stage2 = st->stage2;
+                have = 1;
+            }
+            for (int k = 0; k < slabs; ++k) {
+                cur->slab_copy[cur->n_slabs] = cp;
+                cur->slab_row0[cur->n_slabs] = st->copy_row0[cp] + 16 * k;
+                cur->slab_n[cur->n_slabs] = min(16, st->copy_nrows[cp] - 16 * k);
+                ++cur->n_slabs;
+            }
+            add_src(cp);
         }
-        for (int k = 0; k < slabs; ++k) {
-            cur.slab_copy[cur.n_slabs] = cp;
-            cur.slab_row0[cur.n_slabs] = st->copy_row0[cp] + 16 * k;
-            cur.slab_n[cur.n_slabs] = min(16, st->copy_nrows[cp] - 16 * k);
-            ++cur.n_slabs;
-        }
-        add_src(cp);
+        if (have) flush();
+        n_items = n;
     }
-    if (have) flush();
+    __syncthreads();
+    {   // entries of an item beyond its counts are never read
+        const int words = n_items * static_cast<int>(sizeof(StepTile) / 4);
+        int* dst = reinterpret_cast<int*>(c.step_tiles + stile_base);
+        for (int i = tid; i < words; i += 64) dst[i] = reinterpret_cast<const int*>(items)[i];
+    }
+    // the placement back to the device state; other blocks read active, s, e, n_masked, n_copies, stage2 only, which stay
+    SeqState* gst = c.state + seq;
+    if (tid == 0) {
+        gst->in_fwd = 1;
+        gst->row0 = st->row0; gst->n_rows = st->n_rows; gst->lm_row0 = st->lm_row0;
+    }
+    if (tid < st->n_copies) {
+        gst->copy_row0[tid] = st->copy_row0[tid];
+        gst->copy_nrows[tid] = st->copy_nrows[tid];
+    }
 }
+
+typedef unsigned long long Mask;   // bit i: position i of the block (blocks have at most 64 positions)
 
 // Accept rule (Section 3, Observation 3): every masked position whose confidence exceeds tau
 // (strict); if none, the single most confident one (lowest position on a tie).
-__device__ int accept_set(const float* conf, const bool* masked, int B, float tau, bool* acc) {
-    int n = 0, best = -1;
-    for (int i = 0; i < B; ++i) {
-        acc[i] = masked[i] && conf[i] > tau;
-        n += acc[i];
-        if (masked[i] && (best < 0 || conf[i] > conf[best])) best = i;
+__device__ Mask accept_set(const float* conf, Mask masked, float tau) {
+    Mask acc = 0;
+    int best = -1;
+    float best_conf = 0.f;
+    for (Mask left = masked; left; left &= left - 1) {
+        const int i = __ffsll(left) - 1;
+        const float ci = conf[i];
+        if (ci > tau) acc |= 1ull << i;
+        if (best < 0 || ci > best_conf) { best = i; best_conf = ci; }
     }
-    if (n == 0 && best >= 0) { acc[best] = true; n = 1; }
-    return n;
+    if (acc == 0 && best >= 0) acc = 1ull << best;
+    return acc;
 }
 
 // Stochastic reverse step (Section 2.1, Eq. 1) at iteration k of the n_steps a block is decoded in: a masked
 // position stays masked with probability s / t = (n_steps - k - 1) / (n_steps - k), decided by its uniform
 // deviate u (unmask iff u >= s / t, in fp32); the last iteration unmasks everything left.
-__device__ int sample_set(const float* u, const bool* masked, int B, int k, int n_steps, bool* acc) {
-    const bool all = k >= n_steps - 1;
-    const float stay = all ? 0.f : static_cast<float>(n_steps - k - 1) / static_cast<float>(n_steps - k);
-    int n = 0;
-    for (int i = 0; i < B; ++i) {
-        acc[i] = masked[i] && (all || u[i] >= stay);
-        n += acc[i];
+__device__ Mask sample_set(const float* u, Mask masked, int k, int n_steps) {
+    if (k >= n_steps - 1) return masked;
+    const float stay = static_cast<float>(n_steps - k - 1) / static_cast<float>(n_steps - k);
+    Mask acc = 0;
+    for (Mask left = masked; left; left &= left - 1) {
+        const int i = __ffsll(left) - 1;
+        if (u[i] >= stay) acc |= 1ull << i;
     }
-    return n;
+    return acc;
 }
 
 // st / res: the block's shared-memory copies of the sequence's state and result (the decisions are one thread's
@@ -258,20 +286,44 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
     }
     __shared__ float conf[ODB_MAX_COPIES][kMaxBlock];
     __shared__ int tok[ODB_MAX_COPIES][kMaxBlock];
-    __shared__ int xs[kMaxBlock];          // the block's committed tokens (step only)
+    __shared__ int xs[kMaxBlock];          // the block's committed tokens
+    __shared__ int first_eos;
     int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
     const int s = st->s;
-    int n_copies = 1;
-    // After a step the whole block gathers the copies' confidences and tokens and the block's tokens (the
-    // decisions below are taken by thread 0 alone, in the order the method states them)
-    const bool gathered = !dry && !after_refresh;
-    if (gathered) {
-        n_copies = st->n_copies;
+    const int n_copies = after_refresh || dry ? 1 : st->n_copies;
+    // The whole block gathers what the decisions need - the [EOS] scan of a refresh, the copies' confidences and tokens,
+    // the block's tokens; the decisions below are taken by thread 0 alone, in the order the method states them.  (One
+    // thread scanning and gathering a 256-token response: 42 us; the block: 12 us.)
+    if (after_refresh) {
+        // adaptive length prediction (Section 4.1): first [EOS] of the whole predicted response
+        // whose confidence exceeds the truncate threshold cuts the response there (slot kept)
+        const bool alp = p.alp && !dry;
+        if (threadIdx.x == 0) first_eos = 0x7fffffff;
+        __syncthreads();
+        if (alp)
+            for (int q = s + threadIdx.x; q < st->T; q += blockDim.x) {
+                const int r = st->lm_row0 + (q - st->lm_s);
+                if (c.tok[r] == eos_id && c.conf[r] > p.truncate_threshold) { atomicMin(&first_eos, q); break; }
+            }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (first_eos != 0x7fffffff) st->T = first_eos + 1;
+            st->e = min(s + p.block_len, st->T);
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) xs[i] = x[s + i];
+    if (!dry && after_refresh) {
+        for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) {
+            const int r = st->lm_row0 + (s + i - st->lm_s);
+            conf[0][i] = c.conf[r];
+            tok[0][i] = c.tok[r];
+        }
+    } else if (!dry) {
         for (int i = threadIdx.x; i < n_copies * kMaxBlock; i += blockDim.x) {
             conf[i / kMaxBlock][i % kMaxBlock] = -1.f;
             tok[i / kMaxBlock][i % kMaxBlock] = -1;
         }
-        for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) xs[i] = x[s + i];
         __syncthreads();
         for (int cp = 0; cp < n_copies; ++cp) {
             const int r0 = st->copy_row0[cp], r1 = r0 + st->copy_nrows[cp];
@@ -281,20 +333,19 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
                 tok[cp][i] = c.tok[r];
             }
         }
-        __syncthreads();
     }
+    __syncthreads();
     if (threadIdx.x != 0) return;
 
     if (dry) {
         // model without LM head (layer microbenchmark): there is nothing to decide on, so commit
         // nothing and lay out the next step as if no position had been accepted; the speculative
         // fills are the first masked positions with token id 0
-        if (after_refresh) st->e = min(s + p.block_len, st->T);
         const int B = st->e - s;
         int n_masked = 0, n_ranks = 0;
         const int k_ranks = p.n_copies >= 8 ? 4 : p.n_copies >= 4 ? 2 : 0;
         for (int i = 0; i < B; ++i) {
-            if (x[s + i] != mask_id) continue;
+            if (xs[i] != mask_id) continue;
             if (n_ranks < k_ranks) { st->rank_off[n_ranks] = i; st->rank_tok[n_ranks] = 0; ++n_ranks; }
             ++n_masked;
         }
@@ -318,29 +369,13 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         res->block_end = st->e;
         return;
     }
-    if (after_refresh) {
-        // adaptive length prediction (Section 4.1): first [EOS] of the whole predicted response
-        // whose confidence exceeds the truncate threshold cuts the response there (slot kept)
-        if (p.alp) {
-            for (int q = s; q < st->T; ++q) {
-                const int r = st->lm_row0 + (q - st->lm_s);
-                if (c.tok[r] == eos_id && c.conf[r] > p.truncate_threshold) { st->T = q + 1; break; }
-            }
-        }
-        st->e = min(s + p.block_len, st->T);
-        for (int i = 0; i < st->e - s; ++i) {
-            const int r = st->lm_row0 + (s + i - st->lm_s);
-            conf[0][i] = c.conf[r];
-            tok[0][i] = c.tok[r];
-        }
-    }
     const int B = st->e - s;
     if (after_refresh) st->block_iter = 0;
     const int k_iter = st->block_iter < kMaxLoopIters ? st->block_iter : kMaxLoopIters - 1;
     const float* noise = c.noise + (static_cast<size_t>(seq) * kMaxLoopIters + k_iter) * kMaxBlock;
     ++st->block_iter;
-    bool masked0[kMaxBlock], masked[kMaxBlock], acc[kMaxBlock], taken[kMaxBlock];
-    for (int i = 0; i < B; ++i) { masked0[i] = (gathered ? xs[i] : x[s + i]) == mask_id; taken[i] = false; }
+    Mask masked0 = 0, taken = 0;
+    for (int i = 0; i < B; ++i) masked0 |= static_cast<Mask>(xs[i] == mask_id) << i;
 
     // accept-jump walk (Section 4.2.1): start in the main block; a candidate is hit if its
     // position was accepted with the token it had been filled with; jump to the largest copy
@@ -348,14 +383,26 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
     // an earlier link winning at a shared position
     int cur = 0, chain_len = 0, n_acc = 0;
     const bool pick = p.pick_best && !after_refresh;
+    auto commit = [&](int i, int t) {
+        taken |= 1ull << i;
+        x[s + i] = t;
+        if (n_acc < 64) { res->accepted_pos[n_acc] = s + i; res->accepted_tok[n_acc] = t; }
+        ++n_acc;
+    };
+    auto commit_all = [&](Mask m) {   // the block's positions in m that no earlier link has taken
+        for (Mask left = m & ~taken; left; left &= left - 1) {
+            const int i = __ffsll(left) - 1;
+            commit(i, tok[cur][i]);
+        }
+    };
     if (pick) {
         // the compared speculation (Fig. 7(a), Section 5.3): candidates verified in the main block only; the copy
         // filling the largest set of hits is adopted, and its fills and own accept set are the whole result
-        accept_set(conf[0], masked0, B, p.accept_threshold, acc);
+        Mask acc = accept_set(conf[0], masked0, p.accept_threshold);
         int hit = 0;
         for (int r = 0; r < st->n_ranks; ++r) {
             const int o = st->rank_off[r];
-            if (acc[o] && tok[0][o] == st->rank_tok[r]) hit |= 1 << r;
+            if (((acc >> o) & 1) && tok[0][o] == st->rank_tok[r]) hit |= 1 << r;
         }
         for (int cp = 1; cp < n_copies; ++cp) {
             const int Y = st->copy_mask[cp];
@@ -364,24 +411,14 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
                 (__popc(Y) == __popc(st->copy_mask[cur]) && Y < st->copy_mask[cur]))
                 cur = cp;
         }
-        auto commit = [&](int i, int t) {
-            taken[i] = true;
-            x[s + i] = t;
-            if (n_acc < 64) { res->accepted_pos[n_acc] = s + i; res->accepted_tok[n_acc] = t; }
-            ++n_acc;
-        };
         if (cur != 0) {
             const int Y = st->copy_mask[cur];
-            bool any = false;
-            for (int i = 0; i < B; ++i) masked[i] = masked0[i];
+            Mask masked = masked0;
             for (int r = 0; r < st->n_ranks; ++r)
-                if ((Y >> r) & 1) { masked[st->rank_off[r]] = false; commit(st->rank_off[r], st->rank_tok[r]); }
-            for (int i = 0; i < B; ++i) any |= masked[i];
-            if (any) accept_set(conf[cur], masked, B, p.accept_threshold, acc);
-            else for (int i = 0; i < B; ++i) acc[i] = false;
+                if ((Y >> r) & 1) { masked &= ~(1ull << st->rank_off[r]); commit(st->rank_off[r], st->rank_tok[r]); }
+            acc = masked ? accept_set(conf[cur], masked, p.accept_threshold) : 0;
         }
-        for (int i = 0; i < B; ++i)
-            if (acc[i] && !taken[i]) commit(i, tok[cur][i]);
+        commit_all(acc);
         res->chain[0] = cur;
         chain_len = 1;
     }
@@ -389,27 +426,17 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         res->chain[chain_len < ODB_MAX_CHAIN ? chain_len : ODB_MAX_CHAIN - 1] = cur;
         ++chain_len;
         const int X = after_refresh ? 0 : st->copy_mask[cur];
-        bool any = false;
-        for (int i = 0; i < B; ++i) masked[i] = masked0[i];
+        Mask masked = masked0;
         for (int r = 0; r < st->n_ranks; ++r)
-            if ((X >> r) & 1) masked[st->rank_off[r]] = false;
-        for (int i = 0; i < B; ++i) any |= masked[i];
-        if (!any) break;
-        if (p.sampling) sample_set(noise, masked, B, k_iter, p.sample_steps, acc);
-        else accept_set(conf[cur], masked, B, p.accept_threshold, acc);
-        for (int i = 0; i < B; ++i) {
-            if (acc[i] && !taken[i]) {
-                taken[i] = true;
-                x[s + i] = tok[cur][i];
-                if (n_acc < 64) { res->accepted_pos[n_acc] = s + i; res->accepted_tok[n_acc] = tok[cur][i]; }
-                ++n_acc;
-            }
-        }
+            if ((X >> r) & 1) masked &= ~(1ull << st->rank_off[r]);
+        if (!masked) break;
+        const Mask acc = p.sampling ? sample_set(noise, masked, k_iter, p.sample_steps) : accept_set(conf[cur], masked, p.accept_threshold);
+        commit_all(acc);
         if (after_refresh) break;
         int hit = 0;
         for (int r = 0; r < st->n_ranks; ++r) {
             const int o = st->rank_off[r];
-            if (!((X >> r) & 1) && acc[o] && tok[cur][o] == st->rank_tok[r]) hit |= 1 << r;
+            if (!((X >> r) & 1) && ((acc >> o) & 1) && tok[cur][o] == st->rank_tok[r]) hit |= 1 << r;
         }
         int best = -1;
         for (int cp = 0; cp < n_copies; ++cp) {
@@ -425,19 +452,18 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
 
     // state after the walk; next candidates: the most confident still-masked positions of the
     // adopted copy (Section 4.2), ties to the lower position
-    int n_masked = 0;
-    for (int i = 0; i < B; ++i) {
-        masked[i] = masked0[i] && !taken[i];
-        n_masked += masked[i];
-    }
+    Mask open = masked0 & ~taken;
+    const int n_masked = __popcll(open);
     const int k_ranks = p.n_copies >= 8 ? 4 : p.n_copies >= 4 ? 2 : 0;
     int n_ranks = 0;
     for (int r = 0; r < k_ranks; ++r) {
         int best = -1;
-        for (int i = 0; i < B; ++i)
-            if (masked[i] && (best < 0 || conf[cur][i] > conf[cur][best])) best = i;
+        for (Mask left = open; left; left &= left - 1) {
+            const int i = __ffsll(left) - 1;
+            if (best < 0 || conf[cur][i] > conf[cur][best]) best = i;
+        }
         if (best < 0) break;
-        masked[best] = false;
+        open &= ~(1ull << best);
         st->rank_off[n_ranks] = best;
         st->rank_tok[n_ranks] = tok[cur][best];
         ++n_ranks;
@@ -498,7 +524,7 @@ __global__ void accept_kernel(ControlBuffers c, odb_decode_params p, int after_r
     __syncthreads();
     accept_store(c, &sh, c.host_results + blockIdx.x);
     if (blockIdx.x == 0 && threadIdx.x == 0) *c.host_status = *c.status;
-    __threadfence_system();
+    // no fence: the host reads after synchronising the stream, and the kernel's end makes its stores visible
 }
 
 // The accept of the device-resident loop: the same decisions, then the hand-over to the next iteration.
@@ -510,7 +536,7 @@ __global__ void accept_loop_kernel(ControlBuffers c, odb_decode_params p, int ma
     const int seq = blockIdx.x, batch = gridDim.x;
     const int it = *lc.iter;      // stable until every block has arrived below
     accept_store(c, &sh, lc.host_log + static_cast<size_t>(it) * batch + seq);
-    __threadfence_system();
+    __threadfence();              // the state, for the last block; the host log is read after the stream has been synchronised
     __syncthreads();
     if (threadIdx.x != 0) return;
     // fail-safe: the loop ends unless the last block below asks for another pass (block 0 writes this before it
@@ -539,7 +565,6 @@ __global__ void accept_loop_kernel(ControlBuffers c, odb_decode_params p, int ma
     *lc.iter = it + 1;
     *lc.host_iters = it + 1;
     *c.host_status = err;
-    __threadfence_system();
     cudaGraphSetConditional(lc.handle, again ? 1u : 0u);
 }
 
