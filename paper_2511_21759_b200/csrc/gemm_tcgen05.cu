@@ -327,35 +327,48 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             }
             if (po.n > 0 && t == 0) tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);   // behind the loop's last barrier
         } else {
-            // all MMAs have completed, so the stage ring is free: use it to hand the up values over.
-            // Every epilogue warp executes every barrier, whether or not its wait succeeded.
-            float* xch = reinterpret_cast<float*>(tiles);           // [64][33]
-            const int f = n_tile * 64 + (q & 1) * 32 + lane;          // FFN feature of this lane's pair
+            // All MMAs have completed, so the stage ring is free: the warps that own gate features hand the values of the
+            // tile's second half of rows to the warps that own the matching up features, and get the up values of the
+            // first half; behind one barrier every warp then finishes its half.  (Up values handed over chunk by chunk
+            // behind two barriers each, the up warps idle, as CTA pairs: 50 us for the 8B shape's gate/up projection at 128 rows; this
+            // way 47, and 36 instead of 38 at 32 rows.)
+            constexpr int kHalfRows = BN / 2, kPitch = kHalfRows + 1;
+            float* xch = reinterpret_cast<float*>(tiles);             // [gate | up][64 features][kPitch]
+            const int fl = (q & 1) * 32 + lane;                       // feature of this lane within the tile
+            const int f = n_tile * 64 + fl;
+            const bool is_gate = q < 2;
+            const uint32_t tm_lane = tmem_acc + (static_cast<uint32_t>(q * 32) << 16);
+            float* give = xch + (is_gate ? 0 : 64 * kPitch) + fl * kPitch;
+            const float* take = xch + (is_gate ? 64 * kPitch : 0) + fl * kPitch;
+            if (ok) {
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                uint32_t v[32];
-                if (ok) {
-                    tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
+                for (int c = 0; c < kHalfRows; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(tm_lane + static_cast<uint32_t>((is_gate ? kHalfRows : 0) + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                }
-                if (ok && q >= 2) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) xch[((q & 1) * 32 + lane) * 33 + j] = __uint_as_float(v[j]);
+                    for (int j = 0; j < 16; ++j) give[c + j] = __uint_as_float(v[j]);
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (ok && q < 2) {
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");            // every epilogue warp, whether or not its wait succeeded
+            if (ok) {
+                const int r0 = is_gate ? 0 : kHalfRows;
+#pragma unroll 1
+                for (int c = 0; c < kHalfRows; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(tm_lane + static_cast<uint32_t>(r0 + c), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int m = m0 + c * 32 + j;
-                        const float sc = rs.ssq ? sh->scale[c * 32 + j] : 1.0f;
+                    for (int j = 0; j < 16; ++j) {
+                        const int m = m0 + r0 + c + j;
+                        const float sc = rs.ssq ? sh->scale[r0 + c + j] : 1.0f;
                         if (m < M && f < N) {
-                            const float gate = __uint_as_float(v[j]) * sc;
-                            const float up = xch[((q & 1) * 32 + lane) * 33 + j] * sc;
+                            const float own = __uint_as_float(v[j]) * sc, other = take[c + j] * sc;
+                            const float gate = is_gate ? own : other, up = is_gate ? other : own;
                             act_out[static_cast<size_t>(m) * N + f] = __float2bfloat16_rn(gate / (1.0f + expf(-gate)) * up);
                         }
                     }
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
             }
         }
     }
@@ -498,11 +511,13 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
     const int nkb_per_split = (nkb_total + a.splits - 1) / a.splits;
     const uint32_t stage_bytes = kBM * kBK * 2 + kBRows * kBK * 2;
     // two CTAs per SM as long as two accumulators fit TMEM and a CTA stages at most 128 rows
-    const uint32_t budget = kBRows <= 128 ? 100 * 1024 : 200 * 1024;
+    const uint32_t budget = kBRows <= 128 && !PAIR ? 100 * 1024 : 200 * 1024;
     int stages = static_cast<int>(budget / stage_bytes);
     if (stages > 16) stages = 16;
     if (stages > nkb_per_split) stages = nkb_per_split < 2 ? 2 : nkb_per_split;
-    const size_t smem = static_cast<size_t>(stages) * stage_bytes + sizeof(GemmShared) + 1024;
+    size_t smem = static_cast<size_t>(stages) * stage_bytes + sizeof(GemmShared) + 1024;
+    // one pair per two SMs: two pairs' TMEM allocations on the same two SMs could wait for each other
+    if (PAIR && smem < 116 * 1024) smem = 116 * 1024;
     static std::atomic<unsigned long long> attr_done{0};
     e = set_smem_limit_once(attr_done, gemm_kernel<BN, EPI, PAIR>, 227 * 1024);
     if (e != cudaSuccess) return e;
@@ -670,13 +685,10 @@ int gemm_pick_splits(int M, int N, int K) {
 
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     const bool swiglu = a.act_out != nullptr;
-    // The gate/up projection has no K split to balance its CTAs over the SMs (192 tiles on 148 SMs at the 8B
-    // shape: some SMs stage for two CTAs), so from 65 rows up it also runs as pairs, each CTA staging half of
-    // the activation rows (measured at 128 rows: step 4.84 -> 4.72 ms; at 32 rows pairs lose, 3.27 vs 3.26).
     const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
     if (rows_enabled() && use_pair(a.M, n_tiles) && gemm_rows_supported(a, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
     if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of that kernel only
-    const bool pair = use_pair(a.M, n_tiles) || (swiglu && a.M > 64 && pair_enabled() && (n_tiles & 1) == 0);
+    const bool pair = use_pair(a.M, n_tiles);
     const int bn = pick_bn(a.M, pair);
     if (swiglu) {
         if (a.splits != 1) return cudaErrorInvalidValue;
