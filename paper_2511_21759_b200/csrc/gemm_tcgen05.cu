@@ -674,7 +674,9 @@ int gemm_pick_splits(int M, int N, int K) {
             big_target = e ? atoi(e) : 296;
         }
         int sp = tiles >= big_target ? 1 : big_target / tiles;
-        if (sp > nkb / 8) sp = nkb / 8;
+        // at least 12 k-blocks (5 us of main loop) per split: below that its epilogue and the partials' way through memory
+        // cost more than the idle pairs (1118 rows, d 1024: refresh of two layers 267 us with 8, 243 with 12, 246 with 16)
+        if (sp > nkb / 12) sp = nkb / 12;
         return gemm_whole_splits(sp, nkb);
     }
     int splits = target_ctas() / tiles;
