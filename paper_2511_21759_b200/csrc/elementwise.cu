@@ -53,7 +53,11 @@ __device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i
 // not a row scalar.  x = residual stream row (after adding the split-K partials of the preceding projection
 // in split order; all splits are requested at once, one memory round trip); writes bf16(x * gain) as the
 // projection's operand and this slice's sum(x^2) for the projection's consumer.
-__global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __restrict__ h, const float* __restrict__ partial,
+// SPLITS: room for this many partials per row; the loads in flight are registers, and with room for sixteen two blocks
+// fit an SM: the 512 blocks of a 128-row step were 1.7 waves (9 partials: 9.3 us; with room for ten, four blocks per SM,
+// 6.7 to 8 us; layer step of four sequences 162 -> 160 us).
+template <int SPLITS, int BLOCKS>
+__global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(float* __restrict__ h, const float* __restrict__ partial,
                                                                      int splits, size_t pstride, const float* __restrict__ gain,
                                                                      __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                      const int32_t* __restrict__ row_map, int d, L2Prefetch pf,
@@ -73,12 +77,12 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_kernel(float* __re
         if (emb.table) reinterpret_cast<float4*>(hr)[i] = v;   // first norm of a forward
         if (partial) {
             const float* p = partial + static_cast<size_t>(row) * d + 4 * i;
-            float4 t[16];
+            float4 t[SPLITS];
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
+            for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) t[u] = *reinterpret_cast<const float4*>(p + static_cast<size_t>(u) * pstride);
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
+            for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) { v.x += t[u].x; v.y += t[u].y; v.z += t[u].z; v.w += t[u].w; }
             reinterpret_cast<float4*>(hr)[i] = v;
         }
@@ -520,7 +524,7 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
         return launch_norm_rows<kNormRowsMaxSplits, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
                                                            tw, emb);
     }
-    return launch_kernel_if(!first, rmsnorm_kernel, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
+    return launch_kernel_if(!first, splits <= 4 ? rmsnorm_kernel<4, 4> : splits <= 10 ? rmsnorm_kernel<10, 4> : rmsnorm_kernel<16, 2>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
                             st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb);
 }
 
