@@ -1,10 +1,10 @@
 // Many-row projections (more than 128 activation rows): persistent CTA pairs with the ACTIVATION rows on the M side of
 // the tensor-core tile.
 //
-// The pair kernel of gemm_tcgen05.cu gives the M side to the weights; its accumulator then has one weight row per
-// TMEM lane and an epilogue thread owns one output FEATURE of many rows: SwiGLU has to fetch the matching up value
-// from another warp through shared memory behind block barriers (half of the epilogue warps idle), the confidence
-// statistics need a transpose, and every bf16 store is a 2-byte store.  Here the two operands of the same MMA change
+// The kernel of gemm_tcgen05.cu gives the M side to the weights (as the pair kernel before this one did); its
+// accumulator then has one weight row per TMEM lane and an epilogue thread owns one output FEATURE of many rows:
+// SwiGLU has to fetch the matching up value from another warp through shared memory behind a block barrier, the
+// confidence statistics need a transpose, and every bf16 store is a 2-byte store.  Here the two operands of the MMA change
 // places: a cluster of two CTAs issues one tcgen05.mma.cta_group::2 of 256 activation rows x 256 weight rows, each
 // CTA staging 128 activation rows (A) and one packed weight tile of 128 rows (its half of B), so the bytes staged and
 // the MMA rate are the ones of the other kernel, and lane r of a CTA's accumulator is its activation row r with 256
@@ -59,6 +59,7 @@ struct RowsArgs {
     int M, N, nkb_total, nkb_per_split;
     int n_pairs, m_tiles, group, splits;   // pairs of weight tiles, tiles of 256 rows, row tiles that are walked side by side
     uint64_t w_hint;             // L2 policy of the weight tiles
+    int wide;                    // ROWS_PARTIAL: output rows start on 16-byte boundaries
     int* status;
 };
 
@@ -317,15 +318,24 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                     __syncwarp();
                     take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
                         const int n = nc + ch * 4;
-                        if (mw + r >= a.M || n >= a.N) return;       // N % 4 == 0
+                        if (mw + r >= a.M || n >= a.N) return;
                         const size_t off = static_cast<size_t>(mw + r) * a.N + n;
-                        if (EPI == ROWS_ADD) {
+                        if (EPI == ROWS_ADD) {                       // N % 4 == 0
                             red_add4(a.add_to + off, x);
-                        } else if (po.n == 0) {
-                            *reinterpret_cast<uint4*>(a.partial + split_off + off) = x;
-                        } else {   // tensor-parallel partial sums: the tile goes to the receive buffer of every rank
+                            return;
+                        }
+                        // tensor-parallel partial sums: the tile goes to the receive buffer of every rank
 #pragma unroll 1
-                            for (int p = 0; p < po.n; ++p) *reinterpret_cast<uint4*>(po.partial[p] + split_off + off) = x;
+                        for (int p = 0; p < (po.n ? po.n : 1); ++p) {
+                            float* out = (po.n ? po.partial[p] : a.partial) + split_off + off;
+                            if (a.wide) {
+                                *reinterpret_cast<uint4*>(out) = x;
+                            } else {                                 // rows of any length, a base on any 4-byte boundary
+                                out[0] = __uint_as_float(x.x);
+                                if (n + 1 < a.N) out[1] = __uint_as_float(x.y);
+                                if (n + 2 < a.N) out[2] = __uint_as_float(x.z);
+                                if (n + 3 < a.N) out[3] = __uint_as_float(x.w);
+                            }
                         }
                     });
                 }
@@ -474,6 +484,9 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     a.nkb_total = (g.K + kBK - 1) / kBK;
     a.nkb_per_split = (a.nkb_total + g.splits - 1) / g.splits;
     if (a.nkb_per_split * (g.splits - 1) >= a.nkb_total) return cudaErrorInvalidValue;   // an empty split
+    uintptr_t low = static_cast<uintptr_t>(4 * g.N) | reinterpret_cast<uintptr_t>(g.partial);
+    for (int r = 0; r < g.peers.n; ++r) low |= reinterpret_cast<uintptr_t>(g.peers.partial[r]);
+    a.wide = (low & 15) == 0;
     a.n_pairs = n_tiles / 2;
     a.m_tiles = (g.M + 2 * kBM - 1) / (2 * kBM);
     // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (measured with two CTAs per SM at 128 row tiles: groups of
@@ -510,16 +523,8 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
 
 }  // namespace
 
-// Whether a projection with more than 128 rows runs here: an even number of weight tiles (pairs) and row starts on
-// 16-byte boundaries (always so inside a model: d, F multiples of 16, heads of 64 or 128; the GEMM entry points take any N).
-bool gemm_rows_supported(const GemmArgs& a, int n_tiles) {
-    if (a.M <= 128 || (n_tiles & 1)) return false;
-    if (a.act_out || a.conf.part || a.qkv || a.add_to) return a.splits == 1;
-    uintptr_t low = reinterpret_cast<uintptr_t>(a.partial);
-    for (int r = 0; r < a.peers.n; ++r) low |= reinterpret_cast<uintptr_t>(a.peers.partial[r]);
-    return (a.N & 3) == 0 && (low & 15) == 0;
-}
-
+// More than 128 rows and an even number of weight tiles.  Inside a model every row starts on a 16-byte boundary (d and F
+// are multiples of 16, heads have 64 or 128 dims); the GEMM entry points take any N.
 cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st) {
     if (a.act_out) return launch_rows<ROWS_SWIGLU>(a, n_tiles, st);
     if (a.qkv) return a.qkv->hd == 128 ? launch_rows<ROWS_QKV128>(a, n_tiles, st) : launch_rows<ROWS_QKV64>(a, n_tiles, st);

@@ -4,8 +4,9 @@
 // with x the bf16 activations [M][K] (few rows: block_len * copies in a decode step; all
 // positions in a refresh) and w a bf16 weight matrix [N][K].  The 128-row side of the tensor
 // core tile is given to the WEIGHTS (they are the large, streamed operand) and the activation
-// rows ride on the MMA's N dimension (32..256), so a 32-row decode step wastes no tensor-core
-// rows and every weight byte is fetched from HBM exactly once.
+// rows ride on the MMA's N dimension (32..128), so a 32-row decode step wastes no tensor-core
+// rows and every weight byte is fetched from HBM exactly once.  Projections of more than 128 rows with
+// an even number of weight tiles run as CTA pairs in gemm_rows.cu.
 //
 // Weights are stored PACKED: tile (n-tile of 128 rows, k-block of 64 columns) is one contiguous
 // 16 KB chunk, tiles of a row of tiles consecutive in k.  A CTA therefore reads one sequential
@@ -33,58 +34,43 @@ struct alignas(8) GemmShared {
     uint64_t acc_full;
     uint32_t tmem_base;
     int abort;
-    float scale[256];      // RowScale of the tile's activation rows
+    float scale[128];      // RowScale of the tile's activation rows
 };
 
-// BN: activation rows per tile (MMA N): 32, 64, 128 or 256.
+// BN: activation rows per tile (MMA N): 32, 64 or 128.
 // SWIGLU: the weight is the gate/up matrix packed with gate and up rows interleaved in groups of
 // 64 (tile t = gate rows [64t, 64t+64) then up rows [64t, 64t+64)); the epilogue pairs TMEM lane r
 // (gate) with lane r + 64 (up) through shared memory and stores bf16(silu(gate) * up) to
 // g[m][64 t + r]; N is then the FFN width F and there is no K split.
 constexpr int EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_CONF = 3;
+constexpr int kMinStages = 2;
 
-template <int BN, int EPI, bool PAIR>
+template <int BN, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
             float* __restrict__ partial, __nv_bfloat16* __restrict__ act_out, RowScale rs,
             ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int stages,
-            int l2_prefetch, int pair_tiles_x, int pair_tiles_y,
-            int* status, const __grid_constant__ PeerOut po) {
+            int l2_prefetch, int* status, const __grid_constant__ PeerOut po) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr uint32_t kABytes = kBM * kBK * 2;
-    constexpr int kBRows = PAIR ? BN / 2 : BN;        // activation rows this CTA stages
-    constexpr uint32_t kBBytes = kBRows * kBK * 2;
+    constexpr uint32_t kBBytes = BN * kBK * 2;
     constexpr uint32_t kStageBytes = kABytes + kBBytes;
-    constexpr uint32_t kTxBytes = PAIR ? 2 * kStageBytes : kStageBytes;   // bytes reported to a full barrier
-    constexpr uint32_t kTmemCols = BN < 32 ? 32 : BN;
-    const uint32_t pair_rank = PAIR ? cluster_ctarank() : 0u;
-    const bool leader = pair_rank == 0;
+    constexpr uint32_t kTmemCols = BN;
+    // the epilogues exchange values through the stage ring, which holds at least kMinStages stages
+    constexpr uint32_t kExchangeBytes = EPI == EPI_SWIGLU ? 2 * 64 * (BN / 2 + 1) * 4 : EPI == EPI_CONF ? 32 * 129 * 4 : 0;
+    static_assert(kExchangeBytes <= kMinStages * kStageBytes, "the exchange buffer must end inside the ring");
 
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     GemmShared* sh = reinterpret_cast<GemmShared*>(tiles + static_cast<size_t>(stages) * kStageBytes);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    // Work unit of this CTA.  Single CTAs: grid (weight tiles, row tiles, K splits).  Pairs: grid (2, row tiles of
-    // a group, weight-tile pairs x row-tile groups x K splits), scheduled in that order: the row tiles of a group
-    // run side by side on one weight-tile pair (its weights come from HBM once, from L2 for the other row
-    // tiles), and a group's activation rows (a few MB) stay in L2 while every weight-tile pair passes over them.
-    const int n_pairs = PAIR ? pair_tiles_x >> 1 : 0;
-    const int n_tile = PAIR ? 2 * static_cast<int>(blockIdx.z % n_pairs) + static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x);
-    const int n_tiles = PAIR ? pair_tiles_x : static_cast<int>(gridDim.x);
-    const int m_groups = PAIR ? (pair_tiles_y + static_cast<int>(gridDim.y) - 1) / static_cast<int>(gridDim.y) : 1;
-    const int m_tile = PAIR ? static_cast<int>((blockIdx.z / n_pairs) % m_groups) * static_cast<int>(gridDim.y) + static_cast<int>(blockIdx.y)
-                            : static_cast<int>(blockIdx.y);
-    if (PAIR && m_tile >= pair_tiles_y) {   // ragged last group: both CTAs of the pair leave together
-        if (po.n > 0 && threadIdx.x == 0) {
-            pdl_wait();   // the arrival counter is shared with the previous exchanging launch: count only once that one is complete
-            tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);
-        }
-        return;
-    }
+    // work unit of this CTA: grid (weight tiles, row tiles, K splits)
+    const int n_tile = static_cast<int>(blockIdx.x), n_tiles = static_cast<int>(gridDim.x);
+    const int m_tile = static_cast<int>(blockIdx.y);
     const int n0 = n_tile * kBM;
     const int m0 = m_tile * BN;
-    const int split = PAIR ? static_cast<int>(blockIdx.z / (n_pairs * m_groups)) : static_cast<int>(blockIdx.z);
+    const int split = static_cast<int>(blockIdx.z);
     const int kb0 = split * nkb_per_split;
     int nkb = nkb_total - kb0;
     if (nkb > nkb_per_split) nkb = nkb_per_split;
@@ -92,7 +78,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     // packed weights: tile (n-tile, k-block) is the contiguous 16 KB chunk number n_tile * nkb_total + k_block
     const int wtile0 = n_tile * nkb_total + kb0;
 
-    if constexpr (!PAIR) pdl_launch_dependents();
+    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < stages; ++i) {
             mbar_init(&sh->full[i], 1);
@@ -109,25 +95,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     }
     if (warp == 1) {   // whole warp: allocate the accumulator's TMEM columns
         __syncwarp();
-        if constexpr (PAIR) {   // the same warp of both CTAs allocates the same columns in both SMs
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)),
-                         "r"(kTmemCols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)),
-                         "r"(kTmemCols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if constexpr (PAIR) {
-        cluster_barrier();   // the peer's barriers are initialised before anything signals them
-        pdl_launch_dependents();   // a pair needs the same columns in both SMs: no successor may take any before it has them
-    }
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {
@@ -136,15 +111,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // The weights do not depend on the preceding kernel: fill the ring with weight tiles
             // first, then wait for the predecessor and fetch the activation tiles.
             const int pre = nkb < stages ? nkb : stages;
-            const int mb = m0 + static_cast<int>(pair_rank) * kBRows;   // first activation row this CTA stages
             for (int i = 0; i < pre; ++i) {
-                if (leader) mbar_expect_tx(&sh->full[i], kTxBytes);
-                if constexpr (PAIR)
-                    tma_load_3d_pair(tiles + static_cast<size_t>(i) * kStageBytes, &tmap_w, &sh->full[i], 0, 0, wtile0 + i,
-                                     kEvictFirst);
-                else
-                    tma_load_3d(tiles + static_cast<size_t>(i) * kStageBytes, &tmap_w, &sh->full[i], 0, 0, wtile0 + i,
-                                kEvictFirst);
+                mbar_expect_tx(&sh->full[i], kStageBytes);
+                tma_load_3d(tiles + static_cast<size_t>(i) * kStageBytes, &tmap_w, &sh->full[i], 0, 0, wtile0 + i, kEvictFirst);
             }
             // and ask L2 for the weight tiles that follow, so that HBM keeps streaming while the
             // predecessor (a short elementwise kernel) is still running
@@ -156,14 +125,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                              "r"(0), "r"(0), "r"(wtile0 + i)
                              : "memory");
             pdl_wait();
-            for (int i = 0; i < pre; ++i) {
-                if constexpr (PAIR)
-                    tma_load_2d_pair(tiles + static_cast<size_t>(i) * kStageBytes + kABytes, &tmap_x, &sh->full[i],
-                                     (kb0 + i) * kBK, mb, kEvictLast);
-                else
-                    tma_load_2d(tiles + static_cast<size_t>(i) * kStageBytes + kABytes, &tmap_x, &sh->full[i], (kb0 + i) * kBK,
-                                mb, kEvictLast);
-            }
+            for (int i = 0; i < pre; ++i)
+                tma_load_2d(tiles + static_cast<size_t>(i) * kStageBytes + kABytes, &tmap_x, &sh->full[i], (kb0 + i) * kBK, m0, kEvictLast);
             int issued = pre;
             for (int i = pre; i < nkb; ++i) {
                 const int st = i % stages;
@@ -171,19 +134,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                 if (!mbar_wait(&sh->empty[st], ph ^ 1u, cta_abort, status)) break;
                 uint8_t* a_dst = tiles + static_cast<size_t>(st) * kStageBytes;
                 uint8_t* b_dst = a_dst + kABytes;
-                if (leader) mbar_expect_tx(&sh->full[st], kTxBytes);
-                if constexpr (PAIR) {
-                    tma_load_3d_pair(a_dst, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
-                    tma_load_2d_pair(b_dst, &tmap_x, &sh->full[st], (kb0 + i) * kBK, mb, kEvictLast);
-                } else {
-                    tma_load_3d(a_dst, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
-                    tma_load_2d(b_dst, &tmap_x, &sh->full[st], (kb0 + i) * kBK, mb, kEvictLast);
-                }
+                mbar_expect_tx(&sh->full[st], kStageBytes);
+                tma_load_3d(a_dst, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
+                tma_load_2d(b_dst, &tmap_x, &sh->full[st], (kb0 + i) * kBK, m0, kEvictLast);
                 issued = i + 1;
             }
-            if (*cta_abort && leader) {
-                // aborted: let the copies still in flight land before the CTA's shared memory goes away (the
-                // peer of a pair cannot observe its own copies; it is held by the cluster barrier at the end)
+            if (*cta_abort) {
+                // aborted: let the copies still in flight land before the CTA's shared memory goes away
                 const int first = issued > stages ? issued - stages : 0;
                 for (int i = first; i < issued; ++i) {
                     const long long t0 = clock64();
@@ -194,9 +151,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
-            // ---- MMA issuer (the leader's, for both CTAs of a pair) ----
-            constexpr uint32_t idesc = make_instr_desc(PAIR ? 2 * kBM : kBM, BN);
+        if (lane == 0) {
+            // ---- MMA issuer ----
+            constexpr uint32_t idesc = make_instr_desc(kBM, BN);
             bool ok = true;
             for (int i = 0; i < nkb && ok; ++i) {
                 const int st = i % stages;
@@ -207,22 +164,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                 const uint32_t a_addr = smem_u32(tiles + static_cast<size_t>(st) * kStageBytes);
                 const uint32_t b_addr = a_addr + kABytes;
 #pragma unroll
-                for (int k = 0; k < kBK / kUmmaK; ++k) {
-                    if constexpr (PAIR)
-                        umma_bf16_pair(tmem_acc, make_smem_desc(a_addr + k * kUmmaK * 2), make_smem_desc(b_addr + k * kUmmaK * 2),
-                                       idesc, (i > 0 || k > 0) ? 1u : 0u);
-                    else
-                        umma_bf16(tmem_acc, make_smem_desc(a_addr + k * kUmmaK * 2), make_smem_desc(b_addr + k * kUmmaK * 2),
-                                  idesc, (i > 0 || k > 0) ? 1u : 0u);
-                }
-                // frees the stage (in both CTAs of a pair) once these MMAs have read it
-                if constexpr (PAIR) umma_commit_pair(&sh->empty[st]);
-                else umma_commit(&sh->empty[st]);
+                for (int k = 0; k < kBK / kUmmaK; ++k)
+                    umma_bf16(tmem_acc, make_smem_desc(a_addr + k * kUmmaK * 2), make_smem_desc(b_addr + k * kUmmaK * 2), idesc,
+                              (i > 0 || k > 0) ? 1u : 0u);
+                umma_commit(&sh->empty[st]);   // frees the stage once these MMAs have read it
             }
-            if (ok) {
-                if constexpr (PAIR) umma_commit_pair(&sh->acc_full);
-                else umma_commit(&sh->acc_full);
-            }
+            if (ok) umma_commit(&sh->acc_full);
         }
     } else {
         // ---- epilogue: warps 2..5 own TMEM lanes 32*(warp%4) .. +31 ----
@@ -330,8 +277,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // All MMAs have completed, so the stage ring is free: the warps that own gate features hand the values of the
             // tile's second half of rows to the warps that own the matching up features, and get the up values of the
             // first half; behind one barrier every warp then finishes its half.  (Up values handed over chunk by chunk
-            // behind two barriers each, the up warps idle, as CTA pairs: 50 us for the 8B shape's gate/up projection at 128 rows; this
-            // way 47, and 36 instead of 38 at 32 rows.)
+            // behind two barriers each, the up warps idle, in CTA pairs: 50 us for the 8B shape's gate/up projection at
+            // 128 rows; this way 47, and 36 instead of 38 at 32 rows.)
             constexpr int kHalfRows = BN / 2, kPitch = kHalfRows + 1;
             float* xch = reinterpret_cast<float*>(tiles);             // [gate | up][64 features][kPitch]
             const int fl = (q & 1) * 32 + lane;                       // feature of this lane within the tile
@@ -375,14 +322,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     pdl_wait();   // every thread: keeps completion of the launch chain transitive
     tc_fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_barrier();   // neither CTA's shared memory or TMEM goes away while its peer may touch it
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        if constexpr (PAIR)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
     }
 }
 
@@ -477,7 +420,7 @@ __global__ void pack_gate_up_kernel(const __nv_bfloat16* __restrict__ src, __nv_
     reinterpret_cast<uint4*>(dst)[chunk] = v;
 }
 
-// CTA pairs (cta_group::2) are used whenever the number of weight tiles is even (ODB_GEMM_PAIR=0 turns them off).
+// ODB_GEMM_PAIR=0 in the environment: no CTA pairs, many rows run as single CTAs.
 bool pair_enabled() {
     static int v = -1;
     if (v < 0) {
@@ -487,117 +430,61 @@ bool pair_enabled() {
     return v != 0;
 }
 
-int pick_bn(int M, bool pair) {
+// activation rows per tile of a single CTA; two CTAs share an SM (one's epilogue overlaps the other's main loop)
+int pick_bn(int M) {
     static int max_bn = -1;
     if (max_bn < 0) {
         const char* e = getenv("ODB_GEMM_MAX_BN");
         max_bn = e ? atoi(e) : 0;
     }
-    // Up to 128 rows per tile two CTAs share an SM (one's epilogue overlaps the other's main loop).  A CTA
-    // pair stages only half of the rows per CTA, so it affords 256-row tiles at the same occupancy.
-    int bn = M <= 32 ? 32 : M <= 64 ? 64 : M <= 128 ? 128 : pair ? 256 : 128;
-    if (max_bn > 0 && bn > max_bn) bn = max_bn;
-    return bn;
+    const int bn = M <= 32 ? 32 : M <= 64 ? 64 : 128;
+    return max_bn > 0 && bn > max_bn ? (max_bn < 64 ? 32 : 64) : bn;
 }
 
-template <int BN, int EPI, bool PAIR>
+template <int BN, int EPI>
 cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
-    constexpr bool SWIGLU = EPI == EPI_SWIGLU;
-    constexpr int kBRows = PAIR ? BN / 2 : BN;
     CUtensorMap tmx;
-    cudaError_t e = make_tmap_2d(&tmx, a.x, a.M, a.K, kBRows);
+    cudaError_t e = make_tmap_2d(&tmx, a.x, a.M, a.K, BN);
     if (e != cudaSuccess) return e;
     const int nkb_total = (a.K + kBK - 1) / kBK;
     const int nkb_per_split = (nkb_total + a.splits - 1) / a.splits;
-    const uint32_t stage_bytes = kBM * kBK * 2 + kBRows * kBK * 2;
-    // two CTAs per SM as long as two accumulators fit TMEM and a CTA stages at most 128 rows
-    const uint32_t budget = kBRows <= 128 && !PAIR ? 100 * 1024 : 200 * 1024;
-    int stages = static_cast<int>(budget / stage_bytes);
+    constexpr int kStageBytes = (kBM + BN) * kBK * 2;
+    int stages = 100 * 1024 / kStageBytes;   // two CTAs per SM
     if (stages > 16) stages = 16;
-    if (stages > nkb_per_split) stages = nkb_per_split < 2 ? 2 : nkb_per_split;
-    size_t smem = static_cast<size_t>(stages) * stage_bytes + sizeof(GemmShared) + 1024;
-    // one pair per two SMs: two pairs' TMEM allocations on the same two SMs could wait for each other
-    if (PAIR && smem < 116 * 1024) smem = 116 * 1024;
+    if (stages > nkb_per_split) stages = nkb_per_split < kMinStages ? kMinStages : nkb_per_split;
+    const size_t smem = static_cast<size_t>(stages) * kStageBytes + sizeof(GemmShared) + 1024;
     static std::atomic<unsigned long long> attr_done{0};
-    e = set_smem_limit_once(attr_done, gemm_kernel<BN, EPI, PAIR>, 227 * 1024);
+    e = set_smem_limit_once(attr_done, gemm_kernel<BN, EPI>, 227 * 1024);
     if (e != cudaSuccess) return e;
-    // SWIGLU: N is the FFN width and a weight tile holds 64 gate + 64 up rows
-    dim3 grid(SWIGLU ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM, (a.M + BN - 1) / BN, a.splits);
+    // EPI_SWIGLU: N is the FFN width and a weight tile holds 64 gate + 64 up rows
+    dim3 grid(EPI == EPI_SWIGLU ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM, (a.M + BN - 1) / BN, a.splits);
     static int l2_prefetch = -1;
     if (l2_prefetch < 0) {
         const char* env = getenv("ODB_GEMM_L2_PREFETCH");
         l2_prefetch = env ? atoi(env) : 0;   // measured: prefetching into L2 slows the step down
     }
-    if constexpr (PAIR) {
-        if (grid.x & 1) return cudaErrorInvalidValue;
-        const int tiles_x = static_cast<int>(grid.x), tiles_y = static_cast<int>(grid.y);
-        // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (measured at 128 row tiles: groups of 2 / 4 / 8 / 16
-        // give 430 / 414 / 404 / 407 ms of GEMM time per refresh, no grouping 475, one row tile per weight pass 462)
-        const int group = tiles_y < 8 ? tiles_y : 8;
-        const int m_groups = (tiles_y + group - 1) / group;
-        if (static_cast<size_t>(tiles_x / 2) * m_groups * a.splits > 65535) return cudaErrorInvalidValue;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2, group, (tiles_x / 2) * m_groups * a.splits);
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;   // neighbouring weight tiles form the pair
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = pdl_enabled() ? 2 : 1;
-        return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, EPI, PAIR>, a.tmap_w, tmx, a.partial, a.act_out, a.row_scale, a.conf,
-                                  a.M, a.N, nkb_total, nkb_per_split, stages, pdl_enabled() ? l2_prefetch : 0, tiles_x, tiles_y, a.status, a.peers);
-    } else {
-        return launch_kernel(gemm_kernel<BN, EPI, PAIR>, grid, dim3(kThreads), smem, st, a.tmap_w, tmx, a.partial, a.act_out,
-                             a.row_scale, a.conf, a.M, a.N, nkb_total, nkb_per_split, stages,
-                             pdl_enabled() ? l2_prefetch : 0, 0, 0, a.status, a.peers);
-    }
+    return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(kThreads), smem, st, a.tmap_w, tmx, a.partial, a.act_out, a.row_scale, a.conf,
+                         a.M, a.N, nkb_total, nkb_per_split, stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
 }
 
 template <int EPI>
-cudaError_t launch_epi(const GemmArgs& a, int bn, bool pair, cudaStream_t st) {
-    if (pair) {
-        switch (bn) {
-            case 32: return launch_bn<32, EPI, true>(a, st);
-            case 64: return launch_bn<64, EPI, true>(a, st);
-            case 128: return launch_bn<128, EPI, true>(a, st);
-            default: return launch_bn<256, EPI, true>(a, st);
-        }
-    }
-    switch (bn) {
-        case 32: return launch_bn<32, EPI, false>(a, st);
-        case 64: return launch_bn<64, EPI, false>(a, st);
-        case 128: return launch_bn<128, EPI, false>(a, st);
-        default: return launch_bn<256, EPI, false>(a, st);
+cudaError_t launch_epi(const GemmArgs& a, cudaStream_t st) {
+    switch (pick_bn(a.M)) {
+        case 32: return launch_bn<32, EPI>(a, st);
+        case 64: return launch_bn<64, EPI>(a, st);
+        default: return launch_bn<128, EPI>(a, st);
     }
 }
 
-// Whether a projection of M activation rows with n_tiles weight tiles runs as CTA pairs.  Measured on the
-// 8B shape: with many rows (refresh, 768..1024 rows: tensor/L2 bound) pairs with 256-row tiles are 11 %
+// Whether a projection of M activation rows with n_tiles weight tiles runs as CTA pairs (gemm_rows.cu).  Measured on
+// the 8B shape: with many rows (refresh, 768..1024 rows: tensor/L2 bound) pairs with 256-row tiles are 11 %
 // faster than single CTAs with 128-row tiles; up to 128 rows (decode steps: HBM bound) the pair's extra
 // synchronisation costs more than the halved activation traffic saves (3.55 vs 3.41 ms at 32 rows).
-bool use_pair(int M, int n_tiles) {
-    static int min_rows = -1;
-    if (min_rows < 0) {
-        const char* e = getenv("ODB_GEMM_PAIR_MIN_ROWS");
-        min_rows = e ? atoi(e) : 128;
-    }
-    return pair_enabled() && M > min_rows && (n_tiles & 1) == 0;
-}
-
-bool rows_enabled() {
-    static const bool on = !(getenv("ODB_GEMM_ROWS") && getenv("ODB_GEMM_ROWS")[0] == '0');
-    return on;
-}
+bool use_pair(int M, int n_tiles) { return pair_enabled() && M > 128 && (n_tiles & 1) == 0; }
 
 }  // namespace
 
-bool gemm_rows_usable(int M, int N) { return M > 128 && rows_enabled() && use_pair(M, (N + kBM - 1) / kBM); }
+bool gemm_rows_usable(int M, int N) { return use_pair(M, (N + kBM - 1) / kBM); }
 
 cudaError_t make_weight_tmap(CUtensorMap* out, const void* w, int N, int K) { return make_tmap_packed(out, w, N, K); }
 
@@ -660,7 +547,7 @@ int gemm_whole_splits(int splits, int nkb) {
 
 int gemm_pick_splits(int M, int N, int K) {
     const int n_tiles = (N + kBM - 1) / kBM;
-    const int bn = pick_bn(M, use_pair(M, n_tiles));
+    const int bn = use_pair(M, n_tiles) ? 2 * kBM : pick_bn(M);
     const int tiles = n_tiles * ((M + bn - 1) / bn);
     const int nkb = (K + kBK - 1) / kBK;
     // all work units must be resident at once (two CTA slots per SM) and equal in size: a
@@ -688,19 +575,11 @@ int gemm_pick_splits(int M, int N, int K) {
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     const bool swiglu = a.act_out != nullptr;
     const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
-    if (rows_enabled() && use_pair(a.M, n_tiles) && gemm_rows_supported(a, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
-    if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of that kernel only
-    const bool pair = use_pair(a.M, n_tiles);
-    const int bn = pick_bn(a.M, pair);
-    if (swiglu) {
-        if (a.splits != 1) return cudaErrorInvalidValue;
-        return launch_epi<EPI_SWIGLU>(a, bn, pair, st);
-    }
-    if (a.conf.part) {
-        if (a.splits != 1) return cudaErrorInvalidValue;
-        return launch_epi<EPI_CONF>(a, bn, pair, st);
-    }
-    return launch_epi<EPI_PARTIAL>(a, bn, pair, st);
+    if ((swiglu || a.conf.part || a.qkv || a.add_to) && a.splits != 1) return cudaErrorInvalidValue;
+    if (use_pair(a.M, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
+    if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of the many-row kernel only
+    if (swiglu) return launch_epi<EPI_SWIGLU>(a, st);
+    return a.conf.part ? launch_epi<EPI_CONF>(a, st) : launch_epi<EPI_PARTIAL>(a, st);
 }
 
 cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stride, float* out, size_t n,

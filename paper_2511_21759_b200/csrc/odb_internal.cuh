@@ -338,7 +338,6 @@ cudaError_t launch_pack_weight(const void* src_row_major, void* dst_packed, int 
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
 // many-row projections with the activation rows on the M side of the tile (gemm_rows.cu)
 bool gemm_rows_usable(int M, int N);   // whether a projection of this size has the epilogues `qkv` and `add_to`
-bool gemm_rows_supported(const GemmArgs& a, int n_tiles);
 cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stride, float* out, size_t n,
                                    cudaStream_t st);
