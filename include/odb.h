@@ -118,7 +118,7 @@ typedef struct odb_config {
  * [64t, 64t+64) followed by up rows [64t, 64t+64), so that the GEMM epilogue can form
  * silu(gate) * up inside one tile.  The embedding table stays row-major. */
 typedef struct odb_weights {
-    const void* embed;          /* bf16 [vocab][d_model] */
+    const void* embed;          /* bf16 [vocab][d_model], on a 4-byte boundary */
     const void* lm_head;        /* packed bf16 [vocab][d_model], NULL iff with_lm_head == 0 */
     const float* final_norm;    /* fp32 [d_model] */
     const float* const* norm1;  /* fp32 [d_model] per layer */

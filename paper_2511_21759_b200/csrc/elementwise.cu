@@ -44,7 +44,14 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 
 // float4 i of the embedding row of row r's token
 __device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i, int d) {
-    const uint2 x = reinterpret_cast<const uint2*>(e.table + static_cast<size_t>(e.row_tok[r]) * d)[i];
+    const __nv_bfloat16* row = e.table + static_cast<size_t>(e.row_tok[r]) * d;
+    uint2 x;
+    if (e.halves) {
+        x.x = reinterpret_cast<const uint32_t*>(row)[2 * i];
+        x.y = reinterpret_cast<const uint32_t*>(row)[2 * i + 1];
+    } else {
+        x = reinterpret_cast<const uint2*>(row)[i];
+    }
     return make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xffff0000u), __uint_as_float(x.y << 16),
                        __uint_as_float(x.y & 0xffff0000u));
 }

@@ -156,6 +156,9 @@ struct odb_model {
     const void* p_lm;
 };
 
+// whether the embedding's rows can be read 8 bytes at a time (d_model is a multiple of 16)
+static bool embed_wide(const odb_model* m) { return (reinterpret_cast<uintptr_t>(m->embed) & 7) == 0; }
+
 struct odb_session {
     odb_model* m;
     cudaStream_t st;
@@ -256,6 +259,7 @@ int32_t odb_model_create(const odb_config* cfg, const odb_weights* w, odb_model*
     if (!w || !out || !w->embed || !w->final_norm || !w->norm1 || !w->norm2 || !w->wqkv || !w->wo || !w->wgu || !w->wd)
         return ODB_ERR_ARG;
     if ((cfg->with_lm_head != 0) != (w->lm_head != nullptr)) return ODB_ERR_ARG;
+    if (reinterpret_cast<uintptr_t>(w->embed) & 3) return ODB_ERR_ARG;
     odb_model* m = new (std::nothrow) odb_model();
     if (!m) return ODB_ERR_ARG;
     m->cfg = *cfg;
@@ -340,7 +344,7 @@ int32_t odb_session_create(odb_model* m, void* kv, size_t kv_bytes, void* worksp
     s->pinned_log = nullptr;
     s->pinned_iters = nullptr;
     s->ptable_built[0] = s->ptable_built[1] = s->ptable_built[2] = false;
-    s->persistent_off = c.tp_world > 1;
+    s->persistent_off = c.tp_world > 1 || !embed_wide(m);
     cudaError_t e = cudaMallocHost(&s->pinned_state, sizeof(SeqState) * c.max_batch);
     if (e == cudaSuccess) e = cudaMallocHost(&s->pinned_log, sizeof(odb_result) * kMaxLoopIters * c.max_batch);
     if (e == cudaSuccess) e = cudaMallocHost(&s->pinned_iters, 4 * sizeof(int32_t));
@@ -757,7 +761,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
                  gu_bytes = packed_gate_up_bytes(F, d);
     for (int l = 0; l < c.n_layers; ++l) {
         EmbedSource emb;
-        if (l == 0) { emb.table = m->embed; emb.row_tok = s->cb.row_tok; }
+        if (l == 0) { emb.table = m->embed; emb.row_tok = s->cb.row_tok; emb.halves = embed_wide(m) ? 0 : 1; }
         ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d,
                                                         hint_of(m->p_qkv[l], qkv_bytes, 0), st, res_wait, emb));
         int sp = plan_splits(M, 3 * da, d, false);

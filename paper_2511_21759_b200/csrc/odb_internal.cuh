@@ -350,6 +350,7 @@ cudaError_t launch_bulk_read_stream(const void* src, size_t bytes, int grid, int
 struct EmbedSource {
     const __nv_bfloat16* table = nullptr;
     const int32_t* row_tok = nullptr;
+    int halves = 0;                     // the table starts on a 4-byte boundary only (a tensor inside a mapped file)
 };
 // The part of RMSNorm that is not a row scalar, for rows r = map ? map[i] : i of the residual stream:
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's

@@ -46,6 +46,18 @@ def test_pure_host_calls_work_without_gpu():
     assert lib.odb_model_create(ctypes.byref(cfg), None, ctypes.byref(out)) == B.ODB_ERR_ARG
 
 
+def test_an_embedding_table_off_a_4_byte_boundary_is_refused():
+    from paper_2511_21759_b200 import binding as B
+    lib = B.lib()
+    cfg = B.odb_config(1, 256, 4, 64, 688, 2048, 2047, 2046, 500000.0, 1e-5, 1, 64, 16, 1, 0)
+    one = (ctypes.c_void_p * 1)(0x10000)                              # never read: the table is checked first
+    arrays = [ctypes.cast(one, ctypes.POINTER(ctypes.c_void_p))] * 6
+    out = ctypes.c_void_p()
+    for at in (0x10001, 0x10002, 0x10003):
+        w = B.odb_weights(at, None, 0x10000, *arrays)
+        assert lib.odb_model_create(ctypes.byref(cfg), ctypes.byref(w), ctypes.byref(out)) == B.ODB_ERR_ARG, hex(at)
+
+
 def test_struct_layouts_match_header():
     from paper_2511_21759_b200 import binding as B
     assert ctypes.sizeof(B.odb_config) == 17 * 4

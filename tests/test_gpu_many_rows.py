@@ -51,3 +51,34 @@ def test_refresh_of_many_rows(shape, P, L):
     for j, got in ((0, k), (1, v)):                               # the cache holds what the fresh rows hold
         assert np.array_equal(kv[0, -1, j].transpose(1, 0, 2).reshape(P + L, -1), got)
     sess.close(); gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("L", [60, 230])      # 97 rows: one row per block of the first norm; 267: four
+def test_an_embedding_table_on_any_4_byte_boundary(L):
+    """A table that starts 4 bytes behind an 8-byte boundary is read in halves: the same bits."""
+    E = engine()
+    P, x0 = 37, synth.sequence(5, 0, 37, L, HD64)
+    par = E.DecodeParams(block_len=16)
+    got = []
+    for shift in (0, 2):
+        gm = E.Model.from_synth(HD64, seed=5, max_batch=1, max_seq=P + L, max_block=16, max_copies=1)
+        if shift:
+            t = dict(gm.t)
+            table = torch.empty(t["embed"].numel() + shift, dtype=torch.bfloat16, device="cuda")[shift:].view_as(t["embed"])
+            table.copy_(t["embed"])
+            t["embed"] = table
+            assert table.data_ptr() % 8 == 4
+            gm.close()
+            gm = E.Model(HD64, t, max_batch=1, max_seq=P + L, max_block=16, max_copies=1)
+        sess = E.Session(gm, poison=True)
+        sess.set_sequence(0, x0, P)
+        sess.refresh_prefill(par, 0)
+        refreshed = sess.debug_read("hidden")
+        sess.unmask_accept(par, True)
+        sess.block_decode_step(par)
+        got.append((refreshed, sess.debug_read("hidden"), sess.debug_read("conf"), sess.debug_read("tok")))
+        assert sess.status() == 0
+        sess.close(); gm.close()
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
