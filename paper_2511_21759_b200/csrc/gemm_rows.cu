@@ -120,7 +120,10 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&y);
 }
 
+// tcgen05.ld is a whole-warp instruction: the lanes meet first, whatever the code in front made of them (lanes without a
+// row or a column leave the piece before early).
 __device__ __forceinline__ void tmem_read32(uint32_t taddr, uint32_t (&v)[32]) {
+    __syncwarp();
     tmem_ld32(taddr, v);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -281,6 +284,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
 #pragma unroll
                 for (int c = 0; c < 64; c += 16) {
                     uint32_t g[16], u[16];
+                    __syncwarp();
                     tmem_ld16(tmem + c, g);
                     tmem_ld16(tmem + 64 + c, u);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -307,12 +311,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                     const int nc = tile * kBM + c * 32;
                     if (nc >= a.N) break;
                     uint32_t v[32];
-                    tmem_read32(tmem + c * 32, v);
+                    tmem_read32(tmem + c * 32, v);           // the warp meets: the previous piece has been taken
                     if (EPI == ROWS_PARTIAL && a.rs.ssq) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
                     }
-                    __syncwarp();                            // the previous piece has been taken
 #pragma unroll
                     for (int ch = 0; ch < 8; ++ch) put_chunk(patch, lane, ch, v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
                     __syncwarp();

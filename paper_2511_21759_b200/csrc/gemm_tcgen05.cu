@@ -189,6 +189,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
 #pragma unroll 1
                 for (int c = 0; c < BN / 32; ++c) {
                     uint32_t v[32];
+                    __syncwarp();   // tcgen05.ld is a whole-warp instruction, and the stores before are some lanes' only
                     tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (po.n == 0) {
@@ -303,6 +304,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
 #pragma unroll 1
                 for (int c = 0; c < kHalfRows; c += 16) {
                     uint32_t v[16];
+                    __syncwarp();
                     tmem_ld16(tm_lane + static_cast<uint32_t>(r0 + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll

@@ -26,6 +26,9 @@ def _case(M, N, K, seed):
     (300, 768, 512, 0),       # many rows, even number of weight tiles: CTA pairs, two 256-row tiles, second ragged
     (700, 1024, 688, 2),      # CTA pairs with a K split and a K tail; three row tiles, last ragged (188 rows)
     (129, 256, 64, 1),        # CTA pair, one k-block, one row in the second CTA's half
+    (2305, 4060, 320, 1),     # 160 tiles for 74 CTA pairs: the third tile of a pair reuses the first accumulator; the second
+                              # group has two row tiles, the last one a single row; the last weight tile 92 columns
+    (2305, 4060, 320, 2),     # the same with a K split of unequal halves: 320 tiles of three and two k-blocks
     (1, 128, 64, 1),          # smallest
     (48, 2048, 2048, 0),
 ])

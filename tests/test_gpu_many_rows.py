@@ -54,6 +54,37 @@ def test_refresh_of_many_rows(shape, P, L):
 
 
 @requires_gpu
+def test_refresh_of_two_sequences_beyond_one_tile_per_pair():
+    """3120 rows of two sequences, 13 row tiles: the QKV projection hands out 156 tiles (head dim 64, more than two per
+    CTA pair), gate/up 78, and the second sequence's rows go to its own part of the cache, in every layer."""
+    E = engine()
+    shape = dataclasses.replace(HD64, n_heads=16, d_model=1024)
+    lens = [(1500, 220), (1161, 239)]
+    longest = max(p + n for p, n in lens)
+    om = model_from_synth(shape, seed=5)
+    gm = E.Model.from_synth(shape, seed=5, max_batch=2, max_seq=longest, max_block=16, max_copies=1)
+    sess = E.Session(gm, poison=True)
+    for i, (p, n) in enumerate(lens):
+        sess.set_sequence(i, synth.sequence(5, i, p, n, shape), p)
+    sess.refresh_prefill(E.DecodeParams(block_len=16), 0)
+    conf = sess.debug_read("conf")
+    kv = sess.kv.view(torch.bfloat16).view(2, shape.n_layers, 2, shape.n_heads, longest, shape.head_dim).float().cpu().numpy()
+    assert sess.status() == 0
+    at = 0
+    for i, (p, n) in enumerate(lens):
+        cache, oconf, _ = O.refresh_prefill(om, synth.sequence(5, i, p, n, shape), p + n, p)
+        assert np.allclose(conf[at:at + n], oconf, rtol=2e-2)
+        at += n
+        for l in range(shape.n_layers):
+            for j, want in ((0, cache.k[l]), (1, cache.v[l])):
+                got = kv[i, l, j, :, : p + n].transpose(1, 0, 2).reshape(p + n, -1)
+                ok, worst = logits_close(got, want.reshape(p + n, -1), 4e-2)
+                assert ok, (i, l, j, worst)
+    assert at == len(conf)
+    sess.close(); gm.close()
+
+
+@requires_gpu
 @pytest.mark.parametrize("L", [60, 230])      # 97 rows: one row per block of the first norm; 267: four
 def test_an_embedding_table_on_any_4_byte_boundary(L):
     """A table that starts 4 bytes behind an 8-byte boundary is read in halves: the same bits."""
