@@ -331,6 +331,17 @@ cudaError_t launch_step_attention(const StepAttnArgs& a, cudaStream_t st) {
     return a.hd == 128 ? launch_step_hd<128>(a, st) : launch_step_hd<64>(a, st);
 }
 
+// Enough key splits for 296 CTAs, two per SM.  With head dim 128 two CTAs are what an SM holds (80 KB, 181 registers), and
+// a decode step rounds down: 128 items in three splits are 1.3 waves (layer step of four sequences 165 us, 163 with two;
+// three and six sequences 151 -> 150, 212 -> 207).  With head dim 64 three CTAs fit (41 KB, 139 registers), so rounding
+// up still makes one wave, and rounding down leaves slots empty (d 1024, two layers, 5 / 8 / 12 sequences: 167 / 165 /
+// 202 us per step rounded up, 180 / 179 / 223 down; 16 sequences 220 either way).
+int attention_key_splits(int items, int head_dim, bool refresh) {
+    const int target = 2 * 148;
+    const int ks = head_dim == 128 && !refresh ? target / items : (target + items - 1) / items;
+    return ks < 1 ? 1 : ks > 8 ? 8 : ks;
+}
+
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st) {
     if (a.n_tiles == 0) return cudaSuccess;
     return a.hd == 128 ? launch_hd<128>(a, st) : launch_hd<64>(a, st);

@@ -737,9 +737,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     size_t res_stride = 0;
     static const int ks_env = getenv("ODB_ATTN_KS") ? atoi(getenv("ODB_ATTN_KS")) : 0;
     static const bool tc_attention = !(getenv("ODB_ATTN_TC") && getenv("ODB_ATTN_TC")[0] == '0');
-    // key splits for two CTAs per SM; a decode step rounds down (4 x 32 items: three splits are 1.3 waves, 165 us per
-    // layer against 163 with two)
-    int ks = write_cache ? (2 * 148 + n_tiles * H - 1) / (n_tiles * H) : 2 * 148 / (n_tiles * H);
+    int ks = attention_key_splits(n_tiles * H, hd, write_cache);
     if (ks_env > 0 && !write_cache) ks = ks_env;
     if (ks > 8) ks = 8;
     if (static_cast<size_t>(ks) * M > L.attn_rows) ks = static_cast<int>(L.attn_rows / M);

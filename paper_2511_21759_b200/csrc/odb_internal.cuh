@@ -385,6 +385,8 @@ struct AttnArgs {
     int early = 0;                        // 1: tiles and cache were complete before the launch chain began (decode steps)
     L2Prefetch pf;
 };
+// Key splits of the mma.sync attention over `items` pairs of a row tile and a head, 1 .. 8.
+int attention_key_splits(int items, int head_dim, bool refresh);
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st);
 // refresh attention on the tcgen05 tensor cores (head dim 128): a.tiles = work items of up to 128 query rows
 // whose keys are the fresh rows [f0, f0 + n0); status = device status word (bounded waits)

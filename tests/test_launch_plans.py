@@ -1,0 +1,23 @@
+"""The host-side rules that choose how a launch is divided, on a machine without a GPU: the library's own C++ functions,
+called through their exported names."""
+import ctypes
+
+import pytest
+
+
+def _rule(name, *argtypes):
+    from paper_2511_21759_b200 import binding as B
+    f = getattr(B.lib(), name)
+    f.argtypes, f.restype = argtypes, ctypes.c_int
+    return f
+
+
+@pytest.mark.parametrize("items,hd,refresh,splits", [
+    (4, 64, False, 8), (37, 64, False, 8),                          # never more than eight
+    (80, 64, False, 4), (128, 64, False, 3), (192, 64, False, 2), (256, 64, False, 2),   # rounded up: three CTAs fit an SM
+    (296, 64, False, 1), (297, 64, False, 1), (5000, 64, False, 1),
+    (96, 128, False, 3), (128, 128, False, 2), (192, 128, False, 1), (1024, 128, False, 1),   # rounded down: two fit
+    (128, 128, True, 3), (128, 64, True, 3), (300, 128, True, 1),   # a refresh rounds up with either
+])
+def test_key_splits_of_the_attention(items, hd, refresh, splits):
+    assert _rule("_ZN3odb20attention_key_splitsEiib", ctypes.c_int, ctypes.c_int, ctypes.c_bool)(items, hd, refresh) == splits
