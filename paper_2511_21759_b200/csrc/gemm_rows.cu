@@ -65,7 +65,7 @@ struct RowsArgs {
 
 // The tiles in the order they are handed out, round robin, to the pairs: the row tiles of a group side by side on one
 // weight-tile pair (its weights come from HBM once, from L2 for the other row tiles), then the next weight-tile pair
-// (the group's activation rows, a few MB, stay in L2), then the next group, then the next K split.
+// (the group's activation rows stay in L2: 17 MB at K 4096, 50 MB at K 12288), then the next group, then the next K split.
 struct RowsItem {
     int m_tile, pair, split, kb0, nkb;
 };
@@ -319,28 +319,35 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
 #pragma unroll
                     for (int ch = 0; ch < 8; ++ch) put_chunk(patch, lane, ch, v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
                     __syncwarp();
-                    take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
-                        const int n = nc + ch * 4;
-                        if (mw + r >= a.M || n >= a.N) return;
-                        const size_t off = static_cast<size_t>(mw + r) * a.N + n;
-                        if (EPI == ROWS_ADD) {                       // N % 4 == 0
-                            red_add4(a.add_to + off, x);
-                            return;
-                        }
-                        // tensor-parallel partial sums: the tile goes to the receive buffer of every rank
+                    if (EPI == ROWS_ADD || (a.wide && po.n == 0)) {
+                        take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
+                            const int n = nc + ch * 4;
+                            if (mw + r >= a.M || n >= a.N) return;       // N % 4 == 0
+                            const size_t off = static_cast<size_t>(mw + r) * a.N + n;
+                            if (EPI == ROWS_ADD) red_add4(a.add_to + off, x);
+                            else *reinterpret_cast<uint4*>(a.partial + split_off + off) = x;
+                        });
+                    } else {
+                        // tensor-parallel partial sums (the tile goes to the receive buffer of every rank), and rows of any
+                        // length on any 4-byte boundary; apart from the code above, which that made 2 % of a step slower
+                        take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
+                            const int n = nc + ch * 4;
+                            if (mw + r >= a.M || n >= a.N) return;
+                            const size_t off = split_off + static_cast<size_t>(mw + r) * a.N + n;
 #pragma unroll 1
-                        for (int p = 0; p < (po.n ? po.n : 1); ++p) {
-                            float* out = (po.n ? po.partial[p] : a.partial) + split_off + off;
-                            if (a.wide) {
-                                *reinterpret_cast<uint4*>(out) = x;
-                            } else {                                 // rows of any length, a base on any 4-byte boundary
-                                out[0] = __uint_as_float(x.x);
-                                if (n + 1 < a.N) out[1] = __uint_as_float(x.y);
-                                if (n + 2 < a.N) out[2] = __uint_as_float(x.z);
-                                if (n + 3 < a.N) out[3] = __uint_as_float(x.w);
+                            for (int p = 0; p < (po.n ? po.n : 1); ++p) {
+                                float* out = (po.n ? po.partial[p] : a.partial) + off;
+                                if (a.wide) {
+                                    *reinterpret_cast<uint4*>(out) = x;
+                                } else {
+                                    out[0] = __uint_as_float(x.x);
+                                    if (n + 1 < a.N) out[1] = __uint_as_float(x.y);
+                                    if (n + 2 < a.N) out[2] = __uint_as_float(x.z);
+                                    if (n + 3 < a.N) out[3] = __uint_as_float(x.w);
+                                }
                             }
-                        }
-                    });
+                        });
+                    }
                 }
             } else if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
                 // QKV projection: a head's q, k or v of this row is the thread's own, rotate-half partners included.
@@ -492,8 +499,8 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     a.wide = (low & 15) == 0;
     a.n_pairs = n_tiles / 2;
     a.m_tiles = (g.M + 2 * kBM - 1) / (2 * kBM);
-    // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (measured with two CTAs per SM at 128 row tiles: groups of
-    // 2 / 4 / 8 / 16 give 430 / 414 / 404 / 407 ms of GEMM time per refresh, no grouping 475)
+    // row tiles per group: 8 x 256 rows x K x 2 B stay in L2 (refresh of one layer over 25568 rows with groups of 4 / 8 / 16:
+    // 10.7 / 10.2 / 10.25 ms)
     a.group = a.m_tiles < 8 ? a.m_tiles : 8;
     a.status = g.status;
     // with several row tiles a weight tile is read once per row tile of its group, by pairs a few microseconds apart:
