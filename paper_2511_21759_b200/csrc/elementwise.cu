@@ -63,7 +63,8 @@ __device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i
 // SPLITS: room for this many partials per row; the loads in flight are registers, and with room for sixteen two blocks
 // fit an SM: the 512 blocks of a 128-row step were 1.7 waves (9 partials: 9.3 us; with room for ten, four blocks per SM,
 // 6.7 to 8 us; layer step of four sequences 162 -> 160 us).
-template <int SPLITS, int BLOCKS>
+// EMBED: the first norm of a forward, whose residual stream is the embedding row of each row's token (no partials).
+template <int SPLITS, int BLOCKS, bool EMBED>
 __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(float* __restrict__ h, const float* __restrict__ partial,
                                                                      int splits, size_t pstride, const float* __restrict__ gain,
                                                                      __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
@@ -80,9 +81,9 @@ __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(flo
     float ss = 0.f;
     if (i < (d >> 2)) {
         float* hr = h + static_cast<size_t>(row) * d;
-        float4 v = emb.table ? embed_load4(emb, row, i, d) : reinterpret_cast<const float4*>(hr)[i];
-        if (emb.table) reinterpret_cast<float4*>(hr)[i] = v;   // first norm of a forward
-        if (partial) {
+        float4 v = EMBED ? embed_load4(emb, row, i, d) : reinterpret_cast<const float4*>(hr)[i];
+        if (EMBED) reinterpret_cast<float4*>(hr)[i] = v;
+        if (!EMBED && partial) {
             const float* p = partial + static_cast<size_t>(row) * d + 4 * i;
             float4 t[SPLITS];
 #pragma unroll
@@ -531,7 +532,8 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
         return launch_norm_rows<kNormRowsMaxSplits, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
                                                            tw, emb);
     }
-    return launch_kernel_if(!first, splits <= 4 ? rmsnorm_kernel<4, 4> : splits <= 10 ? rmsnorm_kernel<10, 4> : rmsnorm_kernel<16, 2>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
+    return launch_kernel_if(!first, first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
+                            splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<16, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
                             st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb);
 }
 
