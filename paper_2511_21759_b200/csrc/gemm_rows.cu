@@ -19,10 +19,11 @@
 // CTA, and no second pair either: an allocation for a pair needs the same columns in both SMs, so two of them meeting on
 // one pair of SMs, or one meeting single-SM allocations of a successor, could wait for each other.
 //
-// Measured against the kernels this replaces (8B shape, one launch each, 768 / 4096 / 25568 rows):
-//   SwiGLU                                154 -> 108, 793 -> 554 us, 4.52 -> 3.5 ms (1.43, 1.49, 1.47 PFLOP/s; 1.66 is the peak)
-//   QKV + RoPE + cache scatter             72 -> 60, 330 -> 283 us, 2.17 -> 1.8 ms (projection and RoPE kernel before)
+// Measured against the kernels this replaces (8B shape, one launch each, 768 / 4096 / 25600 rows):
+//   SwiGLU                                154 -> 106, 793 -> 515 us, 4.52 -> 3.34 ms (1.46, 1.60, 1.54 PFLOP/s; 1.68 is the peak)
+//   QKV + RoPE + cache scatter             72 -> 59, 330 -> 273 us, 2.17 -> 1.71 ms (projection and RoPE kernel before)
 //   LM head + statistics at 256 rows      321 -> 205 us
+// Tensor pipe busy in 86 % (SwiGLU), 80 % (QKV) of the cycles at 4096 rows.
 #include "odb_internal.cuh"
 #include "tcgen05_common.cuh"
 

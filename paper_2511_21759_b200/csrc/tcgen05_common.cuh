@@ -82,8 +82,8 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// ---- CTA pair (cta_group::2): two CTAs of a cluster on neighbouring SMs issue ONE MMA of 256 weight rows.
-// Each CTA stages its own 128 weight rows and HALF of the activation rows; the leader (cluster rank 0)
+// ---- CTA pair (cta_group::2): two CTAs of a cluster on neighbouring SMs issue ONE MMA of 256 x 256 rows.
+// Each CTA stages 128 rows of either operand; the leader (cluster rank 0)
 // issues the MMAs, which read both CTAs' shared memory and write both CTAs' TMEM.  TMA loads of both
 // CTAs report their bytes to the leader's barrier (the shared::cluster address with the pair bit cleared).
 constexpr uint32_t kPeerBitMask = 0xFEFFFFFFu;
