@@ -43,7 +43,7 @@ extern "C" int32_t odb_gemm_static_scratch(const void* x, const void* w_packed, 
                                            int32_t K, int32_t k_splits, void* stream) {
     if (!x || !w_packed || !out) return ODB_ERR_ARG;
     if (M < 1 || N < 1 || K < 8 || K % 8) return ODB_ERR_SHAPE;
-    int splits = k_splits > 0 ? k_splits : gemm_pick_splits(M, N, K, kScratchBytes / sizeof(float));
+    int splits = k_splits > 0 ? k_splits : gemm_pick_splits(M, N, K);
     const int nkb = (K + 63) / 64;
     if (splits > nkb) splits = nkb;
     while (splits > 1 && ((nkb + splits - 1) / splits) * (splits - 1) >= nkb) --splits;

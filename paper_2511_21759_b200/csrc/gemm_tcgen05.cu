@@ -547,7 +547,7 @@ int gemm_whole_splits(int splits, int nkb) {
     return splits;
 }
 
-int gemm_pick_splits(int M, int N, int K, size_t max_partials) {
+int gemm_pick_splits(int M, int N, int K) {
     const int n_tiles = (N + kBM - 1) / kBM;
     const bool pair = use_pair(M, n_tiles);
     const int bn = pair ? 2 * kBM : pick_bn(M);
@@ -564,20 +564,19 @@ int gemm_pick_splits(int M, int N, int K, size_t max_partials) {
         }
         const int most = tiles >= big_target ? 1 : big_target / tiles;
         const int many = gemm_whole_splits(most < nkb / 8 ? most : nkb / 8, nkb);
-        const int few = gemm_whole_splits(most < nkb / 12 ? most : nkb / 12, nkb);
-        auto fits = [&](int k) { return k == few || static_cast<size_t>(k) * M * N <= max_partials; };
-        if (!pair) return fits(many) ? many : few;
+        if (!pair) return many;
         // Pairs: between 12 and 8 k-blocks per split, the number with the least work in a row.  A k-block of a tile takes
         // 0.42 us; in that unit the waves of 74 pairs cost their length, a partial sum written and read back 2.4e-6 (1 ps,
         // eight bytes mostly in L2), partials at all 2 (the next kernel adds them, a QKV projection needs a RoPE kernel).
         // Splits of 8 / of 12 k-blocks always / this rule, us per refresh of two layers: d 1024 at 160 rows 166.7 / 168.4 /
         // 166.7, at 600 rows 226 / 222 / 221, at 1250 rows 262 / 227 / 227; d 2048 at 160 rows 215 / 198 / 197, at 350 rows
         // 275 / 279 / 277.
+        const int few = gemm_whole_splits(most < nkb / 12 ? most : nkb / 12, nkb);
         constexpr int kPairs = 74;
         int best = few;
         double best_cost = 0;
         for (int k = few; k <= many; ++k) {
-            if (k != gemm_whole_splits(k, nkb) || !fits(k)) continue;
+            if (k != gemm_whole_splits(k, nkb)) continue;
             const double cost = static_cast<double>((tiles / 2 * k + kPairs - 1) / kPairs) * ((nkb + k - 1) / k) +
                                 (k > 1 ? 2 + 2.4e-6 * k * M * N : 0);
             if (k == few || cost < best_cost) { best = k; best_cost = cost; }

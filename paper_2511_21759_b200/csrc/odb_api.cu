@@ -1197,8 +1197,7 @@ int32_t odb_debug_gemm(const void* x, const void* w, float* out, void* scratch, 
                        int32_t N, int32_t K, int32_t k_splits, void* stream) {
     if (!x || !w || !out || !scratch) return ODB_ERR_ARG;
     if (M < 1 || N < 1 || K < 8 || K % 8) return ODB_ERR_SHAPE;
-    const size_t room = scratch_bytes < 512 ? 0 : (scratch_bytes - 512) / sizeof(float);   // behind the partial sums: the status word
-    int splits = k_splits > 0 ? k_splits : gemm_pick_splits(M, N, K, room);
+    int splits = k_splits > 0 ? k_splits : gemm_pick_splits(M, N, K);
     const int nkb = (K + 63) / 64;
     if (splits > nkb) splits = nkb;
     while (splits > 1 && ((nkb + splits - 1) / splits) * (splits - 1) >= nkb) --splits;

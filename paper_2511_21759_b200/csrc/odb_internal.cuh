@@ -321,8 +321,7 @@ struct GemmArgs {
     int splits;
     int* status;           // device status word
 };
-// K splits of a projection; more than 128 rows: no more than max_partials partial sums where 12 k-blocks per split need less
-int gemm_pick_splits(int M, int N, int K, size_t max_partials = ~size_t(0));
+int gemm_pick_splits(int M, int N, int K);
 // the largest number of K splits <= splits that leaves none of them empty: ceil(nkb / splits) * (splits - 1) < nkb
 int gemm_whole_splits(int splits, int nkb);
 

@@ -23,13 +23,6 @@ def test_key_splits_of_the_attention(items, hd, refresh, splits):
     assert _rule("_ZN3odb20attention_key_splitsEiib", ctypes.c_int, ctypes.c_int, ctypes.c_bool)(items, hd, refresh) == splits
 
 
-ANY = (1 << 64) - 1
-
-
-def _pick():
-    return _rule("_ZN3odb16gemm_pick_splitsEiiim", ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_size_t)
-
-
 @pytest.mark.parametrize("M,N,K,splits", [
     # CTA pairs, few rows: as many splits as leave 8 k-blocks each, while they fit one wave of 74 pairs
     (160, 3072, 1024, 2), (160, 1024, 1024, 2), (160, 1024, 2816, 5), (350, 1024, 2816, 5),
@@ -40,24 +33,13 @@ def _pick():
     (129, 256, 64, 1),                     # a single k-block
 ])
 def test_k_splits_of_many_rows(M, N, K, splits):
-    assert _pick()(M, N, K, ANY) == splits
-
-
-@pytest.mark.parametrize("M,N,K,room,splits", [
-    (130, 2048, 5504, 2 << 20, 7),         # 9 splits would be the least work, 7 (12 k-blocks) are what 8 MiB hold
-    (130, 2048, 5504, 9 * 130 * 2048, 9),
-    (130, 2048, 5504, 1, 7),               # too small for any: the caller refuses what it is given
-    (300, 640, 1024, 300 * 640, 1), (300, 640, 1024, 2 * 300 * 640, 2),   # single CTAs
-])
-def test_k_splits_that_fit_a_scratch_buffer(M, N, K, room, splits):
-    """The number of splits never keeps a call out of a buffer that 12 k-blocks per split fit."""
-    assert _pick()(M, N, K, room) == splits
+    assert _rule("_ZN3odb16gemm_pick_splitsEiii", *[ctypes.c_int] * 3)(M, N, K) == splits
 
 
 def test_k_splits_are_never_empty():
-    pick = _pick()
+    pick = _rule("_ZN3odb16gemm_pick_splitsEiii", *[ctypes.c_int] * 3)
     for M in (1, 32, 128, 129, 256, 300, 768, 1118, 4096):
         for N in (64, 128, 255, 640, 1024, 3072, 12288):
             for nkb in list(range(1, 40)) + [64, 86, 192]:
-                s = pick(M, N, 64 * nkb, ANY)
+                s = pick(M, N, 64 * nkb)
                 assert 1 <= s <= max(1, nkb // 4) and -(-nkb // s) * (s - 1) < nkb, (M, N, nkb, s)
