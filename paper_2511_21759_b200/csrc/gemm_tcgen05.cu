@@ -549,42 +549,25 @@ int gemm_whole_splits(int splits, int nkb) {
 
 int gemm_pick_splits(int M, int N, int K) {
     const int n_tiles = (N + kBM - 1) / kBM;
-    const bool pair = use_pair(M, n_tiles);
-    const int bn = pair ? 2 * kBM : pick_bn(M);
+    const int bn = use_pair(M, n_tiles) ? 2 * kBM : pick_bn(M);
     const int tiles = n_tiles * ((M + bn - 1) / bn);
     const int nkb = (K + kBK - 1) / kBK;
+    // all work units must be resident at once (two CTA slots per SM) and equal in size: a
+    // second, partly filled wave would double the kernel's time
     if (M > 128) {
-        // many rows (refresh): compute bound, and every K split costs M x N fp32 partials written and read back, so split
-        // only when the tiles alone cannot occupy the SMs: 296 tiles are one wave of single CTAs (two per SM), and two
-        // waves of CTA pairs (74, two weight tiles each)
+        // many rows (refresh): compute bound, and every K split costs M x N fp32 partials written and
+        // read back, so split only when the tiles alone cannot occupy the SMs
         static int big_target = 0;
         if (!big_target) {
             const char* e = getenv("ODB_GEMM_BIG_TARGET_CTAS");
             big_target = e ? atoi(e) : 296;
         }
-        const int most = tiles >= big_target ? 1 : big_target / tiles;
-        const int many = gemm_whole_splits(most < nkb / 8 ? most : nkb / 8, nkb);
-        if (!pair) return many;
-        // Pairs: between 12 and 8 k-blocks per split, the number with the least work in a row.  A k-block of a tile takes
-        // 0.42 us; in that unit the waves of 74 pairs cost their length, a partial sum written and read back 2.4e-6 (1 ps,
-        // eight bytes mostly in L2), partials at all 2 (the next kernel adds them, a QKV projection needs a RoPE kernel).
-        // Splits of 8 / of 12 k-blocks always / this rule, us per refresh of two layers: d 1024 at 160 rows 166.7 / 168.4 /
-        // 166.7, at 600 rows 226 / 222 / 221, at 1250 rows 262 / 227 / 227; d 2048 at 160 rows 215 / 198 / 197, at 350 rows
-        // 275 / 279 / 277.
-        const int few = gemm_whole_splits(most < nkb / 12 ? most : nkb / 12, nkb);
-        constexpr int kPairs = 74;
-        int best = few;
-        double best_cost = 0;
-        for (int k = few; k <= many; ++k) {
-            if (k != gemm_whole_splits(k, nkb)) continue;
-            const double cost = static_cast<double>((tiles / 2 * k + kPairs - 1) / kPairs) * ((nkb + k - 1) / k) +
-                                (k > 1 ? 2 + 2.4e-6 * k * M * N : 0);
-            if (k == few || cost < best_cost) { best = k; best_cost = cost; }
-        }
-        return best;
+        int sp = tiles >= big_target ? 1 : big_target / tiles;
+        // at least 12 k-blocks (5 us of main loop) per split: below that its epilogue and the partials' way through memory
+        // cost more than the idle pairs (1118 rows, d 1024: refresh of two layers 267 us with 8, 243 with 12, 246 with 16)
+        if (sp > nkb / 12) sp = nkb / 12;
+        return gemm_whole_splits(sp, nkb);
     }
-    // all work units must be resident at once (two CTA slots per SM) and equal in size: a
-    // second, partly filled wave would double the kernel's time
     int splits = target_ctas() / tiles;
     if (splits > nkb / 4) splits = nkb / 4;
     if (splits > 16) splits = 16;
