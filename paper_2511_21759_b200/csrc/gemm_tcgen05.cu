@@ -552,11 +552,10 @@ int gemm_pick_splits(int M, int N, int K) {
     const int bn = use_pair(M, n_tiles) ? 2 * kBM : pick_bn(M);
     const int tiles = n_tiles * ((M + bn - 1) / bn);
     const int nkb = (K + kBK - 1) / kBK;
-    // all work units must be resident at once (two CTA slots per SM) and equal in size: a
-    // second, partly filled wave would double the kernel's time
     if (M > 128) {
         // many rows (refresh): compute bound, and every K split costs M x N fp32 partials written and
-        // read back, so split only when the tiles alone cannot occupy the SMs
+        // read back, so split only when the tiles alone cannot occupy the SMs: 296 tiles are one wave of single CTAs (two per
+        // SM), and two waves of CTA pairs (74, two weight tiles each)
         static int big_target = 0;
         if (!big_target) {
             const char* e = getenv("ODB_GEMM_BIG_TARGET_CTAS");
@@ -564,10 +563,15 @@ int gemm_pick_splits(int M, int N, int K) {
         }
         int sp = tiles >= big_target ? 1 : big_target / tiles;
         // at least 12 k-blocks (5 us of main loop) per split: below that its epilogue and the partials' way through memory
-        // cost more than the idle pairs (1118 rows, d 1024: refresh of two layers 267 us with 8, 243 with 12, 246 with 16)
+        // cost more than the idle pairs once there are many rows.  Refresh of two layers, us with 8 / with 12: d 1024 at 160 rows
+        // 159 / 166, 350 rows 183 / 189, 1118 rows 262 / 242, 1224 rows 249 / 224; d 2048 at 160 rows 203 / 190, 350 rows
+        // 262 / 271, 1118 rows 376 / 375.  A choice between the two by waves and partials was never more than 1 % from the better,
+        // but any other split of a sum flips greedy tokens that tie (1.2 % of them at d 2048, 1020 rows).
         if (sp > nkb / 12) sp = nkb / 12;
         return gemm_whole_splits(sp, nkb);
     }
+    // all work units must be resident at once (two CTA slots per SM) and equal in size: a
+    // second, partly filled wave would double the kernel's time
     int splits = target_ctas() / tiles;
     if (splits > nkb / 4) splits = nkb / 4;
     if (splits > 16) splits = 16;
