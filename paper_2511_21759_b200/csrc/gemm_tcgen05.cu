@@ -14,8 +14,8 @@
 // 128-byte pieces 2K bytes apart and HBM delivers little more than half its bandwidth (measured).
 //
 // One CTA = one 128 x BN output tile over one K range.  Warp 0 lane 0 issues TMA loads into a
-// ring of shared-memory stages, warp 1 lane 0 issues the MMAs (accumulator in TMEM) and frees
-// stages through tcgen05.commit, warps 2..5 read the accumulator back (tcgen05.ld) and store
+// rings of shared-memory stages (weights, activation rows), warp 1 lane 0 issues the MMAs (accumulator in TMEM) and
+// frees stages through tcgen05.commit, the other warps read the accumulator back (tcgen05.ld) and store
 // fp32 partials.  Splits are reduced later in a fixed order by the consumer kernel, so results
 // are run-to-run identical.  Every mbarrier wait is bounded: on expiry the CTA records
 // ODB_ERR_TIMEOUT, stops issuing work, releases its TMEM and exits.
@@ -28,9 +28,11 @@ namespace odb {
 
 namespace {
 
+constexpr int kMaxStages = 5;
+
 struct alignas(8) GemmShared {
-    uint64_t full[16];
-    uint64_t empty[16];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t acc_full;
     uint32_t tmem_base;
     int abort;
@@ -43,13 +45,23 @@ struct alignas(8) GemmShared {
 // (gate) with lane r + 64 (up) through shared memory and stores bf16(silu(gate) * up) to
 // g[m][64 t + r]; N is then the FFN width F and there is no K split.
 constexpr int EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_CONF = 3;
-constexpr int kMinStages = 2;
+constexpr int kMinStages = 3;
+
+// Groups of four epilogue warps; group g takes the activation rows [g, g + 1) * BN / groups of the tile.  Every CTA of a
+// one-wave launch ends at the same time, so an epilogue is paid in full: with four warps the gate/up projection of 128 rows had
+// 14 us that did not grow with K, of 32 rows 7.  Measured (8B shape, us): gate/up at 128 rows 46.5 with one group, 41.3 with
+// two, 41.0 with four; at 64 rows 38.5 -> 36.1; LM head at 128 rows 220 / 190 / 175, at 64 rows 184 -> 163 (32 rows: 161).
+// The partial sums' epilogue is stores alone: more warps make it slower (QKV at 128 rows 21.3 -> 22.4).
+__host__ __device__ constexpr int epilogue_groups(int bn, int epi) {
+    return bn == 32 || epi == EPI_PARTIAL ? 1 : bn == 128 && epi == EPI_CONF ? 4 : 2;
+}
+__host__ __device__ constexpr int gemm_threads(int bn, int epi) { return 64 + 128 * epilogue_groups(bn, epi); }
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(BN, EPI), 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
             float* __restrict__ partial, __nv_bfloat16* __restrict__ act_out, RowScale rs,
-            ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int stages,
+            ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int w_stages, int x_stages,
             int l2_prefetch, int* status, const __grid_constant__ PeerOut po) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr uint32_t kABytes = kBM * kBK * 2;
@@ -57,11 +69,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     constexpr uint32_t kStageBytes = kABytes + kBBytes;
     constexpr uint32_t kTmemCols = BN;
     // the epilogues exchange values through the stage ring, which holds at least kMinStages stages
-    constexpr uint32_t kExchangeBytes = EPI == EPI_SWIGLU ? 2 * 64 * (BN / 2 + 1) * 4 : EPI == EPI_CONF ? 32 * 129 * 4 : 0;
-    static_assert(kExchangeBytes <= kMinStages * kStageBytes, "the exchange buffer must end inside the ring");
+    constexpr int kGroups = epilogue_groups(BN, EPI), kGroupRows = BN / kGroups;
+    constexpr uint32_t kExchangeBytes = EPI == EPI_SWIGLU ? 2 * 64 * (kGroupRows / 2 + 1) * 4 : EPI == EPI_CONF ? 32 * 129 * 4 : 0;
+    static_assert(kGroups * kExchangeBytes <= kMinStages * kStageBytes, "the exchange buffer must end inside the ring");
 
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    GemmShared* sh = reinterpret_cast<GemmShared*>(tiles + static_cast<size_t>(stages) * kStageBytes);
+    // Two rings, not one of whole stages: the weights come from HBM and need more bytes in flight than the activation rows,
+    // which come from L2.  No slack for an alignment: the rings end where the second CTA of the SM begins.
+    uint8_t* tiles = smem_raw;                                                  // [w_stages][128][64] weights
+    uint8_t* xring = tiles + static_cast<size_t>(w_stages) * kABytes;           // [x_stages][BN][64] activation rows
+    GemmShared* sh = reinterpret_cast<GemmShared*>(xring + static_cast<size_t>(x_stages) * kBBytes);
+    if ((smem_u32(smem_raw) & 1023u) != 0) {                // the swizzled tiles need 1024-byte alignment
+        if (threadIdx.x == 0) atomicExch(status, ODB_ERR_CUDA);
+        pdl_wait();
+        return;
+    }
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -80,7 +101,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
 
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
-        for (int i = 0; i < stages; ++i) {
+        for (int i = 0; i < w_stages; ++i) {
             mbar_init(&sh->full[i], 1);
             mbar_init(&sh->empty[i], 1);
         }
@@ -110,11 +131,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // ---- TMA producer ----
             // The weights do not depend on the preceding kernel: fill the ring with weight tiles
             // first, then wait for the predecessor and fetch the activation tiles.
-            const int pre = nkb < stages ? nkb : stages;
-            for (int i = 0; i < pre; ++i) {
-                mbar_expect_tx(&sh->full[i], kStageBytes);
-                tma_load_3d(tiles + static_cast<size_t>(i) * kStageBytes, &tmap_w, &sh->full[i], 0, 0, wtile0 + i, kEvictFirst);
-            }
+            const int pre = nkb < w_stages ? nkb : w_stages, xpre = nkb < x_stages ? nkb : x_stages;
+            auto load_w = [&](int i, int st) {   // arms the barrier of k-block i for its weights and its activation rows
+                mbar_expect_tx(&sh->full[st], kStageBytes);
+                tma_load_3d(tiles + static_cast<size_t>(st) * kABytes, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
+            };
+            auto load_x = [&](int i, int st, int slot) {
+                tma_load_2d(xring + static_cast<size_t>(slot) * kBBytes, &tmap_x, &sh->full[st], (kb0 + i) * kBK, m0, kEvictLast);
+            };
+            for (int i = 0; i < pre; ++i) load_w(i, i);
             // and ask L2 for the weight tiles that follow, so that HBM keeps streaming while the
             // predecessor (a short elementwise kernel) is still running
             int pf = nkb - pre;
@@ -125,26 +150,30 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                              "r"(0), "r"(0), "r"(wtile0 + i)
                              : "memory");
             pdl_wait();
-            for (int i = 0; i < pre; ++i)
-                tma_load_2d(tiles + static_cast<size_t>(i) * kStageBytes + kABytes, &tmap_x, &sh->full[i], (kb0 + i) * kBK, m0, kEvictLast);
+            for (int i = 0; i < xpre; ++i) load_x(i, i, i);
+            // the MMAs of k-block i free its weight stage for k-block i + w_stages and its activation stage for i + x_stages
+            int st = 0, slot = 0, xst = x_stages;   // weight stage and activation slot of i; weight stage of i + x_stages
+            if (xst >= w_stages) xst -= w_stages;
+            uint32_t ph = 0;
             int issued = pre;
-            for (int i = pre; i < nkb; ++i) {
-                const int st = i % stages;
-                const uint32_t ph = static_cast<uint32_t>(i / stages) & 1u;
-                if (!mbar_wait(&sh->empty[st], ph ^ 1u, cta_abort, status)) break;
-                uint8_t* a_dst = tiles + static_cast<size_t>(st) * kStageBytes;
-                uint8_t* b_dst = a_dst + kABytes;
-                mbar_expect_tx(&sh->full[st], kStageBytes);
-                tma_load_3d(a_dst, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
-                tma_load_2d(b_dst, &tmap_x, &sh->full[st], (kb0 + i) * kBK, m0, kEvictLast);
-                issued = i + 1;
+            for (int i = 0; i + x_stages < nkb; ++i) {
+                if (!mbar_wait(&sh->empty[st], ph, cta_abort, status)) break;
+                if (i + w_stages < nkb) {
+                    load_w(i + w_stages, st);
+                    issued = i + w_stages + 1;
+                }
+                load_x(i + x_stages, xst, slot);
+                if (++st == w_stages) { st = 0; ph ^= 1u; }
+                if (++xst == w_stages) xst = 0;
+                if (++slot == x_stages) slot = 0;
             }
             if (*cta_abort) {
-                // aborted: let the copies still in flight land before the CTA's shared memory goes away
-                const int first = issued > stages ? issued - stages : 0;
+                // aborted: let the copies still in flight land before the CTA's shared memory goes away (a k-block whose
+                // activation rows were never asked for takes its wait's whole limit)
+                const int first = issued > w_stages ? issued - w_stages : 0;
                 for (int i = first; i < issued; ++i) {
                     const long long t0 = clock64();
-                    while (!mbar_try_wait_parity(&sh->full[i % stages], static_cast<uint32_t>(i / stages) & 1u) &&
+                    while (!mbar_try_wait_parity(&sh->full[i % w_stages], static_cast<uint32_t>(i / w_stages) & 1u) &&
                            clock64() - t0 < kWaitLimitCycles / 8) {
                     }
                 }
@@ -155,29 +184,34 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // ---- MMA issuer ----
             constexpr uint32_t idesc = make_instr_desc(kBM, BN);
             bool ok = true;
-            for (int i = 0; i < nkb && ok; ++i) {
-                const int st = i % stages;
-                const uint32_t ph = static_cast<uint32_t>(i / stages) & 1u;
+            int st = 0, slot = 0;
+            uint32_t ph = 0;
+            for (int i = 0; i < nkb; ++i) {
                 ok = mbar_wait(&sh->full[st], ph, cta_abort, status);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a_addr = smem_u32(tiles + static_cast<size_t>(st) * kStageBytes);
-                const uint32_t b_addr = a_addr + kABytes;
+                const uint32_t a_addr = smem_u32(tiles + static_cast<size_t>(st) * kABytes);
+                const uint32_t b_addr = smem_u32(xring + static_cast<size_t>(slot) * kBBytes);
 #pragma unroll
                 for (int k = 0; k < kBK / kUmmaK; ++k)
                     umma_bf16(tmem_acc, make_smem_desc(a_addr + k * kUmmaK * 2), make_smem_desc(b_addr + k * kUmmaK * 2), idesc,
                               (i > 0 || k > 0) ? 1u : 0u);
-                umma_commit(&sh->empty[st]);   // frees the stage once these MMAs have read it
+                umma_commit(&sh->empty[st]);   // frees both stages once these MMAs have read them
+                if (++st == w_stages) { st = 0; ph ^= 1u; }
+                if (++slot == x_stages) slot = 0;
             }
             if (ok) umma_commit(&sh->acc_full);
         }
     } else {
-        // ---- epilogue: warps 2..5 own TMEM lanes 32*(warp%4) .. +31 ----
+        // ---- epilogue: the four warps of a group own TMEM lanes 32*(warp%4) .. +31, and the group's activation rows ----
         const int q = warp & 3;
+        const int grp = kGroups == 1 ? 0 : (warp - 2) >> 2, gthread = static_cast<int>(threadIdx.x) - 64 - 128 * grp;
+        const int g0 = grp * kGroupRows;                                   // the group's first row within the tile
+        auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory"); };
         pdl_wait();   // the previous reader of the output buffer has finished; the predecessor's results are visible
         if (rs.ssq) {   // uniform: row scalars of this tile's activation rows, computed while the main loop runs
-            for (int i = threadIdx.x - 64; i < BN; i += 128) sh->scale[i] = m0 + i < M ? row_scale_of(rs, m0 + i) : 1.0f;
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            for (int i = g0 + gthread; i < g0 + kGroupRows; i += 128) sh->scale[i] = m0 + i < M ? row_scale_of(rs, m0 + i) : 1.0f;
+            group_sync();
         }
         const bool ok = nkb > 0 && mbar_wait(&sh->acc_full, 0, cta_abort, status);   // nkb == 0: empty K split
         if (ok) tc_fence_after();
@@ -187,7 +221,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                 const size_t split_off = static_cast<size_t>(split) * M * N;
                 float* out = partial + split_off;
 #pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
+                for (int c = g0 / 32; c < (g0 + kGroupRows) / 32; ++c) {
                     uint32_t v[32];
                     __syncwarp();   // tcgen05.ld is a whole-warp instruction, and the stores before are some lanes' only
                     tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
@@ -213,8 +247,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                     }
                 }
             }
-            if (po.n > 0) {   // uniform: the tile's stores of all four warps, then one arrival for the CTA
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (po.n > 0) {   // uniform: the tile's stores of all epilogue warps, then one arrival for the CTA
+                asm volatile("bar.sync 15, %0;" ::"n"(128 * kGroups) : "memory");
                 if (threadIdx.x == 64) tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);
             }
         } else if constexpr (EPI == EPI_CONF) {
@@ -223,10 +257,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // four threads scan one row's 128 logits (32 each, ascending ids, online max / sum of exp /
             // argmax); the four are merged in id order and one (max, sum, argmax) triple per (row, tile)
             // is stored.  The RMSNorm scalar of the row is applied first; [MASK] and padding are skipped.
-            float* xch = reinterpret_cast<float*>(tiles);           // [32 rows][129]
-            const int t = threadIdx.x - 64;                            // 0..127
+            float* xch = reinterpret_cast<float*>(tiles + grp * kExchangeBytes);   // [32 rows][129]
+            const int t = gthread;                                     // 0..127
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
+            for (int c = g0 / 32; c < (g0 + kGroupRows) / 32; ++c) {
                 uint32_t v[32];
                 if (ok) {
                     tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
@@ -234,7 +268,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                 }
 #pragma unroll
                 for (int j = 0; j < 32; ++j) xch[j * 129 + q * 32 + lane] = ok ? __uint_as_float(v[j]) : 0.f;
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                group_sync();
                 const int m_l = t >> 2, part = t & 3;
                 const int m = m0 + c * 32 + m_l;
                 const float sc = rs.ssq ? sh->scale[c * 32 + m_l] : 1.0f;
@@ -271,17 +305,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                         for (int r = 0; r < po.n; ++r) po.conf[r][static_cast<size_t>(m) * ce.tiles_total + ce.tile0 + n_tile] = p;
                     }
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                group_sync();
             }
-            if (po.n > 0 && t == 0) tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);   // behind the loop's last barrier
+            if (po.n > 0) {
+                asm volatile("bar.sync 15, %0;" ::"n"(128 * kGroups) : "memory");
+                if (threadIdx.x == 64) tp_arrive_and_signal(po, gridDim.x * gridDim.y * gridDim.z);
+            }
         } else {
             // All MMAs have completed, so the stage ring is free: the warps that own gate features hand the values of the
             // tile's second half of rows to the warps that own the matching up features, and get the up values of the
             // first half; behind one barrier every warp then finishes its half.  (Up values handed over chunk by chunk
             // behind two barriers each, the up warps idle, in CTA pairs: 50 us for the 8B shape's gate/up projection at
             // 128 rows; this way 47, and 36 instead of 38 at 32 rows.)
-            constexpr int kHalfRows = BN / 2, kPitch = kHalfRows + 1;
-            float* xch = reinterpret_cast<float*>(tiles);             // [gate | up][64 features][kPitch]
+            constexpr int kHalfRows = kGroupRows / 2, kPitch = kHalfRows + 1;
+            float* xch = reinterpret_cast<float*>(tiles + grp * kExchangeBytes);   // [gate | up][64 features][kPitch]
             const int fl = (q & 1) * 32 + lane;                       // feature of this lane within the tile
             const int f = n_tile * 64 + fl;
             const bool is_gate = q < 2;
@@ -292,15 +329,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
 #pragma unroll 1
                 for (int c = 0; c < kHalfRows; c += 16) {
                     uint32_t v[16];
-                    tmem_ld16(tm_lane + static_cast<uint32_t>((is_gate ? kHalfRows : 0) + c), v);
+                    tmem_ld16(tm_lane + static_cast<uint32_t>(g0 + (is_gate ? kHalfRows : 0) + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int j = 0; j < 16; ++j) give[c + j] = __uint_as_float(v[j]);
                 }
             }
-            asm volatile("bar.sync 1, 128;" ::: "memory");            // every epilogue warp, whether or not its wait succeeded
+            group_sync();                                             // every epilogue warp, whether or not its wait succeeded
             if (ok) {
-                const int r0 = is_gate ? 0 : kHalfRows;
+                const int r0 = g0 + (is_gate ? 0 : kHalfRows);
 #pragma unroll 1
                 for (int c = 0; c < kHalfRows; c += 16) {
                     uint32_t v[16];
@@ -450,11 +487,14 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int nkb_total = (a.K + kBK - 1) / kBK;
     const int nkb_per_split = (nkb_total + a.splits - 1) / a.splits;
-    constexpr int kStageBytes = (kBM + BN) * kBK * 2;
-    int stages = 100 * 1024 / kStageBytes;   // two CTAs per SM
-    if (stages > 16) stages = 16;
-    if (stages > nkb_per_split) stages = nkb_per_split < kMinStages ? kMinStages : nkb_per_split;
-    const size_t smem = static_cast<size_t>(stages) * kStageBytes + sizeof(GemmShared) + 1024;
+    // Two CTAs per SM, up to 112 KB of stages each.  Weight x activation stages at 128 rows, us per layer step of 87 rows: 3 x 3
+    // (whole stages) 158.6, 4 x 3 155.5, 4 x 2 162; at 32 rows 4 x 2 131, 5 x 2 127, 5 x 4 121.5, 6 x 4 122.8.
+    constexpr int kWStages = BN == 128 ? 4 : 5, kXStages = BN == 128 ? 3 : 4;
+    constexpr int kWBytes = kBM * kBK * 2, kXBytes = BN * kBK * 2;
+    static_assert(kWStages * kWBytes + kXStages * kXBytes + sizeof(GemmShared) <= 113 * 1024, "two CTAs share an SM");
+    const int least = nkb_per_split < kMinStages ? kMinStages : nkb_per_split;
+    const int w_stages = kWStages < least ? kWStages : least, x_stages = kXStages < least ? kXStages : least;
+    const size_t smem = static_cast<size_t>(w_stages) * kWBytes + static_cast<size_t>(x_stages) * kXBytes + sizeof(GemmShared);
     static std::atomic<unsigned long long> attr_done{0};
     e = set_smem_limit_once(attr_done, gemm_kernel<BN, EPI>, 227 * 1024);
     if (e != cudaSuccess) return e;
@@ -465,8 +505,8 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
         const char* env = getenv("ODB_GEMM_L2_PREFETCH");
         l2_prefetch = env ? atoi(env) : 0;   // measured: prefetching into L2 slows the step down
     }
-    return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(kThreads), smem, st, a.tmap_w, tmx, a.partial, a.act_out, a.row_scale, a.conf,
-                         a.M, a.N, nkb_total, nkb_per_split, stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
+    return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(gemm_threads(BN, EPI)), smem, st, a.tmap_w, tmx, a.partial, a.act_out, a.row_scale, a.conf,
+                         a.M, a.N, nkb_total, nkb_per_split, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
 }
 
 template <int EPI>
