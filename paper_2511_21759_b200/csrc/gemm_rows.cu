@@ -59,6 +59,7 @@ struct RowsArgs {
     RowScale rs;
     int M, N, nkb_total, nkb_per_split;
     int n_pairs, m_tiles, group, splits;   // pairs of weight tiles, tiles of 256 rows, row tiles that are walked side by side
+    int whole, n_items;          // the items from `whole` on are single weight tiles
     uint64_t w_hint;             // L2 policy of the weight tiles
     int wide;                    // ROWS_PARTIAL: output rows start on 16-byte boundaries
     int* status;
@@ -67,19 +68,31 @@ struct RowsArgs {
 // The tiles in the order they are handed out, round robin, to the pairs: the row tiles of a group side by side on one
 // weight-tile pair (its weights come from HBM once, from L2 for the other row tiles), then the next weight-tile pair
 // (the group's activation rows stay in L2: 17 MB at K 4096, 50 MB at K 12288), then the next group, then the next K split.
+//
+// HALVES: the items that do not fill a last round of the pairs are two items each, of one packed weight tile (256 x 128;
+// either CTA stages half of its rows).
 struct RowsItem {
-    int m_tile, pair, split, kb0, nkb;
+    int m_tile, tile, split, kb0, nkb;   // tile: packed weight tile, the first of two unless half
+    bool half;
 };
+template <bool HALVES>
 __device__ __forceinline__ RowsItem rows_item(const RowsArgs& a, int item) {
     RowsItem w;
+    int second = 0;
+    w.half = HALVES && item >= a.whole;
+    if (w.half) {
+        second = (item - a.whole) & 1;
+        item = a.whole + ((item - a.whole) >> 1);
+    }
     const int per_split = a.m_tiles * a.n_pairs;
     w.split = item / per_split;
     item -= w.split * per_split;
     const int g = item / (a.group * a.n_pairs), m_first = g * a.group;
     const int in_group = min(a.group, a.m_tiles - m_first);
     item -= m_first * a.n_pairs;
-    w.pair = item / in_group;
-    w.m_tile = m_first + item - w.pair * in_group;
+    const int pair = item / in_group;
+    w.m_tile = m_first + item - pair * in_group;
+    w.tile = 2 * pair + second;
     w.kb0 = w.split * a.nkb_per_split;
     w.nkb = min(a.nkb_per_split, a.nkb_total - w.kb0);   // >= 1: the launcher refuses empty splits
     return w;
@@ -138,9 +151,9 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
-template <int EPI>
+template <int EPI, bool HALVES>
 __global__ void __launch_bounds__(kRowsThreads, 1)
-gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RowsArgs a,
+gemm_rows_kernel(const __grid_constant__ WeightMaps maps, const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RowsArgs a,
                  const __grid_constant__ PeerOut po) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -150,7 +163,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int first = static_cast<int>(blockIdx.x) >> 1, step = static_cast<int>(gridDim.x) >> 1;
-    const int n_items = a.m_tiles * a.n_pairs * a.splits;
+    const int n_items = a.n_items;
+    static_assert(!(HALVES && EPI == ROWS_CONF), "the statistics belong to whole tiles");
     volatile int* cta_abort = &sh->abort;
 
     if (threadIdx.x == 0) {
@@ -167,7 +181,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 0 && lane == 0) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_w)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.tile)) : "memory");
+        if (HALVES) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.half)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_x)) : "memory");
     }
     if (warp == 1) {   // the same warp of both CTAs allocates the same columns in both SMs
@@ -181,20 +196,29 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     __syncthreads();
     tc_fence_after();
     cluster_barrier();         // the peer's barriers are initialised before anything signals them
-    pdl_launch_dependents();   // behind the allocation: no successor's allocation can come before it
+    // Behind the allocation: no successor's allocation can come before it.  Not in front of the attention: its CTAs would take
+    // the SMs that this launch leaves free (or leaves first), five on each, and run there side by side (two layers of d 1024,
+    // 1118 rows: 236 -> 232 us; d 256, 2200 rows: 169 -> 126).
+    if (EPI != ROWS_QKV64 && EPI != ROWS_QKV128) pdl_launch_dependents();
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {
         if (lane == 0) {
             // ---- TMA producer: weight tiles of the first stages first (they do not depend on the preceding kernel) ----
-            RowsItem w = rows_item(a, first);
+            RowsItem w = rows_item<HALVES>(a, first);
             const int pre = w.nkb < kRowsStages ? w.nkb : kRowsStages;
-            int wt = (2 * w.pair + static_cast<int>(rank)) * a.nkb_total + w.kb0;
-            int mrow = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM;
-            for (int i = 0; i < pre; ++i) {
-                if (leader) mbar_expect_tx(&sh->full[i], 2 * kRowsStageBytes);   // the loads of both CTAs report to the leader
-                tma_load_3d_pair(ring + i * kRowsStageBytes, &tmap_w, &sh->full[i], 0, 0, wt + i, a.w_hint);
-            }
+            int wt, wrow, mrow;
+            auto begin = [&]() {
+                wt = (w.tile + (w.half ? 0 : static_cast<int>(rank))) * a.nkb_total + w.kb0;
+                wrow = w.half ? static_cast<int>(rank) * (kBM / 2) : 0;
+                mrow = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM;
+            };
+            auto load_w = [&](int i, int st) {   // the loads of both CTAs report to the leader
+                if (leader) mbar_expect_tx(&sh->full[st], w.half ? 3 * kTileBytes : 2 * kRowsStageBytes);
+                tma_load_3d_pair(ring + st * kRowsStageBytes, w.half ? &maps.half : &maps.tile, &sh->full[st], 0, wrow, wt + i, a.w_hint);
+            };
+            begin();
+            for (int i = 0; i < pre; ++i) load_w(i, i);
             pdl_wait();
             for (int i = 0; i < pre; ++i)
                 tma_load_2d_pair(ring + i * kRowsStageBytes + kTileBytes, &tmap_x, &sh->full[i], (w.kb0 + i) * kBK, mrow, kEvictLast);
@@ -207,18 +231,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 for (; i < w.nkb && ok; ++i) {
                     ok = mbar_wait(&sh->empty[st], ph ^ 1u, cta_abort, a.status);   // the first round's stages are free
                     if (!ok) break;
-                    uint8_t* dst = ring + st * kRowsStageBytes;
-                    if (leader) mbar_expect_tx(&sh->full[st], 2 * kRowsStageBytes);
-                    tma_load_3d_pair(dst, &tmap_w, &sh->full[st], 0, 0, wt + i, a.w_hint);
-                    tma_load_2d_pair(dst + kTileBytes, &tmap_x, &sh->full[st], (w.kb0 + i) * kBK, mrow, kEvictLast);
+                    load_w(i, st);
+                    tma_load_2d_pair(ring + st * kRowsStageBytes + kTileBytes, &tmap_x, &sh->full[st], (w.kb0 + i) * kBK, mrow, kEvictLast);
                     ++issued;
                     if (++st == kRowsStages) { st = 0; ph ^= 1u; }
                 }
                 item += step;
                 if (!ok || item >= n_items) break;
-                w = rows_item(a, item);
-                wt = (2 * w.pair + static_cast<int>(rank)) * a.nkb_total + w.kb0;
-                mrow = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM;
+                w = rows_item<HALVES>(a, item);
+                begin();
                 i = 0;
             }
             if (*cta_abort && leader) {
@@ -235,12 +256,13 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     } else if (warp == 1) {
         if (lane == 0 && leader) {
             // ---- MMA issuer (the leader's, for both CTAs): A = activation rows, B = weight rows ----
-            constexpr uint32_t idesc = make_instr_desc(2 * kBM, kRowsN);
             bool ok = true;
             int st = 0, n = 0;
             uint32_t ph = 0;
             for (int item = first; item < n_items && ok; item += step, ++n) {
-                const int nkb = rows_item(a, item).nkb, b = n & 1;
+                const RowsItem w = rows_item<HALVES>(a, item);
+                const int nkb = w.nkb, b = n & 1;
+                const uint32_t idesc = w.half ? make_instr_desc(2 * kBM, kRowsN / 2) : make_instr_desc(2 * kBM, kRowsN);
                 const uint32_t acc = tmem_acc + static_cast<uint32_t>(b * kRowsN);
                 ok = mbar_wait(&sh->acc_empty[b], ((n >> 1) & 1) ^ 1u, cta_abort, a.status);   // free at first
                 tc_fence_after();
@@ -260,20 +282,20 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             }
         }
     } else {
-        // ---- epilogue: warps 2..9 own TMEM lanes 32 * (warp % 4) .. + 31 = activation rows, and the 128 columns of
-        // packed weight tile 2 * pair + t ----
+        // ---- epilogue: warps 2..9 own TMEM lanes 32 * (warp % 4) .. + 31 = activation rows; group t of four warps owns the
+        // 128 columns of an item's packed weight tile t, or half t of the columns of its only one ----
         const int q = warp & 3, t = (warp - 2) >> 2;
         uint8_t* patch = patches + (warp - 2) * kPatchBytes;
         const uint32_t free_bar = leader_address(&sh->acc_empty[0]);
         pdl_wait();   // the previous reader of the output buffer has finished; the predecessor's results are visible
         int n_done = 0;
         for (int item = first; item < n_items; item += step, ++n_done) {
-            const RowsItem w = rows_item(a, item);
+            const RowsItem w = rows_item<HALVES>(a, item);
             const int b = n_done & 1;
             const int mw = w.m_tile * 2 * kBM + static_cast<int>(rank) * kBM + q * 32;   // the warp's first row
             const int m = mw + lane;
-            const int tile = 2 * w.pair + t;
-            const uint32_t tmem = tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * kRowsN + t * kBM);
+            const int tile = w.half ? w.tile : w.tile + t;
+            const uint32_t tmem = tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * kRowsN + (w.half ? 0 : t * kBM));
             const float sc = m < a.M ? row_scale_of(a.rs, m) : 1.0f;
             int pos = 0, seq = 0;
             if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
@@ -284,6 +306,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             if constexpr (EPI == ROWS_SWIGLU) {
 #pragma unroll
                 for (int c = 0; c < 64; c += 16) {
+                    if (w.half && c / 32 != t) continue;
                     uint32_t g[16], u[16];
                     __syncwarp();
                     tmem_ld16(tmem + c, g);
@@ -302,6 +325,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 __syncwarp();
                 take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
                     const int f = tile * 64 + ch * 8;
+                    if (w.half && ch / 4 != t) return;
                     if (mw + r < a.M && f < a.N)             // F % 16 == 0
                         *reinterpret_cast<uint4*>(a.act_out + static_cast<size_t>(mw + r) * a.N + f) = x;
                 });
@@ -309,6 +333,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 const size_t split_off = static_cast<size_t>(w.split) * a.M * a.N;
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
+                    if (w.half && c / 2 != t) continue;
                     const int nc = tile * kBM + c * 32;
                     if (nc >= a.N) break;
                     uint32_t v[32];
@@ -361,6 +386,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 const float2* rope = e.rope_t + pos;
 #pragma unroll 1
                 for (int piece = 0; piece < kBM / 64; ++piece) {
+                    if (w.half && piece != t) continue;
                     const int grp = HD == 128 ? 0 : piece, c0 = HD == 128 ? piece * 32 : 0;
                     const int g = tile * (kBM / HD) + grp;             // head of [Wq; Wk; Wv]
                     if (g >= 3 * e.H) break;
@@ -482,6 +508,12 @@ int sm_pairs() {
     return v;
 }
 
+// Launches of up to this many rounds hand out single weight tiles in their last one.  Such an item takes about 0.7 of a whole
+// one, and a launch that knows both kinds is 3 to 4 % slower on the whole ones.  Measured (us; without / with): one round or
+// less, refresh of 160 rows at d 256 82 / 74, d 1024 98 / 89, of 1100 rows at d 1024 157 / 142; up to two, refresh at d 2048 350 rows
+// 150 / 143.5, 500 rows 153 / 147, at d 4096 160 rows 180 / 174; O and down of 4096 rows at d 4096 (3.5 rounds) 106 / 107, 292 / 296.
+constexpr int kHalvesRounds = 2;
+
 template <int EPI>
 cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     CUtensorMap tmx;
@@ -510,13 +542,22 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     a.w_hint = a.m_tiles > 1 ? kEvictNormal : kEvictFirst;
     const long long items = static_cast<long long>(a.n_pairs) * a.m_tiles * g.splits;
     if (items > (1ll << 30)) return cudaErrorInvalidValue;
+    // Single weight tiles for the last round if they still are one round.
+    const int pairs = sm_pairs(), left = static_cast<int>(items % pairs);
+    const bool halves = EPI != ROWS_CONF && left > 0 && 2 * left <= pairs && items <= static_cast<long long>(kHalvesRounds) * pairs;
+    a.whole = static_cast<int>(items) - (halves ? left : 0);
+    a.n_items = static_cast<int>(items) + (halves ? left : 0);
     constexpr int smem = kRowsStages * kRowsStageBytes + 8 * kPatchBytes + sizeof(RowsShared) + 1024;
     static_assert(smem <= 227 * 1024, "one CTA per SM");
-    static std::atomic<unsigned long long> attr_done{0};
-    e = set_smem_limit_once(attr_done, gemm_rows_kernel<EPI>, smem);
+    void (*kernel)(WeightMaps, CUtensorMap, RowsArgs, PeerOut) = gemm_rows_kernel<EPI, false>;
+    if constexpr (EPI != ROWS_CONF) {
+        if (halves) kernel = gemm_rows_kernel<EPI, true>;
+    }
+    static std::atomic<unsigned long long> attr_done[2];
+    e = set_smem_limit_once(attr_done[halves], kernel, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * static_cast<unsigned>(items < sm_pairs() ? items : sm_pairs()));
+    cfg.gridDim = dim3(2 * static_cast<unsigned>(a.n_items < pairs ? a.n_items : pairs));
     cfg.blockDim = dim3(kRowsThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -529,7 +570,7 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<EPI>, g.tmap_w, tmx, a, g.peers);
+    return cudaLaunchKernelEx(&cfg, kernel, g.w, tmx, a, g.peers);
 }
 
 }  // namespace

@@ -60,7 +60,7 @@ extern "C" int32_t odb_gemm_static_scratch(const void* x, const void* w_packed, 
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return ODB_ERR_CUDA;
 
     GemmArgs ga;
-    if (make_weight_tmap(&ga.tmap_w, w_packed, N, K) != cudaSuccess) return ODB_ERR_CUDA;
+    if (make_weight_maps(&ga.w, w_packed, N, K) != cudaSuccess) return ODB_ERR_CUDA;
     ga.x = x;
     ga.partial = reinterpret_cast<float*>(scratch);
     ga.act_out = nullptr;

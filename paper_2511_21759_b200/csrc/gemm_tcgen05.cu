@@ -409,14 +409,14 @@ cudaError_t make_tmap_2d(CUtensorMap* out, const void* base, int rows, int K, in
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Packed weight [n_tiles * k_blocks][128][64] bf16: one tile = 16 KB contiguous, rows of 128 bytes.
-cudaError_t make_tmap_packed(CUtensorMap* out, const void* base, int N, int K) {
+// Packed weight [n_tiles * k_blocks][128][64] bf16: one tile = 16 KB contiguous, rows of 128 bytes; box = box_rows rows of a tile.
+cudaError_t make_tmap_packed(CUtensorMap* out, const void* base, int N, int K, int box_rows) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t ntiles = static_cast<cuuint64_t>((N + kBM - 1) / kBM) * ((K + kBK - 1) / kBK);
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(kBK), static_cast<cuuint64_t>(kBM), ntiles};
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(kBK) * 2, static_cast<cuuint64_t>(kBK) * kBM * 2};
-    cuuint32_t box[3] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(kBM), 1};
+    cuuint32_t box[3] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(box_rows), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -505,7 +505,7 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
         const char* env = getenv("ODB_GEMM_L2_PREFETCH");
         l2_prefetch = env ? atoi(env) : 0;   // measured: prefetching into L2 slows the step down
     }
-    return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(gemm_threads(BN, EPI)), smem, st, a.tmap_w, tmx, a.partial, a.act_out, a.row_scale, a.conf,
+    return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(gemm_threads(BN, EPI)), smem, st, a.w.tile, tmx, a.partial, a.act_out, a.row_scale, a.conf,
                          a.M, a.N, nkb_total, nkb_per_split, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
 }
 
@@ -528,7 +528,10 @@ bool use_pair(int M, int n_tiles) { return pair_enabled() && M > 128 && (n_tiles
 
 bool gemm_rows_usable(int M, int N) { return use_pair(M, (N + kBM - 1) / kBM); }
 
-cudaError_t make_weight_tmap(CUtensorMap* out, const void* w, int N, int K) { return make_tmap_packed(out, w, N, K); }
+cudaError_t make_weight_maps(WeightMaps* out, const void* w, int N, int K) {
+    const cudaError_t e = make_tmap_packed(&out->tile, w, N, K, kBM);
+    return e == cudaSuccess ? make_tmap_packed(&out->half, w, N, K, kBM / 2) : e;
+}
 
 cudaError_t make_rows_tmap(CUtensorMap* out, const void* base, int rows, int cols, int box_rows) {
     return make_tmap_2d(out, base, rows, cols, box_rows);
@@ -542,8 +545,8 @@ size_t packed_gate_up_bytes(int F, int K) {
     return static_cast<size_t>((F + 63) / 64) * ((K + kBK - 1) / kBK) * kBM * kBK * 2;
 }
 
-cudaError_t make_gate_up_tmap(CUtensorMap* out, const void* w, int F, int K) {
-    return make_tmap_packed(out, w, ((F + 63) / 64) * kBM, K);
+cudaError_t make_gate_up_maps(WeightMaps* out, const void* w, int F, int K) {
+    return make_weight_maps(out, w, ((F + 63) / 64) * kBM, K);
 }
 
 cudaError_t launch_pack_gate_up(const void* src, void* dst, int F, int K, cudaStream_t st) {

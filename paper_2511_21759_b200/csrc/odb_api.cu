@@ -150,8 +150,8 @@ struct odb_model {
     const __nv_bfloat16* embed;
     const float* final_norm;
     std::vector<const float*> norm1, norm2;
-    std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_d;
-    CUtensorMap tm_lm;
+    std::vector<WeightMaps> w_qkv, w_o, w_gu, w_d;
+    WeightMaps w_lm;
     std::vector<const void*> p_qkv, p_o, p_gu;   // packed weight buffers (for L2 prefetch hints)
     const void* p_lm;
 };
@@ -267,7 +267,7 @@ int32_t odb_model_create(const odb_config* cfg, const odb_weights* w, odb_model*
     m->final_norm = w->final_norm;
     m->p_lm = w->lm_head;
     const int d = cfg->d_model, F = ffn_local(*cfg), da = heads_local(*cfg) * cfg->head_dim, nl = cfg->n_layers;
-    m->tm_qkv.resize(nl); m->tm_o.resize(nl); m->tm_gu.resize(nl); m->tm_d.resize(nl);
+    m->w_qkv.resize(nl); m->w_o.resize(nl); m->w_gu.resize(nl); m->w_d.resize(nl);
     cudaError_t e = cudaSuccess;
     for (int l = 0; l < nl && e == cudaSuccess; ++l) {
         if (!w->norm1[l] || !w->norm2[l] || !w->wqkv[l] || !w->wo[l] || !w->wgu[l] || !w->wd[l]) {
@@ -279,10 +279,10 @@ int32_t odb_model_create(const odb_config* cfg, const odb_weights* w, odb_model*
         m->p_qkv.push_back(w->wqkv[l]);
         m->p_o.push_back(w->wo[l]);
         m->p_gu.push_back(w->wgu[l]);
-        e = make_weight_tmap(&m->tm_qkv[l], w->wqkv[l], 3 * da, d);
-        if (e == cudaSuccess) e = make_weight_tmap(&m->tm_o[l], w->wo[l], d, da);
-        if (e == cudaSuccess) e = make_gate_up_tmap(&m->tm_gu[l], w->wgu[l], F, d);
-        if (e == cudaSuccess) e = make_weight_tmap(&m->tm_d[l], w->wd[l], d, F);
+        e = make_weight_maps(&m->w_qkv[l], w->wqkv[l], 3 * da, d);
+        if (e == cudaSuccess) e = make_weight_maps(&m->w_o[l], w->wo[l], d, da);
+        if (e == cudaSuccess) e = make_gate_up_maps(&m->w_gu[l], w->wgu[l], F, d);
+        if (e == cudaSuccess) e = make_weight_maps(&m->w_d[l], w->wd[l], d, F);
     }
     if (e == cudaSuccess && cfg->with_lm_head) {
         int tile0 = 0, rows = cfg->vocab;
@@ -291,7 +291,7 @@ int32_t odb_model_create(const odb_config* cfg, const odb_weights* w, odb_model*
             delete m;
             return ODB_ERR_SHAPE;
         }
-        e = make_weight_tmap(&m->tm_lm, w->lm_head, rows, d);
+        e = make_weight_maps(&m->w_lm, w->lm_head, rows, d);
     }
     if (e != cudaSuccess) {
         delete m;
@@ -557,15 +557,15 @@ int32_t ensure_ptable(odb_session* s, int M) {
     std::vector<PGemmDesc> t(4 * c.n_layers + 1);
     const int kb_d = (d + 63) / 64, kb_F = (F + 63) / 64;
     for (int l = 0; l < c.n_layers; ++l) {
-        step_persistent_fill_desc(t[4 * l + 0], m->tm_qkv[l], tx_a, m->norm1[l], (3 * d + 127) / 128, kb_d, 0, grid);
-        step_persistent_fill_desc(t[4 * l + 1], m->tm_o[l], tx_o, nullptr, (d + 127) / 128, kb_d, 0, grid);
-        step_persistent_fill_desc(t[4 * l + 2], m->tm_gu[l], tx_a, m->norm2[l], (F + 63) / 64, kb_d, 0, grid);
-        step_persistent_fill_desc(t[4 * l + 3], m->tm_d[l], tx_g, nullptr, (d + 127) / 128, kb_F, 0, grid);
+        step_persistent_fill_desc(t[4 * l + 0], m->w_qkv[l].tile, tx_a, m->norm1[l], (3 * d + 127) / 128, kb_d, 0, grid);
+        step_persistent_fill_desc(t[4 * l + 1], m->w_o[l].tile, tx_o, nullptr, (d + 127) / 128, kb_d, 0, grid);
+        step_persistent_fill_desc(t[4 * l + 2], m->w_gu[l].tile, tx_a, m->norm2[l], (F + 63) / 64, kb_d, 0, grid);
+        step_persistent_fill_desc(t[4 * l + 3], m->w_d[l].tile, tx_g, nullptr, (d + 127) / 128, kb_F, 0, grid);
     }
     if (c.with_lm_head)
-        step_persistent_fill_desc(t[4 * c.n_layers], m->tm_lm, tx_a, m->final_norm, (c.vocab + 127) / 128, kb_d, 1, grid);
+        step_persistent_fill_desc(t[4 * c.n_layers], m->w_lm.tile, tx_a, m->final_norm, (c.vocab + 127) / 128, kb_d, 1, grid);
     else
-        step_persistent_fill_desc(t[4 * c.n_layers], m->tm_o[0], tx_a, m->final_norm, 1, 1, 0, grid);   // unused slot
+        step_persistent_fill_desc(t[4 * c.n_layers], m->w_o[0].tile, tx_a, m->final_norm, 1, 1, 0, grid);   // unused slot
     for (int j = 0; j < 4; ++j) {
         s->pmaxp[j] = step_persistent_max_parts(t[j]);
         if (s->pmaxp[j] > 8 || t[j].n_tiles > 256) t[j].g_use = 0;   // beyond the kernel's fixed tables
@@ -646,10 +646,10 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         tw.status = status;
         return tw;
     };
-    auto gemm = [&](const CUtensorMap& tw, const __nv_bfloat16* x, float* out, int rows, int N, int K, int sp,
+    auto gemm = [&](const WeightMaps& w, const __nv_bfloat16* x, float* out, int rows, int N, int K, int sp,
                     const RowScale* row_scale = nullptr, int slot = -1) {
         GemmArgs ga;
-        ga.tmap_w = tw;
+        ga.w = w;
         ga.x = x;
         ga.partial = out;
         ga.act_out = nullptr;
@@ -666,9 +666,9 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         return launch_gemm(ga, st);
     };
     // many rows, no K split: the product goes straight into the residual stream, no partial sums in memory
-    auto gemm_add = [&](const CUtensorMap& tw, const __nv_bfloat16* x, int K) {
+    auto gemm_add = [&](const WeightMaps& w, const __nv_bfloat16* x, int K) {
         GemmArgs ga;
-        ga.tmap_w = tw;
+        ga.w = w;
         ga.x = x;
         ga.partial = nullptr;
         ga.act_out = nullptr;
@@ -725,7 +725,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         } else if (c.with_lm_head) {
             // test mode: the kernel ended with the LM head's operand; the logits are materialised by a plain launch
             int sp = 1;
-            ODB_LAUNCH(ODB_KIND_GEMM, gemm(m->tm_lm, a, s->at<float>(L.logits), M, c.vocab, d, sp, &inv_scale));
+            ODB_LAUNCH(ODB_KIND_GEMM, gemm(m->w_lm, a, s->at<float>(L.logits), M, c.vocab, d, sp, &inv_scale));
             ODB_LAUNCH(ODB_KIND_CONFIDENCE, launch_confidence(s->at<float>(L.logits), M, c.vocab, c.mask_id, s->at<float>(L.conf),
                                                                  s->at<int32_t>(L.tok), s->ws + L.conf_part, st));
         }
@@ -776,7 +776,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         if (sp == 1 && gemm_rows_usable(M, 3 * da)) {
             // many rows: RoPE, the bf16 rows and the cache scatter in the projection's epilogue, no fp32 rows in memory
             GemmArgs ga;
-            ga.tmap_w = m->tm_qkv[l];
+            ga.w = m->w_qkv[l];
             ga.x = a;
             ga.partial = nullptr;
             ga.act_out = nullptr;
@@ -787,7 +787,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             ga.status = status;
             ODB_FWD(ODB_KIND_GEMM, launch_gemm(ga, st));
         } else {
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_qkv[l], a, partial, M, 3 * da, d, sp));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_qkv[l], a, partial, M, 3 * da, d, sp));
             ODB_FWD(ODB_KIND_ELEMENTWISE, launch_qkv_rope(qa, st));
         }
         if (n_step_tiles > 0) {
@@ -853,15 +853,15 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             // epilogue runs behind this rank's RMSNorm (the reader of slot 0) in the launch chain.  Slot 1 likewise,
             // with the roles of the two exchanges swapped; the statistics buffer: a peer reaches its next LM head only
             // through exchanges this rank signals after its merge of the current statistics.
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_o[l], o, nullptr, M, d, da, sp, nullptr, 0));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_o[l], o, nullptr, M, d, da, sp, nullptr, 0));
             o_wait = end_exchange(0);
             o_sum = tp.recv[c.tp_rank];
             o_parts = R * sp;
         } else if (sp == 1 && gemm_rows_usable(M, d)) {
-            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->tm_o[l], o, da));
+            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->w_o[l], o, da));
             o_sum = nullptr;
         } else {
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_o[l], o, partial, M, d, da, sp));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_o[l], o, partial, M, d, da, sp));
         }
         ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, o_sum, o_parts, static_cast<size_t>(M) * d, m->norm2[l], a, inv, nullptr, M,
                                                         d, hint_of(m->p_gu[l], gu_bytes, pf_bytes), st, o_wait));
@@ -874,12 +874,12 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         // measured slower than the fused epilogue: 3.52 / 3.43 against 3.28 ms per step, 5.02 / 4.97 against 4.74 at 128 rows)
         const int gu_sp = (R > 1 && gu_tiles * ((M + 127) / 128) <= 128) ? plan_splits(M, gu_tiles * 128, d, false) : 1;
         if (gu_sp > 1) {
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_gu[l], a, partial, M, gu_tiles * 128, d, gu_sp));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_gu[l], a, partial, M, gu_tiles * 128, d, gu_sp));
             ODB_FWD(ODB_KIND_ELEMENTWISE, launch_swiglu_combine(partial, gu_sp, static_cast<size_t>(M) * gu_tiles * 128, inv_scale, g, M,
                                                                F, st));
         } else {   // gate/up projection with the SwiGLU epilogue: writes bf16 g directly
             GemmArgs ga;
-            ga.tmap_w = m->tm_gu[l];
+            ga.w = m->w_gu[l];
             ga.x = a;
             ga.partial = nullptr;
             ga.act_out = g;
@@ -891,15 +891,15 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         }
         sp = plan_splits(M, d, F, R > 1);
         if (R > 1) {
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_d[l], g, nullptr, M, d, F, sp, nullptr, 1));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_d[l], g, nullptr, M, d, F, sp, nullptr, 1));
             res_wait = end_exchange(1);
             res = tp.recv[c.tp_rank] + L.tp_recv_slot / sizeof(float);
             res_splits = R * sp;
         } else if (sp == 1 && gemm_rows_usable(M, d) && !(c.with_lm_head && l == c.n_layers - 1)) {
-            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->tm_d[l], g, F));
+            ODB_FWD(ODB_KIND_GEMM, gemm_add(m->w_d[l], g, F));
             res = nullptr; res_splits = 0;
         } else {   // also in front of the LM head, whose norm reads the response rows only
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_d[l], g, partial, M, d, F, sp));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_d[l], g, partial, M, d, F, sp));
             res = partial; res_splits = sp;
         }
         res_stride = static_cast<size_t>(M) * d;
@@ -921,14 +921,14 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
                                                         rows, d, hint_of(m->p_lm, packed_weight_bytes(lm_rows_local, d), 0), st, res_wait));
         if (s->dump_logits) {
             int sp = 1;
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->tm_lm, x, logits, rows, c.vocab, d, sp, scale));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_lm, x, logits, rows, c.vocab, d, sp, scale));
             ODB_FWD(ODB_KIND_CONFIDENCE, launch_confidence(logits, rows, c.vocab, c.mask_id, s->at<float>(L.conf) + r0,
                                                                  s->at<int32_t>(L.tok) + r0, s->ws + L.conf_part, st));
         } else {
             // LM head fused with the confidence reduction: per (row, vocabulary tile) statistics instead
             // of logits, merged per row in tile order
             GemmArgs ga;
-            ga.tmap_w = m->tm_lm;
+            ga.w = m->w_lm;
             ga.x = x;
             ga.partial = nullptr;
             ga.act_out = nullptr;
@@ -1207,7 +1207,7 @@ int32_t odb_debug_gemm(const void* x, const void* w, float* out, void* scratch, 
     int* status = reinterpret_cast<int*>(static_cast<uint8_t*>(scratch) + part_bytes);   // behind the partials
     ODB_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
     GemmArgs ga;
-    ODB_CUDA(make_weight_tmap(&ga.tmap_w, w, N, K));
+    ODB_CUDA(make_weight_maps(&ga.w, w, N, K));
     ga.x = x;
     ga.act_out = nullptr;
     ga.partial = static_cast<float*>(scratch);

@@ -304,9 +304,15 @@ struct QkvRopeArgs {
     L2Prefetch pf;
 };
 
+// Tensor maps of a packed weight [n_tile * k_blocks][128][64] bf16 with the 128-byte swizzle: boxes of a whole tile and of
+// half of its rows.
+struct WeightMaps {
+    CUtensorMap tile, half;
+};
+
 // Weight-streaming GEMM: partial[s][M][N] (fp32) = x[M][K_s] * w[N][K_s]^T for each K split s.
 struct GemmArgs {
-    CUtensorMap tmap_w;    // packed bf16 weight tiles [n_tile * k_blocks][128][64], 128B swizzle
+    WeightMaps w;
     const void* x;         // bf16 [M][K] device
     float* partial;        // fp32 [splits][M][N]
     __nv_bfloat16* act_out; // non-null: gate/up GEMM with the SwiGLU epilogue, writes bf16 [M][N = F]; splits == 1
@@ -327,12 +333,12 @@ int gemm_whole_splits(int splits, int nkb);
 
 // Test entry: one block performs the consumers' flag wait (tensor_parallel.cu).
 cudaError_t launch_tp_wait(const TpWait& tw, cudaStream_t st);
-cudaError_t make_weight_tmap(CUtensorMap* out, const void* w_packed, int N, int K);
+cudaError_t make_weight_maps(WeightMaps* out, const void* w_packed, int N, int K);
 // bf16 [rows][cols] row-major; box = 64 columns x box_rows rows, 128-byte swizzle, rows beyond `rows` read as zero
 cudaError_t make_rows_tmap(CUtensorMap* out, const void* base, int rows, int cols, int box_rows);
 size_t packed_weight_bytes(int N, int K);
 size_t packed_gate_up_bytes(int F, int K);
-cudaError_t make_gate_up_tmap(CUtensorMap* out, const void* w_packed, int F, int K);
+cudaError_t make_gate_up_maps(WeightMaps* out, const void* w_packed, int F, int K);
 cudaError_t launch_pack_gate_up(const void* src_gate_then_up, void* dst_packed, int F, int K, cudaStream_t st);
 cudaError_t launch_pack_weight(const void* src_row_major, void* dst_packed, int N, int K, cudaStream_t st);
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
