@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(flo
                                                                      int splits, size_t pstride, const float* __restrict__ gain,
                                                                      __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                      const int32_t* __restrict__ row_map, int d, L2Prefetch pf,
-                                                                     TpWait tw, EmbedSource emb) {
+                                                                     TpWait tw, EmbedSource emb, int compact) {
     __shared__ float red[32];
     pdl_launch_dependents();
     pdl_wait();
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(flo
         float4 v = EMBED ? embed_load4(emb, row, i, d) : reinterpret_cast<const float4*>(hr)[i];
         if (EMBED) reinterpret_cast<float4*>(hr)[i] = v;
         if (!EMBED && partial) {
-            const float* p = partial + static_cast<size_t>(row) * d + 4 * i;
+            const float* p = partial + static_cast<size_t>(compact ? orow : row) * d + 4 * i;
             float4 t[SPLITS];
 #pragma unroll
             for (int u = 0; u < SPLITS; ++u)
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
                                                                           const float* __restrict__ gain,
                                                                           __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                           const int32_t* __restrict__ row_map, int rows_out, int d,
-                                                                          TpWait tw, EmbedSource emb) {
+                                                                          TpWait tw, EmbedSource emb, int compact) {
     __shared__ float red[kNormRows][32];
     pdl_launch_dependents();
     pdl_wait();
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
         if (!in || row[r] < 0) continue;
         v[r] = EMBED ? embed_load4(emb, row[r], i, d) : reinterpret_cast<const float4*>(h + static_cast<size_t>(row[r]) * d)[i];
         if (SPLITS > 0) {
-            const float* p = partial + static_cast<size_t>(row[r]) * d + 4 * i;
+            const float* p = partial + static_cast<size_t>(compact ? orow0 + r : row[r]) * d + 4 * i;
 #pragma unroll
             for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) t[r][u] = *reinterpret_cast<const float4*>(p + static_cast<size_t>(u) * pstride);
@@ -177,6 +177,16 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
         for (int w = 0; w < nw; ++w) total += red[threadIdx.x][w];
         ssq[static_cast<size_t>(orow0 + threadIdx.x) * gridDim.y + blockIdx.y] = total;
     }
+}
+
+// one block per row, 16 bytes per thread and turn
+__global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+                                                          const int32_t* __restrict__ map, int d) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const uint4* from = reinterpret_cast<const uint4*>(src + static_cast<size_t>(map[blockIdx.x]) * d);
+    uint4* to = reinterpret_cast<uint4*>(dst + static_cast<size_t>(blockIdx.x) * d);
+    for (int i = threadIdx.x; i < d / 8; i += 256) to[i] = from[i];
 }
 
 // More than 64 rows: grid (rows, chunks), one thread per FOUR consecutive rotation pairs (float4 loads, 8-byte
@@ -517,10 +527,10 @@ cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink
 template <int SPLITS, bool EMBED>
 static cudaError_t launch_norm_rows(bool first, float* h, const float* partial, int splits, size_t pstride, const float* gain,
                                     __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, cudaStream_t st,
-                                    const TpWait& tw, const EmbedSource& emb) {
+                                    const TpWait& tw, const EmbedSource& emb, int compact) {
     return launch_kernel_if(!first, rmsnorm_rows_kernel<SPLITS, EMBED>,
                             dim3((rows_out + kNormRows - 1) / kNormRows, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4),
-                            0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, emb);
+                            0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, emb, compact);
 }
 
 // The first norm (emb.table set) is the first kernel of a forward.  It is launched WITHOUT programmatic stream
@@ -529,21 +539,25 @@ static cudaError_t launch_norm_rows(bool first, float* h, const float* partial, 
 // attention kernels to read the tile table and the K/V cache before their own griddepcontrol.wait.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb) {
+                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact, int plan_rows) {
     if (splits > 16) return cudaErrorInvalidValue;
     const bool first = emb.table != nullptr;
     if (first && (partial || row_map)) return cudaErrorInvalidValue;
-    if (rows_out >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
-        if (first) return launch_norm_rows<0, true>(true, h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb);
-        if (!partial) return launch_norm_rows<0, false>(false, h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb);
+    if ((rows_out > plan_rows ? rows_out : plan_rows) >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
+        if (first) return launch_norm_rows<0, true>(true, h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb, 0);
+        if (!partial) return launch_norm_rows<0, false>(false, h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
         if (splits == 1)
-            return launch_norm_rows<1, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb);
+            return launch_norm_rows<1, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
         return launch_norm_rows<kNormRowsMaxSplits, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
-                                                           tw, emb);
+                                                           tw, emb, compact);
     }
     return launch_kernel_if(!first, first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
                             splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<16, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
-                            st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb);
+                            st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb, compact ? 1 : 0);
+}
+
+cudaError_t launch_gather_rows(const __nv_bfloat16* src, __nv_bfloat16* dst, const int32_t* map, int n, int d, cudaStream_t st) {
+    return launch_kernel(gather_rows_kernel, dim3(n), dim3(256), 0, st, src, dst, map, d);
 }
 
 cudaError_t launch_qkv_rope(const QkvRopeArgs& a, cudaStream_t st) {

@@ -526,6 +526,11 @@ bool use_pair(int M, int n_tiles) { return pair_enabled() && M > 128 && (n_tiles
 
 }  // namespace
 
+int gemm_tiled_rows(int M, int N, int plan_rows) {
+    const int bn = use_pair(plan_rows, (N + kBM - 1) / kBM) ? 2 * kBM : pick_bn(M);
+    return (M + bn - 1) / bn * bn;
+}
+
 bool gemm_rows_usable(int M, int N) { return use_pair(M, (N + kBM - 1) / kBM); }
 
 cudaError_t make_weight_maps(WeightMaps* out, const void* w, int N, int K) {
@@ -625,7 +630,7 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     const bool swiglu = a.act_out != nullptr;
     const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
     if ((swiglu || a.conf.part || a.qkv || a.add_to) && a.splits != 1) return cudaErrorInvalidValue;
-    if (use_pair(a.M, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
+    if (use_pair(a.plan_rows > a.M ? a.plan_rows : a.M, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
     if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of the many-row kernel only
     if (swiglu) return launch_epi<EPI_SWIGLU>(a, st);
     return a.conf.part ? launch_epi<EPI_CONF>(a, st) : launch_epi<EPI_PARTIAL>(a, st);

@@ -324,6 +324,7 @@ struct GemmArgs {
     float* add_to = nullptr;            // non-null: the product is added to fp32 [M][N] in place (likewise)
     PeerOut peers;                      // peers.n > 0: the partial tiles (or statistics) go to these buffers instead
     int M, N, K;
+    int plan_rows = 0;     // > M: the kernel is the one a projection of this many rows takes (its sums, bit for bit); 0: M
     int splits;
     int* status;           // device status word
 };
@@ -343,6 +344,8 @@ cudaError_t launch_pack_gate_up(const void* src_gate_then_up, void* dst_packed, 
 cudaError_t launch_pack_weight(const void* src_row_major, void* dst_packed, int N, int K, cudaStream_t st);
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
 // many-row projections with the activation rows on the M side of the tile (gemm_rows.cu)
+// rows that the row tiles of a projection of M rows span, in the kernel of a projection of plan_rows >= M rows
+int gemm_tiled_rows(int M, int N, int plan_rows);
 bool gemm_rows_usable(int M, int N);   // whether a projection of this size has the epilogues `qkv` and `add_to`
 cudaError_t launch_gemm_rows(const GemmArgs& a, int n_tiles, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stride, float* out, size_t n,
@@ -362,10 +365,14 @@ struct EmbedSource {
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's
 // operand, ssq[i][t] = sum of h[r]^2 over the t-th slice of kNormSliceCols columns; the projection's consumer
 // multiplies its fp32 output by 1 / sqrt(sum_t ssq / d + eps) (RowScale; the scalar commutes with the matrix
-// product).  splits <= 16.
+// product).  splits <= 16.  compact: partial[s] holds the rows of the map only, in its order.  plan_rows > rows_out: the
+// variant is the one of this many rows (they differ in the order of a row's sum of squares).
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource());
+                           cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource(),
+                           bool compact = false, int plan_rows = 0);
+// dst[i] = src[map[i]] for n rows of d bf16 (d % 8 == 0, 16-byte aligned rows)
+cudaError_t launch_gather_rows(const __nv_bfloat16* src, __nv_bfloat16* dst, const int32_t* map, int n, int d, cudaStream_t st);
 // SwiGLU of a gate/up projection that ran with K splits (few weight tiles: a tensor-parallel shard): partial is fp32
 // [splits][M][tiles * 128] in the packed gate/up order (tile t = gate features [64t, 64t+64), then the same up
 // features); g[m][f] = bf16(silu(gate) * up) with gate, up = the split sums (split order) times the row scalar.
