@@ -21,7 +21,7 @@ struct CtaSync {
     static __device__ __forceinline__ void sync() { __syncthreads(); }
 };
 
-template <int HD>
+template <int HD, bool LONG>
 __global__ void __launch_bounds__(kAttnThreads) attention_kernel(AttnArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     pdl_launch_dependents();
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(AttnArgs a) {
     if (!a.early) pdl_wait();                          // the tile table itself is written by the predecessor chain
     const QTile t = a.tiles[blockIdx.x];
     bool waited = !a.early;
-    attention_item<HD, CtaSync>(a, t, blockIdx.y, blockIdx.z, threadIdx.x, smem, a.early != 0, [&]() {
+    attention_item<HD, LONG, CtaSync>(a, t, blockIdx.y, blockIdx.z, threadIdx.x, smem, a.early != 0, [&]() {
         if (!waited) pdl_wait();
         waited = true;
     });
@@ -76,7 +76,15 @@ __global__ void __launch_bounds__(256) step_attention_kernel(StepAttnArgs a) {
                               static_cast<size_t>(head) * a.max_seq * HD;
     const __nv_bfloat16* cv = ck + per_kv;
 
+    const int nA = t.cA;
+    auto whole = [&](int tile) { return !fresh_cta && (tile + 1) * kTileK <= n_cache; };   // cached keys only: every slab sees all of them
     auto load_tile = [&](int tile, int buf) {
+        const int kv0 = tile * kTileK, kv1 = kv0 + kTileK;
+        if (!fresh_cta && (kv1 <= nA || (kv0 >= nA && kv1 <= n_cache))) {   // cached keys on one side of the block
+            const size_t at = static_cast<size_t>(kv1 <= nA ? kv0 : t.cB0 + (kv0 - nA)) * HD;
+            load_whole_tile<HD, 256>(sK + buf * kTileBytes, sV + buf * kTileBytes, ck + at, cv + at, HD, threadIdx.x);
+            return;
+        }
         for (int c = threadIdx.x; c < kTileK * CH; c += 256) {
             const int key = c / CH, ch = c % CH;
             bool ok;
@@ -170,12 +178,20 @@ __global__ void __launch_bounds__(256) step_attention_kernel(StepAttnArgs a) {
                     mma_bf16(s[2 * np + 1], qa, kb[2], kb[3]);
                 }
             }
+            if (whole(tile)) {
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
+                for (int nt = 0; nt < 8; ++nt) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int col = nt * 8 + (lane & 3) * 2 + (e & 1);
-                    s[nt][e] = valid[col] >= need ? s[nt][e] * scale_log2 : -INFINITY;
+                    for (int e = 0; e < 4; ++e) s[nt][e] *= scale_log2;
+                }
+            } else {
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int col = nt * 8 + (lane & 3) * 2 + (e & 1);
+                        s[nt][e] = valid[col] >= need ? s[nt][e] * scale_log2 : -INFINITY;
+                    }
                 }
             }
 #pragma unroll
@@ -187,13 +203,13 @@ __global__ void __launch_bounds__(256) step_attention_kernel(StepAttnArgs a) {
                 mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
                 const float m_new = fmaxf(m_run[r], mx);
                 const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
-                const float corr = exp2f(m_run[r] - m_use);
+                const float corr = ex2_ftz(m_run[r] - m_use);
                 m_run[r] = m_new;
                 float rs = 0.f;
 #pragma unroll
                 for (int nt = 0; nt < 8; ++nt) {
-                    const float p0 = exp2f(s[nt][2 * r] - m_use);
-                    const float p1 = exp2f(s[nt][2 * r + 1] - m_use);
+                    const float p0 = ex2_ftz(s[nt][2 * r] - m_use);
+                    const float p1 = ex2_ftz(s[nt][2 * r + 1] - m_use);
                     s[nt][2 * r] = p0;
                     s[nt][2 * r + 1] = p1;
                     rs += p0 + p1;
@@ -310,12 +326,15 @@ cudaError_t combine(const float* part_o, const float* part_ml, __nv_bfloat16* o,
 template <int HD>
 cudaError_t launch_hd(const AttnArgs& a, cudaStream_t st) {
     const size_t smem = kTileQ * HD * 2 + 4 * kTileK * HD * 2 + 2 * kTileK;
-    static std::atomic<unsigned long long> attr_done{0};
-    cudaError_t e = set_smem_limit_once(attr_done, attention_kernel<HD>, static_cast<int>(smem));
+    // a refresh, and steps whose keys are not split: several tiles for every CTA
+    const bool walk = !a.early || a.ksplit == 1;
+    void (*kernel)(AttnArgs) = walk ? attention_kernel<HD, true> : attention_kernel<HD, false>;
+    static std::atomic<unsigned long long> attr_done[2];
+    cudaError_t e = set_smem_limit_once(attr_done[walk], kernel, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     dim3 grid(a.n_tiles, a.H, a.ksplit);
     if (a.ksplit > 8) return cudaErrorInvalidValue;
-    e = launch_kernel(attention_kernel<HD>, grid, dim3(kAttnThreads), smem, st, a);
+    e = launch_kernel(kernel, grid, dim3(kAttnThreads), smem, st, a);
     if (e != cudaSuccess || a.ksplit == 1) return e;
     return combine(a.part_o, a.part_ml, a.o, a.M, a.H, HD, a.ksplit, st);
 }

@@ -489,7 +489,7 @@ __device__ __noinline__ void attention_phase(const StepPersistentArgs& A, PShare
     for (int it = cta; it < n_attn; it += G) {
         const int z = it % A.ksplit, head = (it / A.ksplit) % A.H, qt = it / (A.ksplit * A.H);
         const QTile t = A.tiles[qt];
-        attention_item<HD, WorkerSync>(aa, t, head, z, tid, scratch, true, wait_rope);
+        attention_item<HD, false, WorkerSync>(aa, t, head, z, tid, scratch, true, wait_rope);
         WorkerSync::sync();                              // the tiles in shared memory are free for the next item
         if (sh->abort) break;
     }
