@@ -15,6 +15,7 @@ struct BlockIndexParam {
 
 // Rows of a refresh: every position of every active sequence, in sequence order.
 __global__ void build_refresh_rows_kernel(ControlBuffers c, int batch, BlockIndexParam bp) {
+    pdl_launch_dependents();   // the first norm, which waits for the table before it lets its own successor start
     const int seq = blockIdx.x;
     SeqState* st = c.state + seq;
     if (!st->active || bp.block_index[seq] < 0) {
@@ -101,6 +102,7 @@ __device__ int step_tiles_of(const SeqState* st) {
 // One block per sequence.  The state is worked on in shared memory and the sequences in front are counted by one thread
 // each: written as one thread's walk over global memory this was 6 us at batch 1 and 22 us at batch 16.
 __global__ void __launch_bounds__(64) build_step_rows_kernel(ControlBuffers c, int batch, int mask_id) {
+    pdl_launch_dependents();           // as above
     const int seq = blockIdx.x, tid = threadIdx.x;
     __shared__ SeqState sst;
     __shared__ int xs[kMaxBlock];      // the block's committed tokens
@@ -519,6 +521,7 @@ __device__ __forceinline__ void accept_store(const ControlBuffers& c, const Acce
 
 __global__ void accept_kernel(ControlBuffers c, odb_decode_params p, int after_refresh, int mask_id, int eos_id, int dry) {
     __shared__ AcceptShared sh;
+    pdl_wait();   // launched under the last kernel of the forward: its start is not waited for on top of its work
     accept_load(c, &sh);
     accept_body(c, p, after_refresh, mask_id, eos_id, dry, &sh.st, &sh.res);
     __syncthreads();
@@ -600,8 +603,7 @@ cudaError_t launch_build_step_rows(const ControlBuffers& c, int batch, int mask_
 
 cudaError_t launch_accept(const ControlBuffers& c, int batch, const odb_decode_params& p, int after_refresh,
                           int mask_id, int eos_id, int dry, cudaStream_t st) {
-    accept_kernel<<<batch, 64, 0, st>>>(c, p, after_refresh, mask_id, eos_id, dry);
-    return cudaGetLastError();
+    return launch_kernel(accept_kernel, dim3(batch), dim3(64), 0, st, c, p, after_refresh, mask_id, eos_id, dry);
 }
 
 cudaError_t launch_build_refresh_rows(const ControlBuffers& c, int batch, const int32_t* block_index,

@@ -71,8 +71,9 @@ __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(flo
                                                                      const int32_t* __restrict__ row_map, int d, L2Prefetch pf,
                                                                      TpWait tw, EmbedSource emb, int compact) {
     __shared__ float red[32];
-    pdl_launch_dependents();
+    if (!EMBED) pdl_launch_dependents();
     pdl_wait();
+    if (EMBED) pdl_launch_dependents();   // see launch_rmsnorm
     tp_wait_flags(tw);   // tensor parallelism: the partials of every rank have arrived
     l2_prefetch_slice(pf, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
     const int orow = blockIdx.x;
@@ -124,8 +125,9 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
                                                                           const int32_t* __restrict__ row_map, int rows_out, int d,
                                                                           TpWait tw, EmbedSource emb, int compact) {
     __shared__ float red[kNormRows][32];
-    pdl_launch_dependents();
+    if (!EMBED) pdl_launch_dependents();
     pdl_wait();
+    if (EMBED) pdl_launch_dependents();   // see launch_rmsnorm
     if (SPLITS > 0) tp_wait_flags(tw);
     const int i = blockIdx.y * (kNormSliceCols / 4) + threadIdx.x;   // float4 index within the row
     const int orow0 = blockIdx.x * kNormRows;
@@ -525,18 +527,20 @@ cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink
 }
 
 template <int SPLITS, bool EMBED>
-static cudaError_t launch_norm_rows(bool first, float* h, const float* partial, int splits, size_t pstride, const float* gain,
+static cudaError_t launch_norm_rows(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                                     __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, cudaStream_t st,
                                     const TpWait& tw, const EmbedSource& emb, int compact) {
-    return launch_kernel_if(!first, rmsnorm_rows_kernel<SPLITS, EMBED>,
+    return launch_kernel(rmsnorm_rows_kernel<SPLITS, EMBED>,
                             dim3((rows_out + kNormRows - 1) / kNormRows, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4),
                             0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, emb, compact);
 }
 
-// The first norm (emb.table set) is the first kernel of a forward.  It is launched WITHOUT programmatic stream
-// serialization: it starts only when everything enqueued before it (the row and tile tables, the previous accept) has
-// completed, and every later kernel of the chain starts after this one has started.  That is what allows the
-// attention kernels to read the tile table and the K/V cache before their own griddepcontrol.wait.
+// The first norm (emb.table set) is the first kernel of a forward and follows the kernel that builds the row and tile tables,
+// which is launched without programmatic stream serialization: it starts only when everything enqueued before it (the
+// previous accept) has completed.  The norm lets its successor start only behind its own wait for those tables, so every later
+// kernel of the chain starts when they are complete.  That is what allows the attention kernels to read the tile
+// table and the K/V cache before their own griddepcontrol.wait.  (Started only when the tables were complete, and the accept
+// only when the forward was: layer step 122.5 us against 118.5, tiny model 87.2 against 84.)
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
                            cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact, int plan_rows) {
@@ -544,14 +548,14 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
     const bool first = emb.table != nullptr;
     if (first && (partial || row_map)) return cudaErrorInvalidValue;
     if ((rows_out > plan_rows ? rows_out : plan_rows) >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
-        if (first) return launch_norm_rows<0, true>(true, h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb, 0);
-        if (!partial) return launch_norm_rows<0, false>(false, h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
+        if (first) return launch_norm_rows<0, true>(h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb, 0);
+        if (!partial) return launch_norm_rows<0, false>(h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
         if (splits == 1)
-            return launch_norm_rows<1, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
-        return launch_norm_rows<kNormRowsMaxSplits, false>(false, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
+            return launch_norm_rows<1, false>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
+        return launch_norm_rows<kNormRowsMaxSplits, false>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
                                                            tw, emb, compact);
     }
-    return launch_kernel_if(!first, first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
+    return launch_kernel(first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
                             splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<16, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
                             st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb, compact ? 1 : 0);
 }

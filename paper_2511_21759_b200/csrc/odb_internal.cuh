@@ -70,8 +70,7 @@ __device__ __forceinline__ void l2_prefetch_slice(const L2Prefetch& pf, int cta,
 #endif
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_kernel_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                             Args&&... args) {   // early: with programmatic stream serialization
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -81,12 +80,8 @@ cudaError_t launch_kernel_if(bool early, void (*kernel)(KArgs...), dim3 grid, di
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = early && pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = pdl_enabled() ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-template <typename... KArgs, typename... Args>
-cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-    return launch_kernel_if(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------------------
