@@ -282,7 +282,7 @@ int32_t odb_debug_expire_wait(odb_session* s, int64_t limit_cycles);
 /* Copies a device buffer of the last forward to the host.  which: 0 logits fp32 [rows][vocab]
  * (needs the logit dump);
  * 1 conf fp32 [rows]; 2 tok int32 [rows]; 3 residual stream fp32 [rows][d_model] (behind a refresh with
- * LM head the last layer's projections reach the rows with logits only); 4 q, 5 k,
+ * LM head the last layer's FFN reaches the rows with logits only); 4 q, 5 k,
  * 6 v bf16 [rows][d_model] of the LAST layer; 7 attention output bf16 [rows][d_model];
  * 8 row tokens int32 [rows]; 9 row positions int32 [rows]; 10 row copy ids int32 [rows];
  * 11 the raw timing words of the persistent step kernel (see ODB_PERSISTENT_TIMING below; up to cap_bytes).

@@ -181,14 +181,17 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
     }
 }
 
-// one block per row, 16 bytes per thread and turn
-__global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+// one block per row, 16 bytes per thread and turn; the row's sums of squares by its first threads
+__global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* __restrict__ src, const float* __restrict__ ssq, int slots,
+                                                          __nv_bfloat16* __restrict__ dst, float* __restrict__ dst_ssq,
                                                           const int32_t* __restrict__ map, int d) {
     pdl_launch_dependents();
     pdl_wait();
-    const uint4* from = reinterpret_cast<const uint4*>(src + static_cast<size_t>(map[blockIdx.x]) * d);
-    uint4* to = reinterpret_cast<uint4*>(dst + static_cast<size_t>(blockIdx.x) * d);
+    const size_t row = map[blockIdx.x], to_row = blockIdx.x;
+    const uint4* from = reinterpret_cast<const uint4*>(src + row * d);
+    uint4* to = reinterpret_cast<uint4*>(dst + to_row * d);
     for (int i = threadIdx.x; i < d / 8; i += 256) to[i] = from[i];
+    for (int i = threadIdx.x; i < slots; i += 256) dst_ssq[to_row * slots + i] = ssq[row * slots + i];
 }
 
 // More than 64 rows: grid (rows, chunks), one thread per FOUR consecutive rotation pairs (float4 loads, 8-byte
@@ -543,11 +546,11 @@ static cudaError_t launch_norm_rows(float* h, const float* partial, int splits, 
 // only when the forward was: layer step 122.5 us against 118.5, tiny model 87.2 against 84.)
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact, int plan_rows) {
+                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact) {
     if (splits > 16) return cudaErrorInvalidValue;
     const bool first = emb.table != nullptr;
     if (first && (partial || row_map)) return cudaErrorInvalidValue;
-    if ((rows_out > plan_rows ? rows_out : plan_rows) >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
+    if (rows_out >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
         if (first) return launch_norm_rows<0, true>(h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb, 0);
         if (!partial) return launch_norm_rows<0, false>(h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
         if (splits == 1)
@@ -560,8 +563,9 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
                             st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb, compact ? 1 : 0);
 }
 
-cudaError_t launch_gather_rows(const __nv_bfloat16* src, __nv_bfloat16* dst, const int32_t* map, int n, int d, cudaStream_t st) {
-    return launch_kernel(gather_rows_kernel, dim3(n), dim3(256), 0, st, src, dst, map, d);
+cudaError_t launch_gather_rows(const __nv_bfloat16* src, const float* ssq, int slots, __nv_bfloat16* dst, float* dst_ssq,
+                               const int32_t* map, int n, int d, cudaStream_t st) {
+    return launch_kernel(gather_rows_kernel, dim3(n), dim3(256), 0, st, src, ssq, slots, dst, dst_ssq, map, d);
 }
 
 cudaError_t launch_qkv_rope(const QkvRopeArgs& a, cudaStream_t st) {

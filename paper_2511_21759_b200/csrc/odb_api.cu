@@ -759,9 +759,11 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     };
     const size_t qkv_bytes = packed_weight_bytes(3 * da, d), o_bytes = packed_weight_bytes(d, da),
                  gu_bytes = packed_gate_up_bytes(F, d);
-    // A refresh ends with the logits of n_lm rows, and behind the last layer's attention nothing looks at the others: its O, gate/up
-    // and down projections run over those rows only, gathered in the order of lm_rows, as the kernels and K splits of all M
-    // rows would (the same bits).  Where that saves row tiles: a request of 768 rows and 256 response rows, four layers, 1677 -> 1535 us.
+    // A refresh ends with the logits of n_lm rows, and behind the last layer's attention block nothing looks at the others: its
+    // gate/up and down projections run over those rows only, gathered in the order of lm_rows, with the kernels and K splits
+    // that all M rows would take (the same bits).  Where that saves row tiles: a request of 768 rows and 256 response rows, four
+    // layers, 1689 -> 1553 us; 1200 and 200, one layer, 882 -> 650.  The O projection keeps all rows: the residual stream that
+    // odb_debug_read returns holds the last attention block in every one (without it 1539 and 620 us).
     bool tail = false;
     for (int l = 0; l < c.n_layers; ++l) {
         EmbedSource emb;
@@ -848,17 +850,6 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         ODB_FWD(ODB_KIND_ATTENTION, launch_attention(aa, st));
         if (ks > 1 && seg_on()) ++s->launches[ODB_KIND_ATTENTION];   // the split merge is a second kernel
         }
-        tail = write_cache && l == c.n_layers - 1 && R == 1 && n_lm > 0 && n_lm < M && (one_seq || M > 128) &&
-               gemm_tiled_rows(n_lm, d, M) < gemm_tiled_rows(M, d, M);
-        const int rows = tail ? n_lm : M, plan_rows = tail ? M : 0;
-        const __nv_bfloat16* o_rows = o;
-        if (tail && one_seq) {
-            o_rows = o + static_cast<size_t>(M - n_lm) * da;
-        } else if (tail) {   // `a` is free between the QKV projection and the next norm
-            ODB_FWD(ODB_KIND_ELEMENTWISE, launch_gather_rows(o, a, s->cb.lm_rows, n_lm, da, st));
-            o_rows = a;
-        }
-        const int32_t* tail_map = tail ? s->cb.lm_rows : nullptr;
         sp = plan_splits(M, d, da, R > 1);
         const float* o_sum = partial;   // the partial sums the next RMSNorm adds to the residual stream
         int o_parts = sp;
@@ -874,15 +865,29 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             o_wait = end_exchange(0);
             o_sum = tp.recv[c.tp_rank];
             o_parts = R * sp;
-        } else if (sp == 1 && gemm_rows_usable(M, d) && !tail) {
+        } else if (sp == 1 && gemm_rows_usable(M, d)) {
             ODB_FWD(ODB_KIND_GEMM, gemm_add(m->w_o[l], o, da));
             o_sum = nullptr;
         } else {
-            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_o[l], o_rows, partial, rows, d, da, sp, nullptr, -1, plan_rows));
+            ODB_FWD(ODB_KIND_GEMM, gemm(m->w_o[l], o, partial, M, d, da, sp));
         }
-        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, o_sum, o_parts, static_cast<size_t>(rows) * d, m->norm2[l], a, inv, tail_map, rows,
-                                                        d, hint_of(m->p_gu[l], gu_bytes, pf_bytes), st, o_wait, EmbedSource(), tail,
-                                                        plan_rows));
+        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, o_sum, o_parts, static_cast<size_t>(M) * d, m->norm2[l], a, inv, nullptr, M,
+                                                        d, hint_of(m->p_gu[l], gu_bytes, pf_bytes), st, o_wait));
+        tail = write_cache && l == c.n_layers - 1 && R == 1 && n_lm > 0 && n_lm < M && (one_seq || M > 128) &&
+               gemm_tiled_rows(n_lm, d, M) < gemm_tiled_rows(M, d, M);
+        const int rows = tail ? n_lm : M, plan_rows = tail ? M : 0;
+        const __nv_bfloat16* ffn_x = a;
+        RowScale ffn_scale = inv_scale;
+        if (tail && one_seq) {
+            ffn_x = a + static_cast<size_t>(M - n_lm) * d;
+            ffn_scale.ssq = inv + static_cast<size_t>(M - n_lm) * inv_scale.slots;
+        } else if (tail) {   // `partial` is free between the norm and the down projection's epilogue
+            __nv_bfloat16* gathered = reinterpret_cast<__nv_bfloat16*>(partial);
+            float* gathered_ssq = partial + static_cast<size_t>(n_lm) * d / 2;
+            ODB_FWD(ODB_KIND_ELEMENTWISE, launch_gather_rows(a, inv, inv_scale.slots, gathered, gathered_ssq, s->cb.lm_rows, n_lm, d, st));
+            ffn_x = gathered;
+            ffn_scale.ssq = gathered_ssq;
+        }
         // A tensor-parallel shard has few gate/up weight tiles (96 / 48 / 24 at 2 / 4 / 8 ranks of the 8B shape): one CTA
         // per tile would stream a megabyte each at a single CTA's rate, so the projection then runs with K splits like
         // the others and a small kernel forms SwiGLU from the split sums (one rank of 4 / 8, timed alone: 3.43 -> 2.74
@@ -898,10 +903,10 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         } else {   // gate/up projection with the SwiGLU epilogue: writes bf16 g directly
             GemmArgs ga;
             ga.w = m->w_gu[l];
-            ga.x = a;
+            ga.x = ffn_x;
             ga.partial = nullptr;
             ga.act_out = g;
-            ga.row_scale = inv_scale;
+            ga.row_scale = ffn_scale;
             ga.M = rows; ga.N = F; ga.K = d;
             ga.plan_rows = plan_rows;
             ga.splits = 1;

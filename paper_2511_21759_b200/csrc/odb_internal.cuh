@@ -360,14 +360,14 @@ struct EmbedSource {
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's
 // operand, ssq[i][t] = sum of h[r]^2 over the t-th slice of kNormSliceCols columns; the projection's consumer
 // multiplies its fp32 output by 1 / sqrt(sum_t ssq / d + eps) (RowScale; the scalar commutes with the matrix
-// product).  splits <= 16.  compact: partial[s] holds the rows of the map only, in its order.  plan_rows > rows_out: the
-// variant is the one of this many rows (they differ in the order of a row's sum of squares).
+// product).  splits <= 16.  compact: partial[s] holds the rows of the map only, in its order.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
                            cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource(),
-                           bool compact = false, int plan_rows = 0);
-// dst[i] = src[map[i]] for n rows of d bf16 (d % 8 == 0, 16-byte aligned rows)
-cudaError_t launch_gather_rows(const __nv_bfloat16* src, __nv_bfloat16* dst, const int32_t* map, int n, int d, cudaStream_t st);
+                           bool compact = false);
+// dst[i] = src[map[i]] for n rows of d bf16 (d % 8 == 0, 16-byte aligned rows), and likewise their `slots` sums of squares
+cudaError_t launch_gather_rows(const __nv_bfloat16* src, const float* ssq, int slots, __nv_bfloat16* dst, float* dst_ssq,
+                               const int32_t* map, int n, int d, cudaStream_t st);
 // SwiGLU of a gate/up projection that ran with K splits (few weight tiles: a tensor-parallel shard): partial is fp32
 // [splits][M][tiles * 128] in the packed gate/up order (tile t = gate features [64t, 64t+64), then the same up
 // features); g[m][f] = bf16(silu(gate) * up) with gate, up = the split sums (split order) times the row scalar.

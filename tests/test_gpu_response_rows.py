@@ -52,3 +52,36 @@ def test_last_layer_over_the_response_rows(shape, lens):
         # the final norm's sum of squares and the LM head's sum of exponentials in another order: a few 2^-24 of logits below 8 in
         # every term (1e-6), and at most 2^-24 for each of 1980 terms (1.2e-4)
         assert np.allclose(conf, aconf[rows], rtol=1.3e-4, atol=0)
+
+
+@requires_gpu
+@pytest.mark.parametrize("shape,lens", [
+    (HD128, [(500, 140)]),                                           # O with K splits, one sequence
+    (HD64, [(600, 16), (1, 150), (263, 40)]),                        # several
+    (dataclasses.replace(HD64, n_heads=3, d_model=192), [(200, 90), (150, 33)]),
+    (dataclasses.replace(HD128, n_heads=8, d_model=1024, n_layers=1), [(650, 130), (100, 200)]),   # O adds to the stream itself
+    (HD64, [(60, 31)]),                                              # up to 128 rows
+])
+def test_residual_stream_of_the_prompt_rows_holds_the_last_attention_block(shape, lens):
+    """The last layer's FFN reaches the rows with logits only, its attention block every row: with a last down projection of
+    zeros, a refresh in which every row is a response row leaves that residual stream in all of them."""
+    E = engine()
+    gm = E.Model.from_synth(shape, seed=5, max_batch=len(lens), max_seq=max(p + n for p, n in lens), max_block=16, max_copies=1)
+    sess = E.Session(gm, poison=True)
+
+    def hidden(prompts):
+        for i, ((p, n), at) in enumerate(zip(lens, prompts)):
+            sess.set_sequence(i, synth.sequence(5, i, p, n, shape), at)
+        sess.refresh_prefill(E.DecodeParams(block_len=16), 0)
+        out = sess.debug_read("hidden")
+        sess.unmask_accept(E.DecodeParams(block_len=16), True)
+        return out
+
+    got = hidden([p for p, _ in lens])
+    gm.t["wd"][-1].zero_()
+    want = hidden([0] * len(lens))
+    assert sess.status() == 0
+    at = np.cumsum([0] + [p + n for p, n in lens])
+    rows = np.concatenate([np.arange(at[i], at[i] + p) for i, (p, _) in enumerate(lens)])
+    assert len(rows) and np.isfinite(want).all() and np.array_equal(got[rows], want[rows])
+    sess.close(); gm.close()
