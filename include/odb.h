@@ -298,7 +298,7 @@ int32_t odb_debug_read(odb_session* s, int32_t which, void* host, size_t cap_byt
 
 /* out[M][N] (fp32, device) = x[M][K] (bf16, device) * w[N][K]^T (PACKED bf16, device) with the
  * weight-streaming tcgen05 GEMM, K split k_splits ways and reduced in fixed order.  scratch:
- * device buffer of >= k_splits*M*N*4 + 512 bytes.  k_splits = 0 picks the library's heuristic.
+ * device buffer of >= k_splits*M*N*4 + 512 bytes.  k_splits = 0 picks the library's heuristic (at most 16).
  * Runs on `stream` and waits for it; returns ODB_ERR_TIMEOUT if a device-side wait expired. */
 int32_t odb_debug_gemm(const void* x, const void* w, float* out, void* scratch, size_t scratch_bytes,
                        int32_t M, int32_t N, int32_t K, int32_t k_splits, void* stream);

@@ -547,7 +547,7 @@ static cudaError_t launch_norm_rows(float* h, const float* partial, int splits, 
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
                            cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact) {
-    if (splits > 16) return cudaErrorInvalidValue;
+    if (splits > kMaxKSplits) return cudaErrorInvalidValue;
     const bool first = emb.table != nullptr;
     if (first && (partial || row_map)) return cudaErrorInvalidValue;
     if (rows_out >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
@@ -559,7 +559,7 @@ cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t ps
                                                            tw, emb, compact);
     }
     return launch_kernel(first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
-                            splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<16, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
+                            splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<kMaxKSplits, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
                             st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb, compact ? 1 : 0);
 }
 

@@ -616,13 +616,14 @@ int gemm_pick_splits(int M, int N, int K) {
         // 262 / 271, 1118 rows 376 / 375.  A choice between the two by waves and partials was never more than 1 % from the better,
         // but any other split of a sum flips greedy tokens that tie (1.2 % of them at d 2048, 1020 rows).
         if (sp > nkb / 12) sp = nkb / 12;
+        if (sp > kMaxKSplits) sp = kMaxKSplits;
         return gemm_whole_splits(sp, nkb);
     }
     // all work units must be resident at once (two CTA slots per SM) and equal in size: a
     // second, partly filled wave would double the kernel's time
     int splits = target_ctas() / tiles;
     if (splits > nkb / 4) splits = nkb / 4;
-    if (splits > 16) splits = 16;
+    if (splits > kMaxKSplits) splits = kMaxKSplits;
     return gemm_whole_splits(splits, nkb);
 }
 

@@ -616,13 +616,13 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     const size_t nmax = 3 * static_cast<size_t>(d) > 2 * static_cast<size_t>(F) ? 3 * static_cast<size_t>(d)
                                                                                 : 2 * static_cast<size_t>(F);
     // K splits of a projection with fp32 partial output; `exchanged`: the partials of all R ranks must fit a receive
-    // slot and the consumer's 16-partial limit
+    // slot and the consumer's limit
     auto plan_splits = [&](int rows, int N, int K, bool exchanged) {
         int sp = gemm_pick_splits(rows, N, K);
         size_t cap = L.partial_rows * nmax / (static_cast<size_t>(rows) * N);
         if (exchanged) {   // R blocks of `sp` partials in a receive slot (sized for at least one partial per rank)
             cap = L.tp_recv_slot / sizeof(float) / (static_cast<size_t>(rows) * N * R);
-            if (cap > static_cast<size_t>(16 / R)) cap = 16 / R;
+            if (cap > static_cast<size_t>(kMaxKSplits / R)) cap = kMaxKSplits / R;
         }
         if (static_cast<size_t>(sp) > cap) sp = gemm_whole_splits(static_cast<int>(cap < 1 ? 1 : cap), (K + 63) / 64);
         return sp;

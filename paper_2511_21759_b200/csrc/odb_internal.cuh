@@ -323,7 +323,8 @@ struct GemmArgs {
     int splits;
     int* status;           // device status word
 };
-int gemm_pick_splits(int M, int N, int K);
+int gemm_pick_splits(int M, int N, int K);   // 1 .. kMaxKSplits
+constexpr int kMaxKSplits = 16;              // partial sums of one element that the RMSNorm kernels add up at most
 // the largest number of K splits <= splits that leaves none of them empty: ceil(nkb / splits) * (splits - 1) < nkb
 int gemm_whole_splits(int splits, int nkb);
 
@@ -360,7 +361,7 @@ struct EmbedSource {
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's
 // operand, ssq[i][t] = sum of h[r]^2 over the t-th slice of kNormSliceCols columns; the projection's consumer
 // multiplies its fp32 output by 1 / sqrt(sum_t ssq / d + eps) (RowScale; the scalar commutes with the matrix
-// product).  splits <= 16.  compact: partial[s] holds the rows of the map only, in its order.
+// product).  splits <= kMaxKSplits.  compact: partial[s] holds the rows of the map only, in its order.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
                            cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource(),

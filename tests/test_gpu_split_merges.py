@@ -18,3 +18,9 @@ from test_gpu_many_rows import HD64, HD128, test_refresh_of_many_rows as check_r
 def test_merges_at_their_edges(shape, P, L):
     v = shape.vocab
     check_refresh(dataclasses.replace(shape, mask_id=v - 1, eos_id=v - 2), P, L)
+
+
+@requires_gpu
+@pytest.mark.parametrize("rows,ffn", [(129, 13056), (200, 28672)])   # a down projection of 204 and 448 k-blocks: sixteen splits
+def test_refresh_with_a_long_down_projection(rows, ffn):
+    check_refresh(dataclasses.replace(HD64, n_layers=1, n_heads=16, d_model=1024, d_ffn=ffn), rows - 60, 60)

@@ -21,3 +21,12 @@ def _rule(name, *argtypes):
 ])
 def test_key_splits_of_the_attention(items, hd, refresh, splits):
     assert _rule("_ZN3odb20attention_key_splitsEiib", ctypes.c_int, ctypes.c_int, ctypes.c_bool)(items, hd, refresh) == splits
+
+
+@pytest.mark.parametrize("M,N,K,splits", [
+    (200, 1024, 13056, 16), (200, 1024, 28672, 16), (129, 64, 1 << 17, 16),   # the consumers add up sixteen partials at most
+    (256, 2304, 12480, 15), (256, 2304, 13056, 16), (768, 4096, 4096, 3),     # many rows: at least 12 k-blocks each
+    (32, 4096, 12288, 9), (128, 1024, 28672, 16),                             # up to 128 rows: one wave
+])
+def test_k_splits_of_a_projection(M, N, K, splits):
+    assert _rule("_ZN3odb16gemm_pick_splitsEiii", ctypes.c_int, ctypes.c_int, ctypes.c_int)(M, N, K) == splits
