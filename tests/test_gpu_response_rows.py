@@ -1,4 +1,4 @@
-"""A refresh with LM head runs the last layer's O, gate/up and down projections over the response rows only.  The same
+"""A refresh with LM head runs the last layer's gate/up and down projections over the response rows only.  The same
 token ids with no prompt make every row a response row, so that every projection runs over all of them: the
 confidences and tokens of the rows both have are the same, and the keys and values too."""
 import dataclasses
@@ -14,11 +14,11 @@ from test_gpu_many_rows import HD64, HD128
 ONE = dataclasses.replace(HD64, n_layers=1)
 
 
-def _refresh(E, gm, seqs, prompts):
+def _refresh(E, gm, seqs, prompts, block=0):
     sess = E.Session(gm, poison=True)
     for i, (x, p) in enumerate(zip(seqs, prompts)):
         sess.set_sequence(i, x, p)
-    sess.refresh_prefill(E.DecodeParams(block_len=16), 0)
+    sess.refresh_prefill(E.DecodeParams(block_len=16), block)
     out = sess.debug_read("conf"), sess.debug_read("tok"), sess.debug_read("o"), sess.kv.clone()
     assert sess.status() == 0
     sess.close()
@@ -85,3 +85,24 @@ def test_residual_stream_of_the_prompt_rows_holds_the_last_attention_block(shape
     rows = np.concatenate([np.arange(at[i], at[i] + p) for i, (p, _) in enumerate(lens)])
     assert len(rows) and np.isfinite(want).all() and np.array_equal(got[rows], want[rows])
     sess.close(); gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("lens,block", [
+    ([(300, 2100)], 0),                       # 2100 rows through the LM head: a second chunk of 52
+    ([(200, 1100), (150, 1000)], 0),          # gathered
+    ([(500, 140)], 2),                        # the rows with logits start two blocks behind the prompt
+    ([(263, 90), (1, 200)], 1),
+])
+def test_rows_with_logits_in_chunks_and_behind_later_blocks(lens, block):
+    E = engine()
+    shape = dataclasses.replace(HD64, n_layers=1)
+    gm = E.Model.from_synth(shape, seed=5, max_batch=len(lens), max_seq=max(p + n for p, n in lens), max_block=16, max_copies=1)
+    seqs = [synth.sequence(5, i, p, n, shape) for i, (p, n) in enumerate(lens)]
+    conf, tok, o, kv = _refresh(E, gm, seqs, [p for p, _ in lens], block)
+    aconf, atok, ao, akv = _refresh(E, gm, seqs, [0] * len(lens))
+    gm.close()
+    at = np.cumsum([0] + [p + n for p, n in lens])
+    rows = np.concatenate([np.arange(at[i] + p + 16 * block, at[i + 1]) for i, (p, _) in enumerate(lens)])
+    assert len(conf) == len(rows) and np.array_equal(tok, atok[rows]) and np.array_equal(o, ao) and torch.equal(kv, akv)
+    assert np.allclose(conf, aconf[rows], rtol=1.3e-4, atol=0)       # as above: the chunks of the two runs differ in length

@@ -49,3 +49,43 @@ def test_step_without_key_splits(shape, batch):
         rms = np.sqrt((want ** 2).mean(-1, keepdims=True))
         assert (np.abs(got - want) <= 2.0 ** -8 * 1.01 * np.abs(want) + 2.0 ** -13 * rms).all(), i
     sess.close(); gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("copies,decoded", [(4, 0), (8, 22)])          # 22 of 32 decoded: the decoded-share layout
+@pytest.mark.parametrize("heads", [4, 32])                             # one cached tile per key split, and two
+def test_step_with_copies_around_whole_tiles(heads, copies, decoded):
+    """101 keys in front of the block and 232 behind it: a tile that holds keys of both sides is followed by whole ones that
+    start off a multiple of 64, and the last ends early.  Every row sees its own copy's rows; in the decoded-share layout
+    copy 0's decoded ones too."""
+    E = engine()
+    shape = dataclasses.replace(HD64, n_layers=1, n_heads=heads, d_model=64 * heads)
+    P, L, block = 101, 264, 32
+    gm = E.Model.from_synth(shape, seed=5, max_batch=1, max_seq=P + L, max_block=block, max_copies=8)
+    sess = E.Session(gm, poison=True)
+    x0 = synth.sequence(5, 0, P, L, shape)
+    at = np.random.default_rng(1).permutation(block)[:decoded]
+    x0[P + at] = 7 + at                                                # ids other than [MASK] and [EOS]
+    sess.set_sequence(0, x0, P)
+    par = E.DecodeParams(block_len=block, n_copies=copies, alp=False)
+    sess.refresh_prefill(par, 0)
+    sess.unmask_accept(par, True)
+    sess.block_decode_step(par)
+    x, copy, pos = sess.get_tokens(0), sess.debug_read("row_copy"), sess.debug_read("row_pos")
+    q, k, v, o = (torch.from_numpy(bf16_bits_to_f64(sess.debug_read(n))).view(-1, heads, 64) for n in "qkvo")
+    assert sess.status() == 0 and len(set(copy.tolist())) == copies
+    share = len(copy) < copies * block
+    assert share == (copies == 8)
+    sees = copy[:, None] == copy[None, :]
+    if share:
+        sees |= ((copy == 0) & (x[pos] != shape.mask_id))[None, :]
+    kv = sess.kv.view(torch.bfloat16).view(2, heads, -1, 64).double().cpu()
+    out = [j for j in range(P + L) if not P <= j < P + block]
+    keys, vals = (torch.cat([kv[j][:, out], r.transpose(0, 1)], 1) for j, r in ((0, k), (1, v)))
+    s = torch.einsum("qhd,hkd->hqk", q, keys) / math.sqrt(64)
+    s[:, :, len(out):].masked_fill_(~torch.from_numpy(sees)[None], -math.inf)
+    want = torch.einsum("hqk,hkd->qhd", torch.softmax(s, -1), vals).numpy()
+    # the bound of the test above
+    rms = np.sqrt((want ** 2).mean(-1, keepdims=True))
+    assert (np.abs(o.numpy() - want) <= 2.0 ** -8 * 1.01 * np.abs(want) + 2.0 ** -13 * rms).all()
+    sess.close(); gm.close()
