@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(256) step_attention_kernel(StepAttnArgs a) {
     uint8_t* sValid = sV + 2 * kTileBytes;           // [2][64]: 0 invalid, 1 valid, 2 valid and decoded
 
     pdl_launch_dependents();
-    // the tile table and the K/V cache were complete before this step's launch chain began: the splits
-    // that stream cached keys request their first two tiles before waiting for the predecessor
+    // the K/V cache was complete before this step began, and the tile table before anything behind its first norm could
+    // start: the splits that stream cached keys request their first two tiles before waiting for the predecessor
     const StepTile& t = a.tiles[blockIdx.x];
     const int head = blockIdx.y;
     const int z = blockIdx.z, ks = gridDim.z;
@@ -326,7 +326,11 @@ cudaError_t combine(const float* part_o, const float* part_ml, __nv_bfloat16* o,
 template <int HD>
 cudaError_t launch_hd(const AttnArgs& a, cudaStream_t st) {
     const size_t smem = kTileQ * HD * 2 + 4 * kTileK * HD * 2 + 2 * kTileK;
-    // a refresh, and steps whose keys are not split: several tiles for every CTA
+    // LONG by the kind of launch: a refresh, and steps whose keys are not split.  us per call, always short / always long: refresh of
+    // two layers, d 1024, 1118 rows (nine tiles per CTA) 227.5 / 217.3, 300 rows 166.3 / 164.4, 128 rows at d 256 (one tile) 102.0 /
+    // 100.4; unsplit steps of 16 sequences at d 1024 190.3 / 182.9.  Steps with key splits, one or two tiles per CTA: tiny step 84.1 /
+    // 84.4, 8B layer step 117.9 / 118.5, resident loop of four layers 3079 / 3105.  With four and more tiles per split the short form, which
+    // they keep, is the slower one: four 8B sequences 150.7 / 149.4, six 202.8 / 200.6, 1800 keys 127.2 / 126.5, at d 1024 114.7 / 112.5.
     const bool walk = !a.early || a.ksplit == 1;
     void (*kernel)(AttnArgs) = walk ? attention_kernel<HD, true> : attention_kernel<HD, false>;
     static std::atomic<unsigned long long> attr_done[2];

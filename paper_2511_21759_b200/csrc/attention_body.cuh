@@ -84,9 +84,9 @@ __device__ __forceinline__ void load_whole_tile(uint8_t* sK, uint8_t* sV, const 
 template <int HD>
 constexpr size_t attention_smem_bytes() { return kTileQ * HD * 2 + 4 * kTileK * HD * 2 + 2 * kTileK; }
 
-// LONG: for items of several key tiles per split (whole tiles loaded by their base address and used without masks, the bare
-// exponential instruction): 30.1 -> 25.5 us for 1118 rows x 16 heads of 64, 9 tiles each.  It is more code, and a launch whose
-// CTAs take one or two tiles pays for fetching it: 0.4 us of the 7.8 of a batch-1 step (resident loop of four layers 3092 -> 3117).
+// LONG: whole tiles loaded by their base address and used without masks, the bare exponential instruction: 30.1 -> 25.5 us for
+// 1118 rows x 16 heads of 64, 9 tiles each.  It is more code, and a step whose CTAs take one or two tiles pays for fetching it:
+// 0.4 us of the 7.8 of a batch-1 step.  Which launches take it, with both sides measured: launch_hd.
 template <int HD, bool LONG, class Sync, class Wait>
 __device__ __forceinline__ void attention_item(const AttnArgs& a, const QTile& t, int head, int z, int tid, uint8_t* smem,
                                                bool early, Wait wait_inputs) {
@@ -97,8 +97,8 @@ __device__ __forceinline__ void attention_item(const AttnArgs& a, const QTile& t
     uint8_t* sV = sK + 2 * kTileBytes;               // [2][64][HD]
     uint8_t* sValid = sV + 2 * kTileBytes;           // [2][64]
 
-    // early (decode steps): the tile table and the K/V cache were complete before this forward began, so
-    // cached key tiles are requested before waiting for the producer of q and of the fresh k / v
+    // early (decode steps): the K/V cache was complete before this forward began and the tile table before this kernel
+    // could start, so cached key tiles are requested before waiting for the producer of q and of the fresh k / v
     if (!early) wait_inputs();
     const int warp = tid >> 5, lane = tid & 31;
     const int d = a.H * HD;

@@ -58,7 +58,7 @@ struct RowsArgs {
     QkvRopeArgs qkv;             // ROWS_QKV64 / ROWS_QKV128 (head dim)
     RowScale rs;
     int M, N, nkb_total, nkb_per_split;
-    int n_pairs, m_tiles, group, splits;   // pairs of weight tiles, tiles of 256 rows, row tiles that are walked side by side
+    int n_pairs, m_tiles, group;           // pairs of weight tiles, tiles of 256 rows, row tiles that are walked side by side
     int whole, n_items;          // the items from `whole` on are single weight tiles
     uint64_t w_hint;             // L2 policy of the weight tiles
     int wide;                    // ROWS_PARTIAL: output rows start on 16-byte boundaries
@@ -523,7 +523,6 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     a.partial = g.partial; a.act_out = g.act_out; a.ce = g.conf; a.rs = g.row_scale; a.add_to = g.add_to;
     a.qkv = g.qkv ? *g.qkv : QkvRopeArgs();
     a.M = g.M; a.N = g.N;
-    a.splits = g.splits;
     a.nkb_total = (g.K + kBK - 1) / kBK;
     a.nkb_per_split = (a.nkb_total + g.splits - 1) / g.splits;
     if (a.nkb_per_split * (g.splits - 1) >= a.nkb_total) return cudaErrorInvalidValue;   // an empty split

@@ -29,11 +29,16 @@ cudaError_t set_smem_limit_once(std::atomic<unsigned long long>& done, Kernel ke
 }
 
 // ---------------------------------------------------------------------------------------
-// programmatic dependent launch: every kernel of a forward lets its successor start early
-// (launch_dependents at entry) and waits for its predecessor's results (wait) only where it
-// first needs them, so prologues, tensor-map fetches and weight prefetches overlap the
-// predecessor's tail.  Every such kernel executes pdl_wait() before it exits, which keeps the
-// completion order of the chain transitive.
+// programmatic dependent launch: a kernel of a forward lets its successor start early
+// (launch_dependents) and waits for its predecessor's results (wait) only where it first
+// needs them, so prologues, tensor-map fetches and weight prefetches overlap the predecessor's
+// tail.  Every such kernel executes pdl_wait() before it exits, which keeps the completion order
+// of the chain transitive.  The successor is let go at entry, but for
+//   - the first norm: behind its wait for the kernel that builds the row and tile tables.  That
+//     alone makes the tables complete before any later kernel of the chain starts, and lets the
+//     attention read its work items (and a step the K/V cache) before its own wait;
+//   - kernels that allocate TMEM for CTA pairs, and the tensor-core attention: behind the allocation;
+//   - many-row QKV projections with the RoPE epilogue: not at all (gemm_rows.cu).
 // ---------------------------------------------------------------------------------------
 
 #ifdef __CUDACC__
@@ -391,7 +396,8 @@ struct AttnArgs {
     __nv_bfloat16* o;                     // [M][H*hd]
     float* part_o; float* part_ml;        // split workspaces [ks][M][H][hd], [ks][M][H][2]
     int layer, n_layers, H, hd, max_seq, M, ksplit;
-    int early = 0;                        // 1: tiles and cache were complete before the launch chain began (decode steps)
+    int early = 0;                        // 1: the cache was complete before the forward began (decode steps); the tiles are
+                                          // complete before any kernel behind the first norm starts
     L2Prefetch pf;
 };
 // Key splits of the mma.sync attention over `items` pairs of a row tile and a head, 1 .. 8.
