@@ -403,7 +403,7 @@ struct AttnArgs {
 // Key splits of the mma.sync attention over `items` pairs of a row tile and a head, 1 .. 8.
 int attention_key_splits(int items, int head_dim, bool refresh);
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st);
-// refresh attention on the tcgen05 tensor cores (head dim 128): a.tiles = work items of up to 128 query rows
+// refresh attention on the tcgen05 tensor cores: a.tiles = work items of up to 128 query rows
 // whose keys are the fresh rows [f0, f0 + n0); status = device status word (bounded waits)
 cudaError_t launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
 
@@ -419,8 +419,8 @@ struct StepAttnArgs {
     L2Prefetch pf;
 };
 cudaError_t launch_step_attention(const StepAttnArgs& a, cudaStream_t st);
-// the same work items on the tcgen05 tensor cores (head dim 128): writes the split partials only;
-// cache_rows = rows of the K/V cache viewed as [rows][128]
+// the same work items on the tcgen05 tensor cores: with key splits it writes the partials only;
+// cache_rows = rows of the K/V cache viewed as [rows][hd]
 cudaError_t launch_step_attention_tc(const StepAttnArgs& a, size_t cache_rows, int* status, cudaStream_t st);
 cudaError_t launch_attention_combine(const float* part_o, const float* part_ml, __nv_bfloat16* o, int M, int H, int hd,
                                      int ksplit, cudaStream_t st);
