@@ -814,11 +814,15 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
             if (sks < 2) sks = 2;
             sa.ksplit = sks;
             sa.pf = hint_of(m->p_gu[l], gu_bytes, 0);
-            // tensor-core work items for head dim 128 (batched steps: 33.5 -> 22.5 ms at 16 sequences x 256 rows with the
+            // tensor-core work items; head dim 128 (batched steps: 33.5 -> 22.5 ms at 16 sequences x 256 rows with the
             // first, two-pass version of that kernel, when a single 128-row item per head still lost to mma.sync, 1.20
             // vs 1.12 ms per step at batch 1; in one pass it wins there too: 1.00 vs 1.13 ms, step 4.82 -> 4.63 ms)
-            static const int tc_step_min = getenv("ODB_ATTN_TC_STEP_MIN") ? atoi(getenv("ODB_ATTN_TC_STEP_MIN")) : 1;
-            if (hd == 128 && tc_attention && n_step_tiles * H >= tc_step_min) {
+            // Head dim 64, two layers of d 1024, us per step, mma.sync / tensor cores: 16 items 133.4 / 129.8 and 146.8 / 145.7, 32 items
+            // 149.7 / 147.3, 64 items 172 / 161 and 196 / 179, 128 items 214 / 187, 512 items of 64-row blocks 558 / 373; d 256, 4 items
+            // 112 / 109.  Below 32 items the two are as good as equal, and those steps keep the sums that they had.
+            static const int tc_step_env = getenv("ODB_ATTN_TC_STEP_MIN") ? atoi(getenv("ODB_ATTN_TC_STEP_MIN")) : 0;
+            const int tc_step_min = tc_step_env > 0 ? tc_step_env : hd == 128 ? 1 : 32;
+            if (tc_attention && n_step_tiles * H >= tc_step_min) {
                 const size_t cache_rows = static_cast<size_t>(c.max_batch) * c.n_layers * 2 * H * c.max_seq;
                 // with a work item for every CTA slot there is nothing to gain from key splits: one CTA per item takes
                 // the cached and the fresh keys and writes the final output (no partials, no merge kernel)
@@ -830,8 +834,11 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
                 ODB_FWD(ODB_KIND_ATTENTION, launch_step_attention(sa, st));
                 if (seg_on()) ++s->launches[ODB_KIND_ATTENTION];
             }
-        } else if (write_cache && hd == 128 && n_big_tiles > 0 && tc_attention) {
-            // refresh with head dim 128: 128-row work items on the tcgen05 tensor cores, no key split
+        } else if (write_cache && tc_attention && n_big_tiles * H >= (hd == 128 ? 1 : 74)) {
+            // refresh: 128-row work items on the tcgen05 tensor cores, no key split.  Head dim 64, us per refresh of two layers, mma.sync
+            // (64-row items, keys split to fill the chip) / tensor cores: d 1024, 128 items 226 / 195, 96 items 203 / 188, 64 items 163 / 158, 32
+            // items 151.5 / 149.2; d 256, 512 items 426 / 327, 64 items 181 / 171, 16 items 116 / 121.  With fewer items than every
+            // other SM could take, a few per cent either way, the refresh keeps the key splits.
             AttnArgs aa;
             aa.tiles = s->cb.big_tiles; aa.n_tiles = n_big_tiles;
             aa.q = q; aa.k = k; aa.v = v; aa.cache = s->kv; aa.row_flags = s->cb.row_flags; aa.o = o;

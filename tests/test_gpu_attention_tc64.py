@@ -1,0 +1,94 @@
+"""The tensor-core attention with head dim 64, where launches have enough work items for it: refreshes around the edges of the
+128-row items and 64-key tiles, steps of several copies with and without key splits, in both row layouts."""
+import dataclasses
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+from gpu_common import bf16_bits_to_f64, engine, requires_gpu
+from test_gpu_many_rows import HD64
+
+HEADS = 32
+SHAPE = dataclasses.replace(HD64, n_layers=1, n_heads=HEADS, d_model=64 * HEADS, d_ffn=256)
+
+
+def rows(sess, name):
+    return torch.from_numpy(bf16_bits_to_f64(sess.debug_read(name))).view(-1, HEADS, 64)
+
+
+def check(o, q, keys, vals, visible=None):
+    s = torch.einsum("qhd,hkd->hqk", q, keys) / math.sqrt(64)
+    if visible is not None:
+        s = s.masked_fill(~visible[None], -math.inf)
+    want = torch.einsum("hqk,hkd->qhd", torch.softmax(s, -1), vals).numpy()
+    # the output is rounded to bf16 (half of the last of seven fraction bits: 2^-8 of the value at worst); fp32 scores and
+    # sums, P as two bf16 terms: 2^-16 of the row's size
+    rms = np.sqrt((want ** 2).mean(-1, keepdims=True))
+    assert (np.abs(o.numpy() - want) <= 2.0 ** -8 * 1.01 * np.abs(want) + 2.0 ** -13 * rms).all()
+
+
+@requires_gpu
+@pytest.mark.parametrize("lens", [
+    [(257, 64)],                          # three items (96 with 32 heads): the last has 65 rows; six key tiles, the last of one key
+    [(320, 64)],                          # whole items and whole tiles
+    [(100, 28), (1, 64), (70, 100)],      # one whole item, one of 65 rows, one and 42 rows
+    [(1000, 70), (30, 33)],               # seventeen key tiles and one
+])
+def test_refresh(lens):
+    E = engine()
+    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=len(lens), max_seq=max(p + n for p, n in lens), max_block=16, max_copies=1)
+    sess = E.Session(gm, poison=True)
+    for i, (p, n) in enumerate(lens):
+        sess.set_sequence(i, synth.sequence(5, i, p, n, SHAPE), p)
+    sess.refresh_prefill(E.DecodeParams(block_len=16), 0)
+    q, k, v, o = (rows(sess, x) for x in "qkvo")
+    assert sess.status() == 0
+    r0 = 0
+    for p, n in lens:
+        r = slice(r0, r0 + p + n)
+        check(o[r], q[r], k[r].transpose(0, 1), v[r].transpose(0, 1))
+        r0 += p + n
+    assert r0 == len(o)
+    sess.close(); gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("copies,decoded,block,batch", [
+    (4, 0, 32, 1),       # one item per head, seven cached key splits and the fresh one
+    (4, 5, 24, 2),       # 96 rows an item
+    (8, 22, 32, 3),      # the decoded-share layout: copies see copy 0's decoded rows
+    (4, 0, 64, 5),       # ten items per head: no key splits, the outputs are final
+    (8, 44, 64, 5),
+])
+def test_step_with_copies(copies, decoded, block, batch):
+    E = engine()
+    lens = [(101 + 37 * i, 200 - 19 * i) for i in range(batch)]
+    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=batch, max_seq=max(p + n for p, n in lens), max_block=block, max_copies=8)
+    sess = E.Session(gm, poison=True)
+    for i, (p, n) in enumerate(lens):
+        x = synth.sequence(5, i, p, n, SHAPE)
+        at = np.random.default_rng(i).permutation(block)[:decoded]
+        x[p + at] = 7 + at                                             # ids other than [MASK] and [EOS]
+        sess.set_sequence(i, x, p)
+    par = E.DecodeParams(block_len=block, n_copies=copies, alp=False)
+    sess.refresh_prefill(par, 0)
+    sess.unmask_accept(par, True)
+    sess.block_decode_step(par)
+    copy, pos = sess.debug_read("row_copy"), sess.debug_read("row_pos")
+    seq = np.cumsum((copy == 0) & (np.roll(copy, 1) != 0)) - 1          # the rows are in sequence order, copy 0 first
+    q, k, v, o = (rows(sess, x) for x in "qkvo")
+    assert sess.status() == 0
+    kv = sess.kv.view(torch.bfloat16).view(batch, 2, HEADS, -1, 64).double().cpu()
+    for i, (p, n) in enumerate(lens):
+        r = np.flatnonzero(seq == i)
+        x = sess.get_tokens(i)
+        sees = copy[r][:, None] == copy[r][None, :]
+        if len(r) < copies * block:
+            sees |= ((copy[r] == 0) & (x[pos[r]] != SHAPE.mask_id))[None, :]
+        out = [j for j in range(p + n) if not p <= j < p + block]
+        keys, vals = (torch.cat([kv[i, j][:, out], f[r].transpose(0, 1)], 1) for j, f in ((0, k), (1, v)))
+        check(o[r], q[r], keys, vals, torch.cat([torch.ones(len(r), len(out), dtype=torch.bool), torch.from_numpy(sees)], 1))
+    sess.close(); gm.close()
