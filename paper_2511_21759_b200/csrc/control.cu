@@ -1,242 +1,11 @@
-// Control kernels: row tables of a refresh / a block step, and the unmask/accept kernel
-// (threshold accept rule, accept-jump walk over the block copies, adaptive length prediction,
-// choice of the next speculative candidates).  A few hundred scalars per sequence: one small
-// block per sequence, the sequential parts on thread 0.
+// Control kernels: the unmask/accept kernel (threshold accept rule, accept-jump walk over the block copies, adaptive
+// length prediction, choice of the next speculative candidates).  A few hundred scalars per sequence: one small
+// block per sequence, the sequential parts on thread 0.  (The row tables: first_norm.cu.)
 #include "odb_internal.cuh"
 
 namespace odb {
 
 namespace {
-
-struct BlockIndexParam {
-    int32_t block_index[64];
-    int32_t block_len;
-};
-
-// Rows of a refresh: every position of every active sequence, in sequence order.
-__global__ void build_refresh_rows_kernel(ControlBuffers c, int batch, BlockIndexParam bp) {
-    pdl_launch_dependents();   // the first norm, which waits for the table before it lets its own successor start
-    const int seq = blockIdx.x;
-    SeqState* st = c.state + seq;
-    if (!st->active || bp.block_index[seq] < 0) {
-        if (threadIdx.x == 0) st->in_fwd = 0;
-        return;
-    }
-    // what the sequences in front take: one thread per sequence (serially, sixteen sequences were 9 us of dependent loads)
-    __shared__ int row0, lm0, tile0, big0;
-    if (threadIdx.x == 0) row0 = lm0 = tile0 = big0 = 0;
-    __syncthreads();
-    if (threadIdx.x < seq) {
-        const SeqState* o = c.state + threadIdx.x;
-        if (o->active && bp.block_index[threadIdx.x] >= 0) {
-            atomicAdd(&row0, o->T);
-            atomicAdd(&lm0, o->T - (o->P + bp.block_index[threadIdx.x] * bp.block_len));
-            atomicAdd(&tile0, (o->T + 63) / 64);
-            atomicAdd(&big0, (o->T + 127) / 128);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int s = st->P + bp.block_index[seq] * bp.block_len;
-        st->in_fwd = 1;
-        st->block_idx = bp.block_index[seq];
-        st->s = s;
-        st->e = min(s + bp.block_len, st->T);
-        st->row0 = row0;
-        st->n_rows = st->T;
-        st->lm_row0 = lm0;
-        st->lm_s = s;
-        st->lm_n = st->T - s;
-        st->n_ranks = 0;
-        st->n_copies = 1;
-        st->copy_mask[0] = 0;
-        st->stage2 = 0;
-    }
-    const int T = st->T;
-    const int s = st->P + bp.block_index[seq] * bp.block_len;
-    const int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
-    for (int p = threadIdx.x; p < T; p += blockDim.x) {
-        const int row = row0 + p;
-        c.row_tok[row] = x[p];
-        c.row_pos[row] = p;
-        c.row_seq[row] = seq;
-        c.row_copy[row] = 0;
-        c.row_flags[row] = 0;
-        if (p >= s) c.lm_rows[lm0 + (p - s)] = row;
-    }
-    for (int j = threadIdx.x; j < (T + 63) / 64; j += blockDim.x) {
-        QTile q;
-        q.q_row0 = row0 + 64 * j;
-        q.nq = min(64, T - 64 * j);
-        q.seq = seq;
-        q.cA = 0; q.cB0 = 0; q.cB1 = 0;
-        q.f0 = row0; q.n0 = T;
-        q.f1 = 0; q.n1 = 0;
-        c.tiles[tile0 + j] = q;
-    }
-    for (int j = threadIdx.x; j < (T + 127) / 128; j += blockDim.x) {
-        QTile q;
-        q.q_row0 = row0 + 128 * j;
-        q.nq = min(128, T - 128 * j);
-        q.seq = seq;
-        q.cA = 0; q.cB0 = 0; q.cB1 = 0;
-        q.f0 = row0; q.n0 = T;
-        q.f1 = 0; q.n1 = 0;
-        c.big_tiles[big0 + j] = q;
-    }
-}
-
-// Rows of a block step (Section 4.2; decoded-share layout: Section 4.2.2, caption of Fig. 8):
-// copy 0 holds the whole block; a speculative copy holds the whole block (stage 1) or only the
-// positions still masked in the committed state (stage 2).  Position ids are the true positions.
-__device__ int step_rows_of(const SeqState* st) {
-    const int B = st->e - st->s;
-    return st->stage2 ? B + (st->n_copies - 1) * st->n_masked : st->n_copies * B;
-}
-
-__device__ int step_tiles_of(const SeqState* st) {
-    const int B = st->e - st->s;
-    return step_tiles_of_counts(st->n_copies, B, st->stage2 ? st->n_masked : B);
-}
-
-// One block per sequence.  The state is worked on in shared memory and the sequences in front are counted by one thread
-// each: written as one thread's walk over global memory this was 6 us at batch 1 and 22 us at batch 16.
-__global__ void __launch_bounds__(64) build_step_rows_kernel(ControlBuffers c, int batch, int mask_id) {
-    pdl_launch_dependents();           // as above
-    const int seq = blockIdx.x, tid = threadIdx.x;
-    __shared__ SeqState sst;
-    __shared__ int xs[kMaxBlock];      // the block's committed tokens
-    __shared__ unsigned masked_w[2];   // bit i: position i of the block is masked
-    __shared__ int row_base, tile_base, stile_base;
-    __shared__ StepTile items[ODB_MAX_COPIES];
-    {
-        const int* gs = reinterpret_cast<const int*>(c.state + seq);
-        for (int i = tid; i < static_cast<int>(sizeof(SeqState) / 4); i += 64) reinterpret_cast<int*>(&sst)[i] = gs[i];
-        if (tid == 0) row_base = tile_base = stile_base = 0;
-    }
-    __syncthreads();
-    SeqState* st = &sst;
-    if (!st->active || st->n_masked <= 0) {
-        if (tid == 0) c.state[seq].in_fwd = 0;
-        return;
-    }
-    const int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
-    const int s = st->s, e = st->e, B = e - s;   // B <= kMaxBlock = blockDim
-    const int my_tok = tid < B ? x[s + tid] : 0;
-    if (tid < seq) {
-        const SeqState* o = c.state + tid;
-        if (o->active && o->n_masked > 0) {
-            atomicAdd(&row_base, step_rows_of(o));
-            atomicAdd(&tile_base, o->n_copies);
-            atomicAdd(&stile_base, step_tiles_of(o));
-        }
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, tid < B && my_tok == mask_id);
-    if ((tid & 31) == 0) masked_w[tid >> 5] = bal;
-    xs[tid] = my_tok;
-    __syncthreads();
-    if (tid == 0) {
-        const int nm = __popc(masked_w[0]) + __popc(masked_w[1]);
-        int row = row_base;
-        st->in_fwd = 1;
-        st->row0 = row;
-        // copy 0 holds the whole block; a speculative copy the whole block or, in the decoded-share layout, the
-        // positions still masked
-        for (int cp = 0; cp < st->n_copies; ++cp) {
-            st->copy_row0[cp] = row;
-            st->copy_nrows[cp] = (st->stage2 && cp > 0) ? nm : B;
-            row += st->copy_nrows[cp];
-        }
-        st->n_rows = row - st->row0;
-        st->lm_row0 = st->row0;
-    }
-    __syncthreads();
-    const unsigned long long masked = static_cast<unsigned long long>(masked_w[1]) << 32 | masked_w[0];
-    // one thread per (copy, position): the rows of the copies, copy after copy
-    for (int it = tid; it < st->n_copies * B; it += 64) {
-        const int cp = it / B, i = it % B;
-        const bool decoded = !((masked >> i) & 1ull);
-        const bool shared = st->stage2 && cp > 0;
-        if (shared && decoded) continue;
-        const int row = st->copy_row0[cp] + (shared ? __popcll(masked & ((1ull << i) - 1ull)) : i);
-        int tok = xs[i];
-        for (int r = 0; r < st->n_ranks; ++r)
-            if (((st->copy_mask[cp] >> r) & 1) && st->rank_off[r] == i) tok = st->rank_tok[r];
-        c.row_tok[row] = tok;
-        c.row_pos[row] = s + i;
-        c.row_seq[row] = seq;
-        c.row_copy[row] = cp;
-        c.row_flags[row] = decoded ? kRowDecoded : 0;
-        c.lm_rows[row] = row;
-    }
-    if (tid < st->n_copies) {
-        const int cp = tid;
-        QTile q;
-        q.q_row0 = st->copy_row0[cp];
-        q.nq = st->copy_nrows[cp];
-        q.seq = seq;
-        q.cA = s; q.cB0 = e; q.cB1 = st->T;
-        q.f0 = q.q_row0; q.n0 = q.nq;
-        const bool shared = st->stage2 && cp > 0;
-        q.f1 = shared ? st->copy_row0[0] : 0;
-        q.n1 = shared ? st->copy_nrows[0] : 0;
-        c.tiles[tile_base + cp] = q;
-    }
-    // attention work items that share the cached K/V among copies: copies are packed, in order, into
-    // items of at most 8 slabs of 16 rows (the host counts them with the same rule, step_tiles_of)
-    __shared__ int n_items;
-    if (tid == 32) {
-        int have = 0, n = 0;
-        StepTile* cur = items;
-        auto add_src = [&](int cp) {
-            for (int i = 0; i < cur->n_src; ++i)
-                if (cur->src_copy[i] == cp) return;
-            cur->src_copy[cur->n_src] = cp;
-            cur->src_row0[cur->n_src] = st->copy_row0[cp];
-            cur->src_n[cur->n_src] = st->copy_nrows[cp];
-            ++cur->n_src;
-        };
-        auto flush = [&]() {
-            if (st->stage2) add_src(0);   // copy 0's decoded rows are visible to every speculative copy
-            ++cur; ++n;
-            have = 0;
-        };
-        for (int cp = 0; cp < st->n_copies; ++cp) {
-            const int slabs = (st->copy_nrows[cp] + 15) / 16;
-            if (have && cur->n_slabs + slabs > 8) flush();
-            if (!have) {
-                cur->seq = seq; cur->cA = s; cur->cB0 = e; cur->cB1 = st->T;
-                cur->n_slabs = 0; cur->n_src = 0; cur->stage2 = st->stage2;
-                have = 1;
-            }
-            for (int k = 0; k < slabs; ++k) {
-                cur->slab_copy[cur->n_slabs] = cp;
-                cur->slab_row0[cur->n_slabs] = st->copy_row0[cp] + 16 * k;
-                cur->slab_n[cur->n_slabs] = min(16, st->copy_nrows[cp] - 16 * k);
-                ++cur->n_slabs;
-            }
-            add_src(cp);
-        }
-        if (have) flush();
-        n_items = n;
-    }
-    __syncthreads();
-    {   // entries of an item beyond its counts are never read
-        const int words = n_items * static_cast<int>(sizeof(StepTile) / 4);
-        int* dst = reinterpret_cast<int*>(c.step_tiles + stile_base);
-        for (int i = tid; i < words; i += 64) dst[i] = reinterpret_cast<const int*>(items)[i];
-    }
-    // the placement back to the device state; other blocks read active, s, e, n_masked, n_copies, stage2 only, which stay
-    SeqState* gst = c.state + seq;
-    if (tid == 0) {
-        gst->in_fwd = 1;
-        gst->row0 = st->row0; gst->n_rows = st->n_rows; gst->lm_row0 = st->lm_row0;
-    }
-    if (tid < st->n_copies) {
-        gst->copy_row0[tid] = st->copy_row0[tid];
-        gst->copy_nrows[tid] = st->copy_nrows[tid];
-    }
-}
 
 typedef unsigned long long Mask;   // bit i: position i of the block (blocks have at most 64 positions)
 
@@ -270,10 +39,15 @@ __device__ Mask sample_set(const float* u, Mask masked, int k, int n_steps) {
     return acc;
 }
 
-// st / res: the block's shared-memory copies of the sequence's state and result (the decisions are one thread's
-// serial walk: every field it touches would otherwise be a dependent global load)
+// rank set i of the copies of a step, one byte each: {}, {1}, {2}, {1,2}, {3}, {1,2,3}, {4}, {1,2,3,4}
+__device__ __forceinline__ int copy_set(int i) { return static_cast<int>(0x0f08070403020100ull >> (8 * i)) & 0xff; }
+
+// Block of 64 threads.  st / res: the block's shared-memory copies of the sequence's state and result (the decisions are one
+// thread's serial walk: every field it touches would otherwise be a dependent global load).  wait_forward() returns when the
+// forward's confidences and tokens are there; what stands in front of it needs the states and tokens alone.
+template <class Wait>
 __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p, int after_refresh, int mask_id, int eos_id,
-                            int dry, SeqState* st, odb_result* res) {
+                            int dry, SeqState* st, odb_result* res, Wait wait_forward) {
     const int seq = blockIdx.x;
     if (!st->active || !st->in_fwd) {
         if (threadIdx.x == 0) {
@@ -288,11 +62,18 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
     }
     __shared__ float conf[ODB_MAX_COPIES][kMaxBlock];
     __shared__ int tok[ODB_MAX_COPIES][kMaxBlock];
-    __shared__ int xs[kMaxBlock];          // the block's committed tokens
+    __shared__ unsigned masked_w[2];       // bit i: position i of the block is masked
     __shared__ int first_eos;
     int32_t* x = c.x + static_cast<size_t>(seq) * c.max_seq;
     const int s = st->s;
     const int n_copies = after_refresh || dry ? 1 : st->n_copies;
+    {   // up to the block's end before a length prediction, which can only move it forward
+        const int i = threadIdx.x;
+        const bool masked = s + i < (after_refresh ? min(s + p.block_len, st->T) : st->e) && __ldcg(x + s + i) == mask_id;
+        const unsigned w = __ballot_sync(0xffffffffu, masked);
+        if ((i & 31) == 0) masked_w[i >> 5] = w;
+    }
+    if (!dry) wait_forward();
     // The whole block gathers what the decisions need - the [EOS] scan of a refresh, the copies' confidences and tokens,
     // the block's tokens; the decisions below are taken by thread 0 alone, in the order the method states them.  (One
     // thread scanning and gathering a 256-token response: 42 us; the block: 12 us.)
@@ -314,7 +95,6 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         }
         __syncthreads();
     }
-    for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) xs[i] = x[s + i];
     if (!dry && after_refresh) {
         for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) {
             const int r = st->lm_row0 + (s + i - st->lm_s);
@@ -338,28 +118,29 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
+    const int B = st->e - s;
+    const Mask masked0 = (static_cast<Mask>(masked_w[1]) << 32 | masked_w[0]) & (B >= 64 ? ~0ull : (1ull << B) - 1ull);
 
     if (dry) {
         // model without LM head (layer microbenchmark): there is nothing to decide on, so commit
         // nothing and lay out the next step as if no position had been accepted; the speculative
         // fills are the first masked positions with token id 0
-        const int B = st->e - s;
-        int n_masked = 0, n_ranks = 0;
+        int n_ranks = 0;
         const int k_ranks = p.n_copies >= 8 ? 4 : p.n_copies >= 4 ? 2 : 0;
-        for (int i = 0; i < B; ++i) {
-            if (xs[i] != mask_id) continue;
-            if (n_ranks < k_ranks) { st->rank_off[n_ranks] = i; st->rank_tok[n_ranks] = 0; ++n_ranks; }
-            ++n_masked;
+        for (Mask left = masked0; left && n_ranks < k_ranks; left &= left - 1) {
+            st->rank_off[n_ranks] = __ffsll(left) - 1;
+            st->rank_tok[n_ranks] = 0;
+            ++n_ranks;
         }
+        const int n_masked = __popcll(masked0);
         st->n_ranks = n_ranks;
         st->n_masked = n_masked;
         const int thr = p.stage2_min_decoded >= 0 ? p.stage2_min_decoded : (4 * B + 6) / 7;
         const int stage2 = (p.n_copies >= 8 && (B - n_masked) >= thr) ? 1 : 0;
         const int want = p.n_copies >= 8 ? (stage2 ? 8 : 4) : p.n_copies >= 4 ? 4 : 1;
-        const int all_masks[ODB_MAX_COPIES] = {0, 1, 2, 3, 4, 7, 8, 15};
         int nc = 0;
         for (int i = 0; i < want; ++i)
-            if ((all_masks[i] >> n_ranks) == 0) st->copy_mask[nc++] = all_masks[i];
+            if ((copy_set(i) >> n_ranks) == 0) st->copy_mask[nc++] = copy_set(i);
         st->n_copies = nc;
         st->stage2 = stage2;
         res->masks_left = n_masked;
@@ -371,13 +152,11 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         res->block_end = st->e;
         return;
     }
-    const int B = st->e - s;
     if (after_refresh) st->block_iter = 0;
     const int k_iter = st->block_iter < kMaxLoopIters ? st->block_iter : kMaxLoopIters - 1;
     const float* noise = c.noise + (static_cast<size_t>(seq) * kMaxLoopIters + k_iter) * kMaxBlock;
     ++st->block_iter;
-    Mask masked0 = 0, taken = 0;
-    for (int i = 0; i < B; ++i) masked0 |= static_cast<Mask>(xs[i] == mask_id) << i;
+    Mask taken = 0;
 
     // accept-jump walk (Section 4.2.1): start in the main block; a candidate is hit if its
     // position was accepted with the token it had been filled with; jump to the largest copy
@@ -477,10 +256,9 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
     const int thr = p.stage2_min_decoded >= 0 ? p.stage2_min_decoded : (4 * B + 6) / 7;
     const int stage2 = (p.n_copies >= 8 && (B - n_masked) >= thr) ? 1 : 0;
     const int want = p.n_copies >= 8 ? (stage2 ? 8 : 4) : p.n_copies >= 4 ? 4 : 1;
-    const int all_masks[ODB_MAX_COPIES] = {0, 1, 2, 3, 4, 7, 8, 15};
     int nc = 0;
     for (int i = 0; i < want; ++i)
-        if ((all_masks[i] >> n_ranks) == 0) st->copy_mask[nc++] = all_masks[i];
+        if ((copy_set(i) >> n_ranks) == 0) st->copy_mask[nc++] = copy_set(i);
     st->n_copies = nc;
     st->stage2 = stage2;
 
@@ -498,12 +276,13 @@ struct AcceptShared {
     SeqState st;
     odb_result res;
 };
+// from L2: in front of the wait nothing else orders these reads behind an L1 line of an earlier kernel
 __device__ __forceinline__ void accept_load(const ControlBuffers& c, AcceptShared* sh) {
     const int seq = blockIdx.x;
     const int* gs = reinterpret_cast<const int*>(c.state + seq);
     const int* gr = reinterpret_cast<const int*>(c.results + seq);
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(SeqState) / 4); i += blockDim.x) reinterpret_cast<int*>(&sh->st)[i] = gs[i];
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(odb_result) / 4); i += blockDim.x) reinterpret_cast<int*>(&sh->res)[i] = gr[i];
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(SeqState) / 4); i += blockDim.x) reinterpret_cast<int*>(&sh->st)[i] = __ldcg(gs + i);
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(odb_result) / 4); i += blockDim.x) reinterpret_cast<int*>(&sh->res)[i] = __ldcg(gr + i);
     __syncthreads();
 }
 // state and result back to the device copies and out to pinned host memory (host_res: where this call's results go)
@@ -519,11 +298,15 @@ __device__ __forceinline__ void accept_store(const ControlBuffers& c, const Acce
     for (int i = threadIdx.x; i < static_cast<int>(sizeof(odb_result) / 4); i += blockDim.x) { gr[i] = sr[i]; hr[i] = sr[i]; }
 }
 
-__global__ void accept_kernel(ControlBuffers c, odb_decode_params p, int after_refresh, int mask_id, int eos_id, int dry) {
+// Launched under the last kernel of the forward, and it starts when the forward's first kernel has written the tables and the
+// states (first_norm.cu): it reads states and tokens, which nothing behind that kernel writes, before it waits for the forward.
+// Without an LM head that is all it decides on.  Behind the wait are stores alone: us in an 8B layer step with one copy / four,
+// 3.7 / 5.0 when it waited first and one thread walked over the block's tokens.
+__global__ void __launch_bounds__(kMaxBlock) accept_kernel(ControlBuffers c, odb_decode_params p, int after_refresh, int mask_id, int eos_id, int dry) {
     __shared__ AcceptShared sh;
-    pdl_wait();   // launched under the last kernel of the forward: its start is not waited for on top of its work
     accept_load(c, &sh);
-    accept_body(c, p, after_refresh, mask_id, eos_id, dry, &sh.st, &sh.res);
+    accept_body(c, p, after_refresh, mask_id, eos_id, dry, &sh.st, &sh.res, []() { pdl_wait(); });
+    pdl_wait();
     __syncthreads();
     accept_store(c, &sh, c.host_results + blockIdx.x);
     if (blockIdx.x == 0 && threadIdx.x == 0) *c.host_status = *c.status;
@@ -531,10 +314,11 @@ __global__ void accept_kernel(ControlBuffers c, odb_decode_params p, int after_r
 }
 
 // The accept of the device-resident loop: the same decisions, then the hand-over to the next iteration.
-__global__ void accept_loop_kernel(ControlBuffers c, odb_decode_params p, int mask_id, int eos_id, int dry, LoopControl lc) {
+__global__ void __launch_bounds__(kMaxBlock) accept_loop_kernel(ControlBuffers c, odb_decode_params p, int mask_id, int eos_id, int dry, LoopControl lc) {
     __shared__ AcceptShared sh;
     accept_load(c, &sh);
-    accept_body(c, p, 0, mask_id, eos_id, dry, &sh.st, &sh.res);
+    accept_body(c, p, 0, mask_id, eos_id, dry, &sh.st, &sh.res, []() { pdl_wait(); });
+    pdl_wait();
     __syncthreads();
     const int seq = blockIdx.x, batch = gridDim.x;
     const int it = *lc.iter;      // stable until every block has arrived below
@@ -592,27 +376,12 @@ cudaError_t launch_expire_wait(long long limit_cycles, int* status, cudaStream_t
 
 cudaError_t launch_accept_loop(const ControlBuffers& c, int batch, const odb_decode_params& p, int mask_id, int eos_id,
                                int dry, const LoopControl& lc, cudaStream_t st) {
-    accept_loop_kernel<<<batch, 64, 0, st>>>(c, p, mask_id, eos_id, dry, lc);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_build_step_rows(const ControlBuffers& c, int batch, int mask_id, cudaStream_t st) {
-    build_step_rows_kernel<<<batch, 64, 0, st>>>(c, batch, mask_id);
-    return cudaGetLastError();
+    return launch_kernel(accept_loop_kernel, dim3(batch), dim3(kMaxBlock), 0, st, c, p, mask_id, eos_id, dry, lc);
 }
 
 cudaError_t launch_accept(const ControlBuffers& c, int batch, const odb_decode_params& p, int after_refresh,
                           int mask_id, int eos_id, int dry, cudaStream_t st) {
-    return launch_kernel(accept_kernel, dim3(batch), dim3(64), 0, st, c, p, after_refresh, mask_id, eos_id, dry);
-}
-
-cudaError_t launch_build_refresh_rows(const ControlBuffers& c, int batch, const int32_t* block_index,
-                                           int block_len, cudaStream_t st) {
-    BlockIndexParam bp;
-    for (int i = 0; i < 64; ++i) bp.block_index[i] = i < batch ? block_index[i] : 0;
-    bp.block_len = block_len;
-    build_refresh_rows_kernel<<<batch, 256, 0, st>>>(c, batch, bp);
-    return cudaGetLastError();
+    return launch_kernel(accept_kernel, dim3(batch), dim3(kMaxBlock), 0, st, c, p, after_refresh, mask_id, eos_id, dry);
 }
 
 }  // namespace odb

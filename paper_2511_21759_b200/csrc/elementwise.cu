@@ -1,34 +1,11 @@
 // Small memory-bound kernels between the GEMMs: residual (at first: the embedding) + split-K reduction
 // + RMSNorm operand, split-K reduction + RoPE + K/V cache scatter, and the vocab-wide confidence
 // reduction (SwiGLU lives in the gate/up GEMM's epilogue).  All reductions run in a fixed order (bitwise reproducible).
-#include "odb_internal.cuh"
+#include "norm_common.cuh"
 
 namespace odb {
 
 namespace {
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(c, d);
-    uint2 pk;
-    pk.x = *reinterpret_cast<const uint32_t*>(&lo);
-    pk.y = *reinterpret_cast<const uint32_t*>(&hi);
-    return pk;
-}
-
-// x^2 + y^2 + z^2 + w^2 with the roundings spelled out, so that every variant of an RMSNorm kernel gives the same bits
-// (a last bit here flips bf16 roundings in every layer behind): SECOND_FIRST starts with y^2, as the few-row kernel does.
-template <bool SECOND_FIRST>
-__device__ __forceinline__ float squares4(const float4& v) {
-    const float t = SECOND_FIRST ? __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)) : __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x));
-    return __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, t));
-}
 
 // block-wide sum, same value returned to every thread; `red` has >= 32 floats
 __device__ __forceinline__ float block_sum(float v, float* red) {
@@ -42,20 +19,6 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
     return t;
 }
 
-// float4 i of the embedding row of row r's token
-__device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i, int d) {
-    const __nv_bfloat16* row = e.table + static_cast<size_t>(e.row_tok[r]) * d;
-    uint2 x;
-    if (e.halves) {
-        x.x = reinterpret_cast<const uint32_t*>(row)[2 * i];
-        x.y = reinterpret_cast<const uint32_t*>(row)[2 * i + 1];
-    } else {
-        x = reinterpret_cast<const uint2*>(row)[i];
-    }
-    return make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xffff0000u), __uint_as_float(x.y << 16),
-                       __uint_as_float(x.y & 0xffff0000u));
-}
-
 // grid (output rows, slices of kNormSliceCols columns), one float4 per thread: the part of RMSNorm that is
 // not a row scalar.  x = residual stream row (after adding the split-K partials of the preceding projection
 // in split order; all splits are requested at once, one memory round trip); writes bf16(x * gain) as the
@@ -63,17 +26,16 @@ __device__ __forceinline__ float4 embed_load4(const EmbedSource& e, int r, int i
 // SPLITS: room for this many partials per row; the loads in flight are registers, and with room for sixteen two blocks
 // fit an SM: the 512 blocks of a 128-row step were 1.7 waves (9 partials: 9.3 us; with room for ten, four blocks per SM,
 // 6.7 to 8 us; layer step of four sequences 162 -> 160 us).
-// EMBED: the first norm of a forward, whose residual stream is the embedding row of each row's token (no partials).
-template <int SPLITS, int BLOCKS, bool EMBED>
+// (The first norm of a forward: first_norm.cu.)
+template <int SPLITS, int BLOCKS>
 __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(float* __restrict__ h, const float* __restrict__ partial,
                                                                      int splits, size_t pstride, const float* __restrict__ gain,
                                                                      __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                      const int32_t* __restrict__ row_map, int d, L2Prefetch pf,
-                                                                     TpWait tw, EmbedSource emb, int compact) {
+                                                                     TpWait tw, int compact) {
     __shared__ float red[32];
-    if (!EMBED) pdl_launch_dependents();
+    pdl_launch_dependents();
     pdl_wait();
-    if (EMBED) pdl_launch_dependents();   // see launch_rmsnorm
     tp_wait_flags(tw);   // tensor parallelism: the partials of every rank have arrived
     l2_prefetch_slice(pf, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
     const int orow = blockIdx.x;
@@ -82,9 +44,8 @@ __global__ void __launch_bounds__(kNormSliceCols / 4, BLOCKS) rmsnorm_kernel(flo
     float ss = 0.f;
     if (i < (d >> 2)) {
         float* hr = h + static_cast<size_t>(row) * d;
-        float4 v = EMBED ? embed_load4(emb, row, i, d) : reinterpret_cast<const float4*>(hr)[i];
-        if (EMBED) reinterpret_cast<float4*>(hr)[i] = v;
-        if (!EMBED && partial) {
+        float4 v = reinterpret_cast<const float4*>(hr)[i];
+        if (partial) {
             const float* p = partial + static_cast<size_t>(compact ? orow : row) * d + 4 * i;
             float4 t[SPLITS];
 #pragma unroll
@@ -116,18 +77,16 @@ constexpr int kNormRowsMaxSplits = 4;
 // SPLITS: most partials per row (0: the projection in front has added to the residual stream itself), a template
 // parameter because the loads in flight are registers: with room for four splits two blocks fit an SM, without any
 // eight do (25568 rows x 4096: 247 us with one partial in the four-split kernel, 90 us with none).
-// EMBED: the first norm of a forward; the residual stream is the embedding row of each row's token.
-template <int SPLITS, bool EMBED>
+template <int SPLITS>
 __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float* __restrict__ h, const float* __restrict__ partial,
                                                                           int splits, size_t pstride,
                                                                           const float* __restrict__ gain,
                                                                           __nv_bfloat16* __restrict__ out, float* __restrict__ ssq,
                                                                           const int32_t* __restrict__ row_map, int rows_out, int d,
-                                                                          TpWait tw, EmbedSource emb, int compact) {
+                                                                          TpWait tw, int compact) {
     __shared__ float red[kNormRows][32];
-    if (!EMBED) pdl_launch_dependents();
+    pdl_launch_dependents();
     pdl_wait();
-    if (EMBED) pdl_launch_dependents();   // see launch_rmsnorm
     if (SPLITS > 0) tp_wait_flags(tw);
     const int i = blockIdx.y * (kNormSliceCols / 4) + threadIdx.x;   // float4 index within the row
     const int orow0 = blockIdx.x * kNormRows;
@@ -142,7 +101,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
 #pragma unroll
     for (int r = 0; r < kNormRows; ++r) {
         if (!in || row[r] < 0) continue;
-        v[r] = EMBED ? embed_load4(emb, row[r], i, d) : reinterpret_cast<const float4*>(h + static_cast<size_t>(row[r]) * d)[i];
+        v[r] = reinterpret_cast<const float4*>(h + static_cast<size_t>(row[r]) * d)[i];
         if (SPLITS > 0) {
             const float* p = partial + static_cast<size_t>(compact ? orow0 + r : row[r]) * d + 4 * i;
 #pragma unroll
@@ -163,7 +122,7 @@ __global__ void __launch_bounds__(kNormSliceCols / 4) rmsnorm_rows_kernel(float*
             for (int u = 0; u < SPLITS; ++u)
                 if (u < splits) { x.x += t[r][u].x; x.y += t[r][u].y; x.z += t[r][u].z; x.w += t[r][u].w; }
         }
-        if (SPLITS > 0 || EMBED) reinterpret_cast<float4*>(h + static_cast<size_t>(row[r]) * d)[i] = x;
+        if (SPLITS > 0) reinterpret_cast<float4*>(h + static_cast<size_t>(row[r]) * d)[i] = x;
         ss[r] = squares4<false>(x);
         reinterpret_cast<uint2*>(out + static_cast<size_t>(orow0 + r) * d)[i] = pack4_bf16(x.x * g.x, x.y * g.y, x.z * g.z, x.w * g.w);
     }
@@ -529,38 +488,27 @@ cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink
     return cudaGetLastError();
 }
 
-template <int SPLITS, bool EMBED>
+template <int SPLITS>
 static cudaError_t launch_norm_rows(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                                     __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, cudaStream_t st,
-                                    const TpWait& tw, const EmbedSource& emb, int compact) {
-    return launch_kernel(rmsnorm_rows_kernel<SPLITS, EMBED>,
+                                    const TpWait& tw, int compact) {
+    return launch_kernel(rmsnorm_rows_kernel<SPLITS>,
                             dim3((rows_out + kNormRows - 1) / kNormRows, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4),
-                            0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, emb, compact);
+                            0, st, h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, tw, compact);
 }
 
-// The first norm (emb.table set) is the first kernel of a forward and follows the kernel that builds the row and tile tables,
-// which is launched without programmatic stream serialization: it starts only when everything enqueued before it (the
-// previous accept) has completed.  The norm lets its successor start only behind its own wait for those tables, so every later
-// kernel of the chain starts when they are complete.  That is what allows the attention kernels to read the tile
-// table and the K/V cache before their own griddepcontrol.wait.  (Started only when the tables were complete, and the accept
-// only when the forward was: layer step 122.5 us against 118.5, tiny model 87.2 against 84.)
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw, const EmbedSource& emb, bool compact) {
+                           cudaStream_t st, const TpWait& tw, bool compact) {
     if (splits > kMaxKSplits) return cudaErrorInvalidValue;
-    const bool first = emb.table != nullptr;
-    if (first && (partial || row_map)) return cudaErrorInvalidValue;
     if (rows_out >= 256 && (!partial || splits <= kNormRowsMaxSplits)) {
-        if (first) return launch_norm_rows<0, true>(h, nullptr, 0, 0, gain, out, ssq, nullptr, rows_out, d, st, tw, emb, 0);
-        if (!partial) return launch_norm_rows<0, false>(h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
-        if (splits == 1)
-            return launch_norm_rows<1, false>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, emb, compact);
-        return launch_norm_rows<kNormRowsMaxSplits, false>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st,
-                                                           tw, emb, compact);
+        if (!partial) return launch_norm_rows<0>(h, nullptr, 0, 0, gain, out, ssq, row_map, rows_out, d, st, tw, compact);
+        if (splits == 1) return launch_norm_rows<1>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, compact);
+        return launch_norm_rows<kNormRowsMaxSplits>(h, partial, splits, pstride, gain, out, ssq, row_map, rows_out, d, st, tw, compact);
     }
-    return launch_kernel(first ? rmsnorm_kernel<1, 4, true> : splits <= 4 ? rmsnorm_kernel<4, 4, false> :
-                            splits <= 10 ? rmsnorm_kernel<10, 4, false> : rmsnorm_kernel<kMaxKSplits, 2, false>, dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0,
-                            st, h, partial, splits, pstride, gain, out, ssq, row_map, d, pf, tw, emb, compact ? 1 : 0);
+    return launch_kernel(splits <= 4 ? rmsnorm_kernel<4, 4> : splits <= 10 ? rmsnorm_kernel<10, 4> : rmsnorm_kernel<kMaxKSplits, 2>,
+                         dim3(rows_out, (d + kNormSliceCols - 1) / kNormSliceCols), dim3(kNormSliceCols / 4), 0, st, h, partial, splits,
+                         pstride, gain, out, ssq, row_map, d, pf, tw, compact ? 1 : 0);
 }
 
 cudaError_t launch_gather_rows(const __nv_bfloat16* src, const float* ssq, int slots, __nv_bfloat16* dst, float* dst_ssq,

@@ -582,10 +582,10 @@ int32_t ensure_ptable(odb_session* s, int M) {
     return ODB_OK;
 }
 
-// One forward over the M rows of the row table already built on the device.
+// One forward over the M rows of `first`, whose tables its first kernel writes.
 // one_seq: the rows are one sequence's, those with logits the last n_lm of them.
-int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, int n_step_tiles = 0, int n_big_tiles = 0,
-                cudaStream_t st = nullptr, bool one_seq = false) {
+int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_tiles, bool write_cache, int n_step_tiles = 0,
+                int n_big_tiles = 0, cudaStream_t st = nullptr, bool one_seq = false) {
     const odb_model* m = s->m;
     const odb_config& c = m->cfg;
     const Layout& L = s->L;
@@ -720,6 +720,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         static const bool ptiming = getenv("ODB_PERSISTENT_TIMING") && getenv("ODB_PERSISTENT_TIMING")[0] == '1';
         pa.timing = (ptiming && c.with_lm_head && !s->dump_logits) ? s->at<unsigned long long>(L.logits) : nullptr;
         ODB_CUDA(step_persistent_configure(pa));
+        ODB_LAUNCH(ODB_KIND_CONTROL, launch_build_step_rows(s->cb, c.max_batch, c.mask_id, st));
         ODB_LAUNCH(ODB_KIND_GEMM, launch_step_persistent(pa, st));
         if (pa.with_lm) {
             ODB_LAUNCH(ODB_KIND_CONFIDENCE, launch_confidence_final(pa.conf_part, (c.vocab + 127) / 128, M, s->at<float>(L.conf),
@@ -766,10 +767,10 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     // odb_debug_read returns holds the last attention block in every one (without it 1539 and 620 us).
     bool tail = false;
     for (int l = 0; l < c.n_layers; ++l) {
-        EmbedSource emb;
-        if (l == 0) { emb.table = m->embed; emb.row_tok = s->cb.row_tok; emb.halves = embed_wide(m) ? 0 : 1; }
-        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d,
-                                                        hint_of(m->p_qkv[l], qkv_bytes, 0), st, res_wait, emb));
+        const L2Prefetch qkv_hint = hint_of(m->p_qkv[l], qkv_bytes, 0);
+        if (l == 0) ODB_FWD(ODB_KIND_ELEMENTWISE, launch_first_norm(h, m->norm1[l], a, inv, M, d, first, qkv_hint, st));
+        else ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d, qkv_hint, st,
+                                                             res_wait));
         int sp = plan_splits(M, 3 * da, d, false);
         QkvRopeArgs qa;
         qa.partial = partial; qa.splits = sp; qa.pstride = static_cast<size_t>(M) * 3 * da;
@@ -951,7 +952,7 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
         ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, tail ? res + static_cast<size_t>(r0) * d : res, res_splits, res_stride,
                                                         m->final_norm, a, inv, s->cb.lm_rows + r0, rows, d,
                                                         hint_of(m->p_lm, packed_weight_bytes(lm_rows_local, d), 0), st, res_wait,
-                                                        EmbedSource(), tail));
+                                                        tail));
         if (s->dump_logits) {
             int sp = 1;
             ODB_FWD(ODB_KIND_GEMM, gemm(m->w_lm, x, logits, rows, c.vocab, d, sp, scale));
@@ -989,6 +990,16 @@ int32_t forward(odb_session* s, int M, int n_lm, int n_tiles, bool write_cache, 
     return ODB_OK;
 }
 
+FirstRows first_rows(const odb_session* s) {
+    FirstRows f;
+    f.cb = s->cb;
+    f.table = s->m->embed;
+    f.halves = embed_wide(s->m) ? 0 : 1;
+    f.batch = s->m->cfg.max_batch;
+    f.mask_id = s->m->cfg.mask_id;
+    return f;
+}
+
 // Work items of the multi-copy step attention for a step of this shape (0: the per-copy kernel is used)
 int step_items(const odb_session* s, const StepShape& sh) {
     return (!sh.multi || static_cast<size_t>(2) * sh.rows > s->L.attn_rows) ? 0 : sh.step_tiles;
@@ -1020,9 +1031,10 @@ int32_t odb_refresh_prefill(odb_session* s, const odb_decode_params* p, const in
     }
     if (M == 0) return ODB_ERR_STATE;
     if (tp_on && static_cast<size_t>(n_lm) > s->L.lm_chunk) return ODB_ERR_SHAPE;   // one exchange of statistics per forward
-    if (!continuing)
-        ODB_LAUNCH(ODB_KIND_CONTROL, launch_build_refresh_rows(s->cb, c.max_batch, block_index, p->block_len, s->st));
-    int32_t rc = forward(s, M, c.with_lm_head ? n_lm : 0, n_tiles, true, 0, n_big, nullptr, n_seq == 1);
+    FirstRows first = first_rows(s);
+    first.block_len = p->block_len;
+    for (int i = 0; i < c.max_batch; ++i) first.block_index[i] = block_index[i];
+    int32_t rc = forward(s, first, M, c.with_lm_head ? n_lm : 0, n_tiles, true, 0, n_big, nullptr, n_seq == 1);
     if (rc != ODB_OK) return rc;
     s->last_rows = M;
     s->last_lm_rows = n_lm;
@@ -1047,8 +1059,9 @@ int32_t odb_block_decode_step(odb_session* s, const odb_decode_params* p) {
         if (trc != ODB_OK) return trc;
     }
     if (tp_on && static_cast<size_t>(M) > s->L.lm_chunk) return ODB_ERR_SHAPE;
-    if (!continuing) ODB_LAUNCH(ODB_KIND_CONTROL, launch_build_step_rows(s->cb, c.max_batch, c.mask_id, s->st));
-    int32_t rc = forward(s, M, c.with_lm_head ? M : 0, sh.tiles, false, step_items(s, sh));
+    FirstRows first = first_rows(s);
+    first.step = 1;
+    int32_t rc = forward(s, first, M, c.with_lm_head ? M : 0, sh.tiles, false, step_items(s, sh));
     if (rc != ODB_OK) return rc;
     s->last_rows = M;
     s->last_lm_rows = M;
@@ -1133,10 +1146,11 @@ int32_t odb_decode_block_resident(odb_session* s, const odb_decode_params* p, in
         lc.host_iters = s->pinned_iters;
         long long before[ODB_PROFILE_KINDS];
         memcpy(before, s->launches, sizeof(before));
-        // the body: row table, forward, accept.  Whatever a launch returns, the recording is closed before leaving.
+        // the body: forward, accept.  Whatever a launch returns, the recording is closed before leaving.
         int32_t rc = [&]() -> int32_t {
-            ODB_LAUNCH(ODB_KIND_CONTROL, launch_build_step_rows(s->cb, c.max_batch, c.mask_id, s->record_st));
-            int32_t frc = forward(s, sh.rows, c.with_lm_head ? sh.rows : 0, sh.tiles, false, step_items(s, sh), 0, s->record_st);
+            FirstRows first = first_rows(s);
+            first.step = 1;
+            int32_t frc = forward(s, first, sh.rows, c.with_lm_head ? sh.rows : 0, sh.tiles, false, step_items(s, sh), 0, s->record_st);
             if (frc != ODB_OK) return frc;
             ODB_LAUNCH(ODB_KIND_CONTROL, launch_accept_loop(s->cb, c.max_batch, *p, c.mask_id, c.eos_id,
                                                             c.with_lm_head ? 0 : 1, lc, s->record_st));

@@ -34,7 +34,7 @@ cudaError_t set_smem_limit_once(std::atomic<unsigned long long>& done, Kernel ke
 // needs them, so prologues, tensor-map fetches and weight prefetches overlap the predecessor's
 // tail.  Every such kernel executes pdl_wait() before it exits, which keeps the completion order
 // of the chain transitive.  The successor is let go at entry, but for
-//   - the first norm: behind its wait for the kernel that builds the row and tile tables.  That
+//   - the first kernel: its blocks that write the row and tile tables behind those stores.  That
 //     alone makes the tables complete before any later kernel of the chain starts, and lets the
 //     attention read its work items (and a step the K/V cache) before its own wait;
 //   - kernels that allocate TMEM for CTA pairs, and the tensor-core attention: behind the allocation;
@@ -356,12 +356,6 @@ cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stri
 cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink, int grid, cudaStream_t st);
 // bulk-copy ring probe; *streamed = the bytes one launch reads (whole chunks per CTA); `status` is a device word
 cudaError_t launch_bulk_read_stream(const void* src, size_t bytes, int grid, int* status, size_t* streamed, cudaStream_t st);
-// table non-null: the residual stream of row r starts as the embedding of token row_tok[r] (first norm of a forward)
-struct EmbedSource {
-    const __nv_bfloat16* table = nullptr;
-    const int32_t* row_tok = nullptr;
-    int halves = 0;                     // the table starts on a 4-byte boundary only (a tensor inside a mapped file)
-};
 // The part of RMSNorm that is not a row scalar, for rows r = map ? map[i] : i of the residual stream:
 // h[r] += sum_s partial[s][r] (if partial; split order), out[i] = bf16(h[r] * gain) is the projection's
 // operand, ssq[i][t] = sum of h[r]^2 over the t-th slice of kNormSliceCols columns; the projection's consumer
@@ -369,8 +363,7 @@ struct EmbedSource {
 // product).  splits <= kMaxKSplits.  compact: partial[s] holds the rows of the map only, in its order.
 cudaError_t launch_rmsnorm(float* h, const float* partial, int splits, size_t pstride, const float* gain,
                            __nv_bfloat16* out, float* ssq, const int32_t* row_map, int rows_out, int d, L2Prefetch pf,
-                           cudaStream_t st, const TpWait& tw = TpWait(), const EmbedSource& emb = EmbedSource(),
-                           bool compact = false);
+                           cudaStream_t st, const TpWait& tw = TpWait(), bool compact = false);
 // dst[i] = src[map[i]] for n rows of d bf16 (d % 8 == 0, 16-byte aligned rows), and likewise their `slots` sums of squares
 cudaError_t launch_gather_rows(const __nv_bfloat16* src, const float* ssq, int slots, __nv_bfloat16* dst, float* dst_ssq,
                                const int32_t* map, int n, int d, cudaStream_t st);
@@ -500,9 +493,23 @@ struct ControlBuffers {
     SeqState* host_state; odb_result* host_results; int* host_status;
     const int* status;        // device status word
 };
-// block_index[seq] < 0: the sequence takes no part in this refresh
-cudaError_t launch_build_refresh_rows(const ControlBuffers& c, int batch, const int32_t* block_index, int block_len,
-                                      cudaStream_t st);
+// Where the rows of a forward come from: a block step of every active sequence with masked positions, or a refresh of the active
+// ones whose block_index is not negative.
+struct FirstRows {
+    ControlBuffers cb;
+    const __nv_bfloat16* table = nullptr;   // embedding
+    int halves = 0;                         // the table starts on a 4-byte boundary only (a tensor inside a mapped file)
+    int batch = 0;
+    int step = 0;
+    int mask_id = 0;                        // step
+    int block_len = 0;                      // refresh
+    int32_t block_index[64] = {};
+};
+// The first kernel of a forward of M rows: row and tile tables, h[r] = embedding of row r's token, and the first norm of them
+// (out, ssq as launch_rmsnorm's).
+cudaError_t launch_first_norm(float* h, const float* gain, __nv_bfloat16* out, float* ssq, int M, int d, const FirstRows& f, L2Prefetch pf,
+                              cudaStream_t st);
+// the tables of a step alone (for the persistent step kernel, which reads the embedding itself)
 cudaError_t launch_build_step_rows(const ControlBuffers& c, int batch, int mask_id, cudaStream_t st);
 
 // Number of StepTiles of a sequence's step: copies packed in order into items of <= 8 slabs of 16 rows.
