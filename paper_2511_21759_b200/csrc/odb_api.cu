@@ -615,6 +615,10 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
     int* status = s->at<int>(L.status);
     const size_t nmax = 3 * static_cast<size_t>(d) > 2 * static_cast<size_t>(F) ? 3 * static_cast<size_t>(d)
                                                                                 : 2 * static_cast<size_t>(F);
+    // A forward that ends in the LM head keeps its sums in the order they have always had: its greedy tokens are whole results, and
+    // another order moves those whose two best logits all but tie (5 % of them in a request over random weights, at the same
+    // distance from 64 bits).  One that ends in the residual stream takes whichever kernel is the fastest.
+    const bool same_order = c.with_lm_head || R > 1;
     // K splits of a projection with fp32 partial output; `exchanged`: the partials of all R ranks must fit a receive
     // slot and the consumer's limit
     auto plan_splits = [&](int rows, int N, int K, bool exchanged) {
@@ -820,10 +824,10 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
             // vs 1.12 ms per step at batch 1; in one pass it wins there too: 1.00 vs 1.13 ms, step 4.82 -> 4.63 ms)
             // Head dim 64, two layers of d 1024, us per step, mma.sync / tensor cores: 16 items 133.4 / 129.8 and 146.8 / 145.7, 32 items
             // 149.7 / 147.3, 64 items 172 / 161 and 196 / 179, 128 items 214 / 187, 512 items of 64-row blocks 558 / 373; d 256, 4 items
-            // 112 / 109.  Below 32 items the two are as good as equal, and those steps keep the sums that they had.
+            // 112 / 109.  Below 32 items the two are as good as equal.
             static const int tc_step_env = getenv("ODB_ATTN_TC_STEP_MIN") ? atoi(getenv("ODB_ATTN_TC_STEP_MIN")) : 0;
             const int tc_step_min = tc_step_env > 0 ? tc_step_env : hd == 128 ? 1 : 32;
-            if (tc_attention && n_step_tiles * H >= tc_step_min) {
+            if (tc_attention && (hd == 128 || !same_order) && n_step_tiles * H >= tc_step_min) {
                 const size_t cache_rows = static_cast<size_t>(c.max_batch) * c.n_layers * 2 * H * c.max_seq;
                 // with a work item for every CTA slot there is nothing to gain from key splits: one CTA per item takes
                 // the cached and the fresh keys and writes the final output (no partials, no merge kernel)
@@ -835,7 +839,7 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
                 ODB_FWD(ODB_KIND_ATTENTION, launch_step_attention(sa, st));
                 if (seg_on()) ++s->launches[ODB_KIND_ATTENTION];
             }
-        } else if (write_cache && tc_attention && n_big_tiles * H >= (hd == 128 ? 1 : 74)) {
+        } else if (write_cache && tc_attention && (hd == 128 || !same_order) && n_big_tiles * H >= (hd == 128 ? 1 : 74)) {
             // refresh: 128-row work items on the tcgen05 tensor cores, no key split.  Head dim 64, us per refresh of two layers, mma.sync
             // (64-row items, keys split to fill the chip) / tensor cores: d 1024, 128 items 226 / 195, 96 items 203 / 188, 64 items 163 / 158, 32
             // items 151.5 / 149.2; d 256, 512 items 426 / 327, 64 items 181 / 171, 16 items 116 / 121.  With fewer items than every

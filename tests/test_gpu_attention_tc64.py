@@ -1,5 +1,6 @@
 """The tensor-core attention with head dim 64, where launches have enough work items for it: refreshes around the edges of the
-128-row items and 64-key tiles, steps of several copies with and without key splits, in both row layouts."""
+128-row items and 64-key tiles, steps of several copies with and without key splits, in both row layouts.  (Models without LM head: those with one stay on
+mma.sync.)"""
 import dataclasses
 import math
 
@@ -39,7 +40,7 @@ def check(o, q, keys, vals, visible=None):
 ])
 def test_refresh(lens):
     E = engine()
-    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=len(lens), max_seq=max(p + n for p, n in lens), max_block=16, max_copies=1)
+    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=len(lens), max_seq=max(p + n for p, n in lens), max_block=16, max_copies=1, with_lm_head=False)
     sess = E.Session(gm, poison=True)
     for i, (p, n) in enumerate(lens):
         sess.set_sequence(i, synth.sequence(5, i, p, n, SHAPE), p)
@@ -66,7 +67,7 @@ def test_refresh(lens):
 def test_step_with_copies(copies, decoded, block, batch):
     E = engine()
     lens = [(101 + 37 * i, 200 - 19 * i) for i in range(batch)]
-    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=batch, max_seq=max(p + n for p, n in lens), max_block=block, max_copies=8)
+    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=batch, max_seq=max(p + n for p, n in lens), max_block=block, max_copies=8, with_lm_head=False)
     sess = E.Session(gm, poison=True)
     for i, (p, n) in enumerate(lens):
         x = synth.sequence(5, i, p, n, SHAPE)
