@@ -514,6 +514,12 @@ int sm_pairs() {
 // 150 / 143.5, 500 rows 153 / 147, at d 4096 160 rows 180 / 174; O and down of 4096 rows at d 4096 (3.5 rounds) 106 / 107, 292 / 296.
 constexpr int kHalvesRounds = 2;
 
+// items handed out as single weight tiles, of `items` whole ones: the last round's, if they still are one round as halves
+int half_items(long long items, int pairs) {
+    const int left = static_cast<int>(items % pairs);
+    return 2 * left <= pairs && items <= static_cast<long long>(kHalvesRounds) * pairs ? left : 0;
+}
+
 template <int EPI>
 cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     CUtensorMap tmx;
@@ -541,11 +547,10 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
     a.w_hint = a.m_tiles > 1 ? kEvictNormal : kEvictFirst;
     const long long items = static_cast<long long>(a.n_pairs) * a.m_tiles * g.splits;
     if (items > (1ll << 30)) return cudaErrorInvalidValue;
-    // Single weight tiles for the last round if they still are one round.
-    const int pairs = sm_pairs(), left = static_cast<int>(items % pairs);
-    const bool halves = EPI != ROWS_CONF && left > 0 && 2 * left <= pairs && items <= static_cast<long long>(kHalvesRounds) * pairs;
-    a.whole = static_cast<int>(items) - (halves ? left : 0);
-    a.n_items = static_cast<int>(items) + (halves ? left : 0);
+    const int pairs = sm_pairs(), left = EPI == ROWS_CONF ? 0 : half_items(items, pairs);
+    const bool halves = left > 0;
+    a.whole = static_cast<int>(items) - left;
+    a.n_items = static_cast<int>(items) + left;
     constexpr int smem = kRowsStages * kRowsStageBytes + 8 * kPatchBytes + sizeof(RowsShared) + 1024;
     static_assert(smem <= 227 * 1024, "one CTA per SM");
     void (*kernel)(WeightMaps, CUtensorMap, RowsArgs, PeerOut) = gemm_rows_kernel<EPI, false>;
@@ -573,6 +578,29 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
 }
 
 }  // namespace
+
+// K splits of the O and down projections of a forward over more than 128 rows without LM head: the cheapest by two terms, the rounds of the CTA
+// pairs (0.45 us per k-block of 256 x 256; a last round of single weight tiles counts 0.68) and the sums themselves (1 us per split
+// and million of them: written, and read by the norm behind; an unsplit product's go into the residual stream, which is
+// as much).  At least eight k-blocks each.  Fitted to and checked against 60 sweeps of one projection's splits, d 1024, 2048 and
+// 4096 and 160 to 3600 rows: on average 0.12 % of the refresh behind the best split, 1.3 % at worst.  Against as many splits as
+// make 296 tiles, the rule of gemm_pick_splits (us per refresh, before / now; one layer at d 4096, two below): d 4096 900 rows, O 2 -> 1
+// splits 449 / 437, down 2 -> 1 449 / 437; 1200 rows, down 1 -> 4 601 / 573 (three 569); d 2048 512
+// rows, down 7 -> 4 240 / 232, 2000 rows, O 2 -> 1 528 / 506; d 1024 3600 rows, down 2 -> 1 369 / 353.
+int gemm_rows_splits(int M, int N, int K) {
+    const int pairs = sm_pairs(), nkb = (K + kBK - 1) / kBK;
+    const long long tiles = static_cast<long long>((N + 2 * kBM - 1) / (2 * kBM)) * ((M + 2 * kBM - 1) / (2 * kBM));
+    int best = 1;
+    double least = 0.;
+    for (int sp = 1; sp <= kMaxKSplits && (sp == 1 || 8 * sp <= nkb); ++sp) {
+        if (gemm_whole_splits(sp, nkb) != sp) continue;
+        const long long items = tiles * sp;
+        const double rounds = half_items(items, pairs) ? items / pairs + 0.68 : static_cast<double>((items + pairs - 1) / pairs);
+        const double cost = rounds * 0.45 * ((nkb + sp - 1) / sp) + 1e-6 * sp * M * N;
+        if (sp == 1 || cost < least) { best = sp; least = cost; }
+    }
+    return best;
+}
 
 // More than 128 rows and an even number of weight tiles.  Inside a model every row starts on a 16-byte boundary (d and F
 // are multiples of 16, heads have 64 or 128 dims); the GEMM entry points take any N.

@@ -617,12 +617,12 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
                                                                                 : 2 * static_cast<size_t>(F);
     // A forward that ends in the LM head keeps its sums in the order they have always had: its greedy tokens are whole results, and
     // another order moves those whose two best logits all but tie (5 % of them in a request over random weights, at the same
-    // distance from 64 bits).  One that ends in the residual stream takes whichever kernel is the fastest.
+    // distance from 64 bits).  One that ends in the residual stream takes whichever kernel and split is the fastest.
     const bool same_order = c.with_lm_head || R > 1;
     // K splits of a projection with fp32 partial output; `exchanged`: the partials of all R ranks must fit a receive
     // slot and the consumer's limit
     auto plan_splits = [&](int rows, int N, int K, bool exchanged) {
-        int sp = gemm_pick_splits(rows, N, K);
+        int sp = !same_order && gemm_rows_usable(rows, N) ? gemm_rows_splits(rows, N, K) : gemm_pick_splits(rows, N, K);
         size_t cap = L.partial_rows * nmax / (static_cast<size_t>(rows) * N);
         if (exchanged) {   // R blocks of `sp` partials in a receive slot (sized for at least one partial per rank)
             cap = L.tp_recv_slot / sizeof(float) / (static_cast<size_t>(rows) * N * R);
@@ -775,7 +775,10 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
         if (l == 0) ODB_FWD(ODB_KIND_ELEMENTWISE, launch_first_norm(h, m->norm1[l], a, inv, M, d, first, qkv_hint, st));
         else ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d, qkv_hint, st,
                                                              res_wait));
-        int sp = plan_splits(M, 3 * da, d, false);
+        // Many rows: not split, whatever the pairs left idle; split sums cost the RoPE kernel and fp32 rows in memory.  us per refresh,
+        // two splits / none, d 2048, two layers: 300 rows 245 / 232, 512 240 / 231, 768 277 / 258, d 1024 2000 rows 270 / 265;
+        // d 4096, one layer, 300 rows 248 / 246.
+        int sp = !same_order && gemm_rows_usable(M, 3 * da) ? 1 : plan_splits(M, 3 * da, d, false);
         QkvRopeArgs qa;
         qa.partial = partial; qa.splits = sp; qa.pstride = static_cast<size_t>(M) * 3 * da;
         qa.scale = inv_scale;

@@ -329,6 +329,7 @@ struct GemmArgs {
     int* status;           // device status word
 };
 int gemm_pick_splits(int M, int N, int K);   // 1 .. kMaxKSplits
+int gemm_rows_splits(int M, int N, int K);   // the same for a projection of a forward that gemm_rows_usable holds for
 constexpr int kMaxKSplits = 16;              // partial sums of one element that the RMSNorm kernels add up at most
 // the largest number of K splits <= splits that leaves none of them empty: ceil(nkb / splits) * (splits - 1) < nkb
 int gemm_whole_splits(int splits, int nkb);
