@@ -312,13 +312,13 @@ gemm_rows_kernel(const __grid_constant__ WeightMaps maps, const __grid_constant_
                     tmem_ld16(tmem + c, g);
                     tmem_ld16(tmem + 64 + c, u);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    float gate[16], up[16], x[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) { gate[j] = __uint_as_float(g[j]) * sc; up[j] = __uint_as_float(u[j]) * sc; }
+                    silu_product(gate, up, x);
                     uint32_t out[8];
 #pragma unroll
-                    for (int j = 0; j < 16; j += 2) {
-                        const float g0 = __uint_as_float(g[j]) * sc, g1 = __uint_as_float(g[j + 1]) * sc;
-                        const float u0 = __uint_as_float(u[j]) * sc, u1 = __uint_as_float(u[j + 1]) * sc;
-                        out[j / 2] = pack2(g0 / (1.0f + expf(-g0)) * u0, g1 / (1.0f + expf(-g1)) * u1);
-                    }
+                    for (int j = 0; j < 8; ++j) out[j] = pack2(x[2 * j], x[2 * j + 1]);
                     put_chunk(patch, lane, c / 8, out[0], out[1], out[2], out[3]);
                     put_chunk(patch, lane, c / 8 + 1, out[4], out[5], out[6], out[7]);
                 }

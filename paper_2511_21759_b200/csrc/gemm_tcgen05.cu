@@ -344,15 +344,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                     __syncwarp();
                     tmem_ld16(tm_lane + static_cast<uint32_t>(r0 + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    float gate[16], up[16], x[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const float sc = rs.ssq ? sh->scale[r0 + c + j] : 1.0f;
+                        const float own = __uint_as_float(v[j]) * sc, other = take[c + j] * sc;
+                        gate[j] = is_gate ? own : other;
+                        up[j] = is_gate ? other : own;
+                    }
+                    silu_product(gate, up, x);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int m = m0 + r0 + c + j;
-                        const float sc = rs.ssq ? sh->scale[r0 + c + j] : 1.0f;
-                        if (m < M && f < N) {
-                            const float own = __uint_as_float(v[j]) * sc, other = take[c + j] * sc;
-                            const float gate = is_gate ? own : other, up = is_gate ? other : own;
-                            act_out[static_cast<size_t>(m) * N + f] = __float2bfloat16_rn(gate / (1.0f + expf(-gate)) * up);
-                        }
+                        if (m < M && f < N) act_out[static_cast<size_t>(m) * N + f] = __float2bfloat16_rn(x[j]);
                     }
                 }
             }
