@@ -142,6 +142,21 @@ __device__ __forceinline__ void tmem_read32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// two pieces of 16 columns; the wait is part of the statement, so that no use of the values can come in front of it
+__device__ __forceinline__ void tmem_read16x2(uint32_t t0, uint32_t t1, uint32_t (&a)[16], uint32_t (&b)[16]) {
+    __syncwarp();
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]),
+          "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]),
+          "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]),
+          "=r"(b[14]), "=r"(b[15])
+        : "r"(t0), "r"(t1)
+        : "memory");
+}
+
 __device__ __forceinline__ uint32_t leader_address(uint64_t* bar) {   // shared::cluster address of the leader's copy of `bar`
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(bar)));
@@ -298,8 +313,19 @@ gemm_rows_kernel(const __grid_constant__ WeightMaps maps, const __grid_constant_
             const uint32_t tmem = tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * kRowsN + (w.half ? 0 : t * kBM));
             const float sc = m < a.M ? row_scale_of(a.rs, m) : 1.0f;
             int pos = 0, seq = 0;
+            // QKV: quarters of the tile's columns that are this warp's, and the (cos, sin) of the first
+            const int first_quarter = w.half ? 2 * t : 0, last_quarter = w.half ? 2 * t + 2 : 4;
+            float2 next_cs[16];
+            auto load_cs = [&](int u) {
+                constexpr int HD = EPI == ROWS_QKV128 ? 128 : 64;
+                const int c = HD == 128 ? u * 16 : (u & 1) * 16;
+                if (tile * (kBM / HD) + (HD == 128 ? 0 : u >> 1) >= 2 * a.qkv.H) return;   // v is not rotated
+#pragma unroll
+                for (int j = 0; j < 16; ++j) next_cs[j] = a.qkv.rope_t[static_cast<size_t>(c + j) * a.qkv.max_seq + pos];
+            };
             if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
                 if (m < a.M) { pos = a.qkv.row_pos[m]; seq = a.qkv.row_seq[m]; }
+                load_cs(first_quarter);
             }
             if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[b], (n_done >> 1) & 1, cta_abort, a.status))) break;
             tc_fence_after();
@@ -378,51 +404,46 @@ gemm_rows_kernel(const __grid_constant__ WeightMaps maps, const __grid_constant_
             } else if constexpr (EPI == ROWS_QKV64 || EPI == ROWS_QKV128) {
                 // QKV projection: a head's q, k or v of this row is the thread's own, rotate-half partners included.
                 // The RMSNorm scalar, RoPE (q and k), bf16 rows and - in a refresh - the K/V cache.  The (cos, sin) table
-                // is read transposed ([pair][position]): the lanes' positions are neighbours, mostly.  A piece is 32
-                // dims of a head's lower half and the 32 they rotate with.
+                // is read transposed ([pair][position]): the lanes' positions are neighbours, mostly.  A quarter is 16
+                // dims of a head's lower half and the 16 they rotate with, two of them a piece; the table's entries of the
+                // next quarter are asked for in front of the work on this one.
                 constexpr int HD = EPI == ROWS_QKV128 ? 128 : 64, kHalf = HD / 2;
                 const QkvRopeArgs& e = a.qkv;
                 const long long crow = (static_cast<long long>(seq) * e.n_layers + e.layer) * 2 * e.H * e.max_seq + pos;
-                const float2* rope = e.rope_t + pos;
 #pragma unroll 1
-                for (int piece = 0; piece < kBM / 64; ++piece) {
-                    if (w.half && piece != t) continue;
-                    const int grp = HD == 128 ? 0 : piece, c0 = HD == 128 ? piece * 32 : 0;
+                for (int u = first_quarter; u < last_quarter; ++u) {
+                    const int grp = HD == 128 ? 0 : u >> 1, c = HD == 128 ? u * 16 : (u & 1) * 16;
                     const int g = tile * (kBM / HD) + grp;             // head of [Wq; Wk; Wv]
                     if (g >= 3 * e.H) break;
                     const int sec = g / e.H, head = g - sec * e.H;
-                    __syncwarp();                                      // the previous piece has been taken
-#pragma unroll 1
-                    for (int cc = 0; cc < 32; cc += 16) {
-                        const int c = c0 + cc;
-                        uint32_t lo[16], hi[16];
-                        tmem_ld16(tmem + grp * HD + c, lo);
-                        tmem_ld16(tmem + grp * HD + kHalf + c, hi);
-                        float2 cs[16];
+                    uint32_t lo[16], hi[16];
+                    if (!(u & 1)) __syncwarp();                        // the previous piece has been taken
+                    tmem_read16x2(tmem + grp * HD + c, tmem + grp * HD + kHalf + c, lo, hi);
+                    float2 cs[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) cs[j] = next_cs[j];
+                    if (u + 1 < last_quarter) load_cs(u + 1);
+                    uint32_t pl[8], ph[8];
+#pragma unroll
+                    for (int j = 0; j < 16; j += 2) {
+                        float x0 = __uint_as_float(lo[j]) * sc, y0 = __uint_as_float(hi[j]) * sc;
+                        float x1 = __uint_as_float(lo[j + 1]) * sc, y1 = __uint_as_float(hi[j + 1]) * sc;
                         if (sec < 2) {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) cs[j] = rope[static_cast<size_t>(c + j) * e.max_seq];
+                            const float a0 = x0 * cs[j].x - y0 * cs[j].y, b0 = y0 * cs[j].x + x0 * cs[j].y;
+                            const float a1 = x1 * cs[j + 1].x - y1 * cs[j + 1].y, b1 = y1 * cs[j + 1].x + x1 * cs[j + 1].y;
+                            x0 = a0; y0 = b0; x1 = a1; y1 = b1;
                         }
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        uint32_t pl[8], ph[8];
-#pragma unroll
-                        for (int j = 0; j < 16; j += 2) {
-                            float x0 = __uint_as_float(lo[j]) * sc, y0 = __uint_as_float(hi[j]) * sc;
-                            float x1 = __uint_as_float(lo[j + 1]) * sc, y1 = __uint_as_float(hi[j + 1]) * sc;
-                            if (sec < 2) {
-                                const float a0 = x0 * cs[j].x - y0 * cs[j].y, b0 = y0 * cs[j].x + x0 * cs[j].y;
-                                const float a1 = x1 * cs[j + 1].x - y1 * cs[j + 1].y, b1 = y1 * cs[j + 1].x + x1 * cs[j + 1].y;
-                                x0 = a0; y0 = b0; x1 = a1; y1 = b1;
-                            }
-                            pl[j / 2] = pack2(x0, x1);
-                            ph[j / 2] = pack2(y0, y1);
-                        }
-                        put_chunk(patch, lane, cc / 8, pl[0], pl[1], pl[2], pl[3]);
-                        put_chunk(patch, lane, cc / 8 + 1, pl[4], pl[5], pl[6], pl[7]);
-                        put_chunk(patch, lane, cc / 8 + 4, ph[0], ph[1], ph[2], ph[3]);
-                        put_chunk(patch, lane, cc / 8 + 5, ph[4], ph[5], ph[6], ph[7]);
+                        pl[j / 2] = pack2(x0, x1);
+                        ph[j / 2] = pack2(y0, y1);
                     }
+                    const int ch = (u & 1) * 2;
+                    put_chunk(patch, lane, ch, pl[0], pl[1], pl[2], pl[3]);
+                    put_chunk(patch, lane, ch + 1, pl[4], pl[5], pl[6], pl[7]);
+                    put_chunk(patch, lane, ch + 4, ph[0], ph[1], ph[2], ph[3]);
+                    put_chunk(patch, lane, ch + 5, ph[4], ph[5], ph[6], ph[7]);
+                    if (!(u & 1)) continue;
                     __syncwarp();
+                    const int c0 = c - 16;
                     __nv_bfloat16* fresh = (sec == 0 ? e.q : sec == 1 ? e.k : e.v) + head * HD;
                     const long long chead = static_cast<long long>((sec - 1) * e.H + head) * e.max_seq;
                     take_rows(patch, lane, [&](int r, int ch, const uint4& x) {
