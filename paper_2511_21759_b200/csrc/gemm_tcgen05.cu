@@ -39,7 +39,7 @@ struct alignas(8) GemmShared {
     float scale[128];      // RowScale of the tile's activation rows
 };
 
-// BN: activation rows per tile (MMA N): 32, 64 or 128.
+// BN: activation rows per tile (MMA N): 32, 64 or 128, or as many less as a launch of a single row tile has (x_rows).
 // SWIGLU: the weight is the gate/up matrix packed with gate and up rows interleaved in groups of
 // 64 (tile t = gate rows [64t, 64t+64) then up rows [64t, 64t+64)); the epilogue pairs TMEM lane r
 // (gate) with lane r + 64 (up) through shared memory and stores bf16(silu(gate) * up) to
@@ -61,23 +61,25 @@ template <int BN, int EPI>
 __global__ void __launch_bounds__(gemm_threads(BN, EPI), 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
             float* __restrict__ partial, __nv_bfloat16* __restrict__ act_out, RowScale rs,
-            ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int w_stages, int x_stages,
+            ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int x_rows, int w_stages, int x_stages,
             int l2_prefetch, int* status, const __grid_constant__ PeerOut po) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr uint32_t kABytes = kBM * kBK * 2;
-    constexpr uint32_t kBBytes = BN * kBK * 2;
-    constexpr uint32_t kStageBytes = kABytes + kBBytes;
+    // x_rows <= BN: activation rows that are loaded and multiplied; the accumulator's columns behind them are never stored
+    const uint32_t x_bytes = static_cast<uint32_t>(x_rows) * (kBK * 2);
+    const uint32_t stage_bytes = kABytes + x_bytes;
+    constexpr uint32_t kLeastStageBytes = kABytes + (BN == 32 ? 16 : BN / 2 + 16) * kBK * 2;
     constexpr uint32_t kTmemCols = BN;
     // the epilogues exchange values through the stage ring, which holds at least kMinStages stages
     constexpr int kGroups = epilogue_groups(BN, EPI), kGroupRows = BN / kGroups;
     constexpr uint32_t kExchangeBytes = EPI == EPI_SWIGLU ? 2 * 64 * (kGroupRows / 2 + 1) * 4 : EPI == EPI_CONF ? 32 * 129 * 4 : 0;
-    static_assert(kGroups * kExchangeBytes <= kMinStages * kStageBytes, "the exchange buffer must end inside the ring");
+    static_assert(kGroups * kExchangeBytes <= kMinStages * kLeastStageBytes, "the exchange buffer must end inside the ring");
 
     // Two rings, not one of whole stages: the weights come from HBM and need more bytes in flight than the activation rows,
     // which come from L2.  No slack for an alignment: the rings end where the second CTA of the SM begins.
     uint8_t* tiles = smem_raw;                                                  // [w_stages][128][64] weights
-    uint8_t* xring = tiles + static_cast<size_t>(w_stages) * kABytes;           // [x_stages][BN][64] activation rows
-    GemmShared* sh = reinterpret_cast<GemmShared*>(xring + static_cast<size_t>(x_stages) * kBBytes);
+    uint8_t* xring = tiles + static_cast<size_t>(w_stages) * kABytes;           // [x_stages][x_rows][64] activation rows
+    GemmShared* sh = reinterpret_cast<GemmShared*>(xring + static_cast<size_t>(x_stages) * x_bytes);
     if ((smem_u32(smem_raw) & 1023u) != 0) {                // the swizzled tiles need 1024-byte alignment
         if (threadIdx.x == 0) atomicExch(status, ODB_ERR_CUDA);
         pdl_wait();
@@ -133,11 +135,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
             // first, then wait for the predecessor and fetch the activation tiles.
             const int pre = nkb < w_stages ? nkb : w_stages, xpre = nkb < x_stages ? nkb : x_stages;
             auto load_w = [&](int i, int st) {   // arms the barrier of k-block i for its weights and its activation rows
-                mbar_expect_tx(&sh->full[st], kStageBytes);
+                mbar_expect_tx(&sh->full[st], stage_bytes);
                 tma_load_3d(tiles + static_cast<size_t>(st) * kABytes, &tmap_w, &sh->full[st], 0, 0, wtile0 + i, kEvictFirst);
             };
             auto load_x = [&](int i, int st, int slot) {
-                tma_load_2d(xring + static_cast<size_t>(slot) * kBBytes, &tmap_x, &sh->full[st], (kb0 + i) * kBK, m0, kEvictLast);
+                tma_load_2d(xring + static_cast<size_t>(slot) * x_bytes, &tmap_x, &sh->full[st], (kb0 + i) * kBK, m0, kEvictLast);
             };
             for (int i = 0; i < pre; ++i) load_w(i, i);
             // and ask L2 for the weight tiles that follow, so that HBM keeps streaming while the
@@ -182,7 +184,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     } else if (warp == 1) {
         if (lane == 0) {
             // ---- MMA issuer ----
-            constexpr uint32_t idesc = make_instr_desc(kBM, BN);
+            const uint32_t idesc = make_instr_desc(kBM, x_rows);
             bool ok = true;
             int st = 0, slot = 0;
             uint32_t ph = 0;
@@ -191,7 +193,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(tiles + static_cast<size_t>(st) * kABytes);
-                const uint32_t b_addr = smem_u32(xring + static_cast<size_t>(slot) * kBBytes);
+                const uint32_t b_addr = smem_u32(xring + static_cast<size_t>(slot) * x_bytes);
 #pragma unroll
                 for (int k = 0; k < kBK / kUmmaK; ++k)
                     umma_bf16(tmem_acc, make_smem_desc(a_addr + k * kUmmaK * 2), make_smem_desc(b_addr + k * kUmmaK * 2), idesc,
@@ -486,8 +488,13 @@ int pick_bn(int M) {
 
 template <int BN, int EPI>
 cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
+    // The rows that there are, in steps of the MMA's sixteen: at 128 an SM takes in as many bytes of activation rows, again and
+    // again from L2, as of weights, and gate/up, 44 SMs of which have two tiles, is as long as that takes.  Layer steps, us, a full tile /
+    // the rows: d 4096, 96 rows 134.6 / 132.2, 87 rows 137.6 / 136.3; d 2048, two layers, 96 rows 152 / 147, 112 rows 155 / 150;
+    // d 1024 96 rows 114.6 / 111.1.  A fourth activation stage in the room of the third of 96 or less rows changes nothing.
+    const int x_rows = a.M < BN ? (a.M + 15) / 16 * 16 : BN;
     CUtensorMap tmx;
-    cudaError_t e = make_tmap_2d(&tmx, a.x, a.M, a.K, BN);
+    cudaError_t e = make_tmap_2d(&tmx, a.x, a.M, a.K, x_rows);
     if (e != cudaSuccess) return e;
     const int nkb_total = (a.K + kBK - 1) / kBK;
     const int nkb_per_split = (nkb_total + a.splits - 1) / a.splits;
@@ -497,11 +504,11 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
     // the LM head with 47 rows 310.7, 315.3, 315.7, 317.4.  At 64 and 128 rows the two CTAs leave less than a kilobyte of
     // the SM's shared memory: no successor's CTA is resident there, prefetching its weights, before one of them ends.
     constexpr int kWStages = BN == 128 ? 4 : 5, kXStages = BN == 128 ? 3 : 4;
-    constexpr int kWBytes = kBM * kBK * 2, kXBytes = BN * kBK * 2;
+    constexpr int kWBytes = kBM * kBK * 2, kXBytes = BN * kBK * 2;   // kXBytes: a full tile's
     static_assert(kWStages * kWBytes + kXStages * kXBytes + sizeof(GemmShared) <= 113 * 1024, "two CTAs share an SM");
     const int least = nkb_per_split < kMinStages ? kMinStages : nkb_per_split;
     const int w_stages = kWStages < least ? kWStages : least, x_stages = kXStages < least ? kXStages : least;
-    const size_t smem = static_cast<size_t>(w_stages) * kWBytes + static_cast<size_t>(x_stages) * kXBytes + sizeof(GemmShared);
+    const size_t smem = static_cast<size_t>(w_stages) * kWBytes + static_cast<size_t>(x_stages) * x_rows * (kBK * 2) + sizeof(GemmShared);
     static std::atomic<unsigned long long> attr_done{0};
     e = set_smem_limit_once(attr_done, gemm_kernel<BN, EPI>, 227 * 1024);
     if (e != cudaSuccess) return e;
@@ -513,7 +520,7 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
         l2_prefetch = env ? atoi(env) : 0;   // measured: prefetching into L2 slows the step down
     }
     return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(gemm_threads(BN, EPI)), smem, st, a.w.tile, tmx, a.partial, a.act_out, a.row_scale, a.conf,
-                         a.M, a.N, nkb_total, nkb_per_split, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
+                         a.M, a.N, nkb_total, nkb_per_split, x_rows, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
 }
 
 template <int EPI>

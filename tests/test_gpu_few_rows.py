@@ -36,3 +36,22 @@ def test_product_over_the_stage_rings(M, kb):
 ])
 def test_refresh_of_few_rows(shape, P, L):
     check_refresh(shape, P, L)
+
+
+@requires_gpu
+@pytest.mark.parametrize("M", [1, 16, 17, 48, 49, 80, 81, 96, 97, 112, 113, 128])    # around the steps of sixteen rows that are loaded
+@pytest.mark.parametrize("kb,splits", [(1, 1), (9, 1), (9, 2)])
+def test_product_of_as_many_rows_as_there_are(M, kb, splits):
+    E = engine()
+    N, K = 384, 64 * kb
+    xb, wb = _case(M, N, K, seed=M + K)
+    out = E.debug_gemm(E.bits_to_device(xb, "cuda"), E.bits_to_device(wb, "cuda"), splits).cpu().numpy().astype(np.float64)
+    xf, wf = synth.bf16_bits_to_f32(xb).astype(np.float64), synth.bf16_bits_to_f32(wb).astype(np.float64)
+    # fp32 accumulation of exact bf16 products, as in the other tests of this kernel
+    assert np.abs(out - xf @ wf.T).max() <= 2e-6 * (np.abs(xf) @ np.abs(wf).T).max()
+
+
+@requires_gpu
+@pytest.mark.parametrize("rows", [16, 17, 48, 80, 81, 96, 112, 113])
+def test_refresh_of_as_many_rows_as_there_are(rows):
+    check_refresh(HD64, rows - rows // 2, rows // 2)
