@@ -6,8 +6,9 @@
 //            cache, the refresh is what writes it); the output is final.
 //   step:    the rows of all copies of one block (a StepTile).  Key splits 0 .. ks-2 stream the cached
 //            K/V of the positions outside the block, visible to every row; the last split takes the fresh
-//            rows, one key tile per source copy: a row sees its own copy's tile and, in the decoded-share
-//            layout, the decoded rows of copy 0's tile.  Copies stay mutually invisible through this
+//            rows: the item's own rows as they lie, the copies one behind the other, and for an item without
+//            copy 0 in the decoded-share layout that copy's rows.  A row sees its own copy's rows and, in the
+//            decoded-share layout, the decoded ones of copy 0.  Copies stay mutually invisible through this
 //            per-row key mask, no mask tensor exists.  Outputs are per-split (max, sum, unnormalised
 //            output) partials merged in split order by the merge kernel of attention.cu.
 // No causal mask.  One pass over the key tiles of 64; per tile S = Q K^T is one 128 x 64 x HD tcgen05.mma group
@@ -244,8 +245,10 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // the first `valid` are keys.  src: 0 = fresh k / v rows of this forward, 1 = the K/V cache.
 struct KeyTile {
     int src, row0, v_row0, valid;
-    int copy;          // fresh tile of a step: the source copy; -1 otherwise (visible to every row)
+    int copy;          // fresh tile of a step: the source copy, or kPacked; -1 otherwise (visible to every row)
 };
+
+constexpr int kPacked = -2;   // consecutive rows of the item's own copies
 
 struct TcArgs {
     const QTile* qtiles;          // refresh work items
@@ -254,6 +257,7 @@ struct TcArgs {
     __nv_bfloat16* o;             // refresh: final output [M][H * HD]
     float* part_o; float* part_ml;   // step: split partials [ks][M][H][HD], [ks][M][H][2]
     int layer, n_layers, H, max_seq, M;
+    int any_order;                // step: the order of sums is free
 };
 
 // 128-byte pieces of a warp's 32 rows, turned in its patch of shared memory (16-byte chunks, XOR-swizzled) so that eight lanes
@@ -345,6 +349,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
     const bool single = STEP && ks == 1;                    // step without key splits
     int n_cached = 0;                                       // step: cached key tiles of this CTA (they come first)
     const StepTile* stp = nullptr;
+    int n_own = 0;                                          // step: packed tiles of the item's own rows; 0: a tile per source copy
     if constexpr (!STEP) {
         const QTile t = a.qtiles[blockIdx.x];
         q_row0 = t.q_row0; nq = t.nq; f0 = t.f0; NK = t.n0;
@@ -356,16 +361,29 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
         cA = stp->cA; cB0 = stp->cB0; cB1 = stp->cB1;
         nA_t = (cA + kTK - 1) / kTK;
         const int nct = nA_t + (cB1 - cB0 + kTK - 1) / kTK;
+        // Fresh keys in tiles of 64 rows as they lie, not a tile per copy (four copies of 32: two tiles, not four; eight of the
+        // decoded-share layout, 24 + 7 x 9 rows: two or three, not eight).  Where the order of sums has to stay, only with
+        // copies of 16, 32 or 64 rows: their keys then fall into the same groups of sixteen and halves of a tile.
+        fresh_split = z == ks - 1;                          // also the only one
+        int nf = 0;
+        if (fresh_split) {
+            const int n0 = stp->src_n[0];
+            const bool other0 = stp->stage2 && stp->slab_copy[0] != 0;   // copy 0 belongs to another item: its tile comes last
+            nf = stp->n_src;
+            if (a.any_order || (!stp->stage2 && n0 >= 16 && (n0 & (n0 - 1)) == 0)) {
+                n_own = (nq + kTK - 1) / kTK;
+                nf = n_own + (other0 ? 1 : 0);
+            }
+        }
         if (single) {
             // one CTA takes every key of the item: the cached tiles, then the fresh ones; its output is final
             n_cached = nct;
-            ntiles = nct + stp->n_src;
+            ntiles = nct + nf;
         } else {
-            fresh_split = z == ks - 1;
             const int tp = (nct + ks - 2) / (ks - 1);
             t_first = fresh_split ? 0 : z * tp;
             n_cached = fresh_split ? 0 : max(0, min(nct, t_first + tp) - t_first);
-            ntiles = fresh_split ? stp->n_src : n_cached;
+            ntiles = fresh_split ? nf : n_cached;
         }
         c_row = ((stp->seq * a.n_layers + a.layer) * 2 * a.H + head) * a.max_seq;   // K; V is H * max_seq rows further
     }
@@ -375,7 +393,11 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
         if constexpr (!STEP) {
             kt.src = 0; kt.row0 = f0 + i * kTK; kt.v_row0 = kt.row0; kt.valid = min(kTK, NK - i * kTK);
         } else if (i >= n_cached) {
-            const int f = i - n_cached;
+            const int fi = i - n_cached, f = n_own ? stp->n_src - 1 : fi;
+            if (fi < n_own) {
+                kt.src = 0; kt.row0 = q_row0 + fi * kTK; kt.v_row0 = kt.row0; kt.valid = min(kTK, nq - fi * kTK); kt.copy = kPacked;
+                return kt;
+            }
             kt.src = 0; kt.row0 = stp->src_row0[f]; kt.v_row0 = kt.row0; kt.valid = stp->src_n[f]; kt.copy = stp->src_copy[f];
         } else {
             const int j = t_first + i;
@@ -518,24 +540,38 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
         const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;   // this warp's TMEM lanes
         bool ok = true;
         int my_copy = -1, stage2 = 0;
-        if constexpr (STEP) {
+        int my_row0 = 0, my_n = 0;                                  // the rows of this row's copy
+        int n_copy0 = 0;                                            // rows of copy 0 at the front of the item
+        if (STEP && fresh_split) {                                  // the splits of cached keys need no copies
             stage2 = stp->stage2;
             const int grow = q_row0 + tid;
             for (int sl = 0; sl < stp->n_slabs; ++sl)
                 if (grow >= stp->slab_row0[sl] && grow < stp->slab_row0[sl] + stp->slab_n[sl]) my_copy = stp->slab_copy[sl];
+            if (my_copy >= 0) {
+                const int f = my_copy - stp->src_copy[0];           // an item's copies are consecutive
+                my_row0 = stp->src_row0[f];
+                my_n = stp->src_n[f];
+            }
+            if (stage2 && stp->src_copy[0] == 0) n_copy0 = stp->src_n[0];
         }
         // which of the tile's 64 keys this row sees (bit j = key j).  Every lane of a warp calls this for the
         // same tile: the branch that uses the ballots is uniform.
         auto tile_mask = [&](const KeyTile& kt) -> unsigned long long {
             const unsigned long long all = kt.valid >= 64 ? ~0ull : ((1ull << kt.valid) - 1ull);
-            if (kt.copy < 0) return all;                            // cached keys, or a refresh
+            if (kt.copy == -1) return all;                          // cached keys, or a refresh
             unsigned long long shared = 0ull;
             if constexpr (STEP) {
-                if (stage2 && kt.copy == 0) {                        // decoded rows of copy 0, shared with every copy
-                    const bool d0 = lane < kt.valid && (a.row_flags[kt.row0 + lane] & kRowDecoded);
-                    const bool d1 = lane + 32 < kt.valid && (a.row_flags[kt.row0 + lane + 32] & kRowDecoded);
+                // decoded rows of copy 0, shared with every copy
+                const int n_shared = kt.copy == kPacked ? min(kt.valid, q_row0 + n_copy0 - kt.row0) : stage2 && kt.copy == 0 ? kt.valid : 0;
+                if (n_shared > 0) {
+                    const bool d0 = lane < n_shared && (a.row_flags[kt.row0 + lane] & kRowDecoded);
+                    const bool d1 = lane + 32 < n_shared && (a.row_flags[kt.row0 + lane + 32] & kRowDecoded);
                     const unsigned lo = __ballot_sync(0xffffffffu, d0), hi = __ballot_sync(0xffffffffu, d1);
                     shared = (static_cast<unsigned long long>(hi) << 32 | lo) & all;
+                }
+                if (kt.copy == kPacked) {
+                    const int k0 = max(0, my_row0 - kt.row0), k1 = min(kt.valid, my_row0 + my_n - kt.row0);
+                    return k1 <= k0 ? shared : shared | ((k1 >= 64 ? ~0ull : (1ull << k1) - 1ull) & ~((1ull << k0) - 1ull));
                 }
             }
             return kt.copy == my_copy ? all : shared;
@@ -553,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
             const uint32_t ts = tmem_s + lane_base + b * kTK;
             const KeyTile kt = key_tile(tile);
             // a whole tile of cached keys (or of a refresh) is seen by every row
-            const bool full = kt.copy < 0 && kt.valid >= 64;
+            const bool full = kt.copy == -1 && kt.valid >= 64;
             const unsigned long long mask = full ? ~0ull : tile_mask(kt);
             ok = wait(&sh->s_full[b], round);
             ok = __all_sync(0xffffffffu, ok);
@@ -726,6 +762,7 @@ cudaError_t launch_step_attention_tc(const StepAttnArgs& a, size_t cache_rows, i
     TcArgs ta{};
     ta.stiles = a.tiles;
     ta.row_flags = a.row_flags;
+    ta.any_order = a.any_order;
     ta.o = a.o;                                            // written when there is no key split
     ta.part_o = a.part_o; ta.part_ml = a.part_ml;
     ta.layer = a.layer; ta.n_layers = a.n_layers; ta.H = a.H; ta.max_seq = a.max_seq; ta.M = a.M;

@@ -184,6 +184,7 @@ struct odb_session {
     // stream of the session's own (the caller's stream may be the default stream, which cannot record)
     struct ResidentGraph {
         StepShape shape;
+        int items;               // of the step attention (step_items)
         odb_decode_params p;
         bool dump_logits;
         cudaGraph_t graph;
@@ -532,6 +533,11 @@ struct LaunchScope {
     }
 };
 
+bool tc_attention() {   // ODB_ATTN_TC=0 in the environment: no tensor-core attention
+    static const bool on = !(getenv("ODB_ATTN_TC") && getenv("ODB_ATTN_TC")[0] == '0');
+    return on;
+}
+
 int bn_index(int M) { return M <= 32 ? 0 : M <= 64 ? 1 : 2; }
 
 // Whether a decode step of M rows runs as the persistent kernel (one cooperative launch for the whole forward).
@@ -743,7 +749,6 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
     int res_splits = 0;
     size_t res_stride = 0;
     static const int ks_env = getenv("ODB_ATTN_KS") ? atoi(getenv("ODB_ATTN_KS")) : 0;
-    static const bool tc_attention = !(getenv("ODB_ATTN_TC") && getenv("ODB_ATTN_TC")[0] == '0');
     int ks = attention_key_splits(n_tiles * H, hd, write_cache);
     if (ks_env > 0 && !write_cache) ks = ks_env;
     if (ks > 8) ks = 8;
@@ -830,11 +835,18 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
             // 112 / 109.  Below 32 items the two are as good as equal.
             static const int tc_step_env = getenv("ODB_ATTN_TC_STEP_MIN") ? atoi(getenv("ODB_ATTN_TC_STEP_MIN")) : 0;
             const int tc_step_min = tc_step_env > 0 ? tc_step_env : hd == 128 ? 1 : 32;
-            if (tc_attention && (hd == 128 || !same_order) && n_step_tiles * H >= tc_step_min) {
+            if (tc_attention() && (hd == 128 || !same_order) && n_step_tiles * H >= tc_step_min) {
                 const size_t cache_rows = static_cast<size_t>(c.max_batch) * c.n_layers * 2 * H * c.max_seq;
                 // with a work item for every CTA slot there is nothing to gain from key splits: one CTA per item takes
                 // the cached and the fresh keys and writes the final output (no partials, no merge kernel)
-                if (ks_env == 1 || (ks_env <= 0 && n_step_tiles * H >= 2 * 148)) sa.ksplit = 1;
+                if (ks_env == 1 || (ks_env <= 0 && n_step_tiles * H >= (same_order ? 2 * 148 : 96))) sa.ksplit = 1;
+                // Where the order of sums is free: no splits from 96 items, four from 32.  The last split takes the fresh keys alone, so
+                // two are one for the cached keys, and the partials' way through memory and the merge are 8 us.  us per step, before
+                // (148 / items, no splits from 296) / now: d 4096, 256 items 392.5 / 369, 128 241.3 / 234.4, 96 235.7 / 228.6, 64 (87 rows)
+                // 132.8 / 127.5, 64 (256 rows) 169 / 169; d 2048, two layers, 256 items 470 / 426, 128 items 305 / 293, 64 items 206 / 189;
+                // d 1024 256 items 257 / 230, 64 items 153 / 147.  None at 64 items: 135.9, 165.7, 199.8, 150.
+                else if (ks_env <= 0 && !same_order && n_step_tiles * H >= 32 && static_cast<size_t>(4) * M <= L.attn_rows) sa.ksplit = 4;
+                sa.any_order = same_order ? 0 : 1;
                 ODB_FWD(ODB_KIND_ATTENTION, launch_step_attention_tc(sa, cache_rows, status, st));
                 if (sa.ksplit > 1)
                     ODB_FWD(ODB_KIND_ATTENTION, launch_attention_combine(sa.part_o, sa.part_ml, o, M, H, hd, sa.ksplit, st));
@@ -842,7 +854,7 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
                 ODB_FWD(ODB_KIND_ATTENTION, launch_step_attention(sa, st));
                 if (seg_on()) ++s->launches[ODB_KIND_ATTENTION];
             }
-        } else if (write_cache && tc_attention && (hd == 128 || !same_order) && n_big_tiles * H >= (hd == 128 ? 1 : 74)) {
+        } else if (write_cache && tc_attention() && (hd == 128 || !same_order) && n_big_tiles * H >= (hd == 128 ? 1 : 74)) {
             // refresh: 128-row work items on the tcgen05 tensor cores, no key split.  Head dim 64, us per refresh of two layers, mma.sync
             // (64-row items, keys split to fill the chip) / tensor cores: d 1024, 128 items 226 / 195, 96 items 203 / 188, 64 items 163 / 158, 32
             // items 151.5 / 149.2; d 256, 512 items 426 / 327, 64 items 181 / 171, 16 items 116 / 121.  With fewer items than every
@@ -1007,9 +1019,22 @@ FirstRows first_rows(const odb_session* s) {
     return f;
 }
 
-// Work items of the multi-copy step attention for a step of this shape (0: the per-copy kernel is used)
+// Work items of the step attention of whole copies for a step of this shape (0: the per-copy kernel is used).
+// Several copies: always.  One copy: with an item for nearly every SM, whose 64-key tiles take the tensor cores as long as the per-copy
+// kernel's two warps of 32 rows, but run in one pass without key splits; only where the order of sums is free, with more than the
+// sixteen rows of one of those warps and 256 positions on average (192 items of 16 rows 137 / 142; 320 items, 136 positions +1.4 %).  us per step, per-copy
+// kernel / this: d 4096, 128 items 140.1 / 137.2, 192 items 177 / 167, 256 items of 64 rows 263 / 247, 512 items 275 / 264; 96 items 133 /
+// 135; d 2048, two layers, 128 items of 64 rows 254 / 233, 256 items 250 / 239.  Head dim 64 (d 1024): 256 items 174 / 160, 192 items
+// 154 / 159, 128 items 129 / 132.
 int step_items(const odb_session* s, const StepShape& sh) {
-    return (!sh.multi || static_cast<size_t>(2) * sh.rows > s->L.attn_rows) ? 0 : sh.step_tiles;
+    const odb_config& c = s->m->cfg;
+    if (static_cast<size_t>(2) * sh.rows > s->L.attn_rows) return 0;
+    if (sh.multi) return sh.step_tiles;
+    if (c.with_lm_head || c.tp_world > 1 || !tc_attention() || sh.step_tiles * c.n_heads < (c.head_dim == 128 ? 128 : 256)) return 0;
+    long long positions = 0;
+    for (const SeqState& st : s->mirror)
+        if (st.active && st.n_masked > 0) positions += st.T;
+    return sh.rows > 16 * sh.step_tiles && positions >= 256ll * sh.step_tiles ? sh.step_tiles : 0;
 }
 
 }  // namespace
@@ -1123,12 +1148,12 @@ int32_t odb_decode_block_resident(odb_session* s, const odb_decode_params* p, in
 
     odb_session::ResidentGraph* g = nullptr;
     for (auto& r : s->resident)
-        if (memcmp(&r.shape, &sh, sizeof(sh)) == 0 && memcmp(&r.p, p, sizeof(*p)) == 0 && r.dump_logits == s->dump_logits)
+        if (memcmp(&r.shape, &sh, sizeof(sh)) == 0 && r.items == step_items(s, sh) && memcmp(&r.p, p, sizeof(*p)) == 0 && r.dump_logits == s->dump_logits)
             g = &r;
     int32_t* loop_words = s->at<int32_t>(s->L.loop);   // [0] iterations done, [1] arrivals, [2] iteration limit
     if (!g) {
         odb_session::ResidentGraph r{};
-        r.shape = sh; r.p = *p; r.dump_logits = s->dump_logits;
+        r.shape = sh; r.items = step_items(s, sh); r.p = *p; r.dump_logits = s->dump_logits;
         ODB_CUDA(cudaGraphCreate(&r.graph, 0));
         LoopControl lc;
         cudaError_t e = cudaGraphConditionalHandleCreate(&lc.handle, r.graph, 1, cudaGraphCondAssignDefault);

@@ -432,6 +432,7 @@ struct StepAttnArgs {
     __nv_bfloat16* o;
     float* part_o; float* part_ml;        // split workspaces, merged by attention_combine
     int layer, n_layers, H, hd, max_seq, M, ksplit;   // ksplit >= 2: the last split handles the fresh keys
+    int any_order = 0;                    // 1: sums may come out in another order (tensor-core kernel: fresh keys packed into tiles)
     L2Prefetch pf;
 };
 cudaError_t launch_step_attention(const StepAttnArgs& a, cudaStream_t st);

@@ -1,6 +1,6 @@
-"""The tensor-core attention with head dim 64, where launches have enough work items for it: refreshes around the edges of the
-128-row items and 64-key tiles, steps of several copies with and without key splits, in both row layouts.  (Models without LM head: those with one stay on
-mma.sync.)"""
+"""The tensor-core attention where the order of sums is free (models without LM head) and launches have enough work items for it:
+refreshes with head dim 64 around the edges of the 128-row items and 64-key tiles, steps of several copies with and without key
+splits, in both row layouts, and batched steps of one copy."""
 import dataclasses
 import math
 
@@ -10,18 +10,18 @@ import torch
 
 import synth
 from gpu_common import bf16_bits_to_f64, engine, requires_gpu
-from test_gpu_many_rows import HD64
+from test_gpu_many_rows import HD64, HD128
 
 HEADS = 32
 SHAPE = dataclasses.replace(HD64, n_layers=1, n_heads=HEADS, d_model=64 * HEADS, d_ffn=256)
 
 
-def rows(sess, name):
-    return torch.from_numpy(bf16_bits_to_f64(sess.debug_read(name))).view(-1, HEADS, 64)
+def rows(sess, name, hd=64):
+    return torch.from_numpy(bf16_bits_to_f64(sess.debug_read(name))).view(-1, HEADS, hd)
 
 
 def check(o, q, keys, vals, visible=None):
-    s = torch.einsum("qhd,hkd->hqk", q, keys) / math.sqrt(64)
+    s = torch.einsum("qhd,hkd->hqk", q, keys) / math.sqrt(q.shape[-1])
     if visible is not None:
         s = s.masked_fill(~visible[None], -math.inf)
     want = torch.einsum("hqk,hkd->qhd", torch.softmax(s, -1), vals).numpy()
@@ -57,20 +57,26 @@ def test_refresh(lens):
 
 
 @requires_gpu
-@pytest.mark.parametrize("copies,decoded,block,batch", [
-    (4, 0, 32, 1),       # one item per head, seven cached key splits and the fresh one
-    (4, 5, 24, 2),       # 96 rows an item
-    (8, 22, 32, 3),      # the decoded-share layout: copies see copy 0's decoded rows
-    (4, 0, 64, 5),       # ten items per head: no key splits, the outputs are final
-    (8, 44, 64, 5),
+@pytest.mark.parametrize("copies,decoded,block,batch,hd", [
+    (4, 0, 32, 1, 64),       # one item per head: three cached key splits and the fresh one, two copies to a tile of fresh keys
+    (4, 5, 24, 2, 64),       # 96 rows an item, copies across the tiles' edges
+    (4, 0, 21, 1, 128),
+    (8, 16, 24, 2, 128),     # the decoded-share layout in two items a sequence: the second sees copy 0's decoded rows in a tile of their own
+    (8, 22, 32, 3, 64),      # in one
+    (4, 0, 64, 5, 64),       # ten items per head: no key splits, the outputs are final
+    (8, 44, 64, 5, 64),
+    (1, 3, 37, 4, 128),      # one copy
+    (1, 5, 17, 10, 64),
+    (1, 60, 64, 8, 64),
 ])
-def test_step_with_copies(copies, decoded, block, batch):
+def test_step_with_copies(copies, decoded, block, batch, hd):
     E = engine()
-    lens = [(101 + 37 * i, 200 - 19 * i) for i in range(batch)]
-    gm = E.Model.from_synth(SHAPE, seed=5, max_batch=batch, max_seq=max(p + n for p, n in lens), max_block=block, max_copies=8, with_lm_head=False)
+    lens = [(101 + 29 * (i % 4), max(block, 220 - 12 * i)) for i in range(batch)]
+    shape = SHAPE if hd == 64 else dataclasses.replace(HD128, n_layers=1, n_heads=HEADS, d_model=128 * HEADS, d_ffn=256)
+    gm = E.Model.from_synth(shape, seed=5, max_batch=batch, max_seq=max(p + n for p, n in lens), max_block=block, max_copies=8, with_lm_head=False)
     sess = E.Session(gm, poison=True)
     for i, (p, n) in enumerate(lens):
-        x = synth.sequence(5, i, p, n, SHAPE)
+        x = synth.sequence(5, i, p, n, shape)
         at = np.random.default_rng(i).permutation(block)[:decoded]
         x[p + at] = 7 + at                                             # ids other than [MASK] and [EOS]
         sess.set_sequence(i, x, p)
@@ -79,16 +85,17 @@ def test_step_with_copies(copies, decoded, block, batch):
     sess.unmask_accept(par, True)
     sess.block_decode_step(par)
     copy, pos = sess.debug_read("row_copy"), sess.debug_read("row_pos")
-    seq = np.cumsum((copy == 0) & (np.roll(copy, 1) != 0)) - 1          # the rows are in sequence order, copy 0 first
-    q, k, v, o = (rows(sess, x) for x in "qkvo")
+    # the rows are in sequence order, copy 0 first; consecutive blocks do not follow one another
+    seq = np.cumsum(np.r_[1, (copy[1:] == 0) & ((copy[:-1] != 0) | (pos[1:] != pos[:-1] + 1))]) - 1
+    q, k, v, o = (rows(sess, x, hd) for x in "qkvo")
     assert sess.status() == 0
-    kv = sess.kv.view(torch.bfloat16).view(batch, 2, HEADS, -1, 64).double().cpu()
+    kv = sess.kv.view(torch.bfloat16).view(batch, 2, HEADS, -1, hd).double().cpu()
     for i, (p, n) in enumerate(lens):
         r = np.flatnonzero(seq == i)
         x = sess.get_tokens(i)
         sees = copy[r][:, None] == copy[r][None, :]
         if len(r) < copies * block:
-            sees |= ((copy[r] == 0) & (x[pos[r]] != SHAPE.mask_id))[None, :]
+            sees |= ((copy[r] == 0) & (x[pos[r]] != shape.mask_id))[None, :]
         out = [j for j in range(p + n) if not p <= j < p + block]
         keys, vals = (torch.cat([kv[i, j][:, out], f[r].transpose(0, 1)], 1) for j, f in ((0, k), (1, v)))
         check(o[r], q[r], keys, vals, torch.cat([torch.ones(len(r), len(out), dtype=torch.bool), torch.from_numpy(sees)], 1))
