@@ -608,11 +608,15 @@ cudaError_t launch_rows(const GemmArgs& g, int n_tiles, cudaStream_t st) {
 // make 296 tiles, the rule of gemm_pick_splits (us per refresh, before / now; one layer at d 4096, two below): d 4096 900 rows, O 2 -> 1
 // splits 449 / 437, down 2 -> 1 449 / 437; 1200 rows, down 1 -> 4 601 / 573 (three 569); d 2048 512
 // rows, down 7 -> 4 240 / 232, 2000 rows, O 2 -> 1 528 / 506; d 1024 3600 rows, down 2 -> 1 369 / 353.
+// Beyond 2048 rows, or two rounds of unsplit tiles, none: the power cap makes the sums' traffic dearer than idle pairs.  By the two terms
+// alone d 4096, 4096 rows would take two for down (step of 16 sequences 1724, unsplit 1708), 3000 three (1269, 1227), 2600 two for O (1166,
+// 1142); d 2048, 2800 three for down (743, 725).
 int gemm_rows_splits(int M, int N, int K) {
     const int pairs = sm_pairs(), nkb = (K + kBK - 1) / kBK;
     const long long tiles = static_cast<long long>((N + 2 * kBM - 1) / (2 * kBM)) * ((M + 2 * kBM - 1) / (2 * kBM));
     int best = 1;
     double least = 0.;
+    if (M > 2048 || tiles > 2 * pairs) return 1;
     for (int sp = 1; sp <= kMaxKSplits && (sp == 1 || 8 * sp <= nkb); ++sp) {
         if (gemm_whole_splits(sp, nkb) != sp) continue;
         const long long items = tiles * sp;

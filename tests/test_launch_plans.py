@@ -34,7 +34,7 @@ def test_k_splits_of_a_projection(M, N, K, splits):
 
 @pytest.mark.parametrize("M,N,K,splits", [
     (768, 4096, 4096, 3), (900, 4096, 4096, 1), (900, 4096, 12288, 1), (1200, 4096, 12288, 4),   # rounds of the pairs against sums
-    (512, 2048, 5504, 4), (2000, 2048, 2048, 1), (25568, 4096, 12288, 1),
+    (512, 2048, 5504, 4), (2000, 2048, 2048, 1), (25568, 4096, 12288, 1), (2600, 4096, 4096, 1), (2800, 2048, 5504, 1),
     (200, 1024, 1024, 2), (200, 1024, 960, 1), (200, 256, 688, 1),                               # at least eight k-blocks each
     (129, 256, 1 << 17, 16),                                                                     # sixteen partials at most
 ])
