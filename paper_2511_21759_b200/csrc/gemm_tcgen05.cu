@@ -21,7 +21,7 @@
 // ODB_ERR_TIMEOUT, stops issuing work, releases its TMEM and exits.
 #include <stdlib.h>
 
-#include "odb_internal.cuh"
+#include "norm_common.cuh"
 #include "tcgen05_common.cuh"
 
 namespace odb {
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, EPI), 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
             float* __restrict__ partial, __nv_bfloat16* __restrict__ act_out, RowScale rs,
             ConfEpilogue ce, int M, int N, int nkb_total, int nkb_per_split, int x_rows, int w_stages, int x_stages,
-            int l2_prefetch, int* status, const __grid_constant__ PeerOut po) {
+            int l2_prefetch, int* status, const __grid_constant__ PeerOut po, const __grid_constant__ NormOut no) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr uint32_t kABytes = kBM * kBK * 2;
     // x_rows <= BN: activation rows that are loaded and multiplied; the accumulator's columns behind them are never stored
@@ -72,6 +72,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     constexpr uint32_t kTmemCols = BN;
     // the epilogues exchange values through the stage ring, which holds at least kMinStages stages
     constexpr int kGroups = epilogue_groups(BN, EPI), kGroupRows = BN / kGroups;
+    constexpr int kNormPitch = 132;                       // floats of a row in the norm's exchange buffer
+    static_assert(32 * kNormPitch * 4 <= kMinStages * kABytes, "the norm's exchange buffer must end inside the ring");
     constexpr uint32_t kExchangeBytes = EPI == EPI_SWIGLU ? 2 * 64 * (kGroupRows / 2 + 1) * 4 : EPI == EPI_CONF ? 32 * 129 * 4 : 0;
     static_assert(kGroups * kExchangeBytes <= kMinStages * kLeastStageBytes, "the exchange buffer must end inside the ring");
 
@@ -217,7 +219,49 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
         }
         const bool ok = nkb > 0 && mbar_wait(&sh->acc_full, 0, cta_abort, status);   // nkb == 0: empty K split
         if (ok) tc_fence_after();
-        if constexpr (EPI == EPI_PARTIAL) {
+        if (EPI == EPI_PARTIAL && BN == 32 && no.h) {
+            // The whole product of an unsplit projection, added to the residual stream here and normalised: what rmsnorm_kernel does, the
+            // sums of squares per 128 columns, which is what a warp of that kernel adds up.  One kernel less in the chain.
+            float* xch = reinterpret_cast<float*>(tiles);                       // [32 rows][kNormPitch]
+            const int col = n0 + lane * 4;                                      // of this lane's four, once a row is a warp's
+            const bool in = col < N;                                            // N % 16 == 0
+            const bool warp_ok = __all_sync(0xffffffffu, ok);
+            const float4 gain = in ? *reinterpret_cast<const float4*>(no.gain + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int c = g0 / 32; c < (g0 + kGroupRows) / 32 && m0 + c * 32 < M; ++c) {
+                if (warp_ok) {
+                    uint32_t v[32];
+                    __syncwarp();
+                    tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) xch[j * kNormPitch + q * 32 + lane] = __uint_as_float(v[j]);
+                }
+                group_sync();                                                   // every warp, whether or not its wait succeeded
+                float4 x[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int m = m0 + c * 32 + r * 4 + q;
+                    if (in && m < M && warp_ok) x[r] = *reinterpret_cast<const float4*>(no.h + static_cast<size_t>(m) * N + col);
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int row = r * 4 + q, m = m0 + c * 32 + row;
+                    float ss = 0.f;
+                    if (in && m < M && warp_ok) {
+                        const float4 t = *reinterpret_cast<const float4*>(xch + row * kNormPitch + lane * 4);
+                        x[r].x += t.x; x[r].y += t.y; x[r].z += t.z; x[r].w += t.w;
+                        *reinterpret_cast<float4*>(no.h + static_cast<size_t>(m) * N + col) = x[r];
+                        *reinterpret_cast<uint2*>(no.out + static_cast<size_t>(m) * N + col) =
+                            pack4_bf16(x[r].x * gain.x, x[r].y * gain.y, x[r].z * gain.z, x[r].w * gain.w);
+                        ss = squares4<true>(x[r]);
+                    }
+                    ss = warp_sum(ss);
+                    if (lane == 0 && m < M) no.ssq[static_cast<size_t>(m) * n_tiles + n_tile] = ss;
+                }
+                group_sync();                                                   // the buffer's next rows
+            }
+        } else if constexpr (EPI == EPI_PARTIAL) {
             const int n = n0 + q * 32 + lane;
             if (ok) {
                 const size_t split_off = static_cast<size_t>(split) * M * N;
@@ -520,7 +564,7 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
         l2_prefetch = env ? atoi(env) : 0;   // measured: prefetching into L2 slows the step down
     }
     return launch_kernel(gemm_kernel<BN, EPI>, grid, dim3(gemm_threads(BN, EPI)), smem, st, a.w.tile, tmx, a.partial, a.act_out, a.row_scale, a.conf,
-                         a.M, a.N, nkb_total, nkb_per_split, x_rows, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers);
+                         a.M, a.N, nkb_total, nkb_per_split, x_rows, w_stages, x_stages, pdl_enabled() ? l2_prefetch : 0, a.status, a.peers, a.norm);
 }
 
 template <int EPI>
@@ -644,7 +688,8 @@ int gemm_pick_splits(int M, int N, int K) {
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     const bool swiglu = a.act_out != nullptr;
     const int n_tiles = swiglu ? (a.N + 63) / 64 : (a.N + kBM - 1) / kBM;
-    if ((swiglu || a.conf.part || a.qkv || a.add_to) && a.splits != 1) return cudaErrorInvalidValue;
+    if ((swiglu || a.conf.part || a.qkv || a.add_to || a.norm.h) && a.splits != 1) return cudaErrorInvalidValue;
+    if (a.norm.h && (a.M > 32 || a.N > kNormOutCols || swiglu || a.conf.part || a.row_scale.ssq || a.peers.n)) return cudaErrorInvalidValue;
     if (use_pair(a.plan_rows > a.M ? a.plan_rows : a.M, n_tiles)) return launch_gemm_rows(a, n_tiles, st);
     if (a.qkv || a.add_to) return cudaErrorInvalidValue;   // epilogues of the many-row kernel only
     if (swiglu) return launch_epi<EPI_SWIGLU>(a, st);

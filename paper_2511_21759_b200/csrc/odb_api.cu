@@ -110,7 +110,8 @@ Layout make_layout(const odb_config& c) {
     L.step_tile_buf = take(sizeof(StepTile) * static_cast<size_t>(c.max_batch) * c.max_copies);
     L.h = take(4 * L.rows * d);
     L.a = take(2 * L.rows * d);
-    L.inv = take(4 * L.rows * ((d + kNormSliceCols - 1) / kNormSliceCols));   // sum-of-squares slices of the current RMSNorm
+    // sum-of-squares slices of the current RMSNorm; of 128 columns each where a projection's epilogue writes them (NormOut)
+    L.inv = take(4 * L.rows * (d <= kNormOutCols ? (d + 127) / 128 : (d + kNormSliceCols - 1) / kNormSliceCols));
     L.q = take(2 * L.rows * d);
     L.k = take(2 * L.rows * d);
     L.v = take(2 * L.rows * d);
@@ -690,6 +691,24 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
         ga.status = status;
         return launch_gemm(ga, st);
     };
+    // One tile of 32 rows, no K split: residual stream and next norm in the projection's epilogue, a kernel less.  Where the order of sums
+    // is free, up to twelve k-blocks go unsplit for it.  us per step of the tiny model (d 256, FFN 688, two layers), with the norm kernels /
+    // O alone / both: 8 rows 77.5 / 75.9 / 75.8, 16 rows 85.0 / 84.8 / 81.0, 32 rows 83.7 / 83.0 / 81.5; more rows, which four warps take one
+    // tile after another, 64 85 / 90 / 90, 128 102 / 110 / 118; d 1024, 32 rows, O and down unsplit for it (16 and 44 k-blocks) 99 / 104 / 119.
+    bool normed = false;                // `a` and `inv` hold the coming norm's results already
+    auto norm_fits = [&](int rows, int sp) { return R == 1 && rows <= 32 && sp == 1 && d <= kNormOutCols; };
+    auto gemm_norm = [&](const WeightMaps& w, const __nv_bfloat16* x, int K, const float* gain) {
+        GemmArgs ga;
+        ga.w = w;
+        ga.x = x;
+        ga.partial = nullptr;
+        ga.act_out = nullptr;
+        ga.norm.h = h; ga.norm.gain = gain; ga.norm.out = a; ga.norm.ssq = inv;
+        ga.M = M; ga.N = d; ga.K = K;
+        ga.splits = 1;
+        ga.status = status;
+        return launch_gemm(ga, st);
+    };
 #define ODB_LAUNCH(kind, call)          \
     do {                                \
         LaunchScope scope__(s, kind);   \
@@ -778,8 +797,9 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
     for (int l = 0; l < c.n_layers; ++l) {
         const L2Prefetch qkv_hint = hint_of(m->p_qkv[l], qkv_bytes, 0);
         if (l == 0) ODB_FWD(ODB_KIND_ELEMENTWISE, launch_first_norm(h, m->norm1[l], a, inv, M, d, first, qkv_hint, st));
-        else ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d, qkv_hint, st,
-                                                             res_wait));
+        else if (!normed) ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->norm1[l], a, inv, nullptr, M, d,
+                                                                          qkv_hint, st, res_wait));
+        inv_scale.slots = normed ? (d + 127) / 128 : (d + kNormSliceCols - 1) / kNormSliceCols;
         // Many rows: not split, whatever the pairs left idle; split sums cost the RoPE kernel and fp32 rows in memory.  us per refresh,
         // two splits / none, d 2048, two layers: 300 rows 245 / 232, 512 240 / 231, 768 277 / 258, d 1024 2000 rows 270 / 265;
         // d 4096, one layer, 300 rows 248 / 246.
@@ -895,11 +915,16 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
         } else if (sp == 1 && gemm_rows_usable(M, d)) {
             ODB_FWD(ODB_KIND_GEMM, gemm_add(m->w_o[l], o, da));
             o_sum = nullptr;
+        } else if (norm_fits(M, sp)) {
+            ODB_FWD(ODB_KIND_GEMM, gemm_norm(m->w_o[l], o, da, m->norm2[l]));
+            o_parts = 0;
         } else {
             ODB_FWD(ODB_KIND_GEMM, gemm(m->w_o[l], o, partial, M, d, da, sp));
         }
-        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, o_sum, o_parts, static_cast<size_t>(M) * d, m->norm2[l], a, inv, nullptr, M,
-                                                        d, hint_of(m->p_gu[l], gu_bytes, pf_bytes), st, o_wait));
+        if (o_parts > 0)
+            ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, o_sum, o_parts, static_cast<size_t>(M) * d, m->norm2[l], a, inv, nullptr, M,
+                                                            d, hint_of(m->p_gu[l], gu_bytes, pf_bytes), st, o_wait));
+        inv_scale.slots = o_parts == 0 ? (d + 127) / 128 : (d + kNormSliceCols - 1) / kNormSliceCols;
         tail = write_cache && l == c.n_layers - 1 && R == 1 && n_lm > 0 && n_lm < M && (one_seq || M > 128) &&
                gemm_tiled_rows(n_lm, d, M) < gemm_tiled_rows(M, d, M);
         const int rows = tail ? n_lm : M, plan_rows = tail ? M : 0;
@@ -941,6 +966,8 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
             ODB_FWD(ODB_KIND_GEMM, launch_gemm(ga, st));
         }
         sp = plan_splits(M, d, F, R > 1);
+        normed = false;
+        if (!same_order && norm_fits(M, 1) && F <= 12 * 64) sp = 1;
         if (R > 1) {
             ODB_FWD(ODB_KIND_GEMM, gemm(m->w_d[l], g, nullptr, M, d, F, sp, nullptr, 1));
             res_wait = end_exchange(1);
@@ -949,6 +976,10 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
         } else if (sp == 1 && gemm_rows_usable(M, d) && !(c.with_lm_head && l == c.n_layers - 1)) {
             ODB_FWD(ODB_KIND_GEMM, gemm_add(m->w_d[l], g, F));
             res = nullptr; res_splits = 0;
+        } else if (norm_fits(M, sp) && !(c.with_lm_head && l == c.n_layers - 1)) {
+            ODB_FWD(ODB_KIND_GEMM, gemm_norm(m->w_d[l], g, F, l + 1 < c.n_layers ? m->norm1[l + 1] : m->final_norm));
+            res = nullptr; res_splits = 0;
+            normed = true;
         } else {   // also in front of the LM head, whose norm reads the response rows only
             ODB_FWD(ODB_KIND_GEMM, gemm(m->w_d[l], g, partial, rows, d, F, sp, nullptr, -1, plan_rows));
             res = partial; res_splits = sp;
@@ -957,10 +988,11 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
     }
     if (!c.with_lm_head) {
         // fold the last projection into the residual stream (the normalised copy is not used)
-        ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->final_norm, a, inv, nullptr, M, d,
+        if (!normed) ODB_FWD(ODB_KIND_ELEMENTWISE, launch_rmsnorm(h, res, res_splits, res_stride, m->final_norm, a, inv, nullptr, M, d,
                                                         L2Prefetch{nullptr, 0}, st, res_wait));
         return ODB_OK;
     }
+    inv_scale.slots = (d + kNormSliceCols - 1) / kNormSliceCols;
     float* logits = s->at<float>(L.logits);
     int lm_tile0_local = 0, lm_rows_local = c.vocab;
     vocab_shard(c, c.tp_rank, &lm_tile0_local, &lm_rows_local);
