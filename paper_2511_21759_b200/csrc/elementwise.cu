@@ -153,9 +153,11 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* _
     for (int i = threadIdx.x; i < slots; i += 256) dst_ssq[to_row * slots + i] = ssq[row * slots + i];
 }
 
-// More than 64 rows: grid (rows, chunks), one thread per FOUR consecutive rotation pairs (float4 loads, 8-byte
-// stores; 1.5 x the throughput of the one-pair kernel below, which stays the faster one on the few rows of a
-// decode step, where the kernel is a single memory round trip on the dependency chain).  Sums the
+// More than 64 rows: grid (rows, chunks, q / k / v), one thread per FOUR consecutive rotation pairs of one of the three (float4
+// loads, 8-byte stores, four splits in flight; with all three in a thread two splits were, and the third waited for them: 8B
+// layer step of 128 rows 139.6 -> 137.0 us with that of four sequences 145.8 -> 144.1, d 2048 154 -> 151).  1.5 x the throughput of
+// the one-pair kernel below, which stays the faster one on the few rows of a
+// decode step, where the kernel is a single memory round trip on the dependency chain.  Sums the
 // QKV partials in split order, applies the RMSNorm scalar, rotates q and k (rotate-half pairing: element i
 // pairs with i + hd/2; angle = pos * theta^(-2i/hd), table precomputed), rounds to bf16 and writes the
 // row-major fresh q/k/v; in a refresh also the K/V cache [seq][layer][k|v][head][pos][hd].  hd/2 is a
@@ -164,67 +166,58 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* _
 __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 __device__ __forceinline__ void scale4(float4& a, float s) { a.x *= s; a.y *= s; a.z *= s; a.w *= s; }
 
-__global__ void qkv_rope_vec4_kernel(QkvRopeArgs a) {
+__global__ void __launch_bounds__(128) qkv_rope_vec4_kernel(QkvRopeArgs a) {
     pdl_launch_dependents();
     pdl_wait();
-    l2_prefetch_slice(a.pf, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    const int sec = blockIdx.z;                       // 0 q, 1 k, 2 v
+    l2_prefetch_slice(a.pf, (sec * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x * gridDim.y * 3);
     const int row = blockIdx.x;
     const int d = a.H * a.hd, half = a.hd / 2;
     const int pos = a.row_pos[row];
     const int seq = a.row_seq[row];
     const float* p0 = a.partial + static_cast<size_t>(row) * 3 * d;
     const float2* rope = a.rope + static_cast<size_t>(pos) * half;
-    __nv_bfloat16* ck = nullptr;
-    __nv_bfloat16* cv = nullptr;
-    if (a.cache) {
-        const size_t per_kv = static_cast<size_t>(a.H) * a.max_seq * a.hd;
-        ck = a.cache + (static_cast<size_t>(seq) * a.n_layers + a.layer) * 2 * per_kv;
-        cv = ck + per_kv;
-    }
     const float inv = row_scale_of(a.scale, row);   // scalar of the RMSNorm folded behind the projection
-    for (int t = (blockIdx.y * blockDim.x + threadIdx.x) * 4; t < d / 2; t += gridDim.y * blockDim.x * 4) {
-        const int head = t / half, i = t % half;
-        const int e0 = head * a.hd + i, e1 = e0 + half;
-        float4 q0 = {0.f, 0.f, 0.f, 0.f}, q1 = q0, k0 = q0, k1 = q0, v0 = q0, v1 = q0;
-        for (int sb = 0; sb < a.splits; sb += 2) {
-            float4 tt[2][6];
+    const int t = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
+    if (t >= d / 2) return;
+    const int head = t / half, i = t % half;
+    const int e0 = head * a.hd + i, e1 = e0 + half;
+    p0 += sec * d;
+    float4 x0 = {0.f, 0.f, 0.f, 0.f}, x1 = x0;
+    for (int sb = 0; sb < a.splits; sb += 4) {
+        float4 tt[4][2];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (sb + u < a.splits) {
-                    const float* p = p0 + static_cast<size_t>(sb + u) * a.pstride;
-                    tt[u][0] = *reinterpret_cast<const float4*>(p + e0); tt[u][1] = *reinterpret_cast<const float4*>(p + e1);
-                    tt[u][2] = *reinterpret_cast<const float4*>(p + d + e0); tt[u][3] = *reinterpret_cast<const float4*>(p + d + e1);
-                    tt[u][4] = *reinterpret_cast<const float4*>(p + 2 * d + e0); tt[u][5] = *reinterpret_cast<const float4*>(p + 2 * d + e1);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (sb + u < a.splits) {
-                    add4(q0, tt[u][0]); add4(q1, tt[u][1]); add4(k0, tt[u][2]); add4(k1, tt[u][3]); add4(v0, tt[u][4]); add4(v1, tt[u][5]);
-                }
+        for (int u = 0; u < 4; ++u) {
+            if (sb + u < a.splits) {
+                const float* p = p0 + static_cast<size_t>(sb + u) * a.pstride;
+                tt[u][0] = *reinterpret_cast<const float4*>(p + e0);
+                tt[u][1] = *reinterpret_cast<const float4*>(p + e1);
             }
         }
-        scale4(q0, inv); scale4(q1, inv); scale4(k0, inv); scale4(k1, inv); scale4(v0, inv); scale4(v1, inv);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sb + u < a.splits) { add4(x0, tt[u][0]); add4(x1, tt[u][1]); }
+    }
+    scale4(x0, inv); scale4(x1, inv);
+    uint2 r0, r1;
+    if (sec < 2) {
         const float4 c01 = *reinterpret_cast<const float4*>(rope + i);       // (cos, sin) of pairs i, i + 1
         const float4 c23 = *reinterpret_cast<const float4*>(rope + i + 2);   // and of pairs i + 2, i + 3
-        const uint2 rq0 = pack4_bf16(q0.x * c01.x - q1.x * c01.y, q0.y * c01.z - q1.y * c01.w, q0.z * c23.x - q1.z * c23.y,
-                                     q0.w * c23.z - q1.w * c23.w);
-        const uint2 rq1 = pack4_bf16(q1.x * c01.x + q0.x * c01.y, q1.y * c01.z + q0.y * c01.w, q1.z * c23.x + q0.z * c23.y,
-                                     q1.w * c23.z + q0.w * c23.w);
-        const uint2 rk0 = pack4_bf16(k0.x * c01.x - k1.x * c01.y, k0.y * c01.z - k1.y * c01.w, k0.z * c23.x - k1.z * c23.y,
-                                     k0.w * c23.z - k1.w * c23.w);
-        const uint2 rk1 = pack4_bf16(k1.x * c01.x + k0.x * c01.y, k1.y * c01.z + k0.y * c01.w, k1.z * c23.x + k0.z * c23.y,
-                                     k1.w * c23.z + k0.w * c23.w);
-        const uint2 rv0 = pack4_bf16(v0.x, v0.y, v0.z, v0.w), rv1 = pack4_bf16(v1.x, v1.y, v1.z, v1.w);
-        const size_t o = static_cast<size_t>(row) * d;
-        *reinterpret_cast<uint2*>(a.q + o + e0) = rq0; *reinterpret_cast<uint2*>(a.q + o + e1) = rq1;
-        *reinterpret_cast<uint2*>(a.k + o + e0) = rk0; *reinterpret_cast<uint2*>(a.k + o + e1) = rk1;
-        *reinterpret_cast<uint2*>(a.v + o + e0) = rv0; *reinterpret_cast<uint2*>(a.v + o + e1) = rv1;
-        if (ck) {
-            const size_t c = (static_cast<size_t>(head) * a.max_seq + pos) * a.hd;
-            *reinterpret_cast<uint2*>(ck + c + i) = rk0; *reinterpret_cast<uint2*>(ck + c + i + half) = rk1;
-            *reinterpret_cast<uint2*>(cv + c + i) = rv0; *reinterpret_cast<uint2*>(cv + c + i + half) = rv1;
-        }
+        r0 = pack4_bf16(x0.x * c01.x - x1.x * c01.y, x0.y * c01.z - x1.y * c01.w, x0.z * c23.x - x1.z * c23.y, x0.w * c23.z - x1.w * c23.w);
+        r1 = pack4_bf16(x1.x * c01.x + x0.x * c01.y, x1.y * c01.z + x0.y * c01.w, x1.z * c23.x + x0.z * c23.y, x1.w * c23.z + x0.w * c23.w);
+    } else {
+        r0 = pack4_bf16(x0.x, x0.y, x0.z, x0.w);
+        r1 = pack4_bf16(x1.x, x1.y, x1.z, x1.w);
+    }
+    __nv_bfloat16* out = (sec == 0 ? a.q : sec == 1 ? a.k : a.v) + static_cast<size_t>(row) * d;
+    *reinterpret_cast<uint2*>(out + e0) = r0;
+    *reinterpret_cast<uint2*>(out + e1) = r1;
+    if (a.cache && sec > 0) {
+        const size_t per_kv = static_cast<size_t>(a.H) * a.max_seq * a.hd;
+        __nv_bfloat16* cache = a.cache + ((static_cast<size_t>(seq) * a.n_layers + a.layer) * 2 + (sec - 1)) * per_kv +
+                               (static_cast<size_t>(head) * a.max_seq + pos) * a.hd;
+        *reinterpret_cast<uint2*>(cache + i) = r0;
+        *reinterpret_cast<uint2*>(cache + i + half) = r1;
     }
 }
 
@@ -520,7 +513,7 @@ cudaError_t launch_qkv_rope(const QkvRopeArgs& a, cudaStream_t st) {
     if (a.M > 64) {   // measured at 128 rows: 0.97 vs 1.09 ms of elementwise time per step; at 32 rows the one-pair kernel wins
         const int quads = a.H * a.hd / 8;             // four rotation pairs per thread
         const int threads = quads >= 128 ? 128 : 32 * ((quads + 31) / 32);
-        return launch_kernel(qkv_rope_vec4_kernel, dim3(a.M, (quads + threads - 1) / threads), dim3(threads), 0, st, a);
+        return launch_kernel(qkv_rope_vec4_kernel, dim3(a.M, (quads + threads - 1) / threads, 3), dim3(threads), 0, st, a);
     }
     const int pairs = a.H * a.hd / 2;
     return launch_kernel(qkv_rope_kernel, dim3(a.M, (pairs + 255) / 256), dim3(256), 0, st, a);
