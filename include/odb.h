@@ -61,9 +61,9 @@ enum {
 enum {
     ODB_KIND_GEMM = 0,        /* tcgen05 weight-streaming GEMMs (QKV, O, gate/up, down, LM head) */
     ODB_KIND_ATTENTION = 1,   /* block-query attention (+ its split merge) */
-    ODB_KIND_ELEMENTWISE = 2, /* embedding, RMSNorm, RoPE/cache scatter, SwiGLU */
+    ODB_KIND_ELEMENTWISE = 2, /* row tables with embedding and first RMSNorm, RMSNorm, RoPE/cache scatter, SwiGLU */
     ODB_KIND_CONFIDENCE = 3,  /* vocab-wide max / sum / argmax */
-    ODB_KIND_CONTROL = 4,     /* row tables, accept / jump / ALP */
+    ODB_KIND_CONTROL = 4,     /* accept / jump / ALP (and the row tables of a persistent step) */
     ODB_PROFILE_KINDS = 5
 };
 
