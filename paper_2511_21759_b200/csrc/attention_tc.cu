@@ -21,9 +21,10 @@
 //   (128 x HD x 64, V taken MN-major straight from its [key][dim] tile), O in TMEM.
 // Exact softmax (rescaling by powers of two changes no bit of a normal number).  Warp-specialised: warps 0..3 = softmax (one query row per thread),
 // warp 4 lane 0 = MMA issuer, warp 5 lane 0 = loader (TMA: boxes of 64 rows x 64 columns with the 128-byte
-// swizzle land in the canonical operand layout, one 64-column atom per 64 dims; rows past a buffer's
-// end read as zero, rows that are not keys of this work item are masked in the softmax and hold finite
-// values, the K/V cache being zeroed when a session is created).  The roles meet only through mbarriers.  Two CTAs share an SM
+// swizzle land in the canonical operand layout, one 64-column atom per 64 dims).  Rows of a tile behind its last key are other
+// sequences' or what a slot's earlier occupant left in the cache: the softmax masks their scores and sets their V to zero, for a
+// zero of P times an infinity or NaN there would be a NaN in this sequence's output.  (Copies of one sequence share their tiles: there a
+// row that is not finite reaches the block's other copies, as in a dense softmax under a mask.)  The roles meet only through mbarriers.  Two CTAs share an SM
 // (256 TMEM columns each, 112 or 64 KB of shared memory).  Every mbarrier wait is bounded; on expiry the CTA records
 // ODB_ERR_TIMEOUT, every role stops, the CTA releases its TMEM and exits.
 //
@@ -137,6 +138,7 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // The wait belongs to the instruction: as a statement of its own nothing would keep a use of the values behind it.
@@ -220,7 +222,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 
 struct alignas(8) TcShared {
     uint64_t q_full;       // Q tile landed                                   (loader -> MMA)
-    uint64_t full[6];      // K or V tile landed in the ring's slot            (loader -> MMA)
+    uint64_t full[6];      // K or V tile landed in the ring's slot            (loader -> MMA, softmax)
     uint64_t empty[6];     // the MMAs have read the slot                      (MMA -> loader)
     uint64_t s_full[3];    // S = Q K^T into S buffer i has completed          (MMA -> softmax)
     uint64_t p_full[3];    // P has taken its place                           (softmax -> MMA, 4 arrivals)
@@ -645,6 +647,22 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
             }
             tmem_st32(ts, hi);
             tmem_st32(ts + kTK / 2, lo);
+            if (kt.valid < kTK) {
+                // V's rows behind the keys, once it has landed.  i: V(tile)'s place in the loader's order.  The parity is not ambiguous:
+                // the load before it in this slot is a K or V tile multiplied before S(tile) was, the one behind it waits for P V(tile).
+                // us per call, without / with: 8B step of four sequences (three such tiles an item) 141.2 / 142.6, d 1024 refresh of two layers
+                // 177.8 / 178.9, 8B refresh of 768 rows equal.  Only non-finite rows, or the rest of a group of 16 alone (P V of the
+                // others left out), takes as long: it is the wait in front of P's arrival.  By the MMA warp's other lanes 142.0 and 180.4.
+                const int i = tile < ntiles - kFirst ? kFirst + 2 * tile + 1 : ntiles + tile, slot = i % kRing;
+                ok = __all_sync(0xffffffffu, wait(&sh->full[slot], static_cast<uint32_t>(i / kRing) & 1u));
+                if (!ok) break;
+                const uint32_t v = smem_u32(ring) + slot * kK;
+#pragma unroll
+                for (int at = 0; at < kAtoms; ++at)
+                    for (uint32_t off = kt.valid * 128 + tid * 16; off < kTK * 128; off += 128 * 16)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(v + at * kTK * 128 + off), "r"(0) : "memory");
+                proxy_fence();
+            }
             if (rescale) {                                           // warp-uniform; rows that keep their shift multiply by 1
                 // P V(tile - 1) has been added to O.  The parity is not ambiguous: S(tile) was issued behind P V(tile - kBufs), so
                 // P V(tile - 3), which the same barrier counts, has completed; P V(tile + 1) cannot have, it is behind this P.
