@@ -619,7 +619,19 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
                 if (M_row != -INFINITY) factor = exp2f(M_row - M_new);   // an exact power of two
                 M_row = M_new;
             }
-            const bool rescale = __any_sync(0xffffffffu, factor != 1.0f);
+            // The exponentials take a score's exact product with scale_log2, the shift comes from the rounded one: from 2^22 on they lie up
+            // to 0.25 and more apart (from 2^31 on P overflowed or vanished), and the scores are rounded first.
+            const bool far = fabsf(mt_log2) >= 0x1p22f && mt_log2 != -INFINITY;
+            bool rescale = false;
+            uint64_t mult2 = scale2;
+            if (__any_sync(0xffffffffu, factor != 1.0f || far)) {
+                rescale = __any_sync(0xffffffffu, factor != 1.0f);
+                if (__any_sync(0xffffffffu, far)) {
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) sv[j] = __float_as_uint(__uint_as_float(sv[j]) * scale_log2);
+                    mult2 = pack2f(1.0f, 1.0f);
+                }
+            }
             const float m_log2 = M_row == -INFINITY ? 0.f : M_row;   // a row that has seen no key: every P is 0
             const uint64_t shift2 = pack2f(-m_log2, -m_log2);
             float l_tile = 0.f;
@@ -630,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_tc_kernel(const __grid_
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
                     // arguments are <= kSlack: the hardware exponential needs no range handling (far below zero it returns 0)
-                    const float2 x = unpack2f(fma2(pack2u(sv[half * 32 + 2 * u], sv[half * 32 + 2 * u + 1]), scale2, shift2));
+                    const float2 x = unpack2f(fma2(pack2u(sv[half * 32 + 2 * u], sv[half * 32 + 2 * u + 1]), mult2, shift2));
                     const float p0 = ex2_approx(x.x), p1 = ex2_approx(x.y);
                     const uint64_t p = pack2f(p0, p1);
                     sum = add2(sum, p);

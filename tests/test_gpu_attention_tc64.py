@@ -100,3 +100,36 @@ def test_step_with_copies(copies, decoded, block, batch, hd):
         keys, vals = (torch.cat([kv[i, j][:, out], f[r].transpose(0, 1)], 1) for j, f in ((0, k), (1, v)))
         check(o[r], q[r], keys, vals, torch.cat([torch.ones(len(r), len(out), dtype=torch.bool), torch.from_numpy(sees)], 1))
     sess.close(); gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("log2_gain", [11, 17, 40])     # scores of about 2^22, 2^34 and 2^80 in the log2 domain
+def test_refresh_with_scores_far_beyond_the_range_of_their_differences(hd, log2_gain):
+    """Every row sees one key alone: its output is that key's v."""
+    E = engine()
+    shape = SHAPE if hd == 64 else dataclasses.replace(HD128, n_layers=1, n_heads=HEADS, d_model=128 * HEADS, d_ffn=256)
+    p, n = 257, 64
+    kw = dict(max_batch=1, max_seq=p + n, max_block=16, max_copies=1, with_lm_head=False)
+    gm = E.Model.from_synth(shape, seed=5, **kw)
+    t = dict(gm.t)
+    gm.close()
+    t["norm1"] = [t["norm1"][0] * 2.0 ** log2_gain]
+    gm = E.Model(shape, t, **kw)
+    sess = E.Session(gm, poison=True)
+    sess.set_sequence(0, synth.sequence(5, 0, p, n, shape), p)
+    sess.refresh_prefill(E.DecodeParams(block_len=16), 0)
+    q, k, v, o = (rows(sess, x, hd) for x in "qkvo")
+    assert sess.status() == 0
+    s = torch.einsum("qhd,khd->hqk", q, k)
+    # fp32 sums of hd products: 2^-24 of the sum of their sizes for each addition
+    off = hd * 2.0 ** -23 * torch.einsum("qhd,khd->hqk", q.abs(), k.abs()).amax(-1)
+    best = s.topk(2, -1)
+    # the runner-up's weight vanishes where even the computed scores lie 2^5 apart in the log2 domain
+    alone = best.values[..., 0] - best.values[..., 1] > 2 * off + 2.0 ** 5 * math.sqrt(hd) / math.log2(math.e)
+    assert alone.double().mean() > 0.9
+    want = torch.gather(v.transpose(0, 1), 1, best.indices[..., :1].expand(-1, -1, hd)).transpose(0, 1)
+    seen = alone.T[..., None].expand_as(o)
+    # one P alone, in two bf16 terms: 2^-16, then the rounding to bf16; the others' P below 2^-32 together with 320 of them
+    assert ((o - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -20 * want.abs().amax())[seen].all()
+    sess.close(); gm.close()
