@@ -237,6 +237,7 @@ int32_t odb_block_decode_step(odb_session* s, const odb_decode_params* p);
  * (after_refresh = 1: copy 0 only, preceded by the [EOS] scan / truncation when p->alp) or
  * step (after_refresh = 0), commits tokens, ranks the next speculative candidates.
  * results: host array [max_batch].  Waits for the stream.
+ * A row without a greedy token (its logits are all NaN) counts as [EOS] with confidence 0.
  * With a model built without LM head (layer microbenchmark) there are no confidences: the call
  * commits nothing and only lays out the copies of the next step (speculative fills: the first
  * masked positions with token id 0), so masks_left never decreases. */

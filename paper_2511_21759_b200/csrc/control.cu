@@ -95,12 +95,16 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         }
         __syncthreads();
     }
+    // A row whose logits are all NaN has no greedy token (0x7fffffff, with confidence 1 / 0), and one of a forward whose waits ran out
+    // whatever was there: committed or filled in, they would be rows far behind the embedding.  They count as [EOS] with confidence 0.
+    auto gather = [&](int cp, int i, int r) {
+        const int t = c.tok[r];
+        const bool known = t >= 0 && t < c.vocab;
+        conf[cp][i] = known ? c.conf[r] : 0.f;
+        tok[cp][i] = known ? t : eos_id;
+    };
     if (!dry && after_refresh) {
-        for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) {
-            const int r = st->lm_row0 + (s + i - st->lm_s);
-            conf[0][i] = c.conf[r];
-            tok[0][i] = c.tok[r];
-        }
+        for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) gather(0, i, st->lm_row0 + (s + i - st->lm_s));
     } else if (!dry) {
         for (int i = threadIdx.x; i < n_copies * kMaxBlock; i += blockDim.x) {
             conf[i / kMaxBlock][i % kMaxBlock] = -1.f;
@@ -109,11 +113,7 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         __syncthreads();
         for (int cp = 0; cp < n_copies; ++cp) {
             const int r0 = st->copy_row0[cp], r1 = r0 + st->copy_nrows[cp];
-            for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-                const int i = c.row_pos[r] - s;
-                conf[cp][i] = c.conf[r];
-                tok[cp][i] = c.tok[r];
-            }
+            for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) gather(cp, c.row_pos[r] - s, r);
         }
     }
     __syncthreads();

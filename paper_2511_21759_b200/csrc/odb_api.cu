@@ -394,6 +394,7 @@ int32_t odb_session_create(odb_model* m, void* kv, size_t kv_bytes, void* worksp
     cb.big_tiles = s->at<QTile>(L.big_tile_buf);
     cb.host_state = s->pinned_state; cb.host_results = s->pinned_results; cb.host_status = s->pinned_status;
     cb.status = s->at<int>(L.status);
+    cb.vocab = c.vocab;
     cb.step_tiles = s->at<StepTile>(L.step_tile_buf);
     cb.conf = s->at<float>(L.conf);
     cb.tok = s->at<int32_t>(L.tok);

@@ -527,6 +527,7 @@ struct ControlBuffers {
     // reads them after synchronising the stream, no copy is enqueued
     SeqState* host_state; odb_result* host_results; int* host_status;
     const int* status;        // device status word
+    int32_t vocab;
 };
 // Where the rows of a forward come from: a block step of every active sequence with masked positions, or a refresh of the active
 // ones whose block_index is not negative.

@@ -89,3 +89,45 @@ def test_other_sequences_keep_their_bits(hd, heads, copies, block, batch):
     for clean, other in zip(got["reused", False], got["reused", True]):
         assert all(np.isfinite(a).all() and np.array_equal(a, b) for a, b in zip(clean, other))
     gm.close()
+
+
+@requires_gpu
+@pytest.mark.parametrize("copies,resident", [(1, False), (4, False), (4, True), (8, False)])
+def test_a_row_without_a_greedy_token_counts_as_eos(copies, resident):
+    """A NaN prompt: every response row's logits are NaN after a refresh.  What is committed stays inside the vocabulary and the block
+    ends; the other sequences decode what they decode without it."""
+    E = engine()
+    shape = dataclasses.replace(HD128, n_heads=4, d_model=512, d_ffn=256)
+    lens, block, bad = [(40, 32), (37, 32), (50, 24)], 16, 1
+    gm = model(E, shape, True, max_batch=3, max_seq=80, max_block=block, max_copies=8)
+    par = E.DecodeParams(block_len=block, n_copies=copies, alp=False)
+    done = {}
+    for nan in (False, True):
+        sess = E.Session(gm, poison=True)
+        for i, (p, n) in enumerate(lens):
+            x = ids(i, p, n, shape)
+            if nan and i == bad:
+                x[:p] = NAN_ID
+            sess.set_sequence(i, x, p)
+        sess.refresh_prefill(par, 0)
+        assert np.isnan(sess.debug_read("hidden")).any() == nan
+        res = sess.unmask_accept(par, True)
+        if nan:
+            r = res[bad]
+            assert [(r.accepted_pos[j], r.accepted_tok[j]) for j in range(r.n_accepted)] == [(37, shape.eos_id)]
+        left = max(r.masks_left for r in res)
+        for _ in range(block):
+            if left == 0:
+                break
+            if resident:
+                left = max(r.masks_left for r in sess.decode_block_resident(par, block)[-1])
+            else:
+                sess.block_decode_step(par)
+                left = max(r.masks_left for r in sess.unmask_accept(par, False))
+        assert left == 0 and sess.status() == 0
+        done[nan] = [sess.get_tokens(i)[: p + block] for i, (p, n) in enumerate(lens)]
+        sess.close()
+    gm.close()
+    assert ((done[True][bad] >= 0) & (done[True][bad] < shape.vocab) & (done[True][bad] != shape.mask_id)).all()
+    for i in (0, 2):
+        assert np.array_equal(done[False][i], done[True][i])
