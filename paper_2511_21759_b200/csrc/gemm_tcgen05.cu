@@ -220,46 +220,43 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
         const bool ok = nkb > 0 && mbar_wait(&sh->acc_full, 0, cta_abort, status);   // nkb == 0: empty K split
         if (ok) tc_fence_after();
         if (EPI == EPI_PARTIAL && BN == 32 && no.h) {
-            // The whole product of an unsplit projection, added to the residual stream here and normalised: what rmsnorm_kernel does, the
-            // sums of squares per 128 columns, which is what a warp of that kernel adds up.  One kernel less in the chain.
+            // The whole product of an unsplit projection of one row tile, added to the residual stream here and normalised: what
+            // rmsnorm_kernel does, the sums of squares per 128 columns, which is what a warp of that kernel adds up.  One kernel less in
+            // the chain.
             float* xch = reinterpret_cast<float*>(tiles);                       // [32 rows][kNormPitch]
             const int col = n0 + lane * 4;                                      // of this lane's four, once a row is a warp's
             const bool in = col < N;                                            // N % 16 == 0
             const bool warp_ok = __all_sync(0xffffffffu, ok);
             const float4 gain = in ? *reinterpret_cast<const float4*>(no.gain + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-            for (int c = g0 / 32; c < (g0 + kGroupRows) / 32 && m0 + c * 32 < M; ++c) {
-                if (warp_ok) {
-                    uint32_t v[32];
-                    __syncwarp();
-                    tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (warp_ok) {
+                uint32_t v[32];
+                __syncwarp();
+                tmem_ld32(tmem_acc + (static_cast<uint32_t>(q * 32) << 16), v);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) xch[j * kNormPitch + q * 32 + lane] = __uint_as_float(v[j]);
-                }
-                group_sync();                                                   // every warp, whether or not its wait succeeded
-                float4 x[8];
+                for (int j = 0; j < 32; ++j) xch[j * kNormPitch + q * 32 + lane] = __uint_as_float(v[j]);
+            }
+            group_sync();                                                       // every warp, whether or not its wait succeeded
+            float4 x[8];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const int m = m0 + c * 32 + r * 4 + q;
-                    if (in && m < M && warp_ok) x[r] = *reinterpret_cast<const float4*>(no.h + static_cast<size_t>(m) * N + col);
-                }
+            for (int r = 0; r < 8; ++r) {
+                const int m = r * 4 + q;
+                if (in && m < M && warp_ok) x[r] = *reinterpret_cast<const float4*>(no.h + static_cast<size_t>(m) * N + col);
+            }
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const int row = r * 4 + q, m = m0 + c * 32 + row;
-                    float ss = 0.f;
-                    if (in && m < M && warp_ok) {
-                        const float4 t = *reinterpret_cast<const float4*>(xch + row * kNormPitch + lane * 4);
-                        x[r].x += t.x; x[r].y += t.y; x[r].z += t.z; x[r].w += t.w;
-                        *reinterpret_cast<float4*>(no.h + static_cast<size_t>(m) * N + col) = x[r];
-                        *reinterpret_cast<uint2*>(no.out + static_cast<size_t>(m) * N + col) =
-                            pack4_bf16(x[r].x * gain.x, x[r].y * gain.y, x[r].z * gain.z, x[r].w * gain.w);
-                        ss = squares4<true>(x[r]);
-                    }
-                    ss = warp_sum(ss);
-                    if (lane == 0 && m < M) no.ssq[static_cast<size_t>(m) * n_tiles + n_tile] = ss;
+            for (int r = 0; r < 8; ++r) {
+                const int m = r * 4 + q;
+                float ss = 0.f;
+                if (in && m < M && warp_ok) {
+                    const float4 t = *reinterpret_cast<const float4*>(xch + m * kNormPitch + lane * 4);
+                    x[r].x += t.x; x[r].y += t.y; x[r].z += t.z; x[r].w += t.w;
+                    *reinterpret_cast<float4*>(no.h + static_cast<size_t>(m) * N + col) = x[r];
+                    *reinterpret_cast<uint2*>(no.out + static_cast<size_t>(m) * N + col) =
+                        pack4_bf16(x[r].x * gain.x, x[r].y * gain.y, x[r].z * gain.z, x[r].w * gain.w);
+                    ss = squares4<true>(x[r]);
                 }
-                group_sync();                                                   // the buffer's next rows
+                ss = warp_sum(ss);
+                if (lane == 0 && m < M) no.ssq[static_cast<size_t>(m) * n_tiles + n_tile] = ss;
             }
         } else if constexpr (EPI == EPI_PARTIAL) {
             const int n = n0 + q * 32 + lane;
