@@ -393,6 +393,21 @@ __global__ void __launch_bounds__(256) swiglu_combine_kernel(const float* __rest
     g[static_cast<size_t>(m) * F + f] = __float2bfloat16_rn(gate / (1.0f + expf(-gate)) * up);
 }
 
+// silu_product against the division it stands for, gate by gate: out[0] counts the bit patterns whose results differ, out[1] is
+// the lowest of them.
+__global__ void __launch_bounds__(256) silu_bits_kernel(unsigned long long* out) {
+    for (unsigned long long b = static_cast<unsigned long long>(blockIdx.x) * blockDim.x + threadIdx.x; b < (1ull << 32);
+         b += static_cast<unsigned long long>(gridDim.x) * blockDim.x) {
+        const float gate[1] = {__uint_as_float(static_cast<unsigned>(b))}, up[1] = {1.0f};
+        float got[1];
+        silu_product(gate, up, got);
+        if (__float_as_uint(got[0]) != __float_as_uint(gate[0] / (1.0f + expf(-gate[0])) * up[0])) {
+            atomicAdd(out, 1ull);
+            atomicMin(out + 1, b);
+        }
+    }
+}
+
 // Read-only streaming probe: every thread reads 16-byte vectors grid-stride over the buffer and folds them into
 // one word, written out only if it has an (impossible) value, so that the loads cannot be removed.
 __global__ void __launch_bounds__(512) read_stream_kernel(const uint4* __restrict__ src, size_t n_vec, unsigned int* sink) {
@@ -474,6 +489,11 @@ cudaError_t launch_bulk_read_stream(const void* src, size_t bytes, int grid, int
 cudaError_t launch_swiglu_combine(const float* partial, int splits, size_t pstride, const RowScale& scale, __nv_bfloat16* g,
                                   int M, int F, cudaStream_t st) {
     return launch_kernel(swiglu_combine_kernel, dim3(M, (F + 255) / 256), dim3(256), 0, st, partial, splits, pstride, scale, g, F);
+}
+
+cudaError_t launch_silu_bits(unsigned long long* out, cudaStream_t st) {
+    silu_bits_kernel<<<148 * 8, 256, 0, st>>>(out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink, int grid, cudaStream_t st) {

@@ -387,6 +387,8 @@ cudaError_t launch_reduce_partials(const float* partial, int splits, size_t stri
                                    cudaStream_t st);
 
 // read-only streaming kernel over `bytes` of src (a multiple of 16), `grid` blocks of 512 threads
+// test: over all 2^32 gates, out[0] += those whose silu_product is not the plain quotient's bits, out[1] = min(out[1], the lowest)
+cudaError_t launch_silu_bits(unsigned long long* out, cudaStream_t st);
 cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned int* sink, int grid, cudaStream_t st);
 // bulk-copy ring probe; *streamed = the bytes one launch reads (whole chunks per CTA); `status` is a device word
 cudaError_t launch_bulk_read_stream(const void* src, size_t bytes, int grid, int* status, size_t* streamed, cudaStream_t st);

@@ -1,5 +1,6 @@
 """SwiGLU in the gate/up projections' epilogues over the whole range of gates: where e^-gate overflows, where the quotient is too small
 for a normal number, and large positive ones.  Every row is the same known vector, every gate a chosen value."""
+import ctypes
 import dataclasses
 
 import numpy as np
@@ -45,3 +46,15 @@ def test_swiglu_over_all_gates(rows):
     assert (np.abs(got[:, :F] - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -23 * (1 + np.abs(want))).all()
     assert (got[:, F:] == 0).all()
     sess.close(); gm.close()
+
+
+@requires_gpu
+def test_the_corrected_quotient_is_the_division_bit_for_bit():
+    """All 2^32 gates, NaN and infinities among them: -0 alone, whose quotient loses its sign, differs."""
+    engine()
+    from paper_2511_21759_b200 import binding as B
+    f = B.lib()._ZN3odb16launch_silu_bitsEPyP11CUstream_st
+    f.argtypes, f.restype = (ctypes.c_void_p, ctypes.c_void_p), ctypes.c_int
+    out = torch.tensor([0, (1 << 63) - 1], dtype=torch.int64, device="cuda")
+    assert f(out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    assert out.tolist() == [1, 1 << 31]
