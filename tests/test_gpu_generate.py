@@ -195,6 +195,50 @@ def test_resident_loop_equals_call_by_call(copies):
 
 
 @requires_gpu
+@pytest.mark.parametrize("copies", [1, 4])
+def test_resident_loop_without_lm_head_equals_call_by_call(copies):
+    """Nothing is committed and the step's shape stays, but lengths choose the attention of a batched step of one copy: of eight
+    sequences with 32 heads of 64, 256 positions on average and more take the tensor-core kernel (no merge), fewer the per-copy kernel
+    with two key splits.  One session goes from short ones to long ones and back, through recorded loops and call by call."""
+    E = engine()
+    shape = dataclasses.replace(synth.TINY, n_layers=2, n_heads=32, d_model=2048, d_ffn=256, vocab=512, mask_id=511, eos_id=510)
+    Bk, iters = 24, 3
+    gm = E.Model.from_synth(shape, seed=2, max_batch=8, max_seq=360, max_block=Bk, max_copies=4, with_lm_head=False)
+    params = E.DecodeParams(block_len=Bk, n_copies=copies)
+    runs = []
+    for resident in (False, True):
+        sess = E.Session(gm, poison=True)
+        out = []
+        for short in (True, False, True):
+            for i in range(8):
+                P, n = (90 + i, 100) if short else (200 + 3 * i, 130)
+                sess.set_sequence(i, synth.sequence(2, i, P, n, shape), P)
+            sess.refresh_prefill(params, 0)
+            sess.unmask_accept(params, True)
+            sess.profile_read()
+            if resident:
+                log = sess.decode_block_resident(params, iters)
+            else:
+                log = []
+                for _ in range(iters):
+                    sess.block_decode_step(params)
+                    log.append(sess.unmask_accept(params, False))
+            assert len(log) == iters and all(r.masks_left == Bk and r.n_accepted == 0 for it in log for r in it)
+            out.append((sess.debug_read("hidden"), sess.debug_read("row_tok"), sess.debug_read("row_pos"), [bytes(r) for it in log for r in it],
+                        sess.profile_read()[1]))
+        assert sess.status() == 0
+        sess.close()
+        runs.append(out)
+    gm.close()
+    for one, loop in zip(*runs):
+        assert np.isfinite(one[0]).all() and all(np.array_equal(a, b) for a, b in zip(one[:3], loop[:3]))
+        assert one[3] == loop[3] and one[4] == loop[4]
+    if copies == 1:
+        assert [r[4]["attention"] for r in runs[1]] == [2 * 2 * iters, 2 * iters, 2 * 2 * iters]
+    assert np.array_equal(runs[1][0][0], runs[1][2][0])
+
+
+@requires_gpu
 def test_resident_loop_respects_max_iters_and_state():
     E = engine()
     from paper_2511_21759_b200 import binding as B
