@@ -542,8 +542,9 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t st) {
     // Two CTAs per SM, up to 112 KB of stages each.  Weight x activation stages at 128 rows, us per layer step of 87 rows: 3 x 3
     // (whole stages) 158.6, 4 x 3 155.5, 4 x 2 162; at 32 rows 4 x 2 131, 5 x 2 127, 5 x 4 121.5, 6 x 4 122.8; at 64 rows 5 x 4
     // 127.9, 4 x 4 126.2, 5 x 3 127.4, 4 x 3 126.5 (d 2048, two layers: 136.3, 136.1, 133.2, 132.6), but a request through
-    // the LM head with 47 rows 310.7, 315.3, 315.7, 317.4.  At 64 and 128 rows the two CTAs leave less than a kilobyte of
-    // the SM's shared memory: no successor's CTA is resident there, prefetching its weights, before one of them ends.
+    // the LM head with 47 rows 310.7, 315.3, 315.7, 317.4.  With whole tiles of 64 and 128 rows the two CTAs leave less
+    // than a kilobyte of the SM's shared memory, with fewer rows up to 40 KB: either way no successor's CTA that needs the rings is
+    // resident there, prefetching its weights, before one of them ends.
     constexpr int kWStages = BN == 128 ? 4 : 5, kXStages = BN == 128 ? 3 : 4;
     constexpr int kWBytes = kBM * kBK * 2, kXBytes = BN * kBK * 2;   // kXBytes: a full tile's
     static_assert(kWStages * kWBytes + kXStages * kXBytes + sizeof(GemmShared) <= 113 * 1024, "two CTAs share an SM");

@@ -369,9 +369,8 @@ int32_t odb_session_create(odb_model* m, void* kv, size_t kv_bytes, void* worksp
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->ws + L.rope_t, rope_t.data(), rope_t.size() * sizeof(float2), cudaMemcpyHostToDevice, s->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->ws + L.state, 0, L.x - L.state, s->st);   // state, results, status
-    // The tensor-core attention loads whole 64-row boxes: cache rows that are not keys of a work item are masked
-    // in its softmax but still enter the P V product with weight zero, so they must hold finite values; the
-    // q / k / v and output rows past a forward's last row are never read (the tensor maps end at that row).
+    // Zero, so that no result could depend on what the caller's buffer held.  (The attention kernels leave out cache rows that are no
+    // keys; q / k / v and output rows past a forward's last row are never read, the tensor maps end at that row.)
     if (e == cudaSuccess) e = cudaMemsetAsync(kv, 0, odb_kv_bytes(&c), s->st);
     if (e == cudaSuccess && c.tp_world > 1)
         e = cudaMemsetAsync(s->ws + L.tp_flags, 0, sizeof(unsigned int) * kTpFlagWords, s->st);
@@ -694,8 +693,12 @@ int32_t forward(odb_session* s, const FirstRows& first, int M, int n_lm, int n_t
     };
     // One tile of 32 rows, no K split: residual stream and next norm in the projection's epilogue, a kernel less.  Where the order of sums
     // is free, up to twelve k-blocks go unsplit for it.  us per step of the tiny model (d 256, FFN 688, two layers), with the norm kernels /
-    // O alone / both: 8 rows 77.5 / 75.9 / 75.8, 16 rows 85.0 / 84.8 / 81.0, 32 rows 83.7 / 83.0 / 81.5; more rows, which four warps take one
+    // O alone / both: 8 rows 77.5 / 75.9 / 75.8, 16 rows 85.0 / 84.8 / 81.0, 32 rows 83.7 / 83.0 / 81.5; more rows, which four warps took one
     // tile after another, 64 85 / 90 / 90, 128 102 / 110 / 118; d 1024, 32 rows, O and down unsplit for it (16 and 44 k-blocks) 99 / 104 / 119.
+    // Down alone by its k-blocks, with K splits and the norm kernel / unsplit with the norm, 8 rows and 32, two layers: d 256, 8 k-blocks 77.1 /
+    // 75.7 and 82.4 / 78.8, 11 78.5 / 78.3 and 83.8 / 81.4, 12 78.1 / 78.4 and 83.1 / 81.6, 16 79.4 / 80.4 and 83.0 / 83.8; d 512, 11 88.2 / 87.8 and
+    // 91.6 / 91.2, 12 87.8 / 89.1 and 91.0 / 91.9, 16 87.9 / 90.7 and 91.4 / 94.3; d 1024, 11 100.7 / 97.3 and 99.6 / 98.6, 12 99.5 / 97.4 and 99.3 /
+    // 99.3, 16 99.6 / 99.7 and 99.2 / 102.0 (single values move by 1 %).
     bool normed = false;                // `a` and `inv` hold the coming norm's results already
     auto norm_fits = [&](int rows, int sp) { return R == 1 && rows <= 32 && sp == 1 && d <= kNormOutCols; };
     auto gemm_norm = [&](const WeightMaps& w, const __nv_bfloat16* x, int K, const float* gain) {
@@ -1058,7 +1061,9 @@ FirstRows first_rows(const odb_session* s) {
 // sixteen rows of one of those warps and 256 positions on average (192 items of 16 rows 137 / 142; 320 items, 136 positions +1.4 %).  us per step, per-copy
 // kernel / this: d 4096, 128 items 140.1 / 137.2, 192 items 177 / 167, 256 items of 64 rows 263 / 247, 512 items 275 / 264; 96 items 133 /
 // 135; d 2048, two layers, 128 items of 64 rows 254 / 233, 256 items 250 / 239.  Head dim 64 (d 1024): 256 items 174 / 160, 192 items
-// 154 / 159, 128 items 129 / 132.
+// 154 / 159, 128 items 129 / 132.  No upper bound on the lengths: the per-copy kernel's two splits are slower at every one, although each has
+// half of the tiles.  One layer, 300 / 600 / 1200 / 2400 positions: d 4096, 128 items per-copy 137.5 / 145.2 / 160.9 / 188.4, this 134.7 / 140.2 /
+// 155.5 / 170.7, 160 items at 2400 246 / 204; d 1024, 256 items of 64 91.4 / 98.8 / 121.2 / 148.3, 88.5 / 93.7 / 106.8 / 128.7.
 int step_items(const odb_session* s, const StepShape& sh) {
     const odb_config& c = s->m->cfg;
     if (static_cast<size_t>(2) * sh.rows > s->L.attn_rows) return 0;

@@ -332,7 +332,6 @@ struct WeightMaps {
     CUtensorMap tile, half;
 };
 
-// Weight-streaming GEMM: partial[s][M][N] (fp32) = x[M][K_s] * w[N][K_s]^T for each K split s.
 // h non-null: an unsplit projection of at most 32 rows adds its product to the residual stream h and writes the next RMSNorm's operand
 // bf16(h * gain) and the sums of h^2 per 128 columns, ssq [M][N / 128].  Up to kNormOutCols columns: there the sums, added up in order,
 // are the norm kernels' bit for bit.
@@ -343,6 +342,7 @@ struct NormOut {
     float* ssq = nullptr;
 };
 constexpr int kNormOutCols = kNormSliceCols;
+// Weight-streaming GEMM: partial[s][M][N] (fp32) = x[M][K_s] * w[N][K_s]^T for each K split s.
 struct GemmArgs {
     WeightMaps w;
     const void* x;         // bf16 [M][K] device
@@ -354,7 +354,7 @@ struct GemmArgs {
     const QkvRopeArgs* qkv = nullptr;   // non-null: QKV projection whose epilogue applies RoPE and writes q / k / v and the cache
                                         // (many rows, gemm_rows_usable); splits == 1
     float* add_to = nullptr;            // non-null: the product is added to fp32 [M][N] in place (likewise)
-    NormOut norm;
+    NormOut norm;                       // norm.h non-null: product and next norm in the epilogue (at most 32 rows); splits == 1
     PeerOut peers;                      // peers.n > 0: the partial tiles (or statistics) go to these buffers instead
     int M, N, K;
     int plan_rows = 0;     // > M: the kernel is the one a projection of this many rows takes (its sums, bit for bit); 0: M
