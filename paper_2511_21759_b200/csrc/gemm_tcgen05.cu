@@ -103,7 +103,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     // packed weights: tile (n-tile, k-block) is the contiguous 16 KB chunk number n_tile * nkb_total + k_block
     const int wtile0 = n_tile * nkb_total + kb0;
 
-    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < w_stages; ++i) {
             mbar_init(&sh->full[i], 1);
@@ -128,6 +127,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // behind the TMEM allocation, as in every kernel that makes one (at entry instead: steps of all kinds 0 to 0.4 % faster)
+    pdl_launch_dependents();
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {

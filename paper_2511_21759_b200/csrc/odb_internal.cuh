@@ -37,7 +37,9 @@ cudaError_t set_smem_limit_once(std::atomic<unsigned long long>& done, Kernel ke
 //   - the first kernel: its blocks that write the row and tile tables behind those stores.  That
 //     alone makes the tables complete before any later kernel of the chain starts, and lets the
 //     attention read its work items (and a step the K/V cache) before its own wait;
-//   - kernels that allocate TMEM for CTA pairs, and the tensor-core attention: behind the allocation;
+//   - kernels that allocate TMEM: behind the allocation.  A CTA that waits for columns then only waits for kernels in front of its
+//     own.  (Let go at entry, a projection's CTA could find all columns taken by two CTAs of the attention behind it, which fit beside
+//     it with head dim 64 and wait for it.)
 //   - many-row QKV projections with the RoPE epilogue: not at all (gemm_rows.cu).
 // ---------------------------------------------------------------------------------------
 
