@@ -96,12 +96,14 @@ __device__ void accept_body(const ControlBuffers& c, const odb_decode_params& p,
         __syncthreads();
     }
     // A row whose logits are all NaN has no greedy token (0x7fffffff, with confidence 1 / 0), and one of a forward whose waits ran out
-    // whatever was there: committed or filled in, they would be rows far behind the embedding.  They count as [EOS] with confidence 0.
+    // whatever was there: committed or filled in, they would be rows far behind the embedding.  They count as [EOS] with confidence 0 (as another
+    // id where that is [MASK], which committed would stay masked).
+    const int none = eos_id != mask_id ? eos_id : mask_id == 0 ? 1 : 0;
     auto gather = [&](int cp, int i, int r) {
         const int t = c.tok[r];
         const bool known = t >= 0 && t < c.vocab;
         conf[cp][i] = known ? c.conf[r] : 0.f;
-        tok[cp][i] = known ? t : eos_id;
+        tok[cp][i] = known ? t : none;
     };
     if (!dry && after_refresh) {
         for (int i = threadIdx.x; i < st->e - s; i += blockDim.x) gather(0, i, st->lm_row0 + (s + i - st->lm_s));
