@@ -123,12 +123,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ 
                      "r"(kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        pdl_launch_dependents();   // behind the allocation, as in every kernel that makes one; one thread's word is the CTA's
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // behind the TMEM allocation, as in every kernel that makes one (at entry instead: steps of all kinds 0 to 0.4 % faster)
-    pdl_launch_dependents();
     const uint32_t tmem_acc = sh->tmem_base;
 
     if (warp == 0) {
